@@ -145,6 +145,15 @@ def _unit(v):
     return v / v.norm(dim=1, keepdim=True).clamp_min(1e-300)
 
 
+def _rotations(quat):
+    """Rotation matrices (k x 3 x 3) of k quaternions."""
+    w, x, y, z = _unit(quat).unbind(1)
+    return torch.stack([1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y),
+                        2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x),
+                        2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)],
+                       1).view(-1, 3, 3)
+
+
 def _torus(g, n, R=1.0, r=0.3):
     u = 2 * math.pi * _rand(g, 2 * n + 256)
     v = 2 * math.pi * _rand(g, 2 * n + 256)
@@ -184,7 +193,7 @@ def _cloud(shape, n, seed):
         which = torch.randint(0, 40, (n,), generator=g, device=DEV)
         cen = _rand(g, 40, 3)
         axes = 0.04 + 0.11 * _rand(g, 40, 3)
-        rot = torch.linalg.qr(_randn(g, 40, 3, 3))[0]
+        rot = _rotations(_randn(g, 40, 4))
         u = _unit(_randn(g, n, 3))
         pe, ne = axes[which] * u, _unit(u / axes[which])
         pt, nt = _torus(g, n)
