@@ -547,9 +547,7 @@ __device__ __forceinline__ void pair_fold(GrpAcc &A, const PairSums &T, f2 three
 // plain FP32 sums folded into the compensated totals
 // With CLAMP the records are four 16-byte words, the fourth (d2, d2, 0, 0)
 // (d2 = 0 for far nodes), and the terms are those of the modified kernel.
-// UNROLL: records in flight per loop trip (8 in the list evaluation, 3 %
-// faster than 4 there; 4 in the on-the-fly group walk, which spills at 8).
-template <bool GRAD, bool SCREENED, bool CLAMP = false, int UNROLL = 4>
+template <bool GRAD, bool SCREENED, bool CLAMP = false>
 __device__ __forceinline__ void grp_flush(GrpAcc &A, const float4 *buf, int cnt, f2 qx, f2 qy,
                                           f2 qz, const EvalParams &ep)
 {
@@ -562,7 +560,7 @@ __device__ __forceinline__ void grp_flush(GrpAcc &A, const float4 *buf, int cnt,
     PairSums T;
     pair_zero(T);
     const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(buf);
-#pragma unroll UNROLL
+#pragma unroll 4
     for (int j = 0; j < cnt; ++j) {
         const ulonglong2 r0 = rec[RW * j + 0];
         const ulonglong2 r1 = rec[RW * j + 1];
@@ -818,10 +816,14 @@ __global__ void __launch_bounds__(32 * kListWarps)
 // Evaluation of the lists.  A group's terms are one stream of 48-byte
 // records: its far nodes (frec) followed by its near leaves' points (the
 // source records; every leaf is read whole -- the last, partial leaf runs
-// into the padding records, which have zero moment and add exactly 0).  The
-// warp copies the stream in chunks of 64 records into shared memory with
-// cp.async (each lane two records, six 16-byte copies), double-buffered so
-// that the copy of chunk k+1 overlaps the packed evaluation of chunk k.
+// into the padding records, which have zero moment and add exactly 0).  One
+// warp evaluates one work item (below) of the stream for the group's 64
+// queries.  The plain FP32 sums of every kLstChunk = 64 records are folded
+// into two-sum pairs.
+//
+// The warp is split into P parts of 32 / P lanes.  Every part holds all 64
+// queries (P pairs per lane) and takes every P-th chunk of the stream; the
+// parts' (hi, lo) sums are added at the end of the item.
 constexpr int kLstChunk = 64;
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
@@ -833,22 +835,6 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-
-// global address of record r of the group's stream (point records of
-// NEAR_W 16-byte words: 3, or 4 with the modified kernel's radius)
-template <int NEAR_W = 3>
-__device__ __forceinline__ const float4 *lst_record(int64_t r, int64_t nf, int64_t f0, int64_t e0,
-                                                    const int *__restrict__ far_ids,
-                                                    const int *__restrict__ near_ids,
-                                                    const float4 *__restrict__ frec,
-                                                    const float4 *__restrict__ src4, int64_t nleaf,
-                                                    int lg_bucket)
-{
-    if (r < nf) return frec + 3 * (int64_t)far_ids[f0 + r];
-    const int64_t rr = r - nf;  // leaves hold 2^lg_bucket points
-    const int64_t leaf = near_ids[e0 + (rr >> lg_bucket)];
-    return src4 + NEAR_W * (((leaf - nleaf) << lg_bucket) + (rr & ((1 << lg_bucket) - 1)));
-}
 
 // Work items: a group's stream is cut into items of at most kItemRecords
 // records so that no warp is left with a group whose box straddles a jump
@@ -876,6 +862,19 @@ __global__ void k_tree_item_table(const int64_t *__restrict__ item_off, int64_t 
         items[i] = make_int2((int)g, (int)(j * kItemRecords));
 }
 
+// Why the warp is split.  On sm_103a a packed f32x2 instruction takes two
+// issue slots and every other instruction one (measured: 16 packed
+// operations 34.2 cycles alone, 38.9 with four MUFU beside them, 41.8 with
+// eight ALU), so a term costs 2 x 16 (w) or 2 x 27 (w and grad) slots, its
+// four MUFU, and its share of the loads and the loop.  With P = 2 a staged
+// record's three shared loads serve two query pairs a lane instead of one.
+// Screened, a 1M-point blob (2.7e10 terms at the corners): corners 15.13
+// -> 14.13 ms, points 10.91 -> 10.50 ms; 4M points: corners 50.8 -> 47.9,
+// points 23.5 -> 22.5 ms.  P = 4 needs 96 or more registers for w and is
+// 4-6 % slower than P = 2; P = 1 in the same form is 3 % slower.
+constexpr int kLstParts = 2;
+constexpr int kLstUnroll = 4;   // records per loop trip (2 and 8: 2-6 % slower)
+
 template <bool GRAD, bool SCREENED, bool CLAMP = false>
 __device__ __forceinline__ void eval_lists_body(
     const float4 *__restrict__ q, int64_t m, const float4 *__restrict__ frec,
@@ -884,93 +883,186 @@ __device__ __forceinline__ void eval_lists_body(
     const int64_t *__restrict__ near_off, const int *__restrict__ near_ids,
     const int2 *__restrict__ items, int64_t nitems, const EvalParams &ep,
     float *__restrict__ ipart, unsigned long long *__restrict__ counter, const IterState *st,
-    int64_t bid)
+    int64_t it)
 {
     if (st && cloud_idle(st)) return;  // finished cloud of a batch
+    constexpr int P = kLstParts;
     constexpr int NA = GRAD ? 4 : 1;
-    constexpr int RW = CLAMP ? 4 : 3;  // 16-byte words per staged record
-    __shared__ float4 buf_all[kGrpWarps][2][kLstChunk * RW];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t it = bid * kGrpWarps + wid;
+    constexpr int RW = CLAMP ? 4 : 3;           // 16-byte words per staged record
+    constexpr int LPS = 32 / P;                 // lanes of a part
+    constexpr int SREC = kLstChunk / P;         // records of a part per stage
+    constexpr int PAD = 4;                      // the parts' records in different banks
+    constexpr int PSTR = SREC * RW + PAD;       // 16-byte words between the parts' buffers
+    __shared__ float4 buf_all[2][P * PSTR];
     if (it >= nitems) return;
+    const int lane = threadIdx.x;
+    const int part = lane / LPS, sl = lane % LPS;
     const int2 item = items[it];
     const int64_t g = item.x;
     const int64_t q0 = g * kGrpQ;
-    const GrpQueries G = grp_queries(q, m, q0, lane);
-    const f2 qx = pk(G.qa.x, G.qb.x), qy = pk(G.qa.y, G.qb.y), qz = pk(G.qa.z, G.qb.z);
-    const f2 zero = pk(0.f, 0.f);
-    GrpAcc A;
-    A.hw = A.lw = A.hgx = A.lgx = A.hgy = A.lgy = A.hgz = A.lgz = zero;
+    f2 qx[P], qy[P], qz[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const float4 a = q[min(q0 + sl + LPS * (2 * p), m - 1)];
+        const float4 b = q[min(q0 + sl + LPS * (2 * p + 1), m - 1)];
+        qx[p] = pk(a.x, b.x);
+        qy[p] = pk(a.y, b.y);
+        qz[p] = pk(a.z, b.z);
+    }
+    GrpAcc A[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+        A[p].hw = A[p].lw = A[p].hgx = A[p].lgx = A[p].hgy = A[p].lgy = A[p].hgz = A[p].lgz = 0ull;
     const float4 *src4 = reinterpret_cast<const float4 *>(src);
-    const int64_t nleaf = (int64_t)1 << levels;
-    const int64_t f0 = far_off[g], nf = far_off[g + 1] - f0;
-    const int64_t e0 = near_off[g], ne = near_off[g + 1] - e0;
+    const int nleaf = 1 << levels;
+    const int64_t f0 = far_off[g], e0 = near_off[g];
+    const int nf = (int)(far_off[g + 1] - f0), ne = (int)(near_off[g + 1] - e0);
     const int lg_bucket = __ffs(bucket) - 1;  // leaf sizes are powers of two
-    const int64_t r_begin = item.y;
-    const int64_t r_end = min(r_begin + kItemRecords, nf + ne * bucket);
-    const int64_t nchunks = (r_end - r_begin + kLstChunk - 1) / kLstChunk;
-    auto issue = [&](int64_t chunk) {
-        float4 *b = buf_all[wid][chunk & 1];
-        const int64_t r0 = r_begin + chunk * kLstChunk;
+    const int *fi = far_ids + f0, *ni = near_ids + e0;
+    const int r_begin = item.y;
+    const int total = (int)min((int64_t)kItemRecords,
+                               (int64_t)nf + (int64_t)ne * bucket - r_begin);
+    const int nsuper = (total + P * kLstChunk - 1) / (P * kLstChunk);
+    const int tail = min(total - (nsuper - 1) * P * kLstChunk, kLstChunk);
+    const int nstages = total > 0 ? (nsuper - 1) * P + (tail + SREC - 1) / SREC : 0;
+    // this lane's two records of a stage: the list entry (loaded one stage
+    // before its copy is issued), then the copy
+    auto rec_of = [&](int stage, int h) {
+        const int t = lane + 32 * h;
+        return (stage / P) * (P * kLstChunk) + (t / SREC) * kLstChunk + (stage % P) * SREC +
+               t % SREC;
+    };
+    int id[2] = {0, 0};
+    auto fetch = [&](int stage) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = rec_of(stage, h);
+            if (r < total) {
+                const int s = r_begin + r;
+                id[h] = s < nf ? __ldg(fi + s) : __ldg(ni + ((s - nf) >> lg_bucket));
+            }
+        }
+    };
+    auto issue = [&](int stage) {
+        float4 *bb = buf_all[stage & 1];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int t = lane + 32 * h;
-            if (r0 + t < r_end) {
-                const float4 *from = lst_record<RW>(r0 + t, nf, f0, e0, far_ids, near_ids, frec,
-                                                    src4, nleaf, lg_bucket);
-                cp_async16(b + RW * t + 0, from + 0);
-                cp_async16(b + RW * t + 1, from + 1);
-                cp_async16(b + RW * t + 2, from + 2);
+            const int r = rec_of(stage, h);
+            float4 *b = bb + (t / SREC) * PSTR + RW * (t % SREC);
+            if (r < total) {
+                const int s = r_begin + r;
+                const bool far = s < nf;
+                const float4 *from =
+                    far ? frec + 3 * (int64_t)id[h]
+                        : src4 + RW * ((((int64_t)id[h] - nleaf) << lg_bucket) +
+                                       ((s - nf) & (bucket - 1)));
+                cp_async16(b + 0, from + 0);
+                cp_async16(b + 1, from + 1);
+                cp_async16(b + 2, from + 2);
                 if (CLAMP) {
-                    if (r0 + t < nf) b[RW * t + 3] = make_float4(0.f, 0.f, 0.f, 0.f);  // far node
-                    else cp_async16(b + RW * t + 3, from + 3);
+                    if (far) b[3] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    else cp_async16(b + 3, from + 3);
                 }
             }
         }
         cp_async_commit();
     };
-    if (nchunks > 0) issue(0);
-    for (int64_t k = 0; k < nchunks; ++k) {
-        if (k + 1 < nchunks) issue(k + 1);
-        else cp_async_commit();  // an empty group keeps the wait count uniform
-        cp_async_wait1();        // chunk k has landed (this lane's copies)
-        __syncwarp();            // ... and every lane's
-        const int cnt = (int)min((int64_t)kLstChunk, r_end - r_begin - k * kLstChunk);
-        grp_flush<GRAD, SCREENED, CLAMP, 8>(A, buf_all[wid][k & 1], cnt, qx, qy, qz, ep);
-        __syncwarp();  // buffer k & 1 is reused by the copy of chunk k + 2
+    const f2 eps2 = pk(ep.eps2, ep.eps2);
+    const f2 three = pk(3.f, 3.f);
+    const f2 sv = pk(ep.s, ep.s);
+    const f2 s2v = pk(ep.s2, ep.s2);
+    const f2 nl2e = pk(ep.nl2e_s, ep.nl2e_s);
+    PairSums T[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) pair_zero(T[p]);
+    if (nstages > 0) {
+        fetch(0);
+        issue(0);
+        fetch(1);
     }
-    // the item's sums: ipart[((it * NA + a) * 2 + h) * 64 + slot]
+    for (int k = 0; k < nstages; ++k) {
+        if (k + 1 < nstages) {
+            issue(k + 1);
+            fetch(k + 2);
+        } else {
+            cp_async_commit();  // an empty group keeps the wait count uniform
+        }
+        cp_async_wait1();  // stage k has landed (this lane's copies)
+        __syncwarp();      // ... and every lane's
+        const int left = total - ((k / P) * (P * kLstChunk) + part * kLstChunk + (k % P) * SREC);
+        const int cnt = min(left, SREC);
+        const ulonglong2 *rec =
+            reinterpret_cast<const ulonglong2 *>(buf_all[k & 1] + part * PSTR);
+#pragma unroll kLstUnroll
+        for (int j = 0; j < cnt; ++j) {
+            const ulonglong2 r0 = rec[RW * j + 0];
+            const ulonglong2 r1 = rec[RW * j + 1];
+            const ulonglong2 r2v = rec[RW * j + 2];
+            const f2 d2c = CLAMP ? rec[RW * j + 3].x : 0ull;
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                pair_term<GRAD, SCREENED, CLAMP>(T[p], r0, r1, r2v, d2c, qx[p], qy[p], qz[p], eps2,
+                                                 three, sv, s2v, nl2e);
+        }
+        __syncwarp();  // buffer k & 1 is reused by the copy of stage k + 2
+        if (k % P == P - 1 || k + 1 == nstages) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                pair_fold<GRAD, SCREENED>(A[p], T[p], three);
+                pair_zero(T[p]);
+            }
+        }
+    }
+    // the item's sums: ipart[((it * NA + a) * 2 + h) * 64 + slot], the parts
+    // added in order
     float *o = ipart + it * (int64_t)NA * 2 * kGrpQ;
 #pragma unroll
-    for (int h2 = 0; h2 < 2; ++h2) {
-        const int slot = lane + 32 * h2;
-        float a, b;
-        upk(A.hw, a, b); o[0 * kGrpQ + slot] = h2 ? b : a;
-        upk(A.lw, a, b); o[1 * kGrpQ + slot] = h2 ? b : a;
-        if (GRAD) {
-            upk(A.hgx, a, b); o[2 * kGrpQ + slot] = h2 ? b : a;
-            upk(A.lgx, a, b); o[3 * kGrpQ + slot] = h2 ? b : a;
-            upk(A.hgy, a, b); o[4 * kGrpQ + slot] = h2 ? b : a;
-            upk(A.lgy, a, b); o[5 * kGrpQ + slot] = h2 ? b : a;
-            upk(A.hgz, a, b); o[6 * kGrpQ + slot] = h2 ? b : a;
-            upk(A.lgz, a, b); o[7 * kGrpQ + slot] = h2 ? b : a;
+    for (int p = 0; p < P; ++p) {
+        f2 *hv[4] = {&A[p].hw, &A[p].hgx, &A[p].hgy, &A[p].hgz};
+        f2 *lv[4] = {&A[p].lw, &A[p].lgx, &A[p].lgy, &A[p].lgz};
+#pragma unroll
+        for (int a = 0; a < NA; ++a) {
+            f2 h = *hv[a], l = *lv[a];
+#pragma unroll
+            for (int u = 1; u < P; ++u) {
+                const f2 oh = __shfl_sync(0xffffffffu, *hv[a], sl + LPS * u);
+                const f2 ol = __shfl_sync(0xffffffffu, *lv[a], sl + LPS * u);
+                two_sum_acc(h, l, oh);
+                l = add2(l, ol);
+            }
+            if (part == 0) {
+                float x, y;
+                upk(h, x, y);
+                o[(2 * a) * kGrpQ + sl + LPS * (2 * p)] = x;
+                o[(2 * a) * kGrpQ + sl + LPS * (2 * p + 1)] = y;
+                upk(l, x, y);
+                o[(2 * a + 1) * kGrpQ + sl + LPS * (2 * p)] = x;
+                o[(2 * a + 1) * kGrpQ + sl + LPS * (2 * p + 1)] = y;
+            }
         }
     }
     if (counter && r_begin == 0) {
         // terms per query of the whole group: far nodes and the leaves' real points
         int64_t pts = 0;
-        for (int64_t e = lane; e < ne; e += 32) {
-            const int64_t j0 = ((int64_t)near_ids[e0 + e] - nleaf) * bucket;
+        for (int e = lane; e < ne; e += 32) {
+            const int64_t j0 = ((int64_t)ni[e] - nleaf) * bucket;
             pts += min((int64_t)bucket, n - j0);
         }
         for (int o2 = 16; o2 > 0; o2 >>= 1) pts += __shfl_xor_sync(0xffffffffu, pts, o2);
+        const int64_t nvalid = min((int64_t)kGrpQ, m - q0);
         if (lane == 0)
-            atomicAdd(counter, (unsigned long long)(nf + pts) * (unsigned long long)G.nvalid);
+            atomicAdd(counter, (unsigned long long)(nf + pts) * (unsigned long long)nvalid);
     }
 }
 
+// One warp per CTA: the items of a launch differ in length, and a warp that
+// has finished leaves its place to the next item at once (with four-warp CTAs
+// 24 of 32 resident warps were active on average).
+constexpr int lst_resident(bool grad) { return grad ? 16 : 24; }  // CTAs per SM (128, 80 registers)
+
 template <bool GRAD, bool SCREENED, bool CLAMP = false>
-__global__ void __launch_bounds__(32 * kGrpWarps)
+__global__ void __launch_bounds__(32, CLAMP ? (GRAD ? 12 : 16) : lst_resident(GRAD))
     k_tree_eval_lists(const float4 *__restrict__ q, int64_t m, const float4 *__restrict__ frec,
                       const float *__restrict__ src, int64_t n, int levels, int bucket,
                       const int64_t *__restrict__ far_off, const int *__restrict__ far_ids,
@@ -1270,8 +1362,7 @@ static cudaError_t launch_lists_t(Ctx *c, const TreeLists &L, float *part, int64
                                   const IterState *st)
 {
     EvalParams ep = make_eval_params(c);
-    k_tree_eval_lists<GRAD, SCREENED, CLAMP><<<(unsigned)ceil_div(L.nitems, kGrpWarps),
-                                                32 * kGrpWarps, 0, c->stream>>>(
+    k_tree_eval_lists<GRAD, SCREENED, CLAMP><<<(unsigned)L.nitems, 32, 0, c->stream>>>(
         L.q, L.m, c->d_tree_frec, CLAMP ? c->d_src16 : c->d_src, c->n, c->tree_levels,
         c->tree_leaf, L.d_far_off, L.d_far, L.d_near_off, L.d_near, L.d_items, L.nitems, ep,
         L.d_ipart, c->d_counter, st);
@@ -1385,11 +1476,11 @@ __global__ void k_tree_moment_records_b(const CloudIter *__restrict__ cl, const 
 }
 
 // GRAD: the points (w and grad w), else the corners (w).  Held to the
-// registers of the single-cloud kernel (8 or 5 resident CTAs per SM): the
+// registers of the single-cloud kernel: the
 // per-cloud arguments come from memory here, not from the parameter bank,
 // and would otherwise take registers for the whole item.
 template <bool GRAD, bool SCREENED>
-__global__ void __launch_bounds__(32 * kGrpWarps, GRAD ? 5 : 8)
+__global__ void __launch_bounds__(32, lst_resident(GRAD))
     k_tree_eval_lists_b(const CloudIter *__restrict__ cl, const int *__restrict__ off, int ncl)
 {
     const int ci = seg_cloud(off, ncl);
@@ -1417,7 +1508,7 @@ cudaError_t launch_tree_batch(int phase, const CloudIter *cl, const int *off, in
 {
     if (blocks <= 0) return cudaSuccess;
     const unsigned g = (unsigned)blocks;
-    const unsigned T = 32 * kGrpWarps;
+    const unsigned T = 32;
     if (level >= 0) {
         k_tree_level_moments_b<<<g, 256, 0, s>>>(cl, off, ncl, level);
         return cudaGetLastError();
@@ -1462,8 +1553,8 @@ int tree_phase_blocks(const Ctx *c, int phase, int level)
     switch (phase) {
     case kPhLeafMom: return (int)ceil_div(nleaf * c->tree_leaf, kMomTile);
     case kPhMomRec: return (int)ceil_div(nn, 256);
-    case kPhListsP: return lists_p ? (int)ceil_div(c->lists_p.nitems, kGrpWarps) : 0;
-    case kPhListsC: return lists_c ? (int)ceil_div(c->lists_c.nitems, kGrpWarps) : 0;
+    case kPhListsP: return lists_p ? (int)c->lists_p.nitems : 0;
+    case kPhListsC: return lists_c ? (int)c->lists_c.nitems : 0;
     case kPhCombineP: return lists_p ? (int)ceil_div(c->lists_p.m, 256) : 0;
     case kPhCombineC: return lists_c ? (int)ceil_div(c->lists_c.m, 256) : 0;
     default: return 0;
