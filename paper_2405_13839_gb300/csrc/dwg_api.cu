@@ -196,6 +196,7 @@ __global__ void k_iter_reset(IterState *st, int max_iters, unsigned long long *c
     st->max_iters = max_iters;
     st->nfaces = 0;
     st->ndefer = 0;
+    st->nfar = 0;
     st->iso = 0.0;
     st->stat = 0.0;
 }
@@ -543,7 +544,8 @@ void dwg_destroy(dwg_handle h)
                     h->d_state, h->d_tr_iso, h->d_tr_stat, h->d_tr_dn, h->d_tr_faces, h->d_err,
                     h->d_tree_A, h->d_tree_C, h->d_tree_R, h->d_tree_M, h->d_tree_rec,
                     h->d_tree_mrec, h->d_tree_frec, h->d_counter, h->d_mlp_params,
-                    h->d_delta2, h->d_src16, h->d_cell_off, h->d_cell_idx, h->d_tree_dmax};
+                    h->d_delta2, h->d_src16, h->d_cell_off, h->d_cell_idx, h->d_far_q,
+                    h->d_defer, h->d_tree_dmax};
     for (void *p : bufs) cudaFree(p);
     free_lists(h->lists_p);
     free_lists(h->lists_c);
@@ -1619,7 +1621,9 @@ static int phase_blocks(const dwg_ctx *c, int ph)
     case kPhReducePoints: return (int)ceil_div(c->n, 256);
     case kPhReduceW: return ls ? (int)ceil_div(c->ncorners, 256) : 0;
     case kPhMcFaces: return ls ? (int)ceil_div(c->nleaves, 256) : 0;
-    case kPhKnn: return ls ? (int)ceil_div(c->max_faces, 128) : 0;
+    case kPhKnn: return ls && !cell_lists_ready(c) ? (int)ceil_div(c->max_faces, 128) : 0;
+    case kPhKnnLists:
+    case kPhKnnFar: return ls ? knn_phase_blocks(c, ph) : 0;
     case kPhKnnDefer: return ls ? 8 : 0;  // blocks take the cloud's deferred faces in turn
     case kPhUpdate: return (int)ceil_div(c->n, 256);
     case kPhSelHist:
@@ -1808,6 +1812,8 @@ static cudaError_t batch_lane_phases(dwg_ctx *h, const dwg_ctx::Lane &L, bool sc
     ok(launch_eval_batch(kPhReduceW, cl, off(kPhReduceW), ncl, ph[kPhReduceW], s));
     ok(launch_iter_batch(kPhMcFaces, cl, off(kPhMcFaces), ncl, ph[kPhMcFaces], 0, s));
     ok(launch_iter_batch(kPhKnn, cl, off(kPhKnn), ncl, ph[kPhKnn], 0, s));
+    ok(launch_iter_batch(kPhKnnLists, cl, off(kPhKnnLists), ncl, ph[kPhKnnLists], 0, s));
+    ok(launch_iter_batch(kPhKnnFar, cl, off(kPhKnnFar), ncl, ph[kPhKnnFar], 0, s));
     ok(launch_iter_batch(kPhKnnDefer, cl, off(kPhKnnDefer), ncl, ph[kPhKnnDefer], 0, s));
     // normal update and convergence
     ok(launch_iter_batch(kPhUpdate, cl, off(kPhUpdate), ncl, ph[kPhUpdate], 0, s));

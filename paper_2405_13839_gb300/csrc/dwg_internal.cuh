@@ -44,6 +44,7 @@ struct IterState {
     int max_iters;
     int nfaces;          // faces emitted in the current iteration
     int ndefer;          // faces whose k-nearest search was deferred (kNN scatter)
+    int nfar;            // faces in cells without a candidate list (kNN scatter)
     double iso;          // w_bar of the current iteration
     double stat;         // convergence statistic of the current iteration
 };
@@ -158,6 +159,7 @@ struct CloudIter {
     int k;
     const int64_t *cell_off;
     const int *cell_idx;
+    int *far_q;
     double acc_scale;
     unsigned long long *acc;
     // normal update and convergence
@@ -193,7 +195,7 @@ struct CloudIter {
 
 // phases of a batched iteration (one launch each, every cloud's blocks)
 enum BatchPhase {
-    kPhReducePoints, kPhReduceW, kPhIso, kPhMcFaces, kPhKnn, kPhKnnDefer, kPhUpdate, kPhSelHist,
+    kPhReducePoints, kPhReduceW, kPhIso, kPhMcFaces, kPhKnn, kPhKnnLists, kPhKnnFar, kPhKnnDefer, kPhUpdate, kPhSelHist,
     kPhSelFind,
     kPhSelSum, kPhSelFinal, kPhLeafMom, kPhMomRec, kPhListsP, kPhListsC, kPhCombineP,
     kPhCombineC, kPhCount
@@ -274,6 +276,8 @@ struct Ctx {
     int64_t *d_cell_off = nullptr;     // nleaves + 1
     int *d_cell_idx = nullptr;         // sorted point indices
     int cells_k = 0;                   // k the lists were built for (0: none)
+    int *d_far_q = nullptr;            // faces of the iteration in leaves without a list
+    int64_t far_cap = 0;               // entries: six per such leaf
     int *d_leaf_corners = nullptr;     // nleaves x 8 corner indices
     uint64_t *d_corner_keys = nullptr; // Morton keys of corners (sorted)
     float4 *d_corner_pos = nullptr;
@@ -518,6 +522,10 @@ cudaError_t launch_mc_tris(Ctx *c, float *out, int64_t cap, unsigned long long *
 // per-leaf candidate lists for the faces' k nearest points (once per
 // discretisation and k; skipped when they would not fit comfortably)
 int build_cell_lists(Ctx *c);
+// the scatter uses the lists of the current k
+bool cell_lists_ready(const Ctx *c);
+// blocks of a cloud's part of the batched scatter phases (kPhKnnLists, kPhKnnFar)
+int knn_phase_blocks(const Ctx *c, int phase);
 void free_cell_lists(Ctx *c);
 // distance to the 10th nearest other point for m points sampled evenly
 cudaError_t launch_spacing(Ctx *c, int64_t m, float *d_out);

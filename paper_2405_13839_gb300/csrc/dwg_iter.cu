@@ -6,9 +6,12 @@
 //                  the six-tetrahedron split of the leaf cube; one face per
 //                  cut tetrahedron with its vector area (the cross-product
 //                  gradient of Sec. 4.3) oriented toward increasing w;
-//   k_knn_scatter  each face adds its vector to its k nearest input points
-//                  (Eq. 7); sums are 64-bit fixed point, so the result does
-//                  not depend on the order of the atomic additions;
+//   k_knn_lists, k_knn_far  each face adds its vector to its k nearest input
+//                  points (Eq. 7), from its leaf's candidate list or, in a
+//                  leaf without one, by a warp's search of the bucket tree;
+//                  sums are 64-bit fixed point, so the result does not depend
+//                  on the order of the atomic additions (k_knn_scatter: k
+//                  other than 10, or no lists at all);
 //   k_normal_update  n_i <- -sum / |sum| (a point no face chose keeps its
 //                  normal), the per-point change in degrees, next sources;
 //   k_sel_*        convergence statistic of Sec. 5.1: mean of the
@@ -50,6 +53,7 @@ __device__ __forceinline__ void iso_body(const double *__restrict__ wsum_blocks,
         st->iso = sh[0] / (double)n;
         st->nfaces = 0;
         st->ndefer = 0;
+        st->nfar = 0;
     }
 }
 
@@ -489,6 +493,158 @@ __device__ __forceinline__ void knn_scan(const KnnTree &T, F3 q, int k, const in
     }
 }
 
+// ---------------------------------------------------------------------------
+// the same search by a whole warp
+// ---------------------------------------------------------------------------
+// The list is one (key, index) pair per lane, ascending over the lanes.
+__device__ __forceinline__ void warp_cmp_swap(uint64_t &key, int &j, int lane, int mask, bool up)
+{
+    const uint64_t ok = __shfl_xor_sync(0xffffffffu, key, mask);
+    const int oj = __shfl_xor_sync(0xffffffffu, j, mask);
+    // `up`: the lower lane of the pair keeps the smaller key
+    if (((lane & mask) == 0) == up ? ok < key : ok > key) {
+        key = ok;
+        j = oj;
+    }
+}
+
+// bitonic sort of the warp's 32 pairs, ascending over the lanes
+__device__ __forceinline__ void warp_sort(uint64_t &key, int &j, int lane)
+{
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+        for (int m = size >> 1; m > 0; m >>= 1)
+            warp_cmp_swap(key, j, lane, m, (lane & size) == 0 || size == 32);
+}
+
+// The batch (nk, nj), one pair per lane (~0: none), merged into the sorted
+// list: one pair at a time while few are below the k-th key, else by sorting
+// the batch and a bitonic merge of the two lists' 32 smallest.
+__device__ __forceinline__ void warp_merge(uint64_t &key, int &j, uint64_t &kth, uint64_t nk, int nj,
+                                           int k, int lane)
+{
+    unsigned m = __ballot_sync(0xffffffffu, nk < kth);
+    if (__popc(m) > 12) {
+        warp_sort(nk, nj, lane);
+        const uint64_t rk = __shfl_sync(0xffffffffu, nk, 31 - lane);
+        const int rj = __shfl_sync(0xffffffffu, nj, 31 - lane);
+        if (rk < key) {
+            key = rk;
+            j = rj;
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) warp_cmp_swap(key, j, lane, d, true);
+        kth = __shfl_sync(0xffffffffu, key, k - 1);
+        return;
+    }
+    while (m) {
+        const int src = __ffs(m) - 1;
+        m &= m - 1;
+        const uint64_t ck = __shfl_sync(0xffffffffu, nk, src);
+        const int cj = __shfl_sync(0xffffffffu, nj, src);
+        const uint64_t pk = __shfl_up_sync(0xffffffffu, key, 1);
+        const int pj = __shfl_up_sync(0xffffffffu, j, 1);
+        if (key > ck) {
+            const bool shift = lane > 0 && pk > ck;
+            key = shift ? pk : ck;
+            j = shift ? pj : cj;
+        }
+        kth = __shfl_sync(0xffffffffu, key, k - 1);
+        m &= __ballot_sync(0xffffffffu, nk < kth);
+    }
+}
+
+constexpr int kWarpStack = 160;  // 31 siblings stay on the stack per five levels of the tree
+
+// Exact k nearest points of q (k <= 32) by one warp, the keys of knn_search:
+// lane t ends with the t-th nearest point in j (-1: fewer points).  A step
+// tests the up to 32 descendants five levels below a node at once (they are
+// consecutive in the heap: one coalesced load), the nearest of those within
+// the k-th distance is taken next; two buckets are scanned at a time, a lane
+// per point.  The list starts from the 32 points around `seed`, a position
+// in the sorted points.  Budget and *bound as in knn_search.
+__device__ __forceinline__ bool warp_knn(const KnnTree &T, F3 q, int k, int64_t seed, int lane,
+                                         int2 *stack, int &j, int *err, int budget, float *bound)
+{
+    const int64_t s0 = max((int64_t)0, min(seed - 16, T.n - 32)), s1 = min(T.n, s0 + 32);
+    uint64_t key = ~0ull;
+    j = -1;
+    if (s0 + lane < s1) {
+        j = (int)(s0 + lane);
+        key = knn_key(pt_d2(__ldg(&T.p4[j]), q), __ldg(&T.perm[j]));
+    }
+    warp_sort(key, j, lane);
+    uint64_t kth = __shfl_sync(0xffffffffu, key, k - 1);
+    auto worst_of = [](uint64_t kk) {
+        return kk == ~0ull ? INFINITY : __uint_as_float((uint32_t)(kk >> 32));
+    };
+    float worst = worst_of(kth);
+    const unsigned lt = (1u << lane) - 1u;
+    const int nleaf = 1 << T.levels;
+    int sp = 1, work = 0;
+    __syncwarp();
+    if (lane == 0) stack[0] = make_int2(1, 0);
+    __syncwarp();
+    while (sp > 0) {
+        const int2 e = stack[--sp];
+        if (__int_as_float(e.y) > worst) continue;
+        if (budget >= 0 && work > budget) {
+            *bound = worst;
+            return false;
+        }
+        const int lv = 31 - __clz(e.x), step = min(5, T.levels - lv);
+        const int child = (e.x << step) + lane;
+        float cd = INFINITY;
+        const bool in = lane < (1 << step);
+        if (in) cd = box_d2(__ldg(&T.lo[child]), __ldg(&T.hi[child]), q);
+        work += 1 << step;
+        unsigned keep = __ballot_sync(0xffffffffu, in && cd <= worst);
+        if (keep == 0) continue;
+        // the nearest of the kept nodes
+        const unsigned cb = (keep >> lane) & 1u ? __float_as_uint(cd) : 0xffffffffu;
+        const unsigned mn = __reduce_min_sync(0xffffffffu, cb);
+        const int first = __ffs(__ballot_sync(0xffffffffu, cb == mn) & keep) - 1;
+        if (lv + step < T.levels) {  // inner nodes: the nearest on top of the stack
+            const int cnt = __popc(keep);
+            if (sp + cnt > kWarpStack) {
+                if (lane == 0) atomicOr(err, kErrStack);
+                break;
+            }
+            if ((keep >> lane) & 1u) {
+                const int pos = lane == first ? cnt - 1
+                                              : __popc(keep & lt) - (lane > first ? 1 : 0);
+                stack[sp + pos] = make_int2(child, __float_as_int(cd));
+            }
+            sp += cnt;
+            __syncwarp();
+            continue;
+        }
+        // buckets, two at a time, the nearest first
+        const int child0 = child - lane;
+        int a = first;
+        keep &= ~(1u << first);
+        while (a >= 0) {
+            const int b = keep ? __ffs(keep) - 1 : -1;
+            if (b >= 0) keep &= keep - 1;
+            const int mine = lane < 16 ? a : b;
+            const int64_t p = (int64_t)(child0 + mine - nleaf) * kBucket + (lane & 15);
+            uint64_t nk = ~0ull;
+            if (mine >= 0 && p < T.n && !(p >= s0 && p < s1)) {
+                const float d = pt_d2(__ldg(&T.p4[p]), q);
+                if (d <= worst) nk = knn_key(d, __ldg(&T.perm[p]));
+            }
+            work += 32;
+            warp_merge(key, j, kth, nk, (int)p, k, lane);
+            worst = worst_of(kth);
+            keep &= __ballot_sync(0xffffffffu, cd <= worst);
+            a = keep ? __ffs(keep) - 1 : -1;
+            if (a >= 0) keep &= keep - 1;
+        }
+    }
+    return true;
+}
+
 static KnnTree knn_tree(const Ctx *c);
 
 // The scatter's additions are first summed per warp in a shared-memory
@@ -511,6 +667,212 @@ constexpr int kAggProbes = 8;    // entries tried before adding to global memory
 constexpr int64_t kAggMaxPoints = 4000000;
 constexpr size_t kAggSmem =
     (size_t)kAggWarps * kAggSlots * (3 * sizeof(unsigned long long) + sizeof(int));
+
+// Faces whose leaf cell has a candidate list, k = 10: a thread per face.  A
+// candidate is one 32-bit key, its squared distance's bits with the low 8
+// replaced by its place in the list (at most kCellCap = 256 entries), and
+// the 11 smallest keys are kept sorted with integer minima and maxima alone
+// (21 instructions a candidate that enters, no 64-bit compares and no index
+// to move).  Cutting 8 bits can only matter when the tenth and the eleventh
+// key agree above them; that face is scanned again with the full (distance,
+// input index) keys.  Faces without a list are queued for k_knn_far.
+// The sums per warp are 32-bit here: a face vector is below 2^25 units (8
+// finest-cell areas) or goes straight to the points' sums.
+// Bound: the gathers of the candidates (L1 wavefronts 77 % of their peak)
+// and the integer pipe.  With k_knn_far against the one thread per face with
+// 64-bit keys and its own tree search (random normals / 3rd-16th iteration):
+// 2,000-point sphere 0.63 / 0.19 -> 0.10 / 0.05 ms, 100k torus 2.8 / 1.9 ->
+// 0.33 / 0.18 ms, 1M blob 13.5 / 10.2 -> 5.5 / 3.8 ms, 4M union 29 / 14.5 ->
+// 12.1 / 5.2 ms.
+constexpr int kScanK = 10;
+constexpr int kTabBits = 8;
+constexpr int kTabSlots = 1 << kTabBits;
+constexpr int kScanWarps = 4;
+constexpr size_t kTabSmem = (size_t)kScanWarps * kTabSlots * 4 * sizeof(int);
+constexpr long long kTabMax = 1 << 25;
+
+__device__ __forceinline__ void knn_lists_body(const float4 *__restrict__ faces, IterState *st,
+                                               int64_t max_faces, const KnnTree &T,
+                                               const int64_t *__restrict__ cell_off,
+                                               const int *__restrict__ cell_idx, double scale,
+                                               unsigned long long *acc, int *far_q, bool agg,
+                                               int64_t bid)
+{
+    if (cloud_idle(st)) return;  // finished cloud of a batch
+    const int64_t nf = min((int64_t)st->nfaces, max_faces);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (bid * blockDim.x + wid * 32 >= nf) return;  // the whole warp is past the faces
+    extern __shared__ int s_tab[];
+    int *s_key = s_tab + wid * 4 * kTabSlots;
+    int *s_v = s_key + kTabSlots;
+    if (agg)
+        for (int i = lane; i < kTabSlots; i += 32) {
+            s_key[i] = -1;
+            s_v[i] = s_v[kTabSlots + i] = s_v[2 * kTabSlots + i] = 0;
+        }
+    const int64_t f = bid * blockDim.x + threadIdx.x;
+    int bj[kScanK];
+#pragma unroll
+    for (int t = 0; t < kScanK; ++t) bj[t] = -1;
+    long long vx = 0, vy = 0, vz = 0;
+    bool far = false;
+    if (f < nf) {
+        const float4 A = faces[2 * f], C = faces[2 * f + 1];
+        const int leaf = __float_as_int(A.w);
+        const int64_t c0 = __ldg(&cell_off[leaf]);
+        const int len = (int)(__ldg(&cell_off[leaf + 1]) - c0);
+        vx = llrint((double)A.x * scale);
+        vy = llrint((double)A.y * scale);
+        vz = llrint((double)A.z * scale);
+        far = len <= 0;
+        if (!far) {
+            const int *cand = cell_idx + c0;
+            const F3 q{C.x, C.y, C.z};
+            unsigned b[kScanK + 1];
+#pragma unroll
+            for (int t = 0; t <= kScanK; ++t) b[t] = 0xffffffffu;
+            for (int t = 0; t < len; t += 4) {
+                int jj[4];
+                unsigned ky[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) jj[u] = __ldg(&cand[min(t + u, len - 1)]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float d = pt_d2(__ldg(&T.p4[jj[u]]), q);
+                    ky[u] = t + u < len ? (__float_as_uint(d) & 0xffffff00u) | (unsigned)(t + u)
+                                        : 0xffffffffu;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (ky[u] < b[kScanK]) {
+#pragma unroll
+                        for (int i = kScanK; i > 0; --i) b[i] = max(b[i - 1], min(b[i], ky[u]));
+                        b[0] = min(b[0], ky[u]);
+                    }
+                }
+            }
+            if ((b[kScanK - 1] >> 8) == (b[kScanK] >> 8) && b[kScanK] != 0xffffffffu) {
+                knn_scan<kScanK, true>(T, q, kScanK, cell_idx, c0, c0 + len, bj);
+            } else {
+#pragma unroll
+                for (int t = 0; t < kScanK; ++t)
+                    if (b[t] != 0xffffffffu) bj[t] = __ldg(&cand[b[t] & 255u]);
+            }
+        }
+    }
+    const unsigned fm = __ballot_sync(0xffffffffu, far);
+    if (fm) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&st->nfar, __popc(fm));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (far) far_q[base + __popc(fm & ((1u << lane) - 1u))] = (int)f;
+    }
+    auto direct = [&](int j) {
+        unsigned long long *a = acc + 3 * (int64_t)j;
+        atomicAdd(a + 0, (unsigned long long)vx);
+        atomicAdd(a + 1, (unsigned long long)vy);
+        atomicAdd(a + 2, (unsigned long long)vz);
+    };
+    const bool small = agg && llabs(vx) < kTabMax && llabs(vy) < kTabMax && llabs(vz) < kTabMax;
+    __syncwarp();  // the table is cleared
+#pragma unroll
+    for (int t = 0; t < kScanK; ++t) {
+        const int j = bj[t];
+        if (j < 0) continue;
+        bool added = false;
+        if (small) {
+            unsigned h = ((unsigned)j * 2654435761u) >> (32 - kTabBits);
+            for (int p = 0; p < kAggProbes; ++p, h = (h + 1) & (kTabSlots - 1)) {
+                const int prev = atomicCAS(&s_key[h], -1, j);
+                if (prev == -1 || prev == j) {
+                    atomicAdd(&s_v[h], (int)vx);
+                    atomicAdd(&s_v[kTabSlots + h], (int)vy);
+                    atomicAdd(&s_v[2 * kTabSlots + h], (int)vz);
+                    added = true;
+                    break;
+                }
+            }
+        }
+        if (!added) direct(j);  // a large vector, or a crowded table
+    }
+    if (!agg) return;
+    __syncwarp();  // every addition is in the table
+    for (int i = lane; i < kTabSlots; i += 32) {
+        const int j = s_key[i];
+        if (j < 0) continue;
+        unsigned long long *a = acc + 3 * (int64_t)j;
+        atomicAdd(a + 0, (unsigned long long)(long long)s_v[i]);
+        atomicAdd(a + 1, (unsigned long long)(long long)s_v[kTabSlots + i]);
+        atomicAdd(a + 2, (unsigned long long)(long long)s_v[2 * kTabSlots + i]);
+    }
+}
+
+__global__ void __launch_bounds__(32 * kScanWarps, 8)
+    k_knn_lists(const float4 *__restrict__ faces, IterState *st, int64_t max_faces, KnnTree T,
+                const int64_t *__restrict__ cell_off, const int *__restrict__ cell_idx,
+                double scale, unsigned long long *acc, int *far_q, int agg)
+{
+    knn_lists_body(faces, st, max_faces, T, cell_off, cell_idx, scale, acc, far_q, agg != 0,
+                   blockIdx.x);
+}
+
+// The queued faces (in cells far from the points, over kCellCap candidates),
+// a warp per face: as threads of a warp their searches, of very different
+// length, waited for each other and were one chain of dependent loads each.
+constexpr int kFarWarps = 4;
+
+__device__ __forceinline__ void knn_far_body(const float4 *__restrict__ faces, IterState *st,
+                                             const KnnTree &T, const int *__restrict__ far_q,
+                                             double scale, unsigned long long *acc, int2 *defer,
+                                             int budget, int *err, int64_t bid, int64_t nblk)
+{
+    if (cloud_idle(st)) return;  // finished cloud of a batch
+    __shared__ int2 s_stack[kFarWarps][kWarpStack];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nq = st->nfar;
+    for (int64_t i = bid * kFarWarps + wid; i < nq; i += nblk * kFarWarps) {
+        const int f = far_q[i];
+        const float4 A = faces[2 * (int64_t)f], C = faces[2 * (int64_t)f + 1];
+        const F3 q{C.x, C.y, C.z};
+        const int64_t seed = (int64_t)__float_as_int(C.w);
+        int j, bud = budget;
+        float bound = INFINITY;
+        bool own = true;
+        while (!warp_knn(T, q, kScanK, seed, lane, s_stack[wid], j, err, bud, &bound)) {
+            int slot = 0;
+            if (lane == 0) slot = atomicAdd(&st->ndefer, 1);
+            slot = __shfl_sync(0xffffffffu, slot, 0);
+            if (slot < kDeferCap) {
+                if (lane == 0) defer[slot] = make_int2(f, __float_as_int(bound));
+                own = false;  // added by k_knn_deferred
+                break;
+            }
+            bud = -1;
+        }
+        if (own && lane < kScanK && j >= 0) {
+            unsigned long long *a = acc + 3 * (int64_t)j;
+            atomicAdd(a + 0, (unsigned long long)llrint((double)A.x * scale));
+            atomicAdd(a + 1, (unsigned long long)llrint((double)A.y * scale));
+            atomicAdd(a + 2, (unsigned long long)llrint((double)A.z * scale));
+        }
+    }
+}
+
+__global__ void __launch_bounds__(32 * kFarWarps)
+    k_knn_far(const float4 *__restrict__ faces, IterState *st, KnnTree T,
+              const int *__restrict__ far_q, double scale, unsigned long long *acc, int2 *defer,
+              int budget, int *err)
+{
+    knn_far_body(faces, st, T, far_q, scale, acc, defer, budget, err, blockIdx.x, gridDim.x);
+}
+
+// blocks of the far search's launch for a queue of at most cap faces
+static int far_blocks(int64_t cap, int most)
+{
+    return (int)std::min<int64_t>(ceil_div(cap, kFarWarps), most);
+}
+constexpr int kFarBlocks = 152 * 8;      // one cloud
+constexpr int kFarBlocksBatch = 64;      // a cloud's part of a batch
 
 // A face whose own search (no candidate list for its cell) runs past
 // kSearchBudget -- a face far from the points, about as far from many of
@@ -1623,6 +1985,18 @@ cudaError_t launch_iso(Ctx *c)
     return cudaGetLastError();
 }
 
+bool cell_lists_ready(const Ctx *c)
+{
+    return c->knn_lists && c->cells_k == c->knn && c->d_cell_off;
+}
+
+int knn_phase_blocks(const Ctx *c, int phase)
+{
+    if (!cell_lists_ready(c)) return 0;
+    if (phase == kPhKnnLists) return (int)ceil_div(c->max_faces, 32 * kScanWarps);
+    return far_blocks(c->far_cap, kFarBlocksBatch);
+}
+
 // A cloud's entry of the batched iteration's table: the same arguments its
 // own launches pass (launch_reduce_points with the points as queries,
 // launch_iso, launch_reduce_w, launch_mc_faces, launch_knn_scatter,
@@ -1661,9 +2035,10 @@ void fill_cloud_iter(const Ctx *c, CloudIter *o)
     o->knn_budget = c->knn_budget;
     o->T = knn_tree(c);
     o->k = c->knn;
-    const bool lists = c->knn_lists && c->cells_k == c->knn && c->d_cell_off;
+    const bool lists = cell_lists_ready(c);
     o->cell_off = lists ? c->d_cell_off : nullptr;
     o->cell_idx = lists ? c->d_cell_idx : nullptr;
+    o->far_q = lists ? c->d_far_q : nullptr;
     o->acc_scale = c->acc_scale;
     o->acc = c->d_acc;
     o->mode = c->mode;
@@ -1719,14 +2094,25 @@ cudaError_t launch_knn_scatter(Ctx *c)
     // one thread per possible face; threads past the emitted count exit
     unsigned blocks = (unsigned)ceil_div(c->max_faces, 128);
     KnnTree T = knn_tree(c);
-    const bool lists = c->knn_lists && c->cells_k == c->knn && c->d_cell_off;
+    const bool lists = cell_lists_ready(c);
     const int64_t *off = lists ? c->d_cell_off : nullptr;
     const int *idx = lists ? c->d_cell_idx : nullptr;
     // the per-warp sum tables (dynamic shared memory) on clouds up to
     // kAggMaxPoints; batched clouds always take them
     const int agg = c->n <= kAggMaxPoints ? 1 : 0;
     const size_t smem = agg ? kAggSmem : 0;
-    if (c->knn == 10) {
+    if (lists && c->knn == kScanK) {
+        k_knn_lists<<<blocks, 32 * kScanWarps, agg ? kTabSmem : 0, c->stream>>>(
+            c->d_faces, c->d_state, c->max_faces, T, off, idx, c->acc_scale, c->d_acc, c->d_far_q,
+            agg);
+        if (c->far_cap > 0) {
+            k_knn_far<<<far_blocks(c->far_cap, kFarBlocks), 32 * kFarWarps, 0, c->stream>>>(
+                c->d_faces, c->d_state, T, c->d_far_q, c->acc_scale, c->d_acc, c->d_defer,
+                c->knn_budget, c->d_err);
+            k_knn_deferred<10, true><<<kDeferBlocks, defer_threads<10>(), 0, c->stream>>>(
+                c->d_faces, c->d_state, c->d_defer, T, c->knn, c->acc_scale, c->d_acc);
+        }
+    } else if (c->knn == 10) {
         k_knn_scatter<10, true><<<blocks, 128, smem, c->stream>>>(
             c->d_faces, c->d_state, c->max_faces, T, c->knn, off, idx, c->acc_scale, c->d_acc,
             c->d_defer, c->knn_budget, agg, c->d_err);
@@ -1845,12 +2231,24 @@ __global__ void __launch_bounds__(128)
     else if (count != room) atomicOr(err, kErrOverflow);  // the two passes must agree
 }
 
+// leaves without a list (their faces go to the far queue, up to six a leaf)
+__global__ void __launch_bounds__(256)
+    k_cells_without(const int64_t *__restrict__ cnt, int64_t nl, unsigned long long *out)
+{
+    const int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int none = __syncthreads_count(l < nl && cnt[l] == 0);
+    if (threadIdx.x == 0 && none) atomicAdd(out, (unsigned long long)none);
+}
+
 void free_cell_lists(Ctx *c)
 {
     cudaFree(c->d_cell_off);
     cudaFree(c->d_cell_idx);
+    cudaFree(c->d_far_q);
     c->d_cell_off = nullptr;
     c->d_cell_idx = nullptr;
+    c->d_far_q = nullptr;
+    c->far_cap = 0;
     c->cells_k = 0;
 }
 
@@ -1868,7 +2266,7 @@ int build_cell_lists(Ctx *c)
     auto body = [&]() -> int {
         DWG_CUDA_TRY(c, cudaMalloc(&R2, nl * sizeof(float)));
         DWG_CUDA_TRY(c, cudaMalloc(&cnt, nl * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&tot, sizeof(int64_t)));
+        DWG_CUDA_TRY(c, cudaMalloc(&tot, 2 * sizeof(int64_t)));
         DWG_CUDA_TRY(c, cudaMalloc(&c->d_cell_off, (nl + 1) * sizeof(int64_t)));
         const unsigned g = (unsigned)ceil_div(nl, 128);
         if (c->knn == 10)
@@ -1881,10 +2279,15 @@ int build_cell_lists(Ctx *c)
                                                       nullptr, nullptr, cnt, c->d_err);
         int rc = scan_i64(c, cnt, c->d_cell_off, nl, tot);
         if (rc) return rc;
-        int64_t total = 0;
-        DWG_CUDA_TRY(c, cudaMemcpyAsync(&total, tot, sizeof total, cudaMemcpyDeviceToHost,
-                                        c->stream));
+        DWG_CUDA_TRY(c, cudaMemsetAsync(tot + 1, 0, sizeof(int64_t), c->stream));
+        k_cells_without<<<(unsigned)ceil_div(nl, 256), 256, 0, c->stream>>>(
+            cnt, nl, reinterpret_cast<unsigned long long *>(tot + 1));
+        int64_t ht[2] = {0, 0};
+        DWG_CUDA_TRY(c, cudaMemcpyAsync(ht, tot, sizeof ht, cudaMemcpyDeviceToHost, c->stream));
         DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+        const int64_t total = ht[0];
+        c->far_cap = 6 * ht[1];
+        DWG_CUDA_TRY(c, cudaMalloc(&c->d_far_q, std::max<int64_t>(c->far_cap, 1) * sizeof(int)));
         DWG_CUDA_TRY(c, cudaMemcpyAsync(c->d_cell_off + nl, tot, sizeof(int64_t),
                                         cudaMemcpyDeviceToDevice, c->stream));
         // lists only where they fit comfortably (a quarter of the free memory)
@@ -1973,6 +2376,25 @@ __global__ void __launch_bounds__(256)
                   c.faces, c.max_faces, c.err, (int64_t)blockIdx.x - off[ci]);
 }
 
+// a batch has k = 10; clouds without candidate lists search the tree
+__global__ void __launch_bounds__(32 * kScanWarps, 8)
+    k_knn_lists_b(const CloudIter *__restrict__ cl, const int *__restrict__ off, int ncl)
+{
+    const int ci = seg_cloud(off, ncl);
+    const CloudIter &c = cl[ci];
+    knn_lists_body(c.faces, c.st, c.max_faces, c.T, c.cell_off, c.cell_idx, c.acc_scale, c.acc,
+                   c.far_q, true, (int64_t)blockIdx.x - off[ci]);
+}
+
+__global__ void __launch_bounds__(32 * kFarWarps)
+    k_knn_far_b(const CloudIter *__restrict__ cl, const int *__restrict__ off, int ncl)
+{
+    const int ci = seg_cloud(off, ncl);
+    const CloudIter &c = cl[ci];
+    knn_far_body(c.faces, c.st, c.T, c.far_q, c.acc_scale, c.acc, c.defer, c.knn_budget, c.err,
+                 (int64_t)blockIdx.x - off[ci], (int64_t)off[ci + 1] - off[ci]);
+}
+
 template <int KMAX, bool FIXED>
 __global__ void __launch_bounds__(128)
     k_knn_scatter_b(const CloudIter *__restrict__ cl, const int *__restrict__ off, int ncl)
@@ -2042,6 +2464,8 @@ cudaError_t launch_iter_batch(int phase, const CloudIter *cl, const int *off, in
     case kPhIso: k_iso_b<<<(unsigned)ncl, 256, 0, s>>>(cl); break;
     case kPhMcFaces: k_mc_faces_b<<<g, 256, 0, s>>>(cl, off, ncl); break;
     case kPhKnn: k_knn_scatter_b<10, true><<<g, 128, kAggSmem, s>>>(cl, off, ncl); break;
+    case kPhKnnLists: k_knn_lists_b<<<g, 32 * kScanWarps, kTabSmem, s>>>(cl, off, ncl); break;
+    case kPhKnnFar: k_knn_far_b<<<g, 32 * kFarWarps, 0, s>>>(cl, off, ncl); break;
     case kPhKnnDefer:
         k_knn_deferred_b<<<g, defer_threads<10>(), 0, s>>>(cl, off, ncl);
         break;
