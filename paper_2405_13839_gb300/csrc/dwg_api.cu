@@ -68,6 +68,51 @@ bool use_tree(const Ctx *c)
 }
 }  // namespace dwg
 
+namespace dwg {
+cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
+{
+    Scratch &S = c->scratch;
+    const size_t b = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
+    *p = nullptr;
+    // the smallest free block that holds it, none far too large
+    ScratchBlock *best = nullptr;
+    for (ScratchBlock &k : S.blocks)
+        if (!k.scope && k.size >= b && k.size <= 4 * b + ((size_t)1 << 20) &&
+            (!best || k.size < best->size))
+            best = &k;
+    if (best) {
+        best->scope = S.depth;
+        *p = best->p;
+        return cudaSuccess;
+    }
+    const cudaError_t e = cudaMalloc(p, b);
+    if (e == cudaSuccess) S.blocks.push_back({*p, b, S.depth});
+    return e;
+}
+
+ScratchScope::~ScratchScope()
+{
+    Scratch &S = c->scratch;
+    cudaStreamSynchronize(c->stream);  // the scope's work may still use the blocks
+    size_t total = 0;
+    for (ScratchBlock &k : S.blocks) {
+        if (k.scope == S.depth) k.scope = 0;
+        total += k.size;
+    }
+    --S.depth;
+    // the largest free blocks go first
+    while (total > kScratchKeep) {
+        auto big = S.blocks.end();
+        for (auto k = S.blocks.begin(); k != S.blocks.end(); ++k)
+            if (!k->scope && (big == S.blocks.end() || k->size > big->size)) big = k;
+        if (big == S.blocks.end()) break;
+        total -= big->size;
+        cudaFree(big->p);
+        S.blocks.erase(big);
+    }
+}
+}  // namespace dwg
+
 static int fail(Ctx *c, int code, const std::string &msg)
 {
     if (c) c->err = msg;
@@ -463,7 +508,7 @@ static int prepare_normals(Ctx *c)
                 auto run = [&]() -> int {
                     DWG_CUDA_TRY(c, cudaMalloc(&X, c->n * 64 * sizeof(float)));
                     DWG_CUDA_TRY(c, cudaMalloc(&Y, c->n * 3 * sizeof(float)));
-                    DWG_CUDA_TRY(c, cudaMalloc(&cR, 4 * sizeof(double)));
+                    DWG_CUDA_TRY(c, cudaMalloc(&cR, kSumDoubles * sizeof(double)));
                     if (launch_features(c, X, false, cR) != cudaSuccess ||
                         launch_mlp_forward(c->d_mlp_params, X, c->n, Y, c->stream, c->d_err) !=
                             cudaSuccess ||
@@ -547,6 +592,7 @@ void dwg_destroy(dwg_handle h)
                     h->d_delta2, h->d_src16, h->d_cell_off, h->d_cell_idx, h->d_far_q,
                     h->d_defer, h->d_tree_dmax};
     for (void *p : bufs) cudaFree(p);
+    for (ScratchBlock &k : h->scratch.blocks) cudaFree(k.p);
     free_lists(h->lists_p);
     free_lists(h->lists_c);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
@@ -969,7 +1015,7 @@ int dwg_voronoi_weights(dwg_handle h, int m, float *a_out)
     double *scratch = nullptr;
     float *d_out = nullptr;
     auto run = [&]() -> int {
-        DWG_CUDA_TRY(h, cudaMalloc(&scratch, (h->n + 1) * sizeof(double)));
+        DWG_CUDA_TRY(h, cudaMalloc(&scratch, (h->n + kSumDoubles) * sizeof(double)));
         if (a_out) DWG_CUDA_TRY(h, cudaMalloc(&d_out, h->n * sizeof(float)));
         if (launch_voronoi_weights(h, m, scratch, d_out) != cudaSuccess)
             return fail(h, DWG_ERR_CUDA, "Voronoi weights launch failed");
@@ -1461,7 +1507,7 @@ int dwg_mlp_features(dwg_handle h, float *X_out)
     double *cR = nullptr;
     auto run = [&]() -> int {
         DWG_CUDA_TRY(h, cudaMalloc(&X, h->n * 64 * sizeof(float)));
-        DWG_CUDA_TRY(h, cudaMalloc(&cR, 4 * sizeof(double)));
+        DWG_CUDA_TRY(h, cudaMalloc(&cR, kSumDoubles * sizeof(double)));
         if (launch_features(h, X, true, cR) != cudaSuccess)
             return fail(h, DWG_ERR_CUDA, "features launch failed");
         int rc = download(h, X_out, X, h->n * 64 * sizeof(float));

@@ -220,10 +220,27 @@ struct TreeLists {
     bool valid = false;
 };
 
+// Scratch of the calls on a handle.  A call's device buffers are blocks that
+// the handle keeps when the call ends, so that a call repeated at its size
+// allocates nothing (cudaMalloc and cudaFree of a call's buffers cost tens to
+// hundreds of microseconds, and cudaFree waits for the device); together at
+// most kScratchKeep bytes between calls, all given back with the handle.
+struct ScratchBlock {
+    void *p;
+    size_t size;
+    int scope;  // nesting depth of the scope that holds it, 0: free
+};
+struct Scratch {
+    std::vector<ScratchBlock> blocks;
+    int depth = 0;
+};
+constexpr size_t kScratchKeep = (size_t)256 << 20;
+
 // ---------------------------------------------------------------------------
 // engine context
 // ---------------------------------------------------------------------------
 struct Ctx {
+    Scratch scratch;
     int device = 0;
     cudaStream_t stream = nullptr;
     cudaStream_t own_stream = nullptr;
@@ -444,6 +461,21 @@ cudaError_t launch_reduce_w_raw(const float *part, int nchunks, int64_t m, float
                                 cudaStream_t s);
 
 // dwg_api.cu
+// a block of the handle's scratch, held until the innermost ScratchScope ends
+// (which waits for the handle's stream first)
+cudaError_t scratch_get(Ctx *c, void **p, size_t bytes);
+template <class T>
+inline cudaError_t scratch_get(Ctx *c, T **p, size_t bytes)
+{
+    return scratch_get(c, reinterpret_cast<void **>(p), bytes);
+}
+struct ScratchScope {
+    Ctx *c;
+    explicit ScratchScope(Ctx *c_) : c(c_) { ++c->scratch.depth; }
+    ~ScratchScope();
+    ScratchScope(const ScratchScope &) = delete;
+    ScratchScope &operator=(const ScratchScope &) = delete;
+};
 void set_global_error(const std::string &msg);
 bool use_tree(const Ctx *c);
 // iteration buffers, spatial structures and source records of the current
@@ -504,8 +536,11 @@ cudaError_t launch_knn_query(Ctx *c, const float4 *q, int64_t m, int k, int64_t 
 constexpr int kPcaK = 10;
 cudaError_t launch_init_pca(Ctx *c);
 cudaError_t launch_init_gauss(Ctx *c);
-// local-Voronoi area weights of the m nearest points into p4.w (scratch: n + 1
-// doubles; a_out: n floats in input order, device, or null)
+// scratch doubles of launch_voronoi_weights beside its n areas, and of
+// launch_features
+constexpr int kSumDoubles = 4 + 4 * 304;
+// local-Voronoi area weights of the m nearest points into p4.w (scratch: n +
+// kSumDoubles doubles; a_out: n floats in input order, device, or null)
 cudaError_t launch_voronoi_weights(Ctx *c, int m, double *scratch, float *a_out);
 // clamp radii of the modified kernel into d_delta2 (k in [1, 31]); delta_out:
 // n floats in input order (device) or null

@@ -493,6 +493,8 @@ __device__ __forceinline__ void knn_scan(const KnnTree &T, F3 q, int k, const in
     }
 }
 
+static KnnTree knn_tree(const Ctx *c);
+
 // ---------------------------------------------------------------------------
 // the same search by a whole warp
 // ---------------------------------------------------------------------------
@@ -645,7 +647,283 @@ __device__ __forceinline__ bool warp_knn(const KnnTree &T, F3 q, int k, int64_t 
     return true;
 }
 
-static KnnTree knn_tree(const Ctx *c);
+// ---------------------------------------------------------------------------
+// the same search for a warp of neighbouring queries, one per lane
+// ---------------------------------------------------------------------------
+// The lanes' queries lie together (consecutive sorted points, consecutive
+// octree leaves), so their searches visit nearly the same nodes: the warp
+// walks the tree once, each node's box tested by every lane against its own
+// query and radius, four descendants two levels down a step (consecutive in
+// the heap); a node no lane needs is dropped.  A bucket that some lane needs
+// is read once, every point a broadcast, and each lane keeps its K smallest
+// distances with floating-point minima and maxima only.  A second pass over
+// the buckets read collects the points within the K-th distance, which are
+// then ordered by the (distance, input index) keys.  (A test of the box
+// around all the queries prunes 32 nodes at once, but one outlier among
+// them, or a jump of the Morton order, makes it keep most of the tree.)
+constexpr int kShWarps = 4;       // warps per CTA of the kernels that use it
+constexpr int kShStack = 96;      // at most 3 siblings per two levels stay behind
+// A warp stops after this many buckets: the lanes that still need a node (an
+// outlier, a cell far from the points) are searched by a warp each instead,
+// so that one such query does not hold its 31 neighbours.
+constexpr int kShBuckets = 64;
+
+struct ShSmem {
+    int stack[kShStack];
+    int visited[kShBuckets];
+};
+
+// Walks the tree for the warp's queries.  worst(): this lane's radius
+// (squared; negative: nothing needed); on_bucket(b) is called by every lane
+// for each bucket within some lane's radius, the nearest subtree first.  When
+// on_bucket gives up (false), the lanes that need it or a node still on the
+// stack get true.
+template <class WorstFn, class BucketFn>
+__device__ __forceinline__ bool sh_walk(const KnnTree &T, F3 q, int lane, int *stack,
+                                        WorstFn &&worst, BucketFn &&on_bucket)
+{
+    const int nleaf = 1 << T.levels;
+    // the least distance at which a lane needs the node (float bits), ~0: none
+    auto need = [&](int node) {
+        const float d = box_d2(__ldg(&T.lo[node]), __ldg(&T.hi[node]), q);
+        return __reduce_min_sync(0xffffffffu, d <= worst() ? __float_as_uint(d) : 0xffffffffu);
+    };
+    int sp = 1;
+    __syncwarp();
+    if (lane == 0) stack[0] = 1;
+    __syncwarp();
+    while (sp > 0) {
+        const int node = stack[--sp];
+        if (need(node) == 0xffffffffu) continue;
+        if (node >= nleaf) {
+            if (on_bucket(node - nleaf)) continue;
+            bool more = false;
+            for (++sp; sp > 0 && !more;) {
+                const int nd = stack[--sp];
+                more = box_d2(__ldg(&T.lo[nd]), __ldg(&T.hi[nd]), q) <= worst();
+            }
+            __syncwarp();
+            return more;
+        }
+        const int step = node >= nleaf / 2 ? 1 : 2;
+        const int c0 = node << step, nc = 1 << step;
+        unsigned dd[4];
+        int cc[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            cc[i] = c0 + i;
+            dd[i] = i < nc ? need(c0 + i) : 0xffffffffu;
+        }
+        // farthest first onto the stack
+        auto order = [&](int i, int j) {
+            if (dd[i] < dd[j]) {
+                const unsigned t = dd[i]; dd[i] = dd[j]; dd[j] = t;
+                const int u = cc[i]; cc[i] = cc[j]; cc[j] = u;
+            }
+        };
+        order(0, 1); order(2, 3); order(0, 2); order(1, 3); order(1, 2);
+        __syncwarp();  // the pop above is read by every lane
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (dd[i] != 0xffffffffu) {
+                if (lane == 0) stack[sp] = cc[i];
+                ++sp;
+            }
+        __syncwarp();
+    }
+    return false;
+}
+
+// The K smallest distances (squared) of each lane's query in b, ascending,
+// INFINITY where the cloud has fewer points.  `seed`: a sorted position near
+// the queries (the same in every lane), whose four buckets are read first.
+// S.visited holds the *nvis buckets read.  True for a lane whose search did
+// not end within kShBuckets buckets.
+template <int K>
+__device__ __forceinline__ bool sh_smallest(const KnnTree &T, F3 q, int64_t seed, int lane,
+                                            ShSmem &S, int *nvis, float (&b)[K])
+{
+#pragma unroll
+    for (int t = 0; t < K; ++t) b[t] = INFINITY;
+    int nv = 0;
+    auto read = [&](int64_t bucket) {
+        if (lane == 0) S.visited[nv] = (int)bucket;
+        ++nv;
+        const int64_t j0 = bucket * kBucket;
+        const int cnt = (int)min((int64_t)kBucket, T.n - j0);
+#pragma unroll 4
+        for (int u = 0; u < cnt; ++u) {
+            const float d = pt_d2(__ldg(&T.p4[j0 + u]), q);
+            if (d < b[K - 1]) {
+#pragma unroll
+                for (int t = K - 1; t > 0; --t) b[t] = fmaxf(b[t - 1], fminf(b[t], d));
+                b[0] = fminf(b[0], d);
+            }
+        }
+    };
+    const int64_t nb = (T.n + kBucket - 1) / kBucket;
+    const int64_t s0 = max((int64_t)0, min(seed / kBucket - 1, nb - 4)), s1 = min(nb, s0 + 4);
+    for (int64_t s = s0; s < s1; ++s) read(s);
+    const bool more = sh_walk(
+        T, q, lane, S.stack, [&]() { return b[K - 1]; },
+        [&](int bucket) {
+            if (bucket >= s0 && bucket < s1) return true;
+            if ((int64_t)bucket >= nb) return true;  // an empty leaf of the complete tree
+            if (nv == kShBuckets) return false;
+            read(bucket);
+            return true;
+        });
+    *nvis = nv;
+    __syncwarp();
+    return more;
+}
+
+// ---------------------------------------------------------------------------
+// the K nearest points of every point, itself among them
+// ---------------------------------------------------------------------------
+// idx[t * stride + r]: the t-th nearest (ascending keys, sorted position, -1:
+// fewer points) of sorted point i0 + r, r < cnt, as knn_search<K, true>
+// gives it.  Points whose search does not end within the warp's buckets, or
+// whose K-th distance ties with others beyond the K, go to the queue.
+template <int K>
+__global__ void __launch_bounds__(32 * kShWarps)
+    k_knn_points(KnnTree T, int64_t i0, int cnt, int64_t stride, int *__restrict__ idx,
+                 int *__restrict__ queue, int *nqueue)
+{
+    __shared__ ShSmem S_all[kShWarps];
+    __shared__ int cols_all[kShWarps][K][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r - lane >= cnt) return;  // the whole warp
+    ShSmem &S = S_all[wid];
+    int (*cols)[32] = cols_all[wid];
+    const bool valid = r < cnt;
+    const int64_t i = i0 + (valid ? r : cnt - 1);
+    const float4 p = T.p4[i];
+    const F3 q{p.x, p.y, p.z};
+    int nv = 0, found = 0;
+    bool far;
+    {
+        float b[K];
+        far = sh_smallest<K>(T, q, i0 + r - lane + 16, lane, S, &nv, b);
+        const float dk = far ? -1.f : b[K - 1];
+        for (int v = 0; v < nv; ++v) {
+            const int bucket = S.visited[v];
+            const int node = (1 << T.levels) + bucket;
+            const float d = box_d2(__ldg(&T.lo[node]), __ldg(&T.hi[node]), q);
+            if (!__any_sync(0xffffffffu, d <= dk)) continue;
+            const int64_t j0 = (int64_t)bucket * kBucket;
+            const int c = (int)min((int64_t)kBucket, T.n - j0);
+#pragma unroll 4
+            for (int u = 0; u < c; ++u)
+                if (pt_d2(__ldg(&T.p4[j0 + u]), q) <= dk) {
+                    if (found < K) cols[found][lane] = (int)j0 + u;
+                    ++found;
+                }
+        }
+    }
+    far = valid && (far || found > K);
+    const unsigned fm = __ballot_sync(0xffffffffu, far);
+    if (fm) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(nqueue, __popc(fm));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (far) queue[base + __popc(fm & ((1u << lane) - 1u))] = r;
+    }
+    if (!valid || far) return;
+    uint64_t key[K];
+    int bj[K];
+#pragma unroll
+    for (int t = 0; t < K; ++t) {
+        bj[t] = t < found ? cols[t][lane] : -1;
+        key[t] = bj[t] >= 0 ? knn_key(pt_d2(__ldg(&T.p4[bj[t]]), q), __ldg(&T.perm[bj[t]])) : ~0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+#pragma unroll
+        for (int t = u & 1; t + 1 < K; t += 2)
+            if (key[t + 1] < key[t]) {
+                const uint64_t k = key[t];
+                key[t] = key[t + 1];
+                key[t + 1] = k;
+                const int j = bj[t];
+                bj[t] = bj[t + 1];
+                bj[t + 1] = j;
+            }
+#pragma unroll
+    for (int t = 0; t < K; ++t) idx[t * stride + r] = bj[t];
+}
+
+// the queued points, a warp each
+__global__ void __launch_bounds__(32 * kShWarps)
+    k_knn_points_far(KnnTree T, int64_t i0, int64_t stride, int k, int *__restrict__ idx,
+                     const int *__restrict__ queue, const int *__restrict__ nqueue, int *err)
+{
+    __shared__ int2 s_stack[kShWarps][kWarpStack];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nq = *nqueue;
+    for (int u = blockIdx.x * kShWarps + wid; u < nq; u += gridDim.x * kShWarps) {
+        const int r = queue[u];
+        const float4 p = T.p4[i0 + r];
+        int j;
+        float bound;
+        warp_knn(T, F3{p.x, p.y, p.z}, k, i0 + r, lane, s_stack[wid], j, err, -1, &bound);
+        if (lane < k) idx[(int64_t)lane * stride + r] = j;
+    }
+}
+
+constexpr int kShFarBlocks = 152 * 8;
+
+// A table of the K nearest points, filled for one range of points at a time
+// (at most kKnnRange, so that the table stays small beside a large cloud):
+// `use(i0, cnt, stride, table)` launches the kernel that reads it.
+constexpr int64_t kKnnRange = (int64_t)3 << 20;
+
+template <int K, class UseFn>
+static cudaError_t points_nearest(Ctx *c, UseFn &&use)
+{
+    const KnnTree T = knn_tree(c);
+    const int64_t stride = std::min<int64_t>(c->n, kKnnRange);
+    ScratchScope scope(c);
+    int *buf = nullptr;  // K * stride table, queue, its length
+    cudaError_t e = scratch_get(c, &buf, ((K + 1) * stride + 1) * sizeof(int));
+    if (e != cudaSuccess) return e;
+    int *queue = buf + K * stride, *nq = queue + stride;
+    for (int64_t i0 = 0; i0 < c->n && e == cudaSuccess; i0 += stride) {
+        const int cnt = (int)std::min<int64_t>(stride, c->n - i0);
+        e = cudaMemsetAsync(nq, 0, sizeof(int), c->stream);
+        if (e != cudaSuccess) break;
+        k_knn_points<K><<<(unsigned)ceil_div(cnt, 32 * kShWarps), 32 * kShWarps, 0, c->stream>>>(
+            T, i0, cnt, stride, buf, queue, nq);
+        k_knn_points_far<<<(unsigned)std::min<int64_t>(ceil_div(cnt, kShWarps), kShFarBlocks),
+                           32 * kShWarps, 0, c->stream>>>(T, i0, stride, K, buf, queue, nq,
+                                                          c->d_err);
+        use(i0, cnt, stride, (const int *)buf);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
+__device__ __forceinline__ uint64_t point_code(const KnnTree &T, F3 q)
+{
+    return morton3((uint64_t)quant21(q.x, T.cube_lo[0], T.inv_h21),
+                   (uint64_t)quant21(q.y, T.cube_lo[1], T.inv_h21),
+                   (uint64_t)quant21(q.z, T.cube_lo[2], T.inv_h21));
+}
+
+// position of the first code not below `code`, by the warp
+__device__ __forceinline__ int64_t warp_lower_bound(const uint64_t *__restrict__ codes, int64_t n,
+                                                    uint64_t code, int lane)
+{
+    int64_t lo = 0, hi = n;  // the answer lies in [lo, hi]
+    while (hi - lo > 32) {
+        const int64_t s = (hi - lo) >> 5;
+        const int c = __popc(__ballot_sync(0xffffffffu, __ldg(&codes[lo + s * (lane + 1) - 1]) < code));
+        if (c < 32) hi = lo + s * (c + 1) - 1;
+        lo += s * c;
+    }
+    return lo + __popc(__ballot_sync(0xffffffffu, lo + lane < hi && __ldg(&codes[lo + lane]) < code));
+}
 
 // The scatter's additions are first summed per warp in a shared-memory
 // table keyed by point (open addressing, a few probes), then each distinct
@@ -1156,40 +1434,63 @@ cudaError_t launch_spacing(Ctx *c, int64_t m, float *d_out)
 // ---------------------------------------------------------------------------
 // learned warm start: patch features from the 16 nearest other points
 // ---------------------------------------------------------------------------
-__global__ void k_centroid(const float4 *__restrict__ p4, int64_t n, double *out /* cx,cy,cz,R */)
+// Centroid and RMS radius about it, in FP64 relative to the bounding-box
+// centre b (so that mean |p - c|^2 = mean |p - b|^2 - |c - b|^2 loses nothing):
+// per-block sums in a fixed order, then one block over the blocks' sums.  As
+// one block over all points it was a chain of loads: 913 us for 200,000
+// points, 13 us as two launches.
+constexpr int kSumBlocks = 304;
+
+__device__ __forceinline__ double block_sum(double v, double *sh)
 {
-    __shared__ double sh[256][3];
-    double s[3] = {0.0, 0.0, 0.0};
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        float4 p = p4[i];
-        s[0] += p.x; s[1] += p.y; s[2] += p.z;
-    }
-    for (int k = 0; k < 3; ++k) sh[threadIdx.x][k] = s[k];
+    sh[threadIdx.x] = v;
     __syncthreads();
     for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int k = 0; k < 3; ++k) sh[threadIdx.x][k] += sh[threadIdx.x + o][k];
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
-    const double cx = sh[0][0] / n, cy = sh[0][1] / n, cz = sh[0][2] / n;
+    const double r = sh[0];
     __syncthreads();
-    double r = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        float4 p = p4[i];
-        double dx = p.x - cx, dy = p.y - cy, dz = p.z - cz;
-        r += dx * dx + dy * dy + dz * dz;
+    return r;
+}
+
+__global__ void __launch_bounds__(256)
+    k_centroid_part(const float4 *__restrict__ p4, int64_t n, double bx, double by, double bz,
+                    double *__restrict__ part)
+{
+    __shared__ double sh[256];
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const float4 p = p4[i];
+        const double dx = p.x - bx, dy = p.y - by, dz = p.z - bz;
+        s[0] += dx;
+        s[1] += dy;
+        s[2] += dz;
+        s[3] += dx * dx + dy * dy + dz * dz;
     }
-    sh[threadIdx.x][0] = r;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x][0] += sh[threadIdx.x + o][0];
-        __syncthreads();
+    for (int k = 0; k < 4; ++k) {
+        const double v = block_sum(s[k], sh);
+        if (threadIdx.x == 0) part[4 * blockIdx.x + k] = v;
+    }
+}
+
+__global__ void __launch_bounds__(256)
+    k_centroid(const double *__restrict__ part, int nb, int64_t n, double bx, double by, double bz,
+               double *out /* cx,cy,cz,R */)
+{
+    __shared__ double sh[256];
+    double m[4];
+    for (int k = 0; k < 4; ++k) {
+        double v = 0.0;
+        for (int b = threadIdx.x; b < nb; b += blockDim.x) v += part[4 * b + k];
+        m[k] = block_sum(v, sh) / n;
     }
     if (threadIdx.x == 0) {
-        out[0] = cx;
-        out[1] = cy;
-        out[2] = cz;
-        out[3] = sqrt(sh[0][0] / n);
+        out[0] = bx + m[0];
+        out[1] = by + m[1];
+        out[2] = bz + m[2];
+        out[3] = sqrt(fmax(0.0, m[3] - (m[0] * m[0] + m[1] * m[1] + m[2] * m[2])));
     }
 }
 
@@ -1197,20 +1498,19 @@ __global__ void k_centroid(const float4 *__restrict__ p4, int64_t n, double *out
 // ascending order) divided by their RMS length, then (p - c) / R, zero
 // padding to 64.  Rows go to row index perm[i] when by_input is set.
 __global__ void __launch_bounds__(128)
-    k_features(KnnTree T, const double *__restrict__ cR, float *__restrict__ X, int by_input,
-               int *err)
+    k_features(KnnTree T, int64_t i0, int cnt_i, int64_t stride, const int *__restrict__ nbr,
+               const double *__restrict__ cR, float *__restrict__ X, int by_input)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T.n) return;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= cnt_i) return;
+    const int64_t i = i0 + r;
     const float4 pi = T.p4[i];
-    int bj[17];
-    knn_search<17, true>(T, F3{pi.x, pi.y, pi.z}, 17, bj, err);
     float o[48];
     int cnt = 0;
     float ss = 0.f;
 #pragma unroll
     for (int t = 0; t < 17; ++t) {
-        int j = bj[t];
+        int j = __ldg(&nbr[t * stride + r]);
         if (j < 0 || j == (int)i || cnt == 16) continue;
         float4 pj = T.p4[j];
         float dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
@@ -1244,10 +1544,15 @@ __global__ void k_normals_from_y(const float *__restrict__ Y, int64_t n, float4 
 
 cudaError_t launch_features(Ctx *c, float *X, bool by_input, double *cR)
 {
-    k_centroid<<<1, 256, 0, c->stream>>>(c->d_p4, c->n, cR);
-    k_features<<<(unsigned)ceil_div(c->n, 128), 128, 0, c->stream>>>(knn_tree(c), cR, X,
-                                                                      by_input ? 1 : 0, c->d_err);
-    return cudaGetLastError();
+    const int nb = (int)std::min<int64_t>(ceil_div(c->n, 256), kSumBlocks);
+    k_centroid_part<<<nb, 256, 0, c->stream>>>(c->d_p4, c->n, c->bbox_c[0], c->bbox_c[1],
+                                               c->bbox_c[2], cR + 4);
+    k_centroid<<<1, 256, 0, c->stream>>>(cR + 4, nb, c->n, c->bbox_c[0], c->bbox_c[1],
+                                         c->bbox_c[2], cR);
+    return points_nearest<17>(c, [&](int64_t i0, int cnt, int64_t stride, const int *nbr) {
+        k_features<<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(
+            knn_tree(c), i0, cnt, stride, nbr, cR, X, by_input ? 1 : 0);
+    });
 }
 
 cudaError_t launch_normals_from_y(Ctx *c, const float *Y)
@@ -1315,19 +1620,20 @@ __device__ bool sym3_min_eigvec(double a[3][3], double out[3])
 // and +z, then +y, then +x where that dot product is zero.  Where the
 // covariance is zero the random normal already in nrm stays.
 __global__ void __launch_bounds__(128)
-    k_init_pca(KnnTree T, double cx, double cy, double cz, float4 *__restrict__ nrm, int *err)
+    k_init_pca(KnnTree T, int64_t i0, int cnt_i, int64_t stride, const int *__restrict__ nbr,
+               double cx, double cy, double cz, float4 *__restrict__ nrm)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T.n) return;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= cnt_i) return;
+    const int64_t i = i0 + r;
     const float4 pi = T.p4[i];
-    int bj[kPcaK];
-    knn_search<kPcaK, true>(T, F3{pi.x, pi.y, pi.z}, kPcaK, bj, err);
     double d[kPcaK][3], mean[3] = {0.0, 0.0, 0.0};
     int cnt = 0;
 #pragma unroll
     for (int t = 0; t < kPcaK; ++t) {
-        if (bj[t] < 0) continue;
-        const float4 pj = T.p4[bj[t]];
+        const int j = __ldg(&nbr[t * stride + r]);
+        if (j < 0) continue;
+        const float4 pj = T.p4[j];
         d[cnt][0] = (double)pj.x - (double)pi.x;
         d[cnt][1] = (double)pj.y - (double)pi.y;
         d[cnt][2] = (double)pj.z - (double)pi.z;
@@ -1371,9 +1677,10 @@ __global__ void k_init_gauss(const float4 *__restrict__ p4, int64_t n, double cx
 
 cudaError_t launch_init_pca(Ctx *c)
 {
-    k_init_pca<<<(unsigned)ceil_div(c->n, 128), 128, 0, c->stream>>>(
-        knn_tree(c), c->bbox_c[0], c->bbox_c[1], c->bbox_c[2], c->d_nrm, c->d_err);
-    return cudaGetLastError();
+    return points_nearest<kPcaK>(c, [&](int64_t i0, int cnt, int64_t stride, const int *nbr) {
+        k_init_pca<<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(
+            knn_tree(c), i0, cnt, stride, nbr, c->bbox_c[0], c->bbox_c[1], c->bbox_c[2], c->d_nrm);
+    });
 }
 
 cudaError_t launch_init_gauss(Ctx *c)
@@ -1386,22 +1693,34 @@ cudaError_t launch_init_gauss(Ctx *c)
 // ---------------------------------------------------------------------------
 // local-Voronoi area weights (Sec. 5.1, "Computing Area Weights")
 // ---------------------------------------------------------------------------
-// A convex polygon of k vertices (counter-clockwise) clipped by the
+// A convex polygon of k vertices (counter-clockwise) clipped in place by the
 // half-plane ax x + ay y <= b; at most cap output vertices (a convex polygon
 // gains at most one per clip; *over is set if rounding asked for more).
-__device__ int vor_clip(const double *px, const double *py, int k, double ax, double ay, double b,
-                        double *ox, double *oy, int cap, bool *over)
+// False when the half-plane leaves the polygon as it is.  FP64 runs at 1/64
+// of the FP32 rate here and bounds the whole kernel: each vertex is tested
+// once, and a polygon with no vertex outside is not touched.
+template <int CAP>
+__device__ __forceinline__ bool vor_clip(double (&px)[CAP], double (&py)[CAP], int &k, double ax,
+                                         double ay, double b, bool *over)
 {
+    double f[CAP];
+    bool cut = false;
+    for (int t = 0; t < k; ++t) {
+        f[t] = ax * px[t] + ay * py[t] - b;
+        cut = cut || !(f[t] <= 0.0);
+    }
+    if (!cut) return false;
+    double ox[CAP], oy[CAP];
     int o = 0;
     for (int t = 0; t < k; ++t) {
         const int u = t + 1 == k ? 0 : t + 1;
-        const double fp = ax * px[t] + ay * py[t] - b, fq = ax * px[u] + ay * py[u] - b;
+        const double fp = f[t], fq = f[u];
         if (fp <= 0.0) {
-            if (o < cap) { ox[o] = px[t]; oy[o] = py[t]; ++o; } else *over = true;
+            if (o < CAP) { ox[o] = px[t]; oy[o] = py[t]; ++o; } else *over = true;
         }
         if ((fp < 0.0 && fq > 0.0) || (fq < 0.0 && fp > 0.0)) {
             const double s = fp / (fp - fq);
-            if (o < cap) {
+            if (o < CAP) {
                 ox[o] = px[t] + s * (px[u] - px[t]);
                 oy[o] = py[t] + s * (py[u] - py[t]);
                 ++o;
@@ -1410,7 +1729,12 @@ __device__ int vor_clip(const double *px, const double *py, int k, double ax, do
             }
         }
     }
-    return o;
+    k = o;
+    for (int v = 0; v < k; ++v) {
+        px[v] = ox[v];
+        py[v] = oy[v];
+    }
+    return true;
 }
 
 // Area of a convex polygon containing the origin intersected with the disk of
@@ -1426,15 +1750,26 @@ __device__ double vor_disk_area(const double *px, const double *py, int k, doubl
         const double ax = px[t], ay = py[t], dx = px[u] - ax, dy = py[u] - ay;
         const double a = dx * dx + dy * dy, b = ax * dx + ay * dy, c = ax * ax + ay * ay - R2;
         if (a == 0.0) continue;
-        const double disc = b * b - a * c;
+        const double bx = px[u], by = py[u];
+        // both ends well inside the circle: so is the edge (the roots below
+        // would be clamped to 0 and 1), and there are no sectors
+        bool inside = c < -1e-9 * R2 && bx * bx + by * by - R2 < -1e-9 * R2;
         double s1 = 0.0, s2 = 0.0;
-        if (disc > 0.0) {
-            const double r = sqrt(disc);
-            s1 = fmin(fmax((-b - r) / a, 0.0), 1.0);
-            s2 = fmin(fmax((-b + r) / a, 0.0), 1.0);
+        if (!inside) {
+            const double disc = b * b - a * c;
+            if (disc > 0.0) {
+                const double r = sqrt(disc);
+                s1 = fmin(fmax((-b - r) / a, 0.0), 1.0);
+                s2 = fmin(fmax((-b + r) / a, 0.0), 1.0);
+            }
+            inside = s1 == 0.0 && s2 == 1.0;
+        }
+        if (inside) {
+            const double x2 = ax + dx, y2 = ay + dy;
+            total += 0.5 * (ax * y2 - ay * x2);
+            continue;
         }
         const double x1 = ax + s1 * dx, y1 = ay + s1 * dy, x2 = ax + s2 * dx, y2 = ay + s2 * dy;
-        const double bx = px[u], by = py[u];
         // no crossing: s1 = s2 = 0, one sector from A to B
         total += 0.5 * R2 * atan2(ax * y1 - ay * x1, ax * x1 + ay * y1);
         total += 0.5 * (x1 * y2 - y1 * x2);
@@ -1449,14 +1784,21 @@ __device__ double vor_disk_area(const double *px, const double *py, int k, doubl
 // neighbourhood with no extent gives 0 (the caller substitutes the mean).
 template <int KMAX, bool FIXED>
 __global__ void __launch_bounds__(128)
-    k_voronoi_area(KnnTree T, int m, double *__restrict__ area, int *err)
+    k_voronoi_area(KnnTree T, int64_t i0, int cnt_i, int64_t stride, const int *__restrict__ nbr,
+                   int m, double *__restrict__ area, int *err)
 {
     constexpr int CAP = KMAX + 4;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T.n) return;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= cnt_i) return;
+    const int64_t i = i0 + r;
     const float4 pi = T.p4[i];
     int bj[KMAX];
-    knn_search<KMAX, FIXED>(T, F3{pi.x, pi.y, pi.z}, m + 1, bj, err);
+    if constexpr (FIXED) {
+#pragma unroll
+        for (int t = 0; t < KMAX; ++t) bj[t] = __ldg(&nbr[t * stride + r]);
+    } else {
+        knn_search<KMAX, FIXED>(T, F3{pi.x, pi.y, pi.z}, m + 1, bj, err);
+    }
     double d[KMAX][3];
     double mean[3] = {0.0, 0.0, 0.0};
     int cnt = 0;
@@ -1495,53 +1837,71 @@ __global__ void __launch_bounds__(128)
     for (int k = 0; k < 3; ++k) e1[k] /= l1;
     const double e2[3] = {nv[1] * e1[2] - nv[2] * e1[1], nv[2] * e1[0] - nv[0] * e1[2],
                           nv[0] * e1[1] - nv[1] * e1[0]};
-    double qx[KMAX], qy[KMAX], R = 0.0;
+    double qx[KMAX], qy[KMAX], R2m = 0.0;
     for (int t = 0; t < cnt; ++t) {
         qx[t] = d[t][0] * e1[0] + d[t][1] * e1[1] + d[t][2] * e1[2];
         qy[t] = d[t][0] * e2[0] + d[t][1] * e2[1] + d[t][2] * e2[2];
-        R = fmax(R, sqrt(qx[t] * qx[t] + qy[t] * qy[t]));
+        R2m = fmax(R2m, qx[t] * qx[t] + qy[t] * qy[t]);
     }
-    R *= 0.5;
+    const double R = 0.5 * sqrt(R2m);
     if (!(R > 0.0)) return;
-    double ax0[CAP], ay0[CAP], ax1[CAP], ay1[CAP];
+    double ax0[CAP], ay0[CAP];
     ax0[0] = -R; ay0[0] = -R; ax0[1] = R; ay0[1] = -R;
     ax0[2] = R;  ay0[2] = R;  ax0[3] = -R; ay0[3] = R;
     int k = 4;
     bool over = false;
+    // The squared distance of the farthest vertex, in float and rounded up: a
+    // seed more than twice as far cuts nothing and is passed over (its
+    // half-plane's border lies at half its distance).
+    float far2 = 2.01f * (float)(R * R);
     for (int t = 0; t < cnt && k >= 3; ++t) {
         const double r2 = qx[t] * qx[t] + qy[t] * qy[t];
         if (!(r2 > 0.0)) continue;  // a seed on the origin imposes nothing
-        k = vor_clip(ax0, ay0, k, qx[t], qy[t], 0.5 * r2, ax1, ay1, CAP, &over);
+        if ((float)r2 > 4.001f * far2) continue;
+        if (!vor_clip<CAP>(ax0, ay0, k, qx[t], qy[t], 0.5 * r2, &over)) continue;
+        float m2 = 0.f;
         for (int v = 0; v < k; ++v) {
-            ax0[v] = ax1[v];
-            ay0[v] = ay1[v];
+            const float x = (float)ax0[v], y = (float)ay0[v];
+            m2 = fmaxf(m2, fmaf(x, x, y * y));
         }
+        far2 = 1.0001f * m2;
     }
     if (over) atomicOr(err, kErrGeometry);
     if (k >= 3) area[i] = vor_disk_area(ax0, ay0, k, R);
 }
 
-// mean of the positive areas (one block, fixed order)
-__global__ void k_area_mean(const double *__restrict__ area, int64_t n, double *out)
+// mean of the positive areas: per-block sums in a fixed order, then one
+// block over them (1,050 us for 1M points as one block)
+__global__ void __launch_bounds__(256)
+    k_area_part(const double *__restrict__ area, int64_t n, double *__restrict__ part)
 {
-    __shared__ double ss[256];
-    __shared__ double sc[256];
+    __shared__ double sh[256];
     double s = 0.0, c = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x)
-        if (area[i] > 0.0) { s += area[i]; c += 1.0; }
-    ss[threadIdx.x] = s;
-    sc[threadIdx.x] = c;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            ss[threadIdx.x] += ss[threadIdx.x + o];
-            sc[threadIdx.x] += sc[threadIdx.x + o];
-        }
-        __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const double a = area[i];
+        if (a > 0.0) { s += a; c += 1.0; }
     }
+    const double ss = block_sum(s, sh), sc = block_sum(c, sh);
+    if (threadIdx.x == 0) {
+        part[2 * blockIdx.x] = ss;
+        part[2 * blockIdx.x + 1] = sc;
+    }
+}
+
+__global__ void __launch_bounds__(256)
+    k_area_mean(const double *__restrict__ part, int nb, double *out)
+{
+    __shared__ double sh[256];
+    double s = 0.0, c = 0.0;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+        s += part[2 * b];
+        c += part[2 * b + 1];
+    }
+    const double ss = block_sum(s, sh), sc = block_sum(c, sh);
     // no positive area at all (a cloud of one point, or all copies of one):
     // the paper's default weight 1
-    if (threadIdx.x == 0) out[0] = sc[0] > 0.0 ? ss[0] / sc[0] : 1.0;
+    if (threadIdx.x == 0) out[0] = sc > 0.0 ? ss / sc : 1.0;
 }
 
 // install a_i (zero areas take the mean) into p4.w; optionally write them in
@@ -1559,14 +1919,21 @@ __global__ void k_area_install(const double *__restrict__ area, const double *__
     if (a_out) a_out[perm[i]] = f;
 }
 
-cudaError_t launch_voronoi_weights(Ctx *c, int m, double *scratch /* n + 1 */, float *a_out)
+cudaError_t launch_voronoi_weights(Ctx *c, int m, double *scratch, float *a_out)
 {
-    const unsigned g = (unsigned)ceil_div(c->n, 128);
+    cudaError_t e = cudaSuccess;
     if (m == 15)
-        k_voronoi_area<16, true><<<g, 128, 0, c->stream>>>(knn_tree(c), m, scratch, c->d_err);
+        e = points_nearest<16>(c, [&](int64_t i0, int cnt, int64_t stride, const int *nbr) {
+            k_voronoi_area<16, true><<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(
+                knn_tree(c), i0, cnt, stride, nbr, m, scratch, c->d_err);
+        });
     else
-        k_voronoi_area<32, false><<<g, 128, 0, c->stream>>>(knn_tree(c), m, scratch, c->d_err);
-    k_area_mean<<<1, 256, 0, c->stream>>>(scratch, c->n, scratch + c->n);
+        k_voronoi_area<32, false><<<(unsigned)ceil_div(c->n, 128), 128, 0, c->stream>>>(
+            knn_tree(c), 0, (int)c->n, 0, nullptr, m, scratch, c->d_err);
+    if (e != cudaSuccess) return e;
+    const int nb = (int)std::min<int64_t>(ceil_div(c->n, 256), kSumBlocks);
+    k_area_part<<<nb, 256, 0, c->stream>>>(scratch, c->n, scratch + c->n + 1);
+    k_area_mean<<<1, 256, 0, c->stream>>>(scratch + c->n + 1, nb, scratch + c->n);
     k_area_install<<<(unsigned)ceil_div(c->n, 256), 256, 0, c->stream>>>(
         scratch, scratch + c->n, c->d_perm, c->n, c->d_p4, a_out, c->d_err);
     return cudaGetLastError();
@@ -1581,14 +1948,21 @@ cudaError_t launch_voronoi_weights(Ctx *c, int m, double *scratch /* n + 1 */, f
 // order) and, when asked, delta in input order.
 template <int KMAX, bool FIXED>
 __global__ void __launch_bounds__(128)
-    k_clamp_delta(KnnTree T, int k, double vmin, double vmax, float *__restrict__ delta2,
+    k_clamp_delta(KnnTree T, int64_t i0, int cnt_i, int64_t stride, const int *__restrict__ nbr,
+                  int k, double vmin, double vmax, float *__restrict__ delta2,
                   float *__restrict__ delta_out, int *err)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T.n) return;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= cnt_i) return;
+    const int64_t i = i0 + r;
     const float4 pi = T.p4[i];
     int bj[KMAX];
-    knn_search<KMAX, FIXED>(T, F3{pi.x, pi.y, pi.z}, k + 1, bj, err);
+    if constexpr (FIXED) {
+#pragma unroll
+        for (int t = 0; t < KMAX; ++t) bj[t] = __ldg(&nbr[t * stride + r]);
+    } else {
+        knn_search<KMAX, FIXED>(T, F3{pi.x, pi.y, pi.z}, k + 1, bj, err);
+    }
     double sum_in = 0.0, sum_all = 0.0;
     int n_in = 0, cnt = 0;
 #pragma unroll
@@ -1615,13 +1989,13 @@ __global__ void __launch_bounds__(128)
 
 cudaError_t launch_clamp_delta(Ctx *c, int k, double vmin, double vmax, float *delta_out)
 {
-    const unsigned g = (unsigned)ceil_div(c->n, 128);
     if (k == 10)
-        k_clamp_delta<11, true><<<g, 128, 0, c->stream>>>(knn_tree(c), k, vmin, vmax, c->d_delta2,
-                                                           delta_out, c->d_err);
-    else
-        k_clamp_delta<32, false><<<g, 128, 0, c->stream>>>(knn_tree(c), k, vmin, vmax,
-                                                            c->d_delta2, delta_out, c->d_err);
+        return points_nearest<11>(c, [&](int64_t i0, int cnt, int64_t stride, const int *nbr) {
+            k_clamp_delta<11, true><<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(
+                knn_tree(c), i0, cnt, stride, nbr, k, vmin, vmax, c->d_delta2, delta_out, c->d_err);
+        });
+    k_clamp_delta<32, false><<<(unsigned)ceil_div(c->n, 128), 128, 0, c->stream>>>(
+        knn_tree(c), 0, (int)c->n, 0, nullptr, k, vmin, vmax, c->d_delta2, delta_out, c->d_err);
     return cudaGetLastError();
 }
 
@@ -2154,10 +2528,84 @@ __device__ __forceinline__ void cell_centre(int4 L, int d, const KnnTree &T, dou
     hp = 0.5 * e * 1.7320508075688772 + ldexp(mag, -17);
 }
 
-template <int KMAX, bool FIXED>
-__global__ void __launch_bounds__(128)
+// A warp's leaf centres (consecutive leaves, neighbours in space) and a
+// sorted position near them; past the last leaf the last one is repeated.
+__device__ __forceinline__ bool cell_warp(const int4 *__restrict__ leaves, int64_t nl, int d,
+                                          const KnnTree &T, double cube_L, int lane, int64_t &l,
+                                          F3 &cf, double &hp)
+{
+    l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (l - lane >= nl) return false;  // the whole warp
+    cell_centre(leaves[min(l, nl - 1)], d, T, cube_L, cf, hp);
+    return true;
+}
+
+// R^2 of a leaf from the squared distance of its centre's k-th nearest point
+// (INFINITY: fewer than k points, every point is a candidate)
+__device__ __forceinline__ float cell_r2(float dk, F3 cf, double hp)
+{
+    if (dk == INFINITY) return INFINITY;
+    const double rk = sqrt((double)dk);
+    const double R = (rk + 2.0 * hp) * (1.0 + 1e-4) + ldexp(fabs((double)cf.x) + fabs((double)cf.y) +
+                                                             fabs((double)cf.z) + rk, -17);
+    return __double2float_ru(R * R);
+}
+
+// k = 10: the leaves whose search does not end within the warp's buckets go
+// to the queue (a warp each, k_cell_radius_far)
+__global__ void __launch_bounds__(32 * kShWarps)
     k_cell_radius(const int4 *__restrict__ leaves, int64_t nl, int d, double cube_L, KnnTree T,
-                  int k, float *__restrict__ R2, int *err)
+                  float *__restrict__ R2, int *__restrict__ queue, int *nqueue)
+{
+    __shared__ ShSmem S[kShWarps];
+    const int lane = threadIdx.x & 31;
+    int64_t l;
+    F3 cf;
+    double hp;
+    if (!cell_warp(leaves, nl, d, T, cube_L, lane, l, cf, hp)) return;
+    const F3 c0{__shfl_sync(0xffffffffu, cf.x, 16), __shfl_sync(0xffffffffu, cf.y, 16),
+                __shfl_sync(0xffffffffu, cf.z, 16)};
+    const int64_t seed = warp_lower_bound(T.codes, T.n, point_code(T, c0), lane);
+    float b[kScanK];
+    int nv;
+    const bool far = sh_smallest<kScanK>(T, cf, seed, lane, S[threadIdx.x >> 5], &nv, b) && l < nl;
+    const unsigned fm = __ballot_sync(0xffffffffu, far);
+    if (fm) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(nqueue, __popc(fm));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (far) queue[base + __popc(fm & ((1u << lane) - 1u))] = (int)l;
+    }
+    if (l < nl && !far) R2[l] = cell_r2(b[kScanK - 1], cf, hp);
+}
+
+__global__ void __launch_bounds__(32 * kShWarps)
+    k_cell_radius_far(const int4 *__restrict__ leaves, int d, double cube_L, KnnTree T,
+                      float *__restrict__ R2, const int *__restrict__ queue,
+                      const int *__restrict__ nqueue, int *err)
+{
+    __shared__ int2 s_stack[kShWarps][kWarpStack];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nq = *nqueue;
+    for (int u = blockIdx.x * kShWarps + wid; u < nq; u += gridDim.x * kShWarps) {
+        const int l = queue[u];
+        F3 cf;
+        double hp;
+        cell_centre(leaves[l], d, T, cube_L, cf, hp);
+        int j;
+        float bound;
+        warp_knn(T, cf, kScanK, warp_lower_bound(T.codes, T.n, point_code(T, cf), lane), lane,
+                 s_stack[wid], j, err, -1, &bound);
+        const int last = __shfl_sync(0xffffffffu, j, kScanK - 1);
+        if (lane == 0) R2[l] = cell_r2(last < 0 ? INFINITY : pt_d2(T.p4[last], cf), cf, hp);
+    }
+}
+
+// any k, a thread per leaf
+template <int KMAX>
+__global__ void __launch_bounds__(128)
+    k_cell_radius_k(const int4 *__restrict__ leaves, int64_t nl, int d, double cube_L, KnnTree T,
+                    int k, float *__restrict__ R2, int *err)
 {
     int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= nl) return;
@@ -2165,70 +2613,57 @@ __global__ void __launch_bounds__(128)
     double hp;
     cell_centre(leaves[l], d, T, cube_L, cf, hp);
     int bj[KMAX];
-    knn_search<KMAX, FIXED>(T, cf, k, bj, err);
-    const int last = bj[(FIXED ? KMAX : k) - 1];
-    if (last < 0) {  // fewer than k points: every point is a candidate
-        R2[l] = INFINITY;
-        return;
-    }
-    const double rk = sqrt((double)pt_d2(T.p4[last], cf));
-    const double R = (rk + 2.0 * hp) * (1.0 + 1e-4) + ldexp(fabs((double)cf.x) + fabs((double)cf.y) +
-                                                             fabs((double)cf.z) + rk, -17);
-    R2[l] = __double2float_ru(R * R);
+    knn_search<KMAX, false>(T, cf, k, bj, err);
+    const int last = bj[k - 1];
+    R2[l] = cell_r2(last < 0 ? INFINITY : pt_d2(T.p4[last], cf), cf, hp);
 }
 
-// points within the radius (FILL: write them; otherwise count, 0 above the cap)
+// points within the radius (FILL: write them; otherwise count, 0 above the
+// cap), one walk of the tree per warp of leaves
 template <bool FILL>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * kShWarps)
     k_cell_lists(const int4 *__restrict__ leaves, int64_t nl, int d, double cube_L, KnnTree T,
                  const float *__restrict__ R2, const int64_t *__restrict__ off,
                  int *__restrict__ idx, int64_t *__restrict__ cnt, int *err)
 {
-    int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= nl) return;
-    int64_t o0 = 0, room = 0;
-    if (FILL) {
-        o0 = off[l];
-        room = off[l + 1] - o0;
-        if (room <= 0) return;
-    }
+    __shared__ int stack[kShWarps][kShStack];
+    const int lane = threadIdx.x & 31;
+    int64_t l;
     F3 cf;
     double hp;
-    cell_centre(leaves[l], d, T, cube_L, cf, hp);
-    const float r2 = R2[l];
-    const int64_t nleaf = (int64_t)1 << T.levels;
-    int stack[64];
-    int sp = 0;
-    int count = 0;
-    bool over = false;
-    stack[sp++] = 1;
-    while (sp > 0 && !over) {
-        const int node = stack[--sp];
-        if (box_d2(__ldg(&T.lo[node]), __ldg(&T.hi[node]), cf) > r2) continue;
-        if (node >= nleaf) {
-            const int64_t j0 = (int64_t)(node - nleaf) * kBucket;
-            const int64_t j1 = min(j0 + kBucket, T.n);
-            for (int64_t j = j0; j < j1; ++j) {
-                if (pt_d2(__ldg(&T.p4[j]), cf) > r2) continue;
-                if (FILL) {
-                    if (count < room) idx[o0 + count] = (int)j;
-                } else if (count == kCellCap) {
-                    over = true;
-                    break;
-                }
-                ++count;
-            }
-        } else {
-            if (sp + 2 > 64) {
-                atomicOr(err, kErrStack);
-                break;
-            }
-            stack[sp++] = 2 * node + 1;
-            stack[sp++] = 2 * node;
-        }
+    if (!cell_warp(leaves, nl, d, T, cube_L, lane, l, cf, hp)) return;
+    const bool valid = l < nl;
+    float r2 = valid ? R2[l] : -1.f;  // -1: this lane needs nothing (more)
+    int64_t o0 = 0;
+    int room = kCellCap;
+    if (FILL) {
+        o0 = valid ? off[l] : 0;
+        room = valid ? (int)(off[l + 1] - o0) : 0;
+        if (room <= 0) r2 = -1.f;
     }
-    if (!FILL) cnt[l] = over ? 0 : count;
-    else if (count != room) atomicOr(err, kErrOverflow);  // the two passes must agree
+    if (!__any_sync(0xffffffffu, r2 >= 0.f)) {
+        if (!FILL && valid) cnt[l] = 0;
+        return;
+    }
+    int count = 0;
+    sh_walk(
+        T, cf, lane, stack[threadIdx.x >> 5], [&]() { return r2; },
+        [&](int bucket) {
+            const int64_t j0 = (int64_t)bucket * kBucket;
+            if (j0 >= T.n) return true;  // an empty leaf of the complete tree
+            const int c = (int)min((int64_t)kBucket, T.n - j0);
+#pragma unroll 4
+            for (int u = 0; u < c; ++u)
+                if (pt_d2(__ldg(&T.p4[j0 + u]), cf) <= r2) {
+                    if (FILL && count < room) idx[o0 + count] = (int)j0 + u;
+                    ++count;
+                }
+            if (!FILL && count > kCellCap) r2 = -1.f;  // over the cap: no list
+            return true;
+        });
+    if (!valid) return;
+    if (!FILL) cnt[l] = count > kCellCap ? 0 : count;
+    else if (room > 0 && count != room) atomicOr(err, kErrOverflow);  // the two passes must agree
 }
 
 // leaves without a list (their faces go to the far queue, up to six a leaf)
@@ -2263,18 +2698,25 @@ int build_cell_lists(Ctx *c)
     KnnTree T = knn_tree(c);
     float *R2 = nullptr;
     int64_t *cnt = nullptr, *tot = nullptr;
+    int *queue = nullptr;
     auto body = [&]() -> int {
         DWG_CUDA_TRY(c, cudaMalloc(&R2, nl * sizeof(float)));
         DWG_CUDA_TRY(c, cudaMalloc(&cnt, nl * sizeof(int64_t)));
         DWG_CUDA_TRY(c, cudaMalloc(&tot, 2 * sizeof(int64_t)));
         DWG_CUDA_TRY(c, cudaMalloc(&c->d_cell_off, (nl + 1) * sizeof(int64_t)));
         const unsigned g = (unsigned)ceil_div(nl, 128);
-        if (c->knn == 10)
-            k_cell_radius<10, true><<<g, 128, 0, c->stream>>>(c->d_leaves, nl, d, c->cube_L, T,
-                                                               c->knn, R2, c->d_err);
-        else
-            k_cell_radius<32, false><<<g, 128, 0, c->stream>>>(c->d_leaves, nl, d, c->cube_L, T,
-                                                                c->knn, R2, c->d_err);
+        if (c->knn == kScanK) {
+            DWG_CUDA_TRY(c, cudaMalloc(&queue, (nl + 1) * sizeof(int)));
+            DWG_CUDA_TRY(c, cudaMemsetAsync(queue + nl, 0, sizeof(int), c->stream));
+            k_cell_radius<<<g, 128, 0, c->stream>>>(c->d_leaves, nl, d, c->cube_L, T, R2, queue,
+                                                    queue + nl);
+            k_cell_radius_far<<<(unsigned)std::min<int64_t>(ceil_div(nl, kShWarps), kShFarBlocks),
+                                32 * kShWarps, 0, c->stream>>>(c->d_leaves, d, c->cube_L, T, R2,
+                                                               queue, queue + nl, c->d_err);
+        } else {
+            k_cell_radius_k<32><<<g, 128, 0, c->stream>>>(c->d_leaves, nl, d, c->cube_L, T, c->knn,
+                                                          R2, c->d_err);
+        }
         k_cell_lists<false><<<g, 128, 0, c->stream>>>(c->d_leaves, nl, d, c->cube_L, T, R2,
                                                       nullptr, nullptr, cnt, c->d_err);
         int rc = scan_i64(c, cnt, c->d_cell_off, nl, tot);
@@ -2307,6 +2749,7 @@ int build_cell_lists(Ctx *c)
     cudaFree(R2);
     cudaFree(cnt);
     cudaFree(tot);
+    cudaFree(queue);
     if (rc) {
         free_cell_lists(c);  // the tree search serves every face
         if (rc == DWG_ERR_OOM) rc = DWG_OK;
