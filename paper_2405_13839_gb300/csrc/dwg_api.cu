@@ -263,10 +263,12 @@ static int ensure_levelset_buffers(Ctx *c, bool tree)
     if (c->built_depth != c->depth) ++c->bufgen;
     int rc = build_discretization(c, c->depth);
     if (rc) return rc;
-    const int nch_c = tree ? 1 : eval_chunks(c, c->ncorners, false);
+    if (!tree && c->reg_mode == DWG_REG_SOFTEN && c->compensated && (rc = build_lattice(c)))
+        return rc;
+    const int nch_c = tree ? 1 : corners_chunks(c);
     if (nch_c != c->nchunks_c) ++c->bufgen;
     c->nchunks_c = nch_c;
-    size_t need_c = (size_t)c->nchunks_c * 2 * (size_t)c->ncorners;
+    size_t need_c = (size_t)c->nchunks_c * 2 * (size_t)(tree ? c->ncorners : corners_slots(c));
     if (need_c > c->part_c_cap) {
         cudaFree(c->d_part_c);
         c->d_part_c = nullptr;
@@ -375,15 +377,14 @@ static int enqueue_body(Ctx *c, cudaGraphConditionalHandle cond, int use_cond,
             if (launch_tree_iter(c, c->lists_c, c->d_corner_pos, c->ncorners, false, c->d_part_c,
                                  c->ncorners, c->d_state) != cudaSuccess)
                 return fail(c, DWG_ERR_CUDA, "tree launch failed");
-        } else if ((rc = eval_launch(c, c->d_corner_pos, c->ncorners, false, c->nchunks_c,
-                                     c->d_part_c, c->ncorners))) {
+        } else if ((rc = eval_corners(c, c->nchunks_c, c->d_part_c))) {
             return rc;
         }
         mark(4);
         if (snap)
             cudaMemcpyAsync(snap + 1, c->d_counter, sizeof(unsigned long long),
                             cudaMemcpyDeviceToDevice, c->stream);
-        if (launch_reduce_w(c, c->d_part_c, c->nchunks_c, c->ncorners, c->d_wc) != cudaSuccess)
+        if (launch_reduce_corners(c, c->d_part_c, c->nchunks_c, c->d_wc) != cudaSuccess)
             return fail(c, DWG_ERR_CUDA, "reduce_w launch failed");
         mark(5);
         if (launch_mc_faces(c) != cudaSuccess) return fail(c, DWG_ERR_CUDA, "mc launch failed");
@@ -933,14 +934,13 @@ int dwg_extract_level_set(dwg_handle h, float *tri_out, int64_t cap, int64_t *co
                 return fail(h, DWG_ERR_CUDA, "tree launch failed");
         } else {
             int r = eval_launch(h, h->d_p4, h->n, true, h->nchunks_p, h->d_part_p, h->n);
-            if (!r) r = eval_launch(h, h->d_corner_pos, h->ncorners, false, h->nchunks_c,
-                                    h->d_part_c, h->ncorners);
+            if (!r) r = eval_corners(h, h->nchunks_c, h->d_part_c);
             if (r) return r;
         }
         if (launch_reduce_points(h, h->d_part_p, h->nchunks_p, h->n, h->d_p4, 1, true, h->d_wg,
                                  h->d_wsum_blocks) != cudaSuccess ||
             launch_iso(h) != cudaSuccess ||
-            launch_reduce_w(h, h->d_part_c, h->nchunks_c, h->ncorners, h->d_wc) != cudaSuccess)
+            launch_reduce_corners(h, h->d_part_c, h->nchunks_c, h->d_wc) != cudaSuccess)
             return fail(h, DWG_ERR_CUDA, "reduce launch failed");
         DWG_CUDA_TRY(h, cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), h->stream));
         if (launch_mc_tris(h, nullptr, 0, d_cnt) != cudaSuccess)
@@ -1665,7 +1665,8 @@ static int phase_blocks(const dwg_ctx *c, int ph)
     const bool ls = c->mode == DWG_UPDATE_LEVELSET;
     switch (ph) {
     case kPhReducePoints: return (int)ceil_div(c->n, 256);
-    case kPhReduceW: return ls ? (int)ceil_div(c->ncorners, 256) : 0;
+    case kPhReduceW:
+        return ls ? (int)ceil_div(use_tree(c) ? c->ncorners : corners_slots(c), 256) : 0;
     case kPhMcFaces: return ls ? (int)ceil_div(c->nleaves, 256) : 0;
     case kPhKnn: return ls && !cell_lists_ready(c) ? (int)ceil_div(c->max_faces, 128) : 0;
     case kPhKnnLists:
@@ -1769,9 +1770,10 @@ static int batch_tables(dwg_ctx *h)
         for (int pass = 0; pass < 2; ++pass) {
             bool grad = pass == 0;
             if (!grad && c->mode != DWG_UPDATE_LEVELSET) continue;
-            int64_t m = grad ? c->n : c->ncorners;
+            int64_t m = grad ? c->n : corners_slots(c);
             int nch = grad ? c->nchunks_p : c->nchunks_c;
             GwnCloud g;
+            g.lat = lattice_of(c);
             g.src = c->d_src;
             g.ntiles = ntiles;
             g.q = grad ? c->d_p4 : c->d_corner_pos;
@@ -1942,7 +1944,7 @@ static int batch_body_branches(dwg_ctx *h, cudaGraphConditionalHandle cond)
             launch_iso(c) != cudaSuccess)
             return fail(h, DWG_ERR_CUDA, "reduce launch failed");
         if (c->mode == DWG_UPDATE_LEVELSET &&
-            (launch_reduce_w(c, c->d_part_c, c->nchunks_c, c->ncorners, c->d_wc) != cudaSuccess ||
+            (launch_reduce_corners(c, c->d_part_c, c->nchunks_c, c->d_wc) != cudaSuccess ||
              launch_mc_faces(c) != cudaSuccess || launch_knn_scatter(c) != cudaSuccess))
             return fail(h, DWG_ERR_CUDA, "level-set launch failed");
         if (launch_normal_update(c) != cudaSuccess || launch_select(c, cond, 0) != cudaSuccess)

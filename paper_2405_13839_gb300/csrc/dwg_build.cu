@@ -493,6 +493,7 @@ __global__ void k_corner_assign(const uint64_t *__restrict__ keys, const int64_t
 static void free_disc(Ctx *c)
 {
     free_cell_lists(c);  // they index the leaves
+    free_lattice(c);
     cudaFree(c->d_leaves);
     cudaFree(c->d_leaf_corners);
     cudaFree(c->d_corner_keys);
@@ -637,6 +638,142 @@ int build_discretization(Ctx *c, int d)
     cudaFree(nodes_b);
     cudaFree(mask);
     if (rc) free_disc(c);
+    return rc;
+}
+
+// ---------------------------------------------------------------------------
+// the corners as lattice tasks (LatTasks)
+// ---------------------------------------------------------------------------
+// Sorted by (x, y, z), a column's corners are taken two at a time (a piece),
+// and four consecutive pieces of one plane x make a task: 94-98 % of the
+// tasks' places hold a corner (octrees of 2,000 to 100,000 points; aligned
+// 2 x 2 x 2 blocks of the lattice would hold 36-58 %).
+__global__ void k_lat_keys(const uint64_t *__restrict__ corner_keys, int64_t m, int bits,
+                           uint64_t *keys, int64_t *idx)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const uint64_t k = corner_keys[i];
+    keys[i] = (compact3(k) << (2 * bits)) | (compact3(k >> 1) << bits) | compact3(k >> 2);
+    idx[i] = i;
+}
+
+__device__ __forceinline__ int64_t key_lower_bound(const uint64_t *__restrict__ keys, int64_t m,
+                                                   uint64_t key)
+{
+    int64_t lo = 0, hi = m;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (__ldg(&keys[mid]) < key) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// 1 where a piece starts: at even places of a column
+__global__ void k_lat_pieces(const uint64_t *__restrict__ keys, int64_t m, int bits, int64_t *flags)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const uint64_t col = (keys[i] >> bits) << bits;
+    flags[i] = ((i - key_lower_bound(keys, m, col)) & 1) == 0;
+}
+
+// per plane x (and one past the last): its first piece, and its tasks
+__global__ void k_lat_planes(const uint64_t *__restrict__ keys, int64_t m, int bits, int64_t nx,
+                             const int64_t *__restrict__ piece, const int64_t *__restrict__ npieces,
+                             int64_t *first, int64_t *tasks)
+{
+    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= nx) return;
+    auto at = [&](int64_t v) {
+        const int64_t i = key_lower_bound(keys, m, (uint64_t)v << (2 * bits));
+        return i < m ? piece[i] : *npieces;
+    };
+    const int64_t a = at(x);
+    first[x] = a;
+    tasks[x] = (at(x + 1) - a + kLatCols - 1) / kLatCols;
+}
+
+__global__ void k_lat_fill(const uint64_t *__restrict__ keys, const int64_t *__restrict__ idx,
+                           const int64_t *__restrict__ flags, const int64_t *__restrict__ piece,
+                           int64_t m, int bits, const int64_t *__restrict__ first,
+                           const int64_t *__restrict__ base, const float4 *__restrict__ pos,
+                           int64_t ntasks, float *lx, float *ly, float *lz, int *lcorner)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const int64_t x = (int64_t)(keys[i] >> (2 * bits));
+    const int64_t local = piece[i] + flags[i] - 1 - first[x];  // the piece within its plane
+    const int64_t task = base[x] + local / kLatCols;
+    const int col = (int)(local % kLatCols), place = 2 * col + (flags[i] ? 0 : 1);
+    const int64_t slot = (task / kLatThreads) * kLatQ * kLatThreads + (int64_t)place * kLatThreads +
+                         task % kLatThreads;
+    const float4 p = pos[idx[i]];
+    lx[task] = p.x;
+    ly[col * ntasks + task] = p.y;
+    lz[slot] = p.z;
+    lcorner[slot] = (int)idx[i];
+}
+
+void free_lattice(Ctx *c)
+{
+    cudaFree(c->d_lat_x);
+    cudaFree(c->d_lat_y);
+    cudaFree(c->d_lat_z);
+    cudaFree(c->d_lat_corner);
+    c->d_lat_x = c->d_lat_y = c->d_lat_z = nullptr;
+    c->d_lat_corner = nullptr;
+    c->lat_tasks = 0;
+}
+
+int build_lattice(Ctx *c)
+{
+    if (c->lat_tasks > 0 || c->ncorners < 1) return DWG_OK;
+    ++c->bufgen;  // a captured graph holds other buffers
+    const int64_t m = c->ncorners;
+    const int bits = c->built_depth + 1;
+    const int64_t nx = ((int64_t)1 << c->built_depth) + 1;
+    const int B = 256;
+    const unsigned g = (unsigned)ceil_div(m, B), gx = (unsigned)ceil_div(nx, B);
+    ScratchScope scope(c);
+    uint64_t *keys = nullptr;
+    int64_t *idx = nullptr, *flags = nullptr, *piece = nullptr, *first = nullptr, *tasks = nullptr,
+            *base = nullptr, *tot = nullptr;
+    DWG_CUDA_TRY(c, scratch_get(c, &keys, m * sizeof(uint64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &idx, m * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &flags, m * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &piece, m * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &first, nx * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &tasks, nx * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &base, nx * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &tot, 2 * sizeof(int64_t)));
+    k_lat_keys<<<g, B, 0, c->stream>>>(c->d_corner_keys, m, bits, keys, idx);
+    int rc = radix_sort_pairs(c, keys, idx, m, 3 * bits);
+    if (rc) return rc;
+    k_lat_pieces<<<g, B, 0, c->stream>>>(keys, m, bits, flags);
+    if ((rc = scan_i64(c, flags, piece, m, tot))) return rc;
+    k_lat_planes<<<gx, B, 0, c->stream>>>(keys, m, bits, nx, piece, tot, first, tasks);
+    if ((rc = scan_i64(c, tasks, base, nx, tot + 1))) return rc;
+    int64_t nt = 0;
+    if ((rc = read_count(c, tot + 1, &nt))) return rc;
+    nt = ceil_div(nt, kLatThreads) * kLatThreads;
+    auto fill = [&]() -> int {
+        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_x, nt * sizeof(float)));
+        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_y, nt * kLatCols * sizeof(float)));
+        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_z, nt * kLatQ * sizeof(float)));
+        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_corner, nt * kLatQ * sizeof(int)));
+        DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_x, 0, nt * sizeof(float), c->stream));
+        DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_y, 0, nt * kLatCols * sizeof(float), c->stream));
+        DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_z, 0, nt * kLatQ * sizeof(float), c->stream));
+        DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_corner, 0xff, nt * kLatQ * sizeof(int), c->stream));
+        k_lat_fill<<<g, B, 0, c->stream>>>(keys, idx, flags, piece, m, bits, first, base,
+                                           c->d_corner_pos, nt, c->d_lat_x, c->d_lat_y,
+                                           c->d_lat_z, c->d_lat_corner);
+        DWG_CUDA_TRY(c, cudaGetLastError());
+        c->lat_tasks = nt;
+        return DWG_OK;
+    };
+    if ((rc = fill())) free_lattice(c);
     return rc;
 }
 

@@ -224,6 +224,7 @@ int measure_fp32_peaks(int device, double *ffma_lane_ops, double *rsqrt_ops, dou
 // the evaluation kernel
 // ---------------------------------------------------------------------------
 constexpr int kEvalThreads = 128;  // CTA size of the default shapes
+constexpr int kLatUnroll = 4;      // sources per loop trip, lattice tasks
 constexpr int kStages = 4;
 
 // One CTA's work: query tile `qtile` against source chunk `chunk`.  With
@@ -469,6 +470,166 @@ __global__ void __launch_bounds__(kEvalThreads)
     if (C.st && cloud_idle(C.st)) return;
     gwn_block<P, kEvalThreads, GRAD, SCREENED>(C.src, C.ntiles, C.q, C.m, C.tpc, C.part, C.stride,
                                                C.ep, err, (int64_t)it.qtile, it.chunk);
+}
+
+// ---------------------------------------------------------------------------
+// w at the leaf corners: lattice tasks
+// ---------------------------------------------------------------------------
+// The corners lie on a lattice, so a thread's eight (one x, four y, two z
+// each) share most of a term's first nine operations, in the order and
+// rounding of gwn_block: p.x - q.x, its square plus eps^2 and m.x (p.x - q.x)
+// once for all eight, the same with y once per column.  The lanes of a pair
+// are two columns, so nothing is shuffled.  Bound by issue slots (two for a
+// packed instruction, one for any other): 6 + 12 + 24 for the coordinates
+// instead of 72, in all 77 per source and eight corners (plain; 108 in
+// gwn_block<4>) and 117 (screened; 148).  100k-point torus, 389,195 corners:
+// plain 14.76 -> 10.41 ms, screened 19.49 -> 14.95 ms; with scalar
+// instructions 11.26 and 17.08 ms; 2 sources a trip 10.74 and 15.33 ms.
+template <bool SCREENED>
+__device__ __forceinline__ void gwn_lattice_block(const float *__restrict__ src,
+                                                  int64_t ntiles_total, const LatTasks &lat,
+                                                  int tiles_per_chunk, float *__restrict__ part,
+                                                  const EvalParams &ep, int *__restrict__ err,
+                                                  int64_t qtile, int chunk)
+{
+    constexpr int T = kSrcTile;
+    constexpr int TILE_FLOATS = T * kSrcFloats;
+    constexpr uint32_t TILE_BYTES = TILE_FLOATS * 4;
+    __shared__ __align__(128) float sbuf[kStages][TILE_FLOATS];
+    __shared__ __align__(8) uint64_t bar[kStages];
+    __shared__ int s_abort;
+
+    const int tid = threadIdx.x;
+    const int64_t tile0 = (int64_t)chunk * tiles_per_chunk;
+    int ntiles = (int)min((int64_t)tiles_per_chunk, ntiles_total - tile0);
+    if (ntiles < 0) ntiles = 0;
+    if (tid == 0) {
+        for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], 1);
+        fence_mbar_init();
+        s_abort = 0;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int s = 0; s < kStages && s < ntiles; ++s) {
+            mbar_expect_tx(&bar[s], TILE_BYTES);
+            bulk_g2s(sbuf[s], src + (tile0 + s) * TILE_FLOATS, TILE_BYTES, &bar[s]);
+        }
+    }
+    const int64_t task = qtile * kLatThreads + tid;
+    const int64_t slot0 = qtile * (kLatQ * kLatThreads) + tid;
+    const float qxs = lat.x[task];
+    const f2 qx = pk(qxs, qxs);
+    f2 qy[kLatCols / 2], qz[kLatCols];  // pairs: columns 2 c and 2 c + 1
+#pragma unroll
+    for (int c = 0; c < kLatCols / 2; ++c) {
+        qy[c] = pk(lat.y[(2 * c) * lat.ntasks + task], lat.y[(2 * c + 1) * lat.ntasks + task]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            qz[2 * c + i] = pk(lat.z[slot0 + (4 * c + i) * kLatThreads],
+                               lat.z[slot0 + (4 * c + 2 + i) * kLatThreads]);
+    }
+    const f2 eps2 = pk(ep.eps2, ep.eps2);
+    const f2 sv = pk(ep.s, ep.s);
+    const f2 nl2e = pk(ep.nl2e_s, ep.nl2e_s);
+    f2 hw[kLatCols], lw[kLatCols];
+#pragma unroll
+    for (int i = 0; i < kLatCols; ++i) hw[i] = lw[i] = 0ull;
+
+    int t = 0;
+    for (; t < ntiles; ++t) {
+        const int s = t % kStages;
+        const uint32_t parity = (uint32_t)((t / kStages) & 1);
+        if (!mbar_wait_bounded(&bar[s], parity)) {
+            atomicOr(err, kErrTimeout);
+            s_abort = 1;
+        }
+        f2 tw[kLatCols];
+#pragma unroll
+        for (int i = 0; i < kLatCols; ++i) tw[i] = 0ull;
+        if (!s_abort) {
+            const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(sbuf[s]);
+#pragma unroll kLatUnroll
+            for (int j = 0; j < T; ++j) {
+                const ulonglong2 r0 = rec[3 * j], r1 = rec[3 * j + 1], r2 = rec[3 * j + 2];
+                const f2 dx = sub2(r0.x, qx);
+                const f2 rx = fma2(dx, dx, eps2);
+                const f2 mx = mul2(r1.y, dx);
+#pragma unroll
+                for (int c = 0; c < kLatCols / 2; ++c) {
+                    const f2 dy = sub2(r0.y, qy[c]);
+                    const f2 ry = fma2(dy, dy, rx);
+                    const f2 my = fma2(r2.x, dy, mx);
+#pragma unroll
+                    for (int i = 2 * c; i < 2 * c + 2; ++i) {
+                        const f2 dz = sub2(r1.x, qz[i]);
+                        const f2 rr = fma2(dz, dz, ry);
+                        const f2 md = fma2(r2.y, dz, my);
+                        const f2 inv = rsqrt2(rr);
+                        const f2 i2 = mul2(inv, inv);
+                        if (!SCREENED) {
+                            tw[i] = fma2(md, mul2(i2, inv), tw[i]);
+                        } else {
+                            const f2 e = ex22(mul2(mul2(rr, inv), nl2e));
+                            const f2 g = mul2(mul2(i2, add2(inv, sv)), e);
+                            tw[i] = fma2(g, md, tw[i]);
+                        }
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kLatCols; ++i) two_sum_acc(hw[i], lw[i], tw[i]);
+        __syncthreads();  // every thread is done with buffer s
+        if (s_abort) break;
+        if (tid == 0 && t + kStages < ntiles) {
+            mbar_expect_tx(&bar[s], TILE_BYTES);
+            bulk_g2s(sbuf[s], src + (tile0 + t + kStages) * TILE_FLOATS, TILE_BYTES, &bar[s]);
+        }
+    }
+    if (s_abort) {
+        // drain the copies still in flight, the one whose wait gave up included
+        if (tid == 0)
+            for (int u = t; u < ntiles && u < t + kStages; ++u)
+                mbar_wait_bounded(&bar[u % kStages], (uint32_t)((u / kStages) & 1));
+        __syncthreads();
+    }
+    // part[(chunk * 2 + h) * slots + slot]
+    const int64_t slots = lat.ntasks * kLatQ;
+    float *hi = part + ((int64_t)chunk * 2 + 0) * slots + slot0, *lo = hi + slots;
+#pragma unroll
+    for (int c = 0; c < kLatCols / 2; ++c)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float x, y;
+            upk(hw[2 * c + i], x, y);
+            hi[(4 * c + i) * kLatThreads] = x;
+            hi[(4 * c + 2 + i) * kLatThreads] = y;
+            upk(lw[2 * c + i], x, y);
+            lo[(4 * c + i) * kLatThreads] = x;
+            lo[(4 * c + 2 + i) * kLatThreads] = y;
+        }
+}
+
+template <bool SCREENED>
+__global__ void __launch_bounds__(kLatThreads)
+    k_gwn_lattice(const float *__restrict__ src, int64_t ntiles_total, LatTasks lat,
+                  int tiles_per_chunk, float *__restrict__ part, EvalParams ep,
+                  int *__restrict__ err)
+{
+    gwn_lattice_block<SCREENED>(src, ntiles_total, lat, tiles_per_chunk, part, ep, err,
+                                (int64_t)blockIdx.x, (int)blockIdx.y);
+}
+
+template <bool SCREENED>
+__global__ void __launch_bounds__(kLatThreads)
+    k_gwn_lattice_batch(const GwnCloud *__restrict__ clouds, const GwnItem *__restrict__ items,
+                        int *__restrict__ err)
+{
+    const GwnItem it = items[blockIdx.x];
+    const GwnCloud &C = clouds[it.cloud];
+    if (C.st && cloud_idle(C.st)) return;
+    gwn_lattice_block<SCREENED>(C.src, C.ntiles, C.lat, C.tpc, C.part, C.ep, err,
+                                (int64_t)it.qtile, it.chunk);
 }
 
 // ---------------------------------------------------------------------------
@@ -719,7 +880,73 @@ int eval_launch(Ctx *c, const float4 *q, int64_t m, bool grad, int nchunks, floa
 }
 
 constexpr int kPGrad = 2;   // query pairs per thread, gradient kernel (batched launches)
-constexpr int kPW = 4;      // query pairs per thread, w-only kernel (batched and raw launches)
+constexpr int kPW = 4;      // query pairs per thread, w-only kernel (raw launches)
+
+bool corners_on_lattice(const Ctx *c)
+{
+    return c->reg_mode == DWG_REG_SOFTEN && c->compensated && c->lat_tasks > 0;
+}
+
+int64_t corners_slots(const Ctx *c)
+{
+    return corners_on_lattice(c) ? c->lat_tasks * kLatQ : c->ncorners;
+}
+
+static int lattice_slots(bool scr, int dev)
+{
+    static int cached[2][64] = {};
+    if (dev < 0 || dev >= 64) dev = 0;
+    int &slot = cached[scr][dev];
+    if (!slot) {
+        int nb = 0;
+        const cudaError_t e =
+            scr ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_gwn_lattice<true>,
+                                                                kLatThreads, 0)
+                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_gwn_lattice<false>,
+                                                                kLatThreads, 0);
+        if (e != cudaSuccess || nb < 1) {
+            cudaGetLastError();
+            nb = 1;
+        }
+        slot = nb * num_sms(dev);
+    }
+    return slot;
+}
+
+int corners_chunks(const Ctx *c)
+{
+    if (!corners_on_lattice(c)) return eval_chunks(c, c->ncorners, false);
+    return pick_chunks(c->lat_tasks / kLatThreads, c->npad / kSrcTile,
+                       lattice_slots(screened_of(c), c->device));
+}
+
+LatTasks lattice_of(const Ctx *c)
+{
+    return LatTasks{c->d_lat_x, c->d_lat_y, c->d_lat_z, c->lat_tasks};
+}
+
+int eval_corners(Ctx *c, int nchunks, float *part)
+{
+    if (!corners_on_lattice(c))
+        return eval_launch(c, c->d_corner_pos, c->ncorners, false, nchunks, part, c->ncorners);
+    const EvalParams ep = make_eval_params(c);
+    const int64_t ntiles = c->npad / kSrcTile;
+    const int tpc = (int)ceil_div(ntiles, nchunks);
+    const dim3 grid((unsigned)(c->lat_tasks / kLatThreads), (unsigned)nchunks);
+    const LatTasks lat = lattice_of(c);
+    if (ep.screened)
+        k_gwn_lattice<true><<<grid, kLatThreads, 0, c->stream>>>(c->d_src, ntiles, lat, tpc, part,
+                                                                 ep, c->d_err);
+    else
+        k_gwn_lattice<false><<<grid, kLatThreads, 0, c->stream>>>(c->d_src, ntiles, lat, tpc, part,
+                                                                  ep, c->d_err);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        c->err = std::string("lattice kernel launch: ") + cudaGetErrorString(e);
+        return DWG_ERR_CUDA;
+    }
+    return DWG_OK;
+}
 
 // ---------------------------------------------------------------------------
 // reduce: combine chunk partials in chunk order; for gradients add back the
@@ -845,6 +1072,29 @@ __device__ __forceinline__ void reduce_w_body(const float *__restrict__ part, in
     out[i] = __fadd_rn(h, l);
 }
 
+// the same over the lattice slots, each sum to its slot's corner
+__device__ __forceinline__ void reduce_lattice_body(const float *__restrict__ part, int nchunks,
+                                                    int64_t slots, const int *__restrict__ corner,
+                                                    float *__restrict__ out, int64_t bid)
+{
+    const int64_t i = bid * blockDim.x + threadIdx.x;
+    if (i >= slots) return;
+    const int to = corner[i];
+    if (to < 0) return;
+    float h = 0.f, l = 0.f;
+    for (int ch = 0; ch < nchunks; ++ch) {
+        two_sum1(h, l, part[((int64_t)ch * 2 + 0) * slots + i]);
+        l = __fadd_rn(l, part[((int64_t)ch * 2 + 1) * slots + i]);
+    }
+    out[to] = __fadd_rn(h, l);
+}
+
+__global__ void k_reduce_lattice(const float *__restrict__ part, int nchunks, int64_t slots,
+                                 const int *__restrict__ corner, float *__restrict__ out)
+{
+    reduce_lattice_body(part, nchunks, slots, corner, out, blockIdx.x);
+}
+
 __global__ void k_reduce_w(const float *__restrict__ part, int nchunks, int64_t m, int64_t stride,
                            float *__restrict__ out)
 {
@@ -867,8 +1117,11 @@ __global__ void k_reduce_w_b(const CloudIter *__restrict__ cl, const int *__rest
 {
     const int ci = seg_cloud(off, ncl);
     const CloudIter &c = cl[ci];
-    reduce_w_body(c.part_c, c.nchunks_c, c.ncorners, c.ncorners, c.wc,
-                  (int64_t)blockIdx.x - off[ci]);
+    const int64_t bid = (int64_t)blockIdx.x - off[ci];
+    if (c.lat_corner)
+        reduce_lattice_body(c.part_c, c.nchunks_c, c.lat_slots, c.lat_corner, c.wc, bid);
+    else
+        reduce_w_body(c.part_c, c.nchunks_c, c.ncorners, c.ncorners, c.wc, bid);
 }
 
 cudaError_t launch_eval_batch(int phase, const CloudIter *cl, const int *off, int ncl,
@@ -887,6 +1140,16 @@ cudaError_t launch_eval_batch(int phase, const CloudIter *cl, const int *off, in
 cudaError_t launch_reduce_w(Ctx *c, const float *part, int nchunks, int64_t m, float *out)
 {
     k_reduce_w<<<(unsigned)ceil_div(m, 256), 256, 0, c->stream>>>(part, nchunks, m, m, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reduce_corners(Ctx *c, const float *part, int nchunks, float *out)
+{
+    if (use_tree(c) || !corners_on_lattice(c))
+        return launch_reduce_w(c, part, nchunks, c->ncorners, out);
+    const int64_t slots = corners_slots(c);
+    k_reduce_lattice<<<(unsigned)ceil_div(slots, 256), 256, 0, c->stream>>>(
+        part, nchunks, slots, c->d_lat_corner, out);
     return cudaGetLastError();
 }
 
@@ -946,7 +1209,7 @@ cudaError_t launch_reduce_w_raw(const float *part, int nchunks, int64_t m, float
     return cudaGetLastError();
 }
 
-int batch_query_tile(bool grad) { return kEvalThreads * 2 * (grad ? kPGrad : kPW); }
+int batch_query_tile(bool grad) { return grad ? kEvalThreads * 2 * kPGrad : kLatThreads * kLatQ; }
 
 cudaError_t launch_gwn_batch(const GwnCloud *clouds, const GwnItem *items, int64_t nitems,
                              bool grad, bool screened, int *err, cudaStream_t s)
@@ -957,8 +1220,8 @@ cudaError_t launch_gwn_batch(const GwnCloud *clouds, const GwnItem *items, int64
         if (screened) k_gwn_batch<kPGrad, true, true><<<g, kEvalThreads, 0, s>>>(clouds, items, err);
         else k_gwn_batch<kPGrad, true, false><<<g, kEvalThreads, 0, s>>>(clouds, items, err);
     } else {
-        if (screened) k_gwn_batch<kPW, false, true><<<g, kEvalThreads, 0, s>>>(clouds, items, err);
-        else k_gwn_batch<kPW, false, false><<<g, kEvalThreads, 0, s>>>(clouds, items, err);
+        if (screened) k_gwn_lattice_batch<true><<<g, kLatThreads, 0, s>>>(clouds, items, err);
+        else k_gwn_lattice_batch<false><<<g, kLatThreads, 0, s>>>(clouds, items, err);
     }
     return cudaGetLastError();
 }

@@ -87,8 +87,24 @@ struct EvalParams {
     int screened;
 };
 
+// The octree's leaf corners arranged for the exact evaluator of w: a task is
+// a thread's eight corners of one lattice plane x, in four (x, y) columns of
+// two z each (kLatQ; places with no corner repeat the origin).  Tasks are
+// padded to whole CTAs of kLatThreads; slot (task / kLatThreads) * kLatQ *
+// kLatThreads + place * kLatThreads + task % kLatThreads.
+constexpr int kLatThreads = 128;
+constexpr int kLatCols = 4;
+constexpr int kLatQ = 2 * kLatCols;
+struct LatTasks {
+    const float *x;      // per task
+    const float *y;      // [kLatCols][ntasks]
+    const float *z;      // per slot
+    int64_t ntasks;      // padded
+};
+
 // one cloud of a batched evaluation launch
 struct GwnCloud {
+    LatTasks lat;      // the corners of the cloud (w only)
     const float *src;
     int64_t ntiles;
     const float4 *q;
@@ -140,10 +156,13 @@ struct CloudIter {
     float4 *wg;
     double *wsum_blocks;
     int wsum_nb;
-    // w at the corners
+    // w at the corners (lat_corner: the corner of each lattice slot, null on
+    // the Barnes-Hut path)
     const float *part_c;
     int nchunks_c;
     int64_t ncorners;
+    const int *lat_corner;
+    int64_t lat_slots;
     float *wc;
     // level set
     const int *leaf_corners;
@@ -299,6 +318,10 @@ struct Ctx {
     uint64_t *d_corner_keys = nullptr; // Morton keys of corners (sorted)
     float4 *d_corner_pos = nullptr;
     float *d_wc = nullptr;             // w at corners
+    // the corners as lattice tasks (exact path; built when first needed)
+    float *d_lat_x = nullptr, *d_lat_y = nullptr, *d_lat_z = nullptr;
+    int *d_lat_corner = nullptr;
+    int64_t lat_tasks = 0;             // padded to kLatThreads
     float4 *d_faces = nullptr;         // 2 x max_faces: area vector, centroid
     int2 *d_defer = nullptr;           // kDeferCap deferred faces: (face, bound bits)
     unsigned long long *d_acc = nullptr; // n x 3 fixed-point face sums
@@ -430,6 +453,8 @@ cudaError_t launch_gather_points(const float *xyz, const float *a, const int64_t
                                  int64_t n, float4 *p4, cudaStream_t s);
 int build_knn_tree(Ctx *c);
 int build_discretization(Ctx *c, int depth);
+int build_lattice(Ctx *c);
+void free_lattice(Ctx *c);
 
 // dwg_eval.cu
 EvalParams make_eval_params(const Ctx *c);
@@ -449,6 +474,15 @@ cudaError_t launch_reduce_points(Ctx *c, const float *part, int nchunks, int64_t
                                  const float4 *queries, int self_mode, bool grad, float4 *out,
                                  double *wsum_blocks);
 cudaError_t launch_reduce_w(Ctx *c, const float *part, int nchunks, int64_t m, float *out);
+// w at the octree's leaf corners by the exact path: the lattice tasks with
+// the softened, compensated kernel, else the general evaluator.  Partial sums
+// per chunk: 2 * corners_slots floats.
+bool corners_on_lattice(const Ctx *c);
+int64_t corners_slots(const Ctx *c);
+int corners_chunks(const Ctx *c);
+int eval_corners(Ctx *c, int nchunks, float *part);
+LatTasks lattice_of(const Ctx *c);
+cudaError_t launch_reduce_corners(Ctx *c, const float *part, int nchunks, float *out);
 int batch_query_tile(bool grad);
 cudaError_t launch_gwn_batch(const GwnCloud *clouds, const GwnItem *items, int64_t nitems,
                              bool grad, bool screened, int *err, cudaStream_t s);

@@ -2398,6 +2398,9 @@ void fill_cloud_iter(const Ctx *c, CloudIter *o)
     o->part_c = c->d_part_c;
     o->nchunks_c = c->nchunks_c;
     o->ncorners = c->ncorners;
+    const bool lat = !use_tree(c) && corners_on_lattice(c);
+    o->lat_corner = lat ? c->d_lat_corner : nullptr;
+    o->lat_slots = lat ? corners_slots(c) : 0;
     o->wc = c->d_wc;
     o->leaf_corners = c->d_leaf_corners;
     o->leaves = c->d_leaves;

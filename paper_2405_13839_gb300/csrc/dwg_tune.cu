@@ -385,6 +385,15 @@ int autotune(Ctx *c, int what, double budget, const char *cache_path, dwg_tuning
         if ((rc = tune_shape(c, c->d_p4, c->n, true, &vg, &ap_ms_p))) return rc;
         if (lset && (rc = tune_shape(c, c->d_corner_pos, c->ncorners, false, &vw, &ap_ms_c)))
             return rc;
+        if (lset && corners_on_lattice(c)) {  // what an iteration runs at the corners
+            const int nch = corners_chunks(c);
+            Buf part;
+            TUNE_TRY(cudaMalloc(&part.p, (size_t)nch * 2 * corners_slots(c) * sizeof(float)));
+            if ((rc = time_ms(c, [&]() { return eval_corners(c, nch, part.as<float>()); },
+                              &ap_ms_c)) ||
+                (rc = device_error(c)))
+                return rc;
+        }
         eval_variant_shape(true, vg, &t.points_pairs, &t.points_threads);
         eval_variant_shape(false, vw, &t.corners_pairs, &t.corners_threads);
     }
