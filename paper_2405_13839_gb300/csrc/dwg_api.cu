@@ -90,18 +90,14 @@ cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
     return e;
 }
 
-ScratchScope::~ScratchScope()
+// frees free blocks, the largest first, until at most `keep` bytes are held
+// (cudaFree waits for the device)
+void scratch_trim(Ctx *c, size_t keep)
 {
     Scratch &S = c->scratch;
-    cudaStreamSynchronize(c->stream);  // the scope's work may still use the blocks
     size_t total = 0;
-    for (ScratchBlock &k : S.blocks) {
-        if (k.scope == S.depth) k.scope = 0;
-        total += k.size;
-    }
-    --S.depth;
-    // the largest free blocks go first
-    while (total > kScratchKeep) {
+    for (const ScratchBlock &k : S.blocks) total += k.size;
+    while (total > keep) {
         auto big = S.blocks.end();
         for (auto k = S.blocks.begin(); k != S.blocks.end(); ++k)
             if (!k->scope && (big == S.blocks.end() || k->size > big->size)) big = k;
@@ -110,6 +106,15 @@ ScratchScope::~ScratchScope()
         cudaFree(big->p);
         S.blocks.erase(big);
     }
+}
+
+ScratchScope::~ScratchScope()
+{
+    Scratch &S = c->scratch;
+    for (ScratchBlock &k : S.blocks)
+        if (k.scope == S.depth) k.scope = 0;
+    --S.depth;
+    scratch_trim(c, kScratchKeep);
 }
 }  // namespace dwg
 
@@ -164,6 +169,54 @@ static int download(Ctx *c, void *dst, const void *src, size_t bytes)
 {
     DWG_CUDA_TRY(c, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, c->stream));
     return DWG_OK;
+}
+
+// device memory that kernels may access as values of `size` bytes (a copy has
+// no alignment rule, a load has)
+static bool kernel_ptr(const void *p, size_t size)
+{
+    return reinterpret_cast<uintptr_t>(p) % size == 0 && is_device_ptr(p);
+}
+// Before a call's kernels touch a caller's device arrays in place, the work
+// already queued on the device is waited for, on every stream: callers fill
+// and reuse such arrays on streams of their own (a framework's default
+// stream), which the handle's stream is not ordered after.  About a
+// microsecond on an idle device.
+static cudaError_t join_caller(Ctx *c)
+{
+    if (c->scratch.joined) return cudaSuccess;
+    c->scratch.joined = true;
+    return cudaDeviceSynchronize();
+}
+// A caller's float array as kernels on the handle's device read it: the array
+// itself when it is there, else a scratch copy.
+static int caller_in(Ctx *c, const float *p, size_t count, const float **d)
+{
+    if (is_device_ptr(p)) DWG_CUDA_TRY(c, join_caller(c));
+    if (kernel_ptr(p, sizeof(float))) {
+        *d = p;
+        return DWG_OK;
+    }
+    float *q = nullptr;
+    DWG_CUDA_TRY(c, scratch_get(c, &q, count * sizeof(float)));
+    *d = q;
+    return upload(c, q, p, count * sizeof(float));
+}
+// Where kernels write a caller's output: the array itself, or scratch to be
+// copied from (caller_done).
+static int caller_out(Ctx *c, float *p, size_t count, float **d)
+{
+    if (is_device_ptr(p)) DWG_CUDA_TRY(c, join_caller(c));
+    if (kernel_ptr(p, sizeof(float))) {
+        *d = p;
+        return DWG_OK;
+    }
+    DWG_CUDA_TRY(c, scratch_get(c, d, count * sizeof(float)));
+    return DWG_OK;
+}
+static int caller_done(Ctx *c, float *p, const float *d, size_t count)
+{
+    return p == d ? DWG_OK : download(c, p, d, count * sizeof(float));
 }
 
 // ---------------------------------------------------------------------------
@@ -224,6 +277,15 @@ __global__ void k_xyz_to_f4(const float *__restrict__ v, int64_t m, float4 *out)
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) out[i] = make_float4(v[3 * i], v[3 * i + 1], v[3 * i + 2], 0.f);
 }
+// the same with the check of dwg_eval_gwn's queries
+__global__ void k_queries_in(const float *__restrict__ v, int64_t m, float4 *out, int *err)
+{
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const float x = v[3 * i], y = v[3 * i + 1], z = v[3 * i + 2];
+    if (!isfinite(x) || !isfinite(y) || !isfinite(z)) atomicOr(err, kErrNonfinite);
+    out[i] = make_float4(x, y, z, 0.f);
+}
 __global__ void k_weights_in(const float *__restrict__ a, const int64_t *__restrict__ perm,
                              int64_t n, float4 *p4, int *err)
 {
@@ -279,7 +341,7 @@ static int ensure_levelset_buffers(Ctx *c, bool tree)
     return DWG_OK;
 }
 
-static int ensure_iter_buffers(Ctx *c)
+static int iter_buffers(Ctx *c)
 {
     const bool tree = use_tree(c);
     if (tree) {
@@ -328,6 +390,17 @@ static int ensure_iter_buffers(Ctx *c)
         c->trace_cap = c->max_iters;
     }
     return DWG_OK;
+}
+
+// what a build took and the iterations do not need
+constexpr size_t kScratchKeepBuilt = (size_t)16 << 20;
+
+static int ensure_iter_buffers(Ctx *c)
+{
+    const uint64_t gen = c->bufgen;
+    const int rc = iter_buffers(c);
+    if (c->bufgen != gen) scratch_trim(c, kScratchKeepBuilt);
+    return rc;
 }
 
 static void invalidate_graph(Ctx *c)
@@ -504,25 +577,18 @@ static int prepare_normals(Ctx *c)
             if (c->init_mode == DWG_INIT_GAUSS && launch_init_gauss(c) != cudaSuccess)
                 return fail(c, DWG_ERR_CUDA, "Gauss-map normals launch failed");
             if (c->init_mode == DWG_INIT_LEARNED) {
+                ScratchScope scope(c);
                 float *X = nullptr, *Y = nullptr;
                 double *cR = nullptr;
-                auto run = [&]() -> int {
-                    DWG_CUDA_TRY(c, cudaMalloc(&X, c->n * 64 * sizeof(float)));
-                    DWG_CUDA_TRY(c, cudaMalloc(&Y, c->n * 3 * sizeof(float)));
-                    DWG_CUDA_TRY(c, cudaMalloc(&cR, kSumDoubles * sizeof(double)));
-                    if (launch_features(c, X, false, cR) != cudaSuccess ||
-                        launch_mlp_forward(c->d_mlp_params, X, c->n, Y, c->stream, c->d_err) !=
-                            cudaSuccess ||
-                        launch_normals_from_y(c, Y) != cudaSuccess)
-                        return fail(c, DWG_ERR_CUDA, "learned init launch failed");
-                    DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-                    return DWG_OK;
-                };
-                int rc = run();
-                cudaFree(X);
-                cudaFree(Y);
-                cudaFree(cR);
-                if (rc) return rc;
+                DWG_CUDA_TRY(c, scratch_get(c, &X, c->n * 64 * sizeof(float)));
+                DWG_CUDA_TRY(c, scratch_get(c, &Y, c->n * 3 * sizeof(float)));
+                DWG_CUDA_TRY(c, scratch_get(c, &cR, kSumDoubles * sizeof(double)));
+                if (launch_features(c, X, false, cR) != cudaSuccess ||
+                    launch_mlp_forward(c->d_mlp_params, X, c->n, Y, c->stream, c->d_err) !=
+                        cudaSuccess ||
+                    launch_normals_from_y(c, Y) != cudaSuccess)
+                    return fail(c, DWG_ERR_CUDA, "learned init launch failed");
+                DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
             }
         } else {
             DWG_CUDA_TRY(c, cudaMemcpyAsync(c->d_nrm, c->d_nrm_init, c->n * sizeof(float4),
@@ -614,6 +680,7 @@ static int create_impl(dwg_ctx *c, const float *points, int64_t n)
     float *xyz = nullptr;
     bool own_xyz = false;
     if (is_device_ptr(points)) {
+        DWG_CUDA_TRY(c, join_caller(c));
         xyz = const_cast<float *>(points);
     } else {
         DWG_CUDA_TRY(c, cudaMalloc(&xyz, n * 3 * sizeof(float)));
@@ -678,6 +745,7 @@ static int create_impl(dwg_ctx *c, const float *points, int64_t n)
         k_iter_reset<<<1, 1, 0, c->stream>>>(c->d_state, c->max_iters, nullptr);
         DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream));
         DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+        scratch_trim(c, kScratchKeepBuilt);
         c->stats.n_points = n;
         return DWG_OK;
     };
@@ -839,16 +907,14 @@ int dwg_set_weights(dwg_handle h, const float *a)
 {
     if (!h || !a) return DWG_ERR_INVALID;
     cudaSetDevice(h->device);
-    float *d = nullptr;
-    DWG_CUDA_TRY(h, cudaMalloc(&d, h->n * sizeof(float)));
-    int rc = upload(h, d, a, h->n * sizeof(float));
-    if (!rc) {
-        k_weights_in<<<nblk(h->n), 256, 0, h->stream>>>(d, h->d_perm, h->n, h->d_p4, h->d_err);
-        rc = check_device_err(h);
-        h->tree_built = false;  // node centres depend on the weights
-        if (rc == DWG_ERR_NONFINITE) h->err = "weights must be finite and > 0";
-    }
-    cudaFree(d);
+    ScratchScope scope(h);
+    const float *d = nullptr;
+    int rc = caller_in(h, a, h->n, &d);
+    if (rc) return rc;
+    k_weights_in<<<nblk(h->n), 256, 0, h->stream>>>(d, h->d_perm, h->n, h->d_p4, h->d_err);
+    rc = check_device_err(h);
+    h->tree_built = false;  // node centres depend on the weights
+    if (rc == DWG_ERR_NONFINITE) h->err = "weights must be finite and > 0";
     return rc;
 }
 
@@ -881,9 +947,10 @@ int dwg_set_regularization(dwg_handle h, int mode, int k, float vmin, float vmax
     if (!h->d_delta2) DWG_CUDA_TRY(h, cudaMalloc(&h->d_delta2, h->n * sizeof(float)));
     if (!h->d_src16)
         DWG_CUDA_TRY(h, cudaMalloc(&h->d_src16, h->npad * kSrcFloatsClamp * sizeof(float)));
+    ScratchScope scope(h);
     float *d_out = nullptr;
     auto run = [&]() -> int {
-        if (delta_out) DWG_CUDA_TRY(h, cudaMalloc(&d_out, h->n * sizeof(float)));
+        if (delta_out) DWG_CUDA_TRY(h, scratch_get(h, &d_out, h->n * sizeof(float)));
         if (launch_clamp_delta(h, k, (double)vmin, (double)vmax, d_out) != cudaSuccess)
             return fail(h, DWG_ERR_CUDA, "clamp radii launch failed");
         int r = check_device_err(h);
@@ -896,7 +963,6 @@ int dwg_set_regularization(dwg_handle h, int mode, int k, float vmin, float vmax
         cudaError_t e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) rc = fail(h, DWG_ERR_CUDA, cudaGetErrorString(e));
     }
-    cudaFree(d_out);
     if (rc) return rc;
     h->reg_mode = mode;
     ++h->delta_gen;  // tree opening radii and group lists depend on the radii
@@ -918,10 +984,11 @@ int dwg_extract_level_set(dwg_handle h, float *tri_out, int64_t cap, int64_t *co
     if (rc) return rc;
     const bool tree = use_tree(h);
     if ((rc = ensure_levelset_buffers(h, tree))) return rc;
+    ScratchScope scope(h);
     unsigned long long *d_cnt = nullptr;
     float *d_tri = nullptr;
     auto body = [&]() -> int {
-        DWG_CUDA_TRY(h, cudaMalloc(&d_cnt, sizeof(unsigned long long)));
+        DWG_CUDA_TRY(h, scratch_get(h, &d_cnt, sizeof(unsigned long long)));
         k_iter_reset<<<1, 1, 0, h->stream>>>(h->d_state, h->max_iters, nullptr);
         LAUNCH_CHECK(h);
         // w at the points -> w_bar; w at the corners
@@ -958,7 +1025,7 @@ int dwg_extract_level_set(dwg_handle h, float *tri_out, int64_t cap, int64_t *co
         if (!tri_out || (int64_t)nt > cap || nt == 0) return check_device_err(h);
         float *dst = tri_out;
         if (!is_device_ptr(tri_out)) {
-            DWG_CUDA_TRY(h, cudaMalloc(&d_tri, nt * 9 * sizeof(float)));
+            DWG_CUDA_TRY(h, scratch_get(h, &d_tri, nt * 9 * sizeof(float)));
             dst = d_tri;
         }
         DWG_CUDA_TRY(h, cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), h->stream));
@@ -973,8 +1040,6 @@ int dwg_extract_level_set(dwg_handle h, float *tri_out, int64_t cap, int64_t *co
     };
     rc = body();
     cudaStreamSynchronize(h->stream);
-    cudaFree(d_cnt);
-    cudaFree(d_tri);
     return rc;
 }
 
@@ -1012,11 +1077,12 @@ int dwg_voronoi_weights(dwg_handle h, int m, float *a_out)
         return DWG_OK;
     }
     int rc;
+    ScratchScope scope(h);
     double *scratch = nullptr;
     float *d_out = nullptr;
     auto run = [&]() -> int {
-        DWG_CUDA_TRY(h, cudaMalloc(&scratch, (h->n + kSumDoubles) * sizeof(double)));
-        if (a_out) DWG_CUDA_TRY(h, cudaMalloc(&d_out, h->n * sizeof(float)));
+        DWG_CUDA_TRY(h, scratch_get(h, &scratch, (h->n + kSumDoubles) * sizeof(double)));
+        if (a_out) DWG_CUDA_TRY(h, scratch_get(h, &d_out, h->n * sizeof(float)));
         if (launch_voronoi_weights(h, m, scratch, d_out) != cudaSuccess)
             return fail(h, DWG_ERR_CUDA, "Voronoi weights launch failed");
         int r = check_device_err(h);
@@ -1030,22 +1096,18 @@ int dwg_voronoi_weights(dwg_handle h, int m, float *a_out)
         cudaError_t e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) rc = fail(h, DWG_ERR_CUDA, cudaGetErrorString(e));
     }
-    cudaFree(scratch);
-    cudaFree(d_out);
     return rc;
 }
 
 static int normals_from_caller(dwg_handle h, const float *normals, float4 *dst)
 {
-    float *d = nullptr;
-    DWG_CUDA_TRY(h, cudaMalloc(&d, h->n * 3 * sizeof(float)));
-    int rc = upload(h, d, normals, h->n * 3 * sizeof(float));
-    if (!rc) {
-        k_normals_in<<<nblk(h->n), 256, 0, h->stream>>>(d, h->d_perm, h->n, dst, h->d_err);
-        rc = check_device_err(h);
-        if (rc == DWG_ERR_NONFINITE) h->err = "normals must be finite and non-zero";
-    }
-    cudaFree(d);
+    ScratchScope scope(h);
+    const float *d = nullptr;
+    int rc = caller_in(h, normals, 3 * h->n, &d);
+    if (rc) return rc;
+    k_normals_in<<<nblk(h->n), 256, 0, h->stream>>>(d, h->d_perm, h->n, dst, h->d_err);
+    rc = check_device_err(h);
+    if (rc == DWG_ERR_NONFINITE) h->err = "normals must be finite and non-zero";
     return rc;
 }
 
@@ -1107,12 +1169,13 @@ int dwg_get_normals(dwg_handle h, float *normals_out)
         int rc = prepare_normals(h);
         if (rc) return rc;
     }
+    ScratchScope scope(h);
     float *d = nullptr;
-    DWG_CUDA_TRY(h, cudaMalloc(&d, h->n * 3 * sizeof(float)));
+    int rc = caller_out(h, normals_out, 3 * h->n, &d);
+    if (rc) return rc;
     k_normals_out<<<nblk(h->n), 256, 0, h->stream>>>(h->d_nrm, h->d_perm, h->n, d);
-    int rc = download(h, normals_out, d, h->n * 3 * sizeof(float));
+    rc = caller_done(h, normals_out, d, 3 * h->n);
     cudaError_t e = cudaStreamSynchronize(h->stream);
-    cudaFree(d);
     if (!rc && e != cudaSuccess) rc = fail(h, DWG_ERR_CUDA, cudaGetErrorString(e));
     return rc;
 }
@@ -1214,21 +1277,20 @@ int dwg_step(dwg_handle h, float *w_out, float *grad_out, float *dtheta_out, dou
     if (iso_out) *iso_out = st.iso;
     if (stat_out) *stat_out = st.stat;
     if (!w_out && !grad_out && !dtheta_out) return DWG_OK;
-    float *d = nullptr;
-    DWG_CUDA_TRY(h, cudaMalloc(&d, h->n * 4 * sizeof(float)));
-    if (w_out || grad_out) {
-        k_wg_out<<<nblk(h->n), 256, 0, h->stream>>>(h->d_wg, h->d_perm, h->n, d, d + h->n);
-        if (w_out && (rc = download(h, w_out, d, h->n * sizeof(float)))) goto out;
-        if (grad_out && (rc = download(h, grad_out, d + h->n, 3 * h->n * sizeof(float)))) goto out;
-    }
-    if (dtheta_out) {
-        DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-        k_scalar_out<<<nblk(h->n), 256, 0, h->stream>>>(h->d_dtheta, h->d_perm, h->n, d);
-        if ((rc = download(h, dtheta_out, d, h->n * sizeof(float)))) goto out;
-    }
-out:
-    cudaStreamSynchronize(h->stream);
-    cudaFree(d);
+    ScratchScope scope(h);
+    const size_t n = (size_t)h->n;
+    float *w = nullptr, *g = nullptr, *d = nullptr;
+    if (w_out && (rc = caller_out(h, w_out, n, &w))) return rc;
+    if (grad_out && (rc = caller_out(h, grad_out, 3 * n, &g))) return rc;
+    if (dtheta_out && (rc = caller_out(h, dtheta_out, n, &d))) return rc;
+    if (w || g) k_wg_out<<<nblk(h->n), 256, 0, h->stream>>>(h->d_wg, h->d_perm, h->n, w, g);
+    if (d) k_scalar_out<<<nblk(h->n), 256, 0, h->stream>>>(h->d_dtheta, h->d_perm, h->n, d);
+    LAUNCH_CHECK(h);
+    if (w_out) rc = caller_done(h, w_out, w, n);
+    if (!rc && grad_out) rc = caller_done(h, grad_out, g, 3 * n);
+    if (!rc && dtheta_out) rc = caller_done(h, dtheta_out, d, n);
+    const cudaError_t e = cudaStreamSynchronize(h->stream);
+    if (!rc && e != cudaSuccess) rc = fail(h, DWG_ERR_CUDA, cudaGetErrorString(e));
     return rc;
 }
 
@@ -1279,56 +1341,48 @@ int dwg_eval_gwn(dwg_handle h, const float *queries, int64_t m, float *w_out, fl
     cudaSetDevice(h->device);
     int rc;
     if ((rc = prepare_normals(h))) return rc;
-    bool grad = grad_out != nullptr;
-    float *qx = nullptr, *part = nullptr, *o = nullptr;
-    float4 *q4 = nullptr, *wg = nullptr;
-    auto body = [&]() -> int {
-        DWG_CUDA_TRY(h, cudaMalloc(&qx, m * 3 * sizeof(float)));
-        if ((rc = upload(h, qx, queries, m * 3 * sizeof(float)))) return rc;
-        if (launch_check_finite(qx, 3 * m, h->d_err, h->stream) != cudaSuccess)
-            return fail(h, DWG_ERR_CUDA, "finite-check launch failed");
+    const bool grad = grad_out != nullptr;
+    const bool tree = use_tree(h);
+    ScratchScope scope(h);
+    const float *qx = nullptr;
+    float *part = nullptr, *w = nullptr, *g = nullptr;
+    float4 *q4 = nullptr;
+    if ((rc = caller_in(h, queries, 3 * m, &qx))) return rc;
+    DWG_CUDA_TRY(h, scratch_get(h, &q4, m * sizeof(float4)));
+    k_queries_in<<<nblk(m), 256, 0, h->stream>>>(qx, m, q4, h->d_err);
+    LAUNCH_CHECK(h);
+    const int nch = tree ? 1 : eval_chunks(h, m, grad);
+    DWG_CUDA_TRY(h, scratch_get(h, &part, (size_t)nch * (grad ? 8 : 2) * m * sizeof(float)));
+    if ((rc = caller_out(h, w_out, m, &w))) return rc;
+    if (grad && (rc = caller_out(h, grad_out, 3 * m, &g))) return rc;
+    if (tree) {
+        // no walk for queries that are not finite; the exact sums run for
+        // them too and are not written, which saves a wait
         if ((rc = check_device_err(h))) return rc;
-        DWG_CUDA_TRY(h, cudaMalloc(&q4, m * sizeof(float4)));
-        k_xyz_to_f4<<<nblk(m), 256, 0, h->stream>>>(qx, m, q4);
-        const bool tree = use_tree(h);
-        int nch = tree ? 1 : eval_chunks(h, m, grad);
-        DWG_CUDA_TRY(h, cudaMalloc(&part, (size_t)nch * (grad ? 8 : 2) * m * sizeof(float)));
-        if (tree) {
-            if ((rc = build_tree(h)) || (rc = tree_records(h))) return rc;
-            DWG_CUDA_TRY(h, cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned long long), h->stream));
-            if (launch_tree_moments(h) != cudaSuccess ||
-                launch_tree_gwn(h, q4, m, grad, part, m, nullptr) != cudaSuccess)
-                return fail(h, DWG_ERR_CUDA, "tree launch failed");
-        } else if ((rc = eval_launch(h, q4, m, grad, nch, part, m))) {
-            return rc;
-        }
-        DWG_CUDA_TRY(h, cudaMalloc(&wg, m * sizeof(float4)));
-        if (launch_reduce_points(h, part, nch, m, q4, grad ? 2 : 0, grad, wg, nullptr) !=
-            cudaSuccess)
-            return fail(h, DWG_ERR_CUDA, "reduce launch failed");
-        DWG_CUDA_TRY(h, cudaMalloc(&o, m * 4 * sizeof(float)));
-        k_wg_out<<<nblk(m), 256, 0, h->stream>>>(wg, nullptr, m, o, grad ? o + m : nullptr);
-        if ((rc = download(h, w_out, o, m * sizeof(float)))) return rc;
-        if (grad && (rc = download(h, grad_out, o + m, 3 * m * sizeof(float)))) return rc;
+        if ((rc = build_tree(h)) || (rc = tree_records(h))) return rc;
+        DWG_CUDA_TRY(h, cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned long long), h->stream));
+        if (launch_tree_moments(h) != cudaSuccess ||
+            launch_tree_gwn(h, q4, m, grad, part, m, nullptr) != cudaSuccess)
+            return fail(h, DWG_ERR_CUDA, "tree launch failed");
+    } else if ((rc = eval_launch(h, q4, m, grad, nch, part, m))) {
+        return rc;
+    }
+    if (launch_reduce_eval(h, part, nch, m, q4, w, g) != cudaSuccess)
+        return fail(h, DWG_ERR_CUDA, "reduce launch failed");
+    h->stats.interactions_eval = (double)m * (double)h->n;
+    if (tree) {
+        unsigned long long cnt = 0;
+        DWG_CUDA_TRY(h, cudaMemcpyAsync(&cnt, h->d_counter, sizeof(cnt), cudaMemcpyDeviceToHost,
+                                        h->stream));
         DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-        h->stats.interactions_eval = (double)m * (double)h->n;
-        if (tree) {
-            unsigned long long cnt = 0;
-            DWG_CUDA_TRY(h, cudaMemcpyAsync(&cnt, h->d_counter, sizeof(cnt), cudaMemcpyDeviceToHost,
-                                            h->stream));
-            DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-            h->stats.interactions_eval = (double)cnt;
-        }
-        return check_device_err(h);
-    };
-    rc = body();
-    cudaStreamSynchronize(h->stream);
-    cudaFree(qx);
-    cudaFree(q4);
-    cudaFree(part);
-    cudaFree(wg);
-    cudaFree(o);
-    return rc;
+        h->stats.interactions_eval = (double)cnt;
+    }
+    if ((rc = check_device_err(h))) return rc;
+    if (w == w_out && g == grad_out) return DWG_OK;
+    if ((rc = caller_done(h, w_out, w, m))) return rc;
+    if (grad && (rc = caller_done(h, grad_out, g, 3 * m))) return rc;
+    DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    return DWG_OK;
 }
 
 int dwg_autotune(dwg_handle h, int what, double w_budget, const char *cache_path,
@@ -1503,22 +1557,18 @@ int dwg_mlp_features(dwg_handle h, float *X_out)
     if (!h || !X_out) return DWG_ERR_INVALID;
     if (h->is_batch) return fail(h, DWG_ERR_STATE, "not on a batch handle");
     cudaSetDevice(h->device);
+    ScratchScope scope(h);
+    const size_t count = (size_t)h->n * 64;
     float *X = nullptr;
     double *cR = nullptr;
-    auto run = [&]() -> int {
-        DWG_CUDA_TRY(h, cudaMalloc(&X, h->n * 64 * sizeof(float)));
-        DWG_CUDA_TRY(h, cudaMalloc(&cR, kSumDoubles * sizeof(double)));
-        if (launch_features(h, X, true, cR) != cudaSuccess)
-            return fail(h, DWG_ERR_CUDA, "features launch failed");
-        int rc = download(h, X_out, X, h->n * 64 * sizeof(float));
-        if (rc) return rc;
-        DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-        return check_device_err(h);
-    };
-    int rc = run();
-    cudaFree(X);
-    cudaFree(cR);
-    return rc;
+    int rc = caller_out(h, X_out, count, &X);
+    if (rc) return rc;
+    DWG_CUDA_TRY(h, scratch_get(h, &cR, kSumDoubles * sizeof(double)));
+    if (launch_features(h, X, true, cR) != cudaSuccess)
+        return fail(h, DWG_ERR_CUDA, "features launch failed");
+    if ((rc = caller_done(h, X_out, X, count))) return rc;
+    DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    return check_device_err(h);
 }
 
 static int mlp_check(std::initializer_list<const void *> ptrs, int64_t B)
@@ -1565,14 +1615,18 @@ int dwg_mlp_grad(const float *params, const float *X, const float *T, int64_t B,
     int rc = mlp_check({params, X, T, grad}, B);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    double *dl = nullptr;
-    cudaError_t e = cudaMallocAsync(&dl, sizeof(double), s);
+    double *dl = nullptr, hl = 0.0;
+    const int slot = mlp_loss_slot(&dl);  // -1: all taken (calls from many threads)
+    cudaError_t e = slot < 0 ? cudaMallocAsync(&dl, sizeof(double), s) : cudaSuccess;
     if (e == cudaSuccess) e = launch_mlp_grad(params, X, T, B, grad, dl, s);
-    double hl = 0.0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hl, dl, sizeof(double), cudaMemcpyDeviceToHost, s);
     rc = mlp_finish(e, s);
-    cudaFreeAsync(dl, s);
-    cudaStreamSynchronize(s);
+    if (slot >= 0) {
+        mlp_loss_release(slot);
+    } else {
+        cudaFreeAsync(dl, s);
+        cudaStreamSynchronize(s);
+    }
     if (loss) *loss = hl;
     return rc;
 }
@@ -1595,28 +1649,22 @@ int dwg_knn(dwg_handle h, const float *queries, int64_t m, int k, int64_t *idx_o
     if (!h || !queries || !idx_out) return DWG_ERR_INVALID;
     if (m < 1 || k < 1 || k > kMaxK) return fail(h, DWG_ERR_INVALID, "need m >= 1, 1 <= k <= 32");
     cudaSetDevice(h->device);
-    float *qx = nullptr;
+    ScratchScope scope(h);
+    const float *qx = nullptr;
     float4 *q4 = nullptr;
-    int64_t *idx = nullptr;
-    int rc;
-    auto body = [&]() -> int {
-        DWG_CUDA_TRY(h, cudaMalloc(&qx, m * 3 * sizeof(float)));
-        if ((rc = upload(h, qx, queries, m * 3 * sizeof(float)))) return rc;
-        DWG_CUDA_TRY(h, cudaMalloc(&q4, m * sizeof(float4)));
-        k_xyz_to_f4<<<nblk(m), 256, 0, h->stream>>>(qx, m, q4);
-        DWG_CUDA_TRY(h, cudaMalloc(&idx, m * k * sizeof(int64_t)));
-        if (launch_knn_query(h, q4, m, k, idx) != cudaSuccess)
-            return fail(h, DWG_ERR_CUDA, "knn launch failed");
-        if ((rc = download(h, idx_out, idx, m * k * sizeof(int64_t)))) return rc;
-        DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-        return check_device_err(h);
-    };
-    rc = body();
-    cudaStreamSynchronize(h->stream);
-    cudaFree(qx);
-    cudaFree(q4);
-    cudaFree(idx);
-    return rc;
+    int64_t *idx = idx_out;
+    int rc = caller_in(h, queries, 3 * m, &qx);
+    if (rc) return rc;
+    DWG_CUDA_TRY(h, scratch_get(h, &q4, m * sizeof(float4)));
+    k_xyz_to_f4<<<nblk(m), 256, 0, h->stream>>>(qx, m, q4);
+    if (is_device_ptr(idx_out)) DWG_CUDA_TRY(h, join_caller(h));
+    if (!kernel_ptr(idx_out, sizeof(int64_t)))
+        DWG_CUDA_TRY(h, scratch_get(h, &idx, m * k * sizeof(int64_t)));
+    if (launch_knn_query(h, q4, m, k, idx) != cudaSuccess)
+        return fail(h, DWG_ERR_CUDA, "knn launch failed");
+    if (idx != idx_out && (rc = download(h, idx_out, idx, m * k * sizeof(int64_t)))) return rc;
+    DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    return check_device_err(h);
 }
 
 // ---------------------------------------------------------------------------

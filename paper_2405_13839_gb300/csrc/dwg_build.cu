@@ -181,17 +181,15 @@ int scan_i64(Ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *d_tota
     if (nb == 1) {
         k_scan_block<<<1, kScanBlock, 0, c->stream>>>(in, out, n, nullptr);
     } else {
+        ScratchScope scope(c);
         int64_t *sums = nullptr, *soffs = nullptr, *stot = nullptr;
-        DWG_CUDA_TRY(c, cudaMallocAsync(&sums, nb * sizeof(int64_t), c->stream));
-        DWG_CUDA_TRY(c, cudaMallocAsync(&soffs, nb * sizeof(int64_t), c->stream));
-        DWG_CUDA_TRY(c, cudaMallocAsync(&stot, sizeof(int64_t), c->stream));
+        DWG_CUDA_TRY(c, scratch_get(c, &sums, nb * sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &soffs, nb * sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &stot, sizeof(int64_t)));
         k_scan_block<<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, out, n, sums);
         int rc = scan_i64(c, sums, soffs, nb, stot);
         if (rc) return rc;
         k_scan_add<<<(unsigned)ceil_div(n, 256), 256, 0, c->stream>>>(out, n, soffs);
-        cudaFreeAsync(sums, c->stream);
-        cudaFreeAsync(soffs, c->stream);
-        cudaFreeAsync(stot, c->stream);
     }
     k_scan_total<<<1, 1, 0, c->stream>>>(in, out, n, d_total);
     DWG_CUDA_TRY(c, cudaGetLastError());
@@ -269,11 +267,12 @@ int radix_sort_pairs(Ctx *c, uint64_t *keys, int64_t *vals, int64_t n, int key_b
     int nblocks = (int)ceil_div(n, kSortItems);
     uint64_t *k2 = nullptr;
     int64_t *v2 = nullptr, *hist = nullptr, *offs = nullptr, *tot = nullptr;
-    DWG_CUDA_TRY(c, cudaMallocAsync(&k2, n * sizeof(uint64_t), c->stream));
-    DWG_CUDA_TRY(c, cudaMallocAsync(&v2, n * sizeof(int64_t), c->stream));
-    DWG_CUDA_TRY(c, cudaMallocAsync(&hist, (int64_t)256 * nblocks * sizeof(int64_t), c->stream));
-    DWG_CUDA_TRY(c, cudaMallocAsync(&offs, (int64_t)256 * nblocks * sizeof(int64_t), c->stream));
-    DWG_CUDA_TRY(c, cudaMallocAsync(&tot, sizeof(int64_t), c->stream));
+    ScratchScope scope(c);
+    DWG_CUDA_TRY(c, scratch_get(c, &k2, n * sizeof(uint64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &v2, n * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &hist, (int64_t)256 * nblocks * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &offs, (int64_t)256 * nblocks * sizeof(int64_t)));
+    DWG_CUDA_TRY(c, scratch_get(c, &tot, sizeof(int64_t)));
     uint64_t *ka = keys, *kb = k2;
     int64_t *va = vals, *vb = v2;
     int passes = (key_bits + 7) / 8;
@@ -294,11 +293,6 @@ int radix_sort_pairs(Ctx *c, uint64_t *keys, int64_t *vals, int64_t n, int key_b
         DWG_CUDA_TRY(c, cudaMemcpyAsync(vals, va, n * sizeof(int64_t), cudaMemcpyDeviceToDevice,
                                         c->stream));
     }
-    cudaFreeAsync(k2, c->stream);
-    cudaFreeAsync(v2, c->stream);
-    cudaFreeAsync(hist, c->stream);
-    cudaFreeAsync(offs, c->stream);
-    cudaFreeAsync(tot, c->stream);
     DWG_CUDA_TRY(c, cudaGetLastError());
     return DWG_OK;
 }
@@ -534,14 +528,15 @@ int build_discretization(Ctx *c, int d)
     uint64_t *keys = nullptr;
     int64_t *slots = nullptr, *kf = nullptr, *kp = nullptr;
 
+    ScratchScope scope(c);
     auto body = [&]() -> int {
-        DWG_CUDA_TRY(c, cudaMalloc(&flags, n * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&pos, n * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&cnt, n * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&tot, sizeof(int64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&nodes_a, n * sizeof(uint64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&nodes_b, n * sizeof(uint64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&mask, n * sizeof(unsigned)));
+        DWG_CUDA_TRY(c, scratch_get(c, &flags, n * sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &pos, n * sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &cnt, n * sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &tot, sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &nodes_a, n * sizeof(uint64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &nodes_b, n * sizeof(uint64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &mask, n * sizeof(unsigned)));
 
         // unique level-l prefixes of the sorted codes, in Morton order
         auto level_nodes = [&](int lvl, uint64_t *out, int64_t &cntn) -> int {
@@ -590,10 +585,10 @@ int build_discretization(Ctx *c, int d)
 
         // distinct corners: sort the 8 corner keys of every leaf, keep the first of each run
         int64_t m = nleaves * 8;
-        DWG_CUDA_TRY(c, cudaMalloc(&keys, m * sizeof(uint64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&slots, m * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&kf, m * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, cudaMalloc(&kp, m * sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &keys, m * sizeof(uint64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &slots, m * sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &kf, m * sizeof(int64_t)));
+        DWG_CUDA_TRY(c, scratch_get(c, &kp, m * sizeof(int64_t)));
         k_corner_keys<<<(unsigned)ceil_div(m, B), B, 0, c->stream>>>(leaves, nleaves, d, keys,
                                                                       slots);
         int rc = radix_sort_pairs(c, keys, slots, m, 3 * (d + 1));
@@ -625,18 +620,7 @@ int build_discretization(Ctx *c, int d)
         return DWG_OK;
     };
     int rc = body();
-    cudaFree(keys);
-    cudaFree(slots);
-    cudaFree(kf);
-    cudaFree(kp);
     cudaFree(leaves);
-    cudaFree(flags);
-    cudaFree(pos);
-    cudaFree(cnt);
-    cudaFree(tot);
-    cudaFree(nodes_a);
-    cudaFree(nodes_b);
-    cudaFree(mask);
     if (rc) free_disc(c);
     return rc;
 }

@@ -960,7 +960,10 @@ __device__ __forceinline__ void reduce_points_body(const float *__restrict__ par
                                                    const uint64_t *__restrict__ codes,
                                                    int64_t nsrc, int self_mode, const CubeQ &cq,
                                                    const EvalParams &ep, float4 *__restrict__ out,
-                                                   double *__restrict__ wsum_blocks, int64_t bid)
+                                                   double *__restrict__ wsum_blocks, int64_t bid,
+                                                   float *__restrict__ w_raw = nullptr,
+                                                   float *__restrict__ g_raw = nullptr,
+                                                   const int *__restrict__ err = nullptr)
 {
     constexpr int NA = GRAD ? 4 : 1;
     int64_t i = bid * blockDim.x + threadIdx.x;
@@ -1028,7 +1031,16 @@ __device__ __forceinline__ void reduce_points_body(const float *__restrict__ par
             o.y = __fadd_rn(h[2], l[2]);
             o.z = __fadd_rn(h[3], l[3]);
         }
-        out[i] = o;
+        if (out) {
+            out[i] = o;
+        } else if (!(*err & kErrNonfinite)) {  // a caller's arrays: not for invalid queries
+            w_raw[i] = o.w;
+            if (GRAD) {
+                g_raw[3 * i] = o.x;
+                g_raw[3 * i + 1] = o.y;
+                g_raw[3 * i + 2] = o.z;
+            }
+        }
         wloc = (double)h[0] + (double)l[0];
     }
     if (wsum_blocks) {
@@ -1054,6 +1066,18 @@ __global__ void k_reduce_points(const float *__restrict__ part, int nchunks, int
 {
     reduce_points_body<GRAD>(part, nchunks, m, stride, q, src, rec_floats, codes, nsrc,
                              self_mode, cq, ep, out, wsum_blocks, blockIdx.x);
+}
+
+// the queries of dwg_eval_gwn: straight into the caller's layout
+template <bool GRAD>
+__global__ void k_reduce_eval(const float *__restrict__ part, int nchunks, int64_t m,
+                              const float4 *__restrict__ q, const float *__restrict__ src,
+                              int rec_floats, const uint64_t *__restrict__ codes, int64_t nsrc,
+                              CubeQ cq, EvalParams ep, float *__restrict__ w_raw,
+                              float *__restrict__ g_raw, const int *__restrict__ err)
+{
+    reduce_points_body<GRAD>(part, nchunks, m, m, q, src, rec_floats, codes, nsrc, GRAD ? 2 : 0, cq,
+                             ep, nullptr, nullptr, blockIdx.x, w_raw, g_raw, err);
 }
 
 int wsum_block_count(int64_t n) { return (int)ceil_div(n, 256); }
@@ -1173,6 +1197,28 @@ cudaError_t launch_reduce_points(Ctx *c, const float *part, int nchunks, int64_t
         k_reduce_points<false><<<blocks, 256, 0, c->stream>>>(part, nchunks, m, m, queries, src,
                                                               recf, c->d_codes, c->n, 0, cq, ep,
                                                               out, wsum_blocks);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reduce_eval(Ctx *c, const float *part, int nchunks, int64_t m,
+                               const float4 *queries, float *w, float *g)
+{
+    CubeQ cq;
+    for (int k = 0; k < 3; ++k) cq.lo[k] = c->cube_lo[k];
+    cq.inv_h21 = (double)(1 << kMortonBits) / c->cube_L;
+    const EvalParams ep = make_eval_params(c);
+    const unsigned blocks = (unsigned)ceil_div(m, 256);
+    const bool clamp = c->reg_mode == DWG_REG_CLAMP;
+    const float *src = clamp ? c->d_src16 : c->d_src;
+    const int recf = clamp ? kSrcFloatsClamp : kSrcFloats;
+    if (g)
+        k_reduce_eval<true><<<blocks, 256, 0, c->stream>>>(part, nchunks, m, queries, src, recf,
+                                                           c->d_codes, c->n, cq, ep, w, g,
+                                                           c->d_err);
+    else
+        k_reduce_eval<false><<<blocks, 256, 0, c->stream>>>(part, nchunks, m, queries, src, recf,
+                                                            c->d_codes, c->n, cq, ep, w, nullptr,
+                                                            c->d_err);
     return cudaGetLastError();
 }
 

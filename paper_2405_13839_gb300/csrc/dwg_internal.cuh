@@ -252,6 +252,7 @@ struct ScratchBlock {
 struct Scratch {
     std::vector<ScratchBlock> blocks;
     int depth = 0;
+    bool joined = false;  // this call has waited for the device (join_caller)
 };
 constexpr size_t kScratchKeep = (size_t)256 << 20;
 
@@ -473,6 +474,11 @@ cudaError_t launch_pack_sources(const float4 *p4, const float4 *nrm, int64_t n, 
 cudaError_t launch_reduce_points(Ctx *c, const float *part, int nchunks, int64_t m,
                                  const float4 *queries, int self_mode, bool grad, float4 *out,
                                  double *wsum_blocks);
+// w (and grad w unless null) of arbitrary queries into device arrays in the
+// caller's layout; nothing is written once the device error word says that a
+// query was not finite
+cudaError_t launch_reduce_eval(Ctx *c, const float *part, int nchunks, int64_t m,
+                               const float4 *queries, float *w, float *g);
 cudaError_t launch_reduce_w(Ctx *c, const float *part, int nchunks, int64_t m, float *out);
 // w at the octree's leaf corners by the exact path: the lattice tasks with
 // the softened, compensated kernel, else the general evaluator.  Partial sums
@@ -496,16 +502,21 @@ cudaError_t launch_reduce_w_raw(const float *part, int nchunks, int64_t m, float
 
 // dwg_api.cu
 // a block of the handle's scratch, held until the innermost ScratchScope ends
-// (which waits for the handle's stream first)
+// (the work of a handle is ordered on its stream, so a block handed out again
+// is only written after what read it before)
 cudaError_t scratch_get(Ctx *c, void **p, size_t bytes);
 template <class T>
 inline cudaError_t scratch_get(Ctx *c, T **p, size_t bytes)
 {
     return scratch_get(c, reinterpret_cast<void **>(p), bytes);
 }
+void scratch_trim(Ctx *c, size_t keep);
 struct ScratchScope {
     Ctx *c;
-    explicit ScratchScope(Ctx *c_) : c(c_) { ++c->scratch.depth; }
+    explicit ScratchScope(Ctx *c_) : c(c_)
+    {
+        if (++c->scratch.depth == 1) c->scratch.joined = false;
+    }
     ~ScratchScope();
     ScratchScope(const ScratchScope &) = delete;
     ScratchScope &operator=(const ScratchScope &) = delete;
@@ -608,6 +619,10 @@ constexpr int kMlpParamCount = 12675;
 cudaError_t launch_mlp_forward(const float *P, const float *X, int64_t B, float *Y, cudaStream_t s,
                                int *err);
 int mlp_forward_error(cudaStream_t s);
+// a device double for one dwg_mlp_grad call on the current device (its slot,
+// -1: none free); the caller releases it after its stream has finished
+int mlp_loss_slot(double **d);
+void mlp_loss_release(int slot);
 cudaError_t launch_mlp_grad(const float *P, const float *X, const float *T, int64_t B, float *grad,
                             double *loss, cudaStream_t s);
 cudaError_t launch_adam(float *p, const float *g, float *m, float *v, int step, float lr,

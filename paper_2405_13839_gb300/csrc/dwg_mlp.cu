@@ -26,6 +26,8 @@
 //   k_normals_from_y  normalise the network output into initial normals.
 #include <cuda_bf16.h>
 
+#include <mutex>
+
 #include "dwg_internal.cuh"
 
 namespace dwg {
@@ -665,6 +667,39 @@ static int mlp_sms()
 
 // device flag for the forward calls that have no handle (dwg_mlp_forward)
 static __device__ int g_mlp_err;
+
+// Device doubles for the losses of calls that run at the same time (threads,
+// streams), a slot per call: allocating one for each call took most of a
+// small training step (the default pool returns its memory at every wait).
+constexpr int kLossSlots = 64;
+static __device__ double g_mlp_loss[kLossSlots];
+static std::mutex g_loss_mu;
+static uint64_t g_loss_busy[64];  // per device
+
+int mlp_loss_slot(double **d)
+{
+    int dev = 0;
+    void *base = nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 ||
+        cudaGetSymbolAddress(&base, g_mlp_loss) != cudaSuccess) {
+        cudaGetLastError();
+        return -1;
+    }
+    std::lock_guard<std::mutex> lk(g_loss_mu);
+    for (int i = 0; i < kLossSlots; ++i)
+        if (!(g_loss_busy[dev] >> i & 1u)) {
+            g_loss_busy[dev] |= (uint64_t)1 << i;
+            *d = static_cast<double *>(base) + i;
+            return dev * kLossSlots + i;
+        }
+    return -1;
+}
+
+void mlp_loss_release(int slot)
+{
+    std::lock_guard<std::mutex> lk(g_loss_mu);
+    g_loss_busy[slot / kLossSlots] &= ~((uint64_t)1 << (slot % kLossSlots));
+}
 
 cudaError_t launch_mlp_forward(const float *P, const float *X, int64_t B, float *Y, cudaStream_t s,
                                int *err)
