@@ -1361,9 +1361,9 @@ int dwg_eval_gwn(dwg_handle h, const float *queries, int64_t m, float *w_out, fl
         if ((rc = check_device_err(h))) return rc;
         if ((rc = build_tree(h)) || (rc = tree_records(h))) return rc;
         DWG_CUDA_TRY(h, cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned long long), h->stream));
-        if (launch_tree_moments(h) != cudaSuccess ||
-            launch_tree_gwn(h, q4, m, grad, part, m, nullptr) != cudaSuccess)
+        if (launch_tree_moments(h) != cudaSuccess)
             return fail(h, DWG_ERR_CUDA, "tree launch failed");
+        if ((rc = tree_eval_call(h, q4, m, grad, part, m))) return rc;
     } else if ((rc = eval_launch(h, q4, m, grad, nch, part, m))) {
         return rc;
     }

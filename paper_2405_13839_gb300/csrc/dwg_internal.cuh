@@ -208,6 +208,7 @@ struct CloudIter {
     const int *far_ids[2], *near_ids[2];
     const int2 *items[2];
     int64_t nitems[2];
+    int irec[2];
     float *ipart[2];
     float *lpart[2];              // the reduce's chunk-0 partials
 };
@@ -236,6 +237,7 @@ struct TreeLists {
     int2 *d_items = nullptr;
     float *d_ipart = nullptr;
     int64_t nitems = 0;
+    int irec = 0;                    // records of an item
     bool valid = false;
 };
 
@@ -540,6 +542,8 @@ cudaError_t launch_tree_moments(Ctx *c);
 // st: loop state whose end makes the kernel skip its work (NULL: always run)
 cudaError_t launch_tree_gwn(Ctx *c, const float4 *q, int64_t m, bool grad, float *part,
                             int64_t stride, const IterState *st);
+// the queries of one call (dwg_eval_gwn): chunk-0 partials as launch_tree_gwn
+int tree_eval_call(Ctx *c, const float4 *q, int64_t m, bool grad, float *part, int64_t stride);
 // the interaction lists of a query set (group test); *built = false when the
 // lists would not fit in device memory (the walk then runs every iteration)
 int tree_lists(Ctx *c, TreeLists &L, const float4 *q, int64_t m, bool *built);

@@ -2453,6 +2453,7 @@ void fill_cloud_iter(const Ctx *c, CloudIter *o)
         o->near_ids[w] = L[w]->d_near;
         o->items[w] = L[w]->d_items;
         o->nitems[w] = L[w]->nitems;
+        o->irec[w] = L[w]->irec;
         o->ipart[w] = L[w]->d_ipart;
         o->lpart[w] = lp[w];
     }

@@ -227,6 +227,16 @@ __global__ void k_tree_level_moments(int64_t first, double *M)
     level_moments_body(first, M, blockIdx.x);
 }
 
+// the levels of at most 1,024 nodes, from `level` up to the root, by one
+// block: a launch a level took 2.7 us each
+__global__ void __launch_bounds__(1024) k_tree_top_moments(int level, double *M)
+{
+    for (int lv = level; lv >= 0; --lv) {
+        level_moments_body((int64_t)1 << lv, M, 0);
+        __syncthreads();
+    }
+}
+
 // m = M / (4 pi) as float; frec (may be NULL): the node as a 48-byte source
 // record (c and m, each value twice) like the point records, for the list
 // evaluation's bulk copies
@@ -605,9 +615,10 @@ __device__ __forceinline__ GrpQueries grp_queries(const float4 *__restrict__ q, 
 
 // One warp walks the tree for its group, 32 nodes per step (one per lane).
 // A node far from the group's box goes to on_far, a near leaf to on_near,
-// an open node pushes its children.  on_far(is_far, node, record, mask) is
-// called by every lane each step (warp-uniform); on_near(leaf) once per
-// near leaf, by every lane.  Returns false if the stack would overflow.
+// an open node pushes its children.  on_far(is_far, node, record, mask) and
+// on_near(is_near, leaf, mask) are called by every lane, on_far each step
+// and on_near where the mask is not empty (both warp-uniform).  Returns
+// false if the stack would overflow.
 template <class FarFn, class NearFn>
 __device__ __forceinline__ bool grp_walk(int *stack, const float4 *__restrict__ rec,
                                          int64_t nleaf, const GrpQueries &G, int lane,
@@ -644,12 +655,8 @@ __device__ __forceinline__ bool grp_walk(int *stack, const float4 *__restrict__ 
             stack[pos + 1] = 2 * node;
         }
         sp += 2 * no;
-        unsigned nm = __ballot_sync(0xffffffffu, act == 2);
-        while (nm) {
-            const int leader = __ffs(nm) - 1;
-            nm &= nm - 1;
-            on_near(__shfl_sync(0xffffffffu, node, leader));
-        }
+        const unsigned nm = __ballot_sync(0xffffffffu, act == 2);
+        if (nm) on_near(act == 2, node, nm);
         __syncwarp();
     }
     return true;
@@ -752,10 +759,14 @@ __global__ void __launch_bounds__(32 * kGrpWarps)
             }
             far_cnt += nf;
         },
-        [&](int leaf) {
-            const int64_t j0 = ((int64_t)leaf - nleaf) * bucket;
-            grp_take_leaf(src4, j0, (int)min((int64_t)bucket, n - j0), nearb, near_cnt, lane,
-                          flush_near);
+        [&](bool, int node, unsigned nm) {
+            while (nm) {
+                const int leaf = __shfl_sync(0xffffffffu, node, __ffs(nm) - 1);
+                nm &= nm - 1;
+                const int64_t j0 = ((int64_t)leaf - nleaf) * bucket;
+                grp_take_leaf(src4, j0, (int)min((int64_t)bucket, n - j0), nearb, near_cnt, lane,
+                              flush_near);
+            }
         });
     if (!ok) {
         if (lane == 0) atomicOr(err, kErrStack);
@@ -799,9 +810,9 @@ __global__ void __launch_bounds__(32 * kListWarps)
             if (FILL && is_far) far_ids[nf + __popc(fm & lt)] = node;
             nf += __popc(fm);
         },
-        [&](int leaf) {
-            if (FILL && lane == 0) near_ids[nn] = leaf;
-            ++nn;
+        [&](bool is_near, int leaf, unsigned nm) {
+            if (FILL && is_near) near_ids[nn + __popc(nm & lt)] = leaf;
+            nn += __popc(nm);
         });
     if (!ok) {
         if (lane == 0) atomicOr(err, kErrStack);
@@ -842,24 +853,36 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // one warp busy long after the rest of the grid has finished).  Each item
 // writes its (hi, lo) sums for the group's 64 queries; k_tree_combine adds
 // the items of a group in order (deterministic).
+// An item has kItemRecords records, half or a quarter of that where the items
+// of a launch would be fewer than eight or four per resident warp (300,000
+// sources at 110,592 queries, 4,537 items on 2,432 places: 556 -> 473 us as
+// 15,768 items).
 constexpr int kItemRecords = 2048;
 
+__host__ __device__ static int item_records(int64_t records, int64_t ng)
+{
+    const int64_t places = (int64_t)152 * 16;
+    const int64_t items = records / kItemRecords + ng / 2;
+    return items < 4 * places ? kItemRecords / 4 : items < 8 * places ? kItemRecords / 2
+                                                                     : kItemRecords;
+}
+
 __global__ void k_tree_items(const int64_t *__restrict__ far_off, const int64_t *__restrict__ near_off,
-                             int64_t ng, int bucket, int64_t *__restrict__ cnt)
+                             int64_t ng, int bucket, int irec, int64_t *__restrict__ cnt)
 {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ng) return;
     const int64_t total = (far_off[g + 1] - far_off[g]) + (near_off[g + 1] - near_off[g]) * bucket;
-    cnt[g] = max((int64_t)1, (total + kItemRecords - 1) / kItemRecords);
+    cnt[g] = max((int64_t)1, (total + irec - 1) / irec);
 }
 
-__global__ void k_tree_item_table(const int64_t *__restrict__ item_off, int64_t ng,
+__global__ void k_tree_item_table(const int64_t *__restrict__ item_off, int64_t ng, int irec,
                                   int2 *__restrict__ items)
 {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ng) return;
     for (int64_t i = item_off[g], j = 0; i < item_off[g + 1]; ++i, ++j)
-        items[i] = make_int2((int)g, (int)(j * kItemRecords));
+        items[i] = make_int2((int)g, (int)(j * irec));
 }
 
 // Why the warp is split.  On sm_103a a packed f32x2 instruction takes two
@@ -881,7 +904,7 @@ __device__ __forceinline__ void eval_lists_body(
     const float *__restrict__ src, int64_t n, int levels, int bucket,
     const int64_t *__restrict__ far_off, const int *__restrict__ far_ids,
     const int64_t *__restrict__ near_off, const int *__restrict__ near_ids,
-    const int2 *__restrict__ items, int64_t nitems, const EvalParams &ep,
+    const int2 *__restrict__ items, int64_t nitems, int irec, const EvalParams &ep,
     float *__restrict__ ipart, unsigned long long *__restrict__ counter, const IterState *st,
     int64_t it)
 {
@@ -920,7 +943,7 @@ __device__ __forceinline__ void eval_lists_body(
     const int lg_bucket = __ffs(bucket) - 1;  // leaf sizes are powers of two
     const int *fi = far_ids + f0, *ni = near_ids + e0;
     const int r_begin = item.y;
-    const int total = (int)min((int64_t)kItemRecords,
+    const int total = (int)min((int64_t)irec,
                                (int64_t)nf + (int64_t)ne * bucket - r_begin);
     const int nsuper = (total + P * kLstChunk - 1) / (P * kLstChunk);
     const int tail = min(total - (nsuper - 1) * P * kLstChunk, kLstChunk);
@@ -1067,13 +1090,13 @@ __global__ void __launch_bounds__(32, CLAMP ? (GRAD ? 12 : 16) : lst_resident(GR
                       const float *__restrict__ src, int64_t n, int levels, int bucket,
                       const int64_t *__restrict__ far_off, const int *__restrict__ far_ids,
                       const int64_t *__restrict__ near_off, const int *__restrict__ near_ids,
-                      const int2 *__restrict__ items, int64_t nitems, EvalParams ep,
+                      const int2 *__restrict__ items, int64_t nitems, int irec, EvalParams ep,
                       float *__restrict__ ipart, unsigned long long *__restrict__ counter,
                       const IterState *st)
 {
     eval_lists_body<GRAD, SCREENED, CLAMP>(q, m, frec, src, n, levels, bucket, far_off, far_ids,
-                                           near_off, near_ids, items, nitems, ep, ipart, counter,
-                                           st, blockIdx.x);
+                                           near_off, near_ids, items, nitems, irec, ep, ipart,
+                                           counter, st, blockIdx.x);
 }
 
 // per query: the items of its group added in order (two-sum on the hi
@@ -1196,8 +1219,10 @@ int tree_lists(Ctx *c, TreeLists &L, const float4 *q, int64_t m, bool *built)
         size_t free_b = 0, total_b = 0;
         DWG_CUDA_TRY(c, cudaMemGetInfo(&free_b, &total_b));
         const double need = 4.0 * (double)(L.nfar + L.nnear) +
-                            (8.0 + 4.0 * 8 * kGrpQ) * ((double)(L.nfar + L.nnear * c->tree_leaf) /
-                                                           kItemRecords + (double)ng);
+                            (8.0 + 4.0 * 8 * kGrpQ) *
+                                ((double)(L.nfar + L.nnear * c->tree_leaf) /
+                                     item_records(L.nfar + L.nnear * c->tree_leaf, ng) +
+                                 (double)ng);
         if (need > 0.5 * (double)free_b) return DWG_OK;
         DWG_CUDA_TRY(c, cudaMalloc(&L.d_far, std::max<int64_t>(L.nfar, 1) * sizeof(int)));
         DWG_CUDA_TRY(c, cudaMalloc(&L.d_near, std::max<int64_t>(L.nnear, 1) * sizeof(int)));
@@ -1207,8 +1232,9 @@ int tree_lists(Ctx *c, TreeLists &L, const float4 *q, int64_t m, bool *built)
         DWG_CUDA_TRY(c, cudaGetLastError());
         // work items and their partial-sum buffer
         DWG_CUDA_TRY(c, cudaMalloc(&L.d_item_off, (ng + 1) * sizeof(int64_t)));
+        L.irec = item_records(L.nfar + L.nnear * c->tree_leaf, ng);
         k_tree_items<<<(unsigned)ceil_div(ng, 256), 256, 0, c->stream>>>(
-            L.d_far_off, L.d_near_off, ng, c->tree_leaf, cnt_f);
+            L.d_far_off, L.d_near_off, ng, c->tree_leaf, L.irec, cnt_f);
         DWG_CUDA_TRY(c, cudaGetLastError());
         if ((rc = scan_i64(c, cnt_f, L.d_item_off, ng, L.d_item_off + ng))) return rc;
         DWG_CUDA_TRY(c, cudaMemcpyAsync(&L.nitems, L.d_item_off + ng, sizeof(int64_t),
@@ -1217,7 +1243,7 @@ int tree_lists(Ctx *c, TreeLists &L, const float4 *q, int64_t m, bool *built)
         DWG_CUDA_TRY(c, cudaMalloc(&L.d_items, L.nitems * sizeof(int2)));
         DWG_CUDA_TRY(c, cudaMalloc(&L.d_ipart, L.nitems * 8 * kGrpQ * sizeof(float)));
         k_tree_item_table<<<(unsigned)ceil_div(ng, 256), 256, 0, c->stream>>>(L.d_item_off, ng,
-                                                                              L.d_items);
+                                                                              L.irec, L.d_items);
         DWG_CUDA_TRY(c, cudaGetLastError());
         L.q = q;
         L.m = m;
@@ -1333,13 +1359,163 @@ cudaError_t launch_tree_moments(Ctx *c)
     k_tree_leaf_moments<<<(unsigned)ceil_div(nleaf * c->tree_leaf, kMomTile), kMomThreads, 0,
                           c->stream>>>(c->d_p4, c->d_nrm, c->n, nleaf, c->tree_leaf,
                                        c->d_tree_M);
-    for (int lv = c->tree_levels - 1; lv >= 0; --lv) {
+    for (int lv = c->tree_levels - 1; lv > 10; --lv) {
         int64_t first = (int64_t)1 << lv;
         k_tree_level_moments<<<(unsigned)ceil_div(first, B), B, 0, c->stream>>>(first, c->d_tree_M);
     }
+    if (c->tree_levels > 0)
+        k_tree_top_moments<<<1, 1024, 0, c->stream>>>(std::min(c->tree_levels - 1, 10),
+                                                      c->d_tree_M);
     k_tree_moment_records<<<(unsigned)ceil_div(nn, B), B, 0, c->stream>>>(
         nn, c->d_tree_M, c->d_tree_rec, c->d_tree_mrec, c->d_tree_frec);
     return cudaGetLastError();
+}
+
+// The offsets of up to kListRange groups' lists and work items from their
+// counts, by one block (a scan of three arrays at once); totals: far nodes,
+// near leaves, items.  The items' size follows item_records' rule.
+constexpr int kListRange = 16384;
+
+__global__ void __launch_bounds__(1024)
+    k_tree_list_offsets(const int64_t *__restrict__ cnt_f, const int64_t *__restrict__ cnt_n,
+                        int ng, int bucket, int64_t *__restrict__ far_off,
+                        int64_t *__restrict__ near_off, int64_t *__restrict__ item_off,
+                        int64_t *__restrict__ totals)
+{
+    __shared__ int64_t sh[3][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // the records of all groups
+    int64_t rec = 0;
+    for (int g = threadIdx.x; g < ng; g += 1024) rec += cnt_f[g] + cnt_n[g] * bucket;
+    for (int o = 16; o > 0; o >>= 1) rec += __shfl_xor_sync(0xffffffffu, rec, o);
+    if (lane == 0) sh[0][w] = rec;
+    __syncthreads();
+    rec = 0;
+    for (int i = 0; i < 32; ++i) rec += sh[0][i];
+    __syncthreads();
+    const int irec = item_records(rec, ng);
+    int64_t run[3] = {0, 0, 0};
+    for (int g0 = 0; g0 < ng; g0 += 1024) {
+        const int g = g0 + threadIdx.x;
+        int64_t v[3] = {0, 0, 0}, in[3];
+        if (g < ng) {
+            v[0] = cnt_f[g];
+            v[1] = cnt_n[g];
+            v[2] = max((int64_t)1, (v[0] + v[1] * bucket + irec - 1) / irec);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            in[a] = v[a];
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t x = __shfl_up_sync(0xffffffffu, in[a], o);
+                if (lane >= o) in[a] += x;
+            }
+            if (lane == 31) sh[a][w] = in[a];
+        }
+        __syncthreads();
+        if (w < 3) {
+            const int64_t x = sh[w][lane];
+            int64_t i = x;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t y = __shfl_up_sync(0xffffffffu, i, o);
+                if (lane >= o) i += y;
+            }
+            sh[w][lane] = i - x;
+            if (lane == 31) sh[w][32] = i;
+        }
+        __syncthreads();
+        int64_t *out[3] = {far_off, near_off, item_off};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (g < ng) out[a][g] = run[a] + sh[a][w] + in[a] - v[a];
+            run[a] += sh[a][32];
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        far_off[ng] = totals[0] = run[0];
+        near_off[ng] = totals[1] = run[1];
+        item_off[ng] = totals[2] = run[2];
+        totals[3] = irec;
+    }
+}
+
+// One call's evaluation under the group test through lists of its own: the
+// walk of k_tree_group keeps a warp for a whole group, walk and evaluation
+// (110,592 queries are 1,728 warps, 11 an SM, at 43 % of the FMA pipe);
+// here the lists are cut into items of at most kItemRecords records and
+// evaluated by k_tree_eval_lists.  300,000 sources, w and grad w at 110,592
+// lattice queries: 1,392 -> 690 us (walks 204, evaluation 473).  In ranges
+// of groups; a range whose
+// lists would take more than kCallLists bytes (queries in no order open the
+// whole tree) is walked.
+constexpr double kCallLists = 1024.0 * 1024.0 * 1024.0;
+
+template <bool GRAD, bool SCREENED>
+static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, int64_t stride)
+{
+    const EvalParams ep = make_eval_params(c);
+    const int64_t all = ceil_div(m, kGrpQ);
+    for (int64_t g0 = 0; g0 < all; g0 += kListRange) {
+        ScratchScope scope(c);
+        const int ng = (int)std::min<int64_t>(kListRange, all - g0);
+        const float4 *qr = q + g0 * kGrpQ;
+        const int64_t mr = std::min<int64_t>(m - g0 * kGrpQ, (int64_t)ng * kGrpQ);
+        float *pr = part + g0 * kGrpQ;
+        const unsigned blocks = (unsigned)ceil_div(ng, kListWarps);
+        int64_t *buf = nullptr;
+        DWG_CUDA_TRY(c, scratch_get(c, &buf, (5 * (int64_t)ng + 7) * sizeof(int64_t)));
+        int64_t *cnt_f = buf, *cnt_n = cnt_f + ng, *far_off = cnt_n + ng, *near_off = far_off + ng + 1,
+                *item_off = near_off + ng + 1, *tot = item_off + ng + 1;
+        k_tree_lists<false><<<blocks, 32 * kListWarps, 0, c->stream>>>(
+            qr, mr, c->d_tree_rec, c->tree_levels, cnt_f, cnt_n, nullptr, nullptr, c->d_err);
+        k_tree_list_offsets<<<1, 1024, 0, c->stream>>>(cnt_f, cnt_n, ng, c->tree_leaf, far_off,
+                                                       near_off, item_off, tot);
+        DWG_CUDA_TRY(c, cudaGetLastError());
+        int64_t ht[4];
+        DWG_CUDA_TRY(c, cudaMemcpyAsync(ht, tot, sizeof ht, cudaMemcpyDeviceToHost, c->stream));
+        DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+        const size_t item_bytes = (GRAD ? 8 : 2) * kGrpQ * sizeof(float);
+        const double need = 4.0 * ((double)ht[0] + (double)ht[1]) +
+                            (double)ht[2] * (sizeof(int2) + item_bytes);
+        if (need > kCallLists) {
+            DWG_CUDA_TRY(c, launch_tree_gwn(c, qr, mr, GRAD, pr, stride, nullptr));
+            continue;
+        }
+        int *far_ids = nullptr, *near_ids = nullptr;
+        int2 *items = nullptr;
+        float *ipart = nullptr;
+        DWG_CUDA_TRY(c, scratch_get(c, &far_ids, ht[0] * sizeof(int)));
+        DWG_CUDA_TRY(c, scratch_get(c, &near_ids, ht[1] * sizeof(int)));
+        DWG_CUDA_TRY(c, scratch_get(c, &items, ht[2] * sizeof(int2)));
+        DWG_CUDA_TRY(c, scratch_get(c, &ipart, ht[2] * item_bytes));
+        k_tree_lists<true><<<blocks, 32 * kListWarps, 0, c->stream>>>(
+            qr, mr, c->d_tree_rec, c->tree_levels, far_off, near_off, far_ids, near_ids, c->d_err);
+        const int irec = (int)ht[3];
+        k_tree_item_table<<<(unsigned)ceil_div(ng, 256), 256, 0, c->stream>>>(item_off, ng, irec,
+                                                                              items);
+        k_tree_eval_lists<GRAD, SCREENED, false><<<(unsigned)ht[2], 32, 0, c->stream>>>(
+            qr, mr, c->d_tree_frec, c->d_src, c->n, c->tree_levels, c->tree_leaf, far_off, far_ids,
+            near_off, near_ids, items, ht[2], irec, ep, ipart, c->d_counter, nullptr);
+        k_tree_combine<GRAD><<<(unsigned)ceil_div(mr, 256), 256, 0, c->stream>>>(
+            ipart, item_off, mr, pr, stride, nullptr);
+        DWG_CUDA_TRY(c, cudaGetLastError());
+    }
+    return DWG_OK;
+}
+
+int tree_eval_call(Ctx *c, const float4 *q, int64_t m, bool grad, float *part, int64_t stride)
+{
+    if (!c->tree_group || c->reg_mode == DWG_REG_CLAMP) {
+        DWG_CUDA_TRY(c, launch_tree_gwn(c, q, m, grad, part, stride, nullptr));
+        return DWG_OK;
+    }
+    const bool scr = make_eval_params(c).screened != 0;
+    if (grad)
+        return scr ? eval_call_lists_t<true, true>(c, q, m, part, stride)
+                   : eval_call_lists_t<true, false>(c, q, m, part, stride);
+    return scr ? eval_call_lists_t<false, true>(c, q, m, part, stride)
+               : eval_call_lists_t<false, false>(c, q, m, part, stride);
 }
 
 template <bool GRAD, bool SCREENED>
@@ -1364,7 +1540,7 @@ static cudaError_t launch_lists_t(Ctx *c, const TreeLists &L, float *part, int64
     EvalParams ep = make_eval_params(c);
     k_tree_eval_lists<GRAD, SCREENED, CLAMP><<<(unsigned)L.nitems, 32, 0, c->stream>>>(
         L.q, L.m, c->d_tree_frec, CLAMP ? c->d_src16 : c->d_src, c->n, c->tree_levels,
-        c->tree_leaf, L.d_far_off, L.d_far, L.d_near_off, L.d_near, L.d_items, L.nitems, ep,
+        c->tree_leaf, L.d_far_off, L.d_far, L.d_near_off, L.d_near, L.d_items, L.nitems, L.irec, ep,
         L.d_ipart, c->d_counter, st);
     k_tree_combine<GRAD><<<(unsigned)ceil_div(L.m, 256), 256, 0, c->stream>>>(
         L.d_ipart, L.d_item_off, L.m, part, stride, st);
@@ -1488,7 +1664,8 @@ __global__ void __launch_bounds__(32, lst_resident(GRAD))
     constexpr int w = GRAD ? 0 : 1;
     eval_lists_body<GRAD, SCREENED>(c.lq[w], c.lm[w], c.tree_frec, c.src, c.n, c.levels, c.bucket,
                                     c.far_off[w], c.far_ids[w], c.near_off[w], c.near_ids[w],
-                                    c.items[w], c.nitems[w], c.ep, c.ipart[w], c.counter, c.st,
+                                    c.items[w], c.nitems[w], c.irec[w], c.ep, c.ipart[w], c.counter,
+                                    c.st,
                                     (int64_t)blockIdx.x - off[ci]);
 }
 
