@@ -245,6 +245,9 @@ __device__ __forceinline__ void gwn_block(const float *__restrict__ src, int64_t
     constexpr uint32_t TILE_BYTES = TILE_FLOATS * 4;
     constexpr int QB = NT * 2 * P;
     constexpr int NA = GRAD ? 4 : 1;
+    // sources per loop trip: 4 is 2-5 % faster than 2, but for four and more
+    // screened pairs of w (1-4 % slower)
+    constexpr int UNROLL = SCREENED && !GRAD && P >= 4 ? 2 : 4;
 
     __shared__ __align__(128) float sbuf[kStages][TILE_FLOATS];
     __shared__ __align__(8) uint64_t bar[kStages];
@@ -311,7 +314,7 @@ __device__ __forceinline__ void gwn_block(const float *__restrict__ src, int64_t
         }
         if (!s_abort) {
             const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(sbuf[s]);
-#pragma unroll 4  // 2-5 % faster than 2 in every shape but (4, 128) screened (1 % slower)
+#pragma unroll UNROLL
             for (int j = 0; j < T; ++j) {
                 const ulonglong2 r0 = rec[RQ * j + 0];  // (x,x) (y,y)
                 const ulonglong2 r1 = rec[RQ * j + 1];  // (z,z) (mx,mx)
@@ -884,7 +887,9 @@ int eval_launch(Ctx *c, const float4 *q, int64_t m, bool grad, int nchunks, floa
 }
 
 constexpr int kPGrad = 2;   // query pairs per thread, gradient kernel (batched launches)
-constexpr int kPW = 4;      // query pairs per thread, w-only kernel (raw launches)
+// query pairs per thread, w-only kernel (raw launches): 20,000 sources at
+// 60,001 queries, screened, 758 us with 4 pairs, 673 with 2
+constexpr int kPW = 2;
 
 bool corners_on_lattice(const Ctx *c)
 {
@@ -1232,7 +1237,7 @@ cudaError_t launch_reduce_eval(Ctx *c, const float *part, int nchunks, int64_t m
 int gwn_w_chunks_raw(int64_t m, int64_t npad, int device)
 {
     return pick_chunks(ceil_div(m, kEvalThreads * 2 * kPW), npad / kSrcTile,
-                       variant_slots(kVarW[0], false, 0, false, device));
+                       variant_slots(kVarW[1], false, 1, false, device));
 }
 
 cudaError_t launch_gwn_w_raw(const float *src, int64_t npad, const float4 *q, int64_t m,
