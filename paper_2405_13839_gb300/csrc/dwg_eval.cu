@@ -245,10 +245,6 @@ __device__ __forceinline__ void gwn_block(const float *__restrict__ src, int64_t
     constexpr uint32_t TILE_BYTES = TILE_FLOATS * 4;
     constexpr int QB = NT * 2 * P;
     constexpr int NA = GRAD ? 4 : 1;
-    // sources per loop trip: 4 is 2-5 % faster than 2, but for four and more
-    // screened pairs of w (1-4 % slower)
-    constexpr int UNROLL = SCREENED && !GRAD && P >= 4 ? 2 : 4;
-
     __shared__ __align__(128) float sbuf[kStages][TILE_FLOATS];
     __shared__ __align__(8) uint64_t bar[kStages];
     __shared__ int s_abort;
@@ -314,7 +310,7 @@ __device__ __forceinline__ void gwn_block(const float *__restrict__ src, int64_t
         }
         if (!s_abort) {
             const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(sbuf[s]);
-#pragma unroll UNROLL
+#pragma unroll 4  // 2: up to 9 % slower; 8: within 1 %
             for (int j = 0; j < T; ++j) {
                 const ulonglong2 r0 = rec[RQ * j + 0];  // (x,x) (y,y)
                 const ulonglong2 r1 = rec[RQ * j + 1];  // (z,z) (mx,mx)
@@ -450,8 +446,13 @@ __device__ __forceinline__ void gwn_block(const float *__restrict__ src, int64_t
     }
 }
 
+// A minimum of one CTA per SM is named so that the compiler spends registers
+// (up to 160) on overlapping terms: left to itself it holds them down for
+// resident warps, which an issue-bound loop does not need (w at 400,000
+// queries of 100,000 sources: plain 15.0 -> 14.4 ms, screened 20.8 -> 19.0 ms;
+// w and grad w at 100,000: 6.33 -> 6.29, 8.53 -> 8.41 ms).
 template <int P, int NT, bool GRAD, bool SCREENED, bool CLAMP = false, bool COMP = true>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, 1)
     k_gwn(const float *__restrict__ src, int64_t ntiles_total, const float4 *__restrict__ q,
           int64_t m, int tiles_per_chunk, float *__restrict__ part, int64_t stride,
           EvalParams ep, int *__restrict__ err)
@@ -464,7 +465,7 @@ __global__ void __launch_bounds__(NT)
 // Many clouds in one launch: CTA b runs work item items[b] of its cloud;
 // clouds that have converged are skipped.
 template <int P, bool GRAD, bool SCREENED>
-__global__ void __launch_bounds__(kEvalThreads)
+__global__ void __launch_bounds__(kEvalThreads, 1)
     k_gwn_batch(const GwnCloud *__restrict__ clouds, const GwnItem *__restrict__ items,
                 int *__restrict__ err)
 {
@@ -613,8 +614,9 @@ __device__ __forceinline__ void gwn_lattice_block(const float *__restrict__ src,
         }
 }
 
+// (the minimum of one CTA as for k_gwn: 10.9 -> 10.4 ms)
 template <bool SCREENED>
-__global__ void __launch_bounds__(kLatThreads)
+__global__ void __launch_bounds__(kLatThreads, 1)
     k_gwn_lattice(const float *__restrict__ src, int64_t ntiles_total, LatTasks lat,
                   int tiles_per_chunk, float *__restrict__ part, EvalParams ep,
                   int *__restrict__ err)
@@ -624,7 +626,7 @@ __global__ void __launch_bounds__(kLatThreads)
 }
 
 template <bool SCREENED>
-__global__ void __launch_bounds__(kLatThreads)
+__global__ void __launch_bounds__(kLatThreads, 1)
     k_gwn_lattice_batch(const GwnCloud *__restrict__ clouds, const GwnItem *__restrict__ items,
                         int *__restrict__ err)
 {
@@ -888,7 +890,8 @@ int eval_launch(Ctx *c, const float4 *q, int64_t m, bool grad, int nchunks, floa
 
 constexpr int kPGrad = 2;   // query pairs per thread, gradient kernel (batched launches)
 // query pairs per thread, w-only kernel (raw launches): 20,000 sources at
-// 60,001 queries, screened, 758 us with 4 pairs, 673 with 2
+// 60,001 queries, screened, 675 us a call with 4 pairs, 696 with 2; 60,000
+// sources at 200,000 queries 6.27 ms with 4, 6.10 ms with 2
 constexpr int kPW = 2;
 
 bool corners_on_lattice(const Ctx *c)
