@@ -17,9 +17,9 @@
 //                   batch on the warp-level tensor-core instruction
 //                   (mma.sync m16n8k16, the fragments of one layer feed the
 //                   next in registers): dY W4, dZ3 W3, dZ2 W2, weight
-//                   gradients dZ^T H on tensor cores from per-warp shared
-//                   stashes, summed per CTA in shared memory, then added to
-//                   the global gradient;
+//                   gradients dZ^T H on tensor cores from the CTA's 64 rows
+//                   in shared memory, summed in registers over its tiles,
+//                   then added to the global gradient;
 //   k_adam          the Adam update of the fp32 master weights;
 //   k_features      16 nearest neighbours (exact, the bucket-tree search)
 //                   and the feature rows;
@@ -48,10 +48,6 @@ __device__ __forceinline__ uint16_t bf16_bits(float x)
     __nv_bfloat16 v = __float2bfloat16_rn(x);
     return *reinterpret_cast<uint16_t *>(&v);
 }
-__device__ __forceinline__ uint32_t pair16(uint16_t lo, uint16_t hi)
-{
-    return (uint32_t)lo | ((uint32_t)hi << 16);
-}
 
 __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                          uint32_t b1)
@@ -61,45 +57,6 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
         "{%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// shared-memory copy of the weights (bf16) and biases (fp32)
-struct MlpSmem {
-    uint16_t W[3][64 * 64];   // W1, W2, W3 as [out][in]
-    uint16_t W4[8 * 64];      // W4 padded to 8 outputs
-    float b[3][64];
-    float b4[8];
-};
-struct MlpSmemT {
-    uint16_t Wt[2][64 * 64];  // W2^T, W3^T as [in][out]
-    uint16_t W4t[64 * 16];    // W4^T padded to 16 columns
-};
-
-__device__ void load_weights(const float *__restrict__ P, MlpSmem &S, MlpSmemT *T)
-{
-    for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) {
-        S.W[0][i] = bf16_bits(P[kOffW1 + i]);
-        S.W[1][i] = bf16_bits(P[kOffW2 + i]);
-        S.W[2][i] = bf16_bits(P[kOffW3 + i]);
-        if (T) {
-            int o = i / 64, in = i % 64;  // W[o][in] -> Wt[in][o]
-            T->Wt[0][in * 64 + o] = S.W[1][i];
-            T->Wt[1][in * 64 + o] = S.W[2][i];
-        }
-    }
-    for (int i = threadIdx.x; i < 8 * 64; i += blockDim.x)
-        S.W4[i] = i < 3 * 64 ? bf16_bits(P[kOffW4 + i]) : (uint16_t)0;
-    if (T)
-        for (int i = threadIdx.x; i < 64 * 16; i += blockDim.x) {
-            int f = i / 16, c = i % 16;
-            T->W4t[i] = c < 3 ? bf16_bits(P[kOffW4 + c * 64 + f]) : (uint16_t)0;
-        }
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) {
-        S.b[0][i] = P[kOffB1 + i];
-        S.b[1][i] = P[kOffB2 + i];
-        S.b[2][i] = P[kOffB3 + i];
-    }
-    if (threadIdx.x < 8) S.b4[threadIdx.x] = threadIdx.x < 3 ? P[kOffB4 + threadIdx.x] : 0.f;
 }
 
 // A fragments of 16 rows of X (fp32, row-major, 64 columns) -> bf16
@@ -123,62 +80,6 @@ __device__ __forceinline__ void load_x(const float *__restrict__ X, int64_t row0
         a[kk][2] = pack_bf16(v01.x, v01.y);
         a[kk][3] = pack_bf16(v11.x, v11.y);
     }
-}
-
-// acc[nt] = A (16 x 64) x W^T for the 8 output tiles of one layer
-__device__ __forceinline__ void layer_mma(const uint16_t *__restrict__ W, const uint32_t (&a)[4][4],
-                                          float (&acc)[8][4], int lane)
-{
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk)
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const uint16_t *row = W + (8 * nt + g) * 64 + 16 * kk + 2 * t;
-            mma16816(acc[nt], a[kk], *reinterpret_cast<const uint32_t *>(row),
-                     *reinterpret_cast<const uint32_t *>(row + 8));
-        }
-}
-
-// bias + ReLU, the relu mask (bit nt*4+e), and the next layer's A fragments
-__device__ __forceinline__ void bias_relu(float (&acc)[8][4], const float *__restrict__ b,
-                                          uint32_t (&a)[4][4], uint32_t &mask, int lane)
-{
-    const int t = lane & 3;
-    mask = 0;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            float z = acc[nt][e] + b[8 * nt + 2 * t + (e & 1)];
-            if (z > 0.f) mask |= 1u << (nt * 4 + e);
-            acc[nt][e] = z > 0.f ? z : 0.f;
-        }
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-        a[kk][0] = pack_bf16(acc[2 * kk][0], acc[2 * kk][1]);
-        a[kk][1] = pack_bf16(acc[2 * kk][2], acc[2 * kk][3]);
-        a[kk][2] = pack_bf16(acc[2 * kk + 1][0], acc[2 * kk + 1][1]);
-        a[kk][3] = pack_bf16(acc[2 * kk + 1][2], acc[2 * kk + 1][3]);
-    }
-}
-
-// the output layer: y (16 x 8, first 3 columns used)
-__device__ __forceinline__ void out_layer(const MlpSmem &S, const uint32_t (&a)[4][4],
-                                          float (&y)[4], int lane)
-{
-    const int g = lane >> 2, t = lane & 3;
-    y[0] = y[1] = y[2] = y[3] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-        const uint16_t *row = S.W4 + g * 64 + 16 * kk + 2 * t;
-        mma16816(y, a[kk], *reinterpret_cast<const uint32_t *>(row),
-                 *reinterpret_cast<const uint32_t *>(row + 8));
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) y[e] += S.b4[2 * t + (e & 1)];
 }
 
 // --- inference on the 5th-generation tensor cores (tcgen05) -----------------
@@ -422,75 +323,118 @@ __global__ void __launch_bounds__(kTcRows)
 }
 
 // --- training -------------------------------------------------------------
+//
+// A CTA of four warps takes 64 rows at a time, 16 per warp.  Each warp runs
+// its rows forward and back on mma.sync, the fragments of one layer feeding
+// the next in registers, and leaves every layer's input (act) and dZ as
+// bf16 rows in shared memory; after one barrier the weight gradients dZ^T H of
+// all 64 rows are products with K = 64, each warp owning 16 rows of every
+// matrix, and go from the accumulators to the global gradient as pairs.
+// Operands come by ldmatrix (transposed where the product wants the other
+// order, so no transposed copies are kept) from rows of 72 elements: eight
+// rows touch all banks.  With the gradients summed per 16 rows by shared-
+// memory float additions (a compare-and-swap loop each, 48 % of the shared-
+// memory pipe) 8,192 rows took 64 us; 128 CTAs of one tile each now GRADUS.
+constexpr int kLd = 72;  // elements of a shared-memory row of 64
+constexpr int kLdY = 24; // of a row of dY (16)
+
 struct MlpGradSmem {
-    float gW[3][64 * 64];
-    float gW4[3 * 64];
-    float gb[3][64];
-    float gb4[4];
-};
-struct MlpStash {
-    uint16_t act[4][16 * 64];  // x, h1, h2, h3 of the warp's 16 rows, bf16
-    uint16_t dz[16 * 64];      // the current layer's dZ, bf16
-    uint16_t dy[16 * 16];      // dY padded to 16 columns
+    uint16_t W[3][64 * kLd];    // [out][in]
+    uint16_t W4[16 * kLd];      // rows 3..15 zero
+    uint16_t act[4][kMlpRows * kLd];  // x, h1, h2, h3
+    uint16_t dz[3][kMlpRows * kLd];
+    uint16_t dy[kMlpRows * kLdY];
+    float b[3][64];
+    float b4[8];
+    float gb[3][kMlpWarps][64]; // bias gradients per warp
+    float gb4[kMlpWarps][4];
 };
 
-// store a C-layout tile set (16 x 64) as bf16 rows in a stash
-__device__ __forceinline__ void stash_c(const float (&v)[8][4], uint16_t *dst, int lane)
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const uint16_t *p)
 {
-    const int g = lane >> 2, t = lane & 3;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const uint16_t *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+
+// acc = A (16 x 64) x W^T, W as [out][in] rows
+__device__ __forceinline__ void layer_mma(const uint16_t *W, const uint32_t (&a)[4][4],
+                                          float (&acc)[8][4], int lane)
+{
+    const int row = (lane & 7) + ((lane >> 4) & 1) * 8, col = ((lane >> 3) & 1) * 8;
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        int c = 8 * nt + 2 * t;
-        *reinterpret_cast<uint32_t *>(dst + g * 64 + c) = pack_bf16(v[nt][0], v[nt][1]);
-        *reinterpret_cast<uint32_t *>(dst + (g + 8) * 64 + c) = pack_bf16(v[nt][2], v[nt][3]);
+    for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+        for (int nt = 0; nt < 8; nt += 2) {
+            uint32_t r[4];
+            ldsm4(r, W + (8 * nt + row) * kLd + 16 * kk + col);
+            mma16816(acc[nt], a[kk], r[0], r[1]);
+            mma16816(acc[nt + 1], a[kk], r[2], r[3]);
+        }
+}
+
+// acc (16 x 64) += A (16 x 16 KK) x M, M as [k][n] rows
+template <int KK>
+__device__ __forceinline__ void mma_rows(const uint16_t *M, const uint32_t (*a)[4],
+                                         float (&acc)[8][4], int lane)
+{
+    const int row = (lane & 7) + ((lane >> 3) & 1) * 8, col = ((lane >> 4) & 1) * 8;
+#pragma unroll
+    for (int kk = 0; kk < KK; ++kk)
+#pragma unroll
+        for (int nt = 0; nt < 8; nt += 2) {
+            uint32_t r[4];
+            ldsm4t(r, M + (16 * kk + row) * kLd + 8 * nt + col);
+            mma16816(acc[nt], a[kk], r[0], r[1]);
+            mma16816(acc[nt + 1], a[kk], r[2], r[3]);
+        }
+}
+
+// bias + ReLU, the relu mask (bit nt * 4 + e), and the next layer's A fragments
+__device__ __forceinline__ void bias_relu(float (&acc)[8][4], const float *__restrict__ b,
+                                          uint32_t (&a)[4][4], uint32_t &mask, int lane)
+{
+    const int t = lane & 3;
+    mask = 0;
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float z = acc[nt][e] + b[8 * nt + 2 * t + (e & 1)];
+            if (z > 0.f) mask |= 1u << (nt * 4 + e);
+            acc[nt][e] = z > 0.f ? z : 0.f;
+        }
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+        a[kk][0] = pack_bf16(acc[2 * kk][0], acc[2 * kk][1]);
+        a[kk][1] = pack_bf16(acc[2 * kk][2], acc[2 * kk][3]);
+        a[kk][2] = pack_bf16(acc[2 * kk + 1][0], acc[2 * kk + 1][1]);
+        a[kk][3] = pack_bf16(acc[2 * kk + 1][2], acc[2 * kk + 1][3]);
     }
 }
+
+// A fragments of the warp's 16 rows as bf16 rows
 __device__ __forceinline__ void stash_a(const uint32_t (&a)[4][4], uint16_t *dst, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
-        *reinterpret_cast<uint32_t *>(dst + g * 64 + 16 * kk + 2 * t) = a[kk][0];
-        *reinterpret_cast<uint32_t *>(dst + (g + 8) * 64 + 16 * kk + 2 * t) = a[kk][1];
-        *reinterpret_cast<uint32_t *>(dst + g * 64 + 16 * kk + 8 + 2 * t) = a[kk][2];
-        *reinterpret_cast<uint32_t *>(dst + (g + 8) * 64 + 16 * kk + 8 + 2 * t) = a[kk][3];
+        *reinterpret_cast<uint32_t *>(dst + g * kLd + 16 * kk + 2 * t) = a[kk][0];
+        *reinterpret_cast<uint32_t *>(dst + (g + 8) * kLd + 16 * kk + 2 * t) = a[kk][1];
+        *reinterpret_cast<uint32_t *>(dst + g * kLd + 16 * kk + 8 + 2 * t) = a[kk][2];
+        *reinterpret_cast<uint32_t *>(dst + (g + 8) * kLd + 16 * kk + 8 + 2 * t) = a[kk][3];
     }
 }
 
-// gW[o][f] += sum_s D[s][o] * H[s][f] over the warp's 16 rows (tensor cores);
-// D is (16 x ncols_d) bf16 with row stride ld_d, H is (16 x 64) bf16
-__device__ __forceinline__ void weight_grad(const uint16_t *D, int ld_d, int mtiles,
-                                            const uint16_t *H, float *gW, int rows_out, int lane)
-{
-    const int g = lane >> 2, t = lane & 3;
-    for (int mt = 0; mt < mtiles; ++mt) {
-        uint32_t a[4];
-        int o0 = 16 * mt + g, o1 = o0 + 8;
-        a[0] = pair16(D[(2 * t) * ld_d + o0], D[(2 * t + 1) * ld_d + o0]);
-        a[1] = pair16(D[(2 * t) * ld_d + o1], D[(2 * t + 1) * ld_d + o1]);
-        a[2] = pair16(D[(2 * t + 8) * ld_d + o0], D[(2 * t + 9) * ld_d + o0]);
-        a[3] = pair16(D[(2 * t + 8) * ld_d + o1], D[(2 * t + 9) * ld_d + o1]);
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            int f = 8 * nt + g;
-            uint32_t b0 = pair16(H[(2 * t) * 64 + f], H[(2 * t + 1) * 64 + f]);
-            uint32_t b1 = pair16(H[(2 * t + 8) * 64 + f], H[(2 * t + 9) * 64 + f]);
-            float d[4] = {0.f, 0.f, 0.f, 0.f};
-            mma16816(d, a, b0, b1);
-            int c = 8 * nt + 2 * t;
-            if (o0 < rows_out) {
-                atomicAdd(&gW[o0 * 64 + c], d[0]);
-                atomicAdd(&gW[o0 * 64 + c + 1], d[1]);
-            }
-            if (o1 < rows_out) {
-                atomicAdd(&gW[o1 * 64 + c], d[2]);
-                atomicAdd(&gW[o1 * 64 + c + 1], d[3]);
-            }
-        }
-    }
-}
-
-// column sums of a C-layout tile set over the warp's 16 rows -> gb
+// column sums of a C-layout tile set over the warp's 16 rows
 __device__ __forceinline__ void bias_grad(const float (&v)[8][4], float *gb, int lane)
 {
     const int t = lane & 3;
@@ -502,15 +446,20 @@ __device__ __forceinline__ void bias_grad(const float (&v)[8][4], float *gb, int
             s += __shfl_xor_sync(0xffffffffu, s, 4);
             s += __shfl_xor_sync(0xffffffffu, s, 8);
             s += __shfl_xor_sync(0xffffffffu, s, 16);
-            if (lane < 4) atomicAdd(&gb[8 * nt + 2 * t + e], s);
+            if (lane < 4) gb[8 * nt + 2 * t + e] = s;
         }
 }
 
-// dH (16 x 64) = dZ (16 x 64, as A fragments) x W (B operand [in][out] = W^T rows)
-__device__ __forceinline__ void back_mma(const uint16_t *Wt, const uint32_t (&a)[4][4],
-                                         float (&acc)[8][4], int lane)
+// two neighbouring sums onto the global gradient (one pair where the array is
+// aligned for it)
+__device__ __forceinline__ void grad_add2(float *p, float x, float y, bool pair)
 {
-    layer_mma(Wt, a, acc, lane);
+    if (pair) {
+        asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(x), "f"(y) : "memory");
+    } else {
+        atomicAdd(p, x);
+        atomicAdd(p + 1, y);
+    }
 }
 
 __global__ void __launch_bounds__(32 * kMlpWarps)
@@ -519,123 +468,175 @@ __global__ void __launch_bounds__(32 * kMlpWarps)
                double *__restrict__ loss)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    MlpSmem &S = *reinterpret_cast<MlpSmem *>(smem_raw);
-    MlpSmemT &ST = *reinterpret_cast<MlpSmemT *>(smem_raw + sizeof(MlpSmem));
-    MlpGradSmem &G =
-        *reinterpret_cast<MlpGradSmem *>(smem_raw + sizeof(MlpSmem) + sizeof(MlpSmemT));
-    MlpStash *stash = reinterpret_cast<MlpStash *>(smem_raw + sizeof(MlpSmem) + sizeof(MlpSmemT) +
-                                                   sizeof(MlpGradSmem));
-    load_weights(P, S, &ST);
-    {
-        float *z = reinterpret_cast<float *>(&G);
-        for (int i = threadIdx.x; i < (int)(sizeof(MlpGradSmem) / sizeof(float)); i += blockDim.x)
-            z[i] = 0.f;
+    MlpGradSmem &S = *reinterpret_cast<MlpGradSmem *>(smem_raw);
+    for (int i = threadIdx.x; i < 64 * 32; i += blockDim.x) {
+        const int o = i >> 5, k = 2 * (i & 31);
+        const int at = o * 64 + k, to = o * kLd + k;
+        *reinterpret_cast<uint32_t *>(&S.W[0][to]) = pack_bf16(P[kOffW1 + at], P[kOffW1 + at + 1]);
+        *reinterpret_cast<uint32_t *>(&S.W[1][to]) = pack_bf16(P[kOffW2 + at], P[kOffW2 + at + 1]);
+        *reinterpret_cast<uint32_t *>(&S.W[2][to]) = pack_bf16(P[kOffW3 + at], P[kOffW3 + at + 1]);
     }
+    for (int i = threadIdx.x; i < 16 * 32; i += blockDim.x) {
+        const int o = i >> 5, k = 2 * (i & 31);
+        *reinterpret_cast<uint32_t *>(&S.W4[o * kLd + k]) =
+            o < 3 ? pack_bf16(P[kOffW4 + o * 64 + k], P[kOffW4 + o * 64 + k + 1]) : 0u;
+    }
+    if (threadIdx.x < 64) {
+        S.b[0][threadIdx.x] = P[kOffB1 + threadIdx.x];
+        S.b[1][threadIdx.x] = P[kOffB2 + threadIdx.x];
+        S.b[2][threadIdx.x] = P[kOffB3 + threadIdx.x];
+    }
+    if (threadIdx.x < 8) S.b4[threadIdx.x] = threadIdx.x < 3 ? P[kOffB4 + threadIdx.x] : 0.f;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
-    MlpStash &W = stash[warp];
     const float inv2b = 2.f / (float)B;
+    const bool pair = (reinterpret_cast<uintptr_t>(grad) & 7) == 0;
+    const int offw[3] = {kOffW1, kOffW2, kOffW3}, offb[3] = {kOffB1, kOffB2, kOffB3};
+    float gw[3][8][4], gw4[2][4], gbias[3] = {0.f, 0.f, 0.f};  // this CTA's tiles so far
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            gw[0][nt][e] = gw[1][nt][e] = gw[2][nt][e] = 0.f;
+            if (nt < 2) gw4[nt][e] = 0.f;
+        }
     double lsum = 0.0;
-    for (int64_t row0 = ((int64_t)blockIdx.x * kMlpWarps + warp) * 16; row0 < B;
-         row0 += (int64_t)gridDim.x * kMlpRows) {
+    for (int64_t tile = blockIdx.x; tile * kMlpRows < B; tile += gridDim.x) {
+        const int64_t row0 = tile * kMlpRows + warp * 16;
+        const int my = warp * 16;  // this warp's rows in the stashes
         uint32_t a[4][4], mask[3];
-        float acc[8][4], y[4];
+        float acc[8][4];
         load_x(X, row0, B, a, lane);
-        stash_a(a, W.act[0], lane);
+        stash_a(a, S.act[0] + my * kLd, lane);
+#pragma unroll
         for (int l = 0; l < 3; ++l) {
             layer_mma(S.W[l], a, acc, lane);
             bias_relu(acc, S.b[l], a, mask[l], lane);
-            stash_a(a, W.act[l + 1], lane);
+            stash_a(a, S.act[l + 1] + my * kLd, lane);
         }
-        out_layer(S, a, y, lane);
+        // the output layer: y (16 x 8, first 3 columns used)
+        float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            const uint16_t *row = S.W4 + g * kLd + 16 * kk + 2 * t;
+            mma16816(y, a[kk], *reinterpret_cast<const uint32_t *>(row),
+                     *reinterpret_cast<const uint32_t *>(row + 8));
+        }
         // dY = 2 (y - t) / B for the valid rows and the 3 used columns
         float dyv[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            int col = 2 * t + (e & 1);
-            int64_t r = row0 + g + (e >= 2 ? 8 : 0);
+            const int col = 2 * t + (e & 1);
+            const int64_t r = row0 + g + (e >= 2 ? 8 : 0);
             float d = 0.f;
             if (col < 3 && r < B) {
-                float res = y[e] - T[r * 3 + col];
+                const float res = y[e] + S.b4[col] - T[r * 3 + col];
                 lsum += (double)res * (double)res;
                 d = res * inv2b;
             }
             dyv[e] = d;
         }
-        __syncwarp();
-        // stash dY (16 x 16) and take its A fragment (columns 0..7 carry data)
-        *reinterpret_cast<uint32_t *>(W.dy + g * 16 + 2 * t) = pack_bf16(dyv[0], dyv[1]);
-        *reinterpret_cast<uint32_t *>(W.dy + (g + 8) * 16 + 2 * t) = pack_bf16(dyv[2], dyv[3]);
-        *reinterpret_cast<uint32_t *>(W.dy + g * 16 + 8 + 2 * t) = 0u;
-        *reinterpret_cast<uint32_t *>(W.dy + (g + 8) * 16 + 8 + 2 * t) = 0u;
-        uint32_t ad[4][4];
+        uint16_t *dy = S.dy + my * kLdY;
+        uint32_t ad[1][4];
         ad[0][0] = pack_bf16(dyv[0], dyv[1]);
         ad[0][1] = pack_bf16(dyv[2], dyv[3]);
-        ad[0][2] = 0u;
-        ad[0][3] = 0u;
-        // db4 (columns 0..2)
+        ad[0][2] = ad[0][3] = 0u;
+        *reinterpret_cast<uint32_t *>(dy + g * kLdY + 2 * t) = ad[0][0];
+        *reinterpret_cast<uint32_t *>(dy + (g + 8) * kLdY + 2 * t) = ad[0][1];
+        *reinterpret_cast<uint32_t *>(dy + g * kLdY + 8 + 2 * t) = 0u;
+        *reinterpret_cast<uint32_t *>(dy + (g + 8) * kLdY + 8 + 2 * t) = 0u;
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
+        for (int e = 0; e < 2; ++e) {  // db4 (columns 0..2)
             float s = dyv[e] + dyv[e + 2];
             s += __shfl_xor_sync(0xffffffffu, s, 4);
             s += __shfl_xor_sync(0xffffffffu, s, 8);
             s += __shfl_xor_sync(0xffffffffu, s, 16);
-            if (lane < 4 && 2 * t + e < 3) atomicAdd(&G.gb4[2 * t + e], s);
+            if (lane < 2) S.gb4[warp][2 * t + e] = s;
         }
-        __syncwarp();
-        // dW4 (3 x 64) = dY^T h3
-        weight_grad(W.dy, 16, 1, W.act[3], G.gW4, 3, lane);
         // dH3 = dY W4 (K = 16, dY columns 3..15 are zero)
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-            const uint16_t *row = ST.W4t + (8 * nt + g) * 16 + 2 * t;
-            mma16816(acc[nt], ad[0], *reinterpret_cast<const uint32_t *>(row),
-                     *reinterpret_cast<const uint32_t *>(row + 8));
-        }
-        // layers 3, 2, 1: dZ = dH * relu'(Z); db, dW; dH_prev = dZ W
+        for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+        mma_rows<1>(S.W4, ad, acc, lane);
+        // layers 3, 2, 1: dZ = dH * relu'(Z), then dH of the layer below = dZ W
+#pragma unroll
         for (int l = 2; l >= 0; --l) {
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     if (!(mask[l] & (1u << (nt * 4 + e)))) acc[nt][e] = 0.f;
-            bias_grad(acc, G.gb[l], lane);
-            __syncwarp();
-            stash_c(acc, W.dz, lane);
-            __syncwarp();
-            weight_grad(W.dz, 64, 4, W.act[l], G.gW[l], 64, lane);
-            if (l > 0) {
-                uint32_t az[4][4];
+            bias_grad(acc, S.gb[l][warp], lane);
+            uint32_t az[4][4];
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    az[kk][0] = pack_bf16(acc[2 * kk][0], acc[2 * kk][1]);
-                    az[kk][1] = pack_bf16(acc[2 * kk][2], acc[2 * kk][3]);
-                    az[kk][2] = pack_bf16(acc[2 * kk + 1][0], acc[2 * kk + 1][1]);
-                    az[kk][3] = pack_bf16(acc[2 * kk + 1][2], acc[2 * kk + 1][3]);
-                }
-                back_mma(ST.Wt[l - 1], az, acc, lane);
+            for (int kk = 0; kk < 4; ++kk) {
+                az[kk][0] = pack_bf16(acc[2 * kk][0], acc[2 * kk][1]);
+                az[kk][1] = pack_bf16(acc[2 * kk][2], acc[2 * kk][3]);
+                az[kk][2] = pack_bf16(acc[2 * kk + 1][0], acc[2 * kk + 1][1]);
+                az[kk][3] = pack_bf16(acc[2 * kk + 1][2], acc[2 * kk + 1][3]);
             }
-            __syncwarp();
+            stash_a(az, S.dz[l] + my * kLd, lane);
+            if (l > 0) {
+#pragma unroll
+                for (int nt = 0; nt < 8; ++nt)
+                    acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+                mma_rows<4>(S.W[l], az, acc, lane);
+            }
+        }
+        __syncthreads();  // every warp's rows are in the stashes
+        // gW[o][f] += sum_s dZ[s][o] H[s][f]: this warp's 16 rows o
+        const int srow = (lane & 7) + ((lane >> 4) & 1) * 8, scol = ((lane >> 3) & 1) * 8;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+                ldsm4t(a[kk], S.dz[l] + (16 * kk + srow) * kLd + 16 * warp + scol);
+            mma_rows<4>(S.act[l], a, gw[l], lane);
+        }
+        // gW4 (3 x 64): columns 16 warp .. 16 warp + 15
+        const int hrow = (lane & 7) + ((lane >> 3) & 1) * 8, hcol = ((lane >> 4) & 1) * 8;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            uint32_t ay[4], r[4];
+            ldsm4t(ay, S.dy + (16 * kk + srow) * kLdY + scol);
+            ldsm4t(r, S.act[3] + (16 * kk + hrow) * kLd + 16 * warp + hcol);
+            mma16816(gw4[0], ay, r[0], r[1]);
+            mma16816(gw4[1], ay, r[2], r[3]);
+        }
+        // the biases: a thread per output
+        if (threadIdx.x < 64) {
+#pragma unroll
+            for (int l = 0; l < 3; ++l)
+#pragma unroll
+                for (int w = 0; w < kMlpWarps; ++w) gbias[l] += S.gb[l][w][threadIdx.x];
+        } else if (threadIdx.x < 67) {
+#pragma unroll
+            for (int w = 0; w < kMlpWarps; ++w) gbias[0] += S.gb4[w][threadIdx.x - 64];
+        }
+        __syncthreads();  // the stashes are reused by the next tile
+    }
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        float *out = grad + offw[l] + (16 * warp + g) * 64 + 2 * t;
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            grad_add2(out + 8 * nt, gw[l][nt][0], gw[l][nt][1], pair);
+            grad_add2(out + 8 * 64 + 8 * nt, gw[l][nt][2], gw[l][nt][3], pair);
         }
     }
-    // loss and the CTA's gradient sums
+    if (g < 3) {
+        float *out = grad + kOffW4 + g * 64 + 16 * warp + 2 * t;
+        grad_add2(out, gw4[0][0], gw4[0][1], pair);
+        grad_add2(out + 8, gw4[1][0], gw4[1][1], pair);
+    }
+    if (threadIdx.x < 64) {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) atomicAdd(&grad[offb[l] + threadIdx.x], gbias[l]);
+    } else if (threadIdx.x < 67) {
+        atomicAdd(&grad[kOffB4 + threadIdx.x - 64], gbias[0]);
+    }
     for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
     if (lane == 0) atomicAdd(loss, lsum / (double)B);
-    __syncthreads();
-    for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) {
-        atomicAdd(&grad[kOffW1 + i], G.gW[0][i]);
-        atomicAdd(&grad[kOffW2 + i], G.gW[1][i]);
-        atomicAdd(&grad[kOffW3 + i], G.gW[2][i]);
-    }
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) {
-        atomicAdd(&grad[kOffB1 + i], G.gb[0][i]);
-        atomicAdd(&grad[kOffB2 + i], G.gb[1][i]);
-        atomicAdd(&grad[kOffB3 + i], G.gb[2][i]);
-    }
-    for (int i = threadIdx.x; i < 3 * 64; i += blockDim.x) atomicAdd(&grad[kOffW4 + i], G.gW4[i]);
-    if (threadIdx.x < 3) atomicAdd(&grad[kOffB4 + threadIdx.x], G.gb4[threadIdx.x]);
 }
 
 __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
@@ -652,10 +653,7 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
     p[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
 }
 
-size_t mlp_grad_smem_bytes()
-{
-    return sizeof(MlpSmem) + sizeof(MlpSmemT) + sizeof(MlpGradSmem) + kMlpWarps * sizeof(MlpStash);
-}
+size_t mlp_grad_smem_bytes() { return sizeof(MlpGradSmem); }
 
 static int mlp_sms()
 {
@@ -734,7 +732,7 @@ cudaError_t launch_mlp_grad(const float *P, const float *X, const float *T, int6
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(grad, 0, kMlpParams * sizeof(float), s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(loss, 0, sizeof(double), s)) != cudaSuccess) return e;
-    int64_t blocks = std::min<int64_t>(ceil_div(B, kMlpRows), (int64_t)mlp_sms());
+    int64_t blocks = std::min<int64_t>(ceil_div(B, kMlpRows), (int64_t)mlp_sms() * 2);
     k_mlp_grad<<<(unsigned)std::max<int64_t>(blocks, 1), 32 * kMlpWarps, sm, s>>>(P, X, T, B, grad,
                                                                                loss);
     return cudaGetLastError();
