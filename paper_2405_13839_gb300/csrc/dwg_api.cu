@@ -1721,11 +1721,12 @@ static int phase_blocks(const dwg_ctx *c, int ph)
     case kPhKnnFar: return ls ? knn_phase_blocks(c, ph) : 0;
     case kPhKnnDefer: return ls ? 8 : 0;  // blocks take the cloud's deferred faces in turn
     case kPhUpdate: return (int)ceil_div(c->n, 256);
+    case kPhSelSmall: return select_small(c->n) ? 1 : 0;
     case kPhSelHist:
-    case kPhSelSum: return select_blocks(c->n);
-    case kPhIso:
+    case kPhSelSum: return select_small(c->n) ? 0 : select_blocks(c->n);
     case kPhSelFind:
-    case kPhSelFinal: return 1;
+    case kPhSelFinal: return select_small(c->n) ? 0 : 1;
+    case kPhIso: return 1;
     default: return tree_phase_blocks(c, ph, -1);
     }
 }
@@ -1913,6 +1914,7 @@ static cudaError_t batch_lane_phases(dwg_ctx *h, const dwg_ctx::Lane &L, bool sc
     ok(launch_iter_batch(kPhKnnDefer, cl, off(kPhKnnDefer), ncl, ph[kPhKnnDefer], 0, s));
     // normal update and convergence
     ok(launch_iter_batch(kPhUpdate, cl, off(kPhUpdate), ncl, ph[kPhUpdate], 0, s));
+    ok(launch_iter_batch(kPhSelSmall, cl, off(kPhSelSmall), ncl, ph[kPhSelSmall], 0, s));
     for (int level = 0; level < 3; ++level) {
         ok(launch_iter_batch(kPhSelHist, cl, off(kPhSelHist), ncl, ph[kPhSelHist], level, s));
         ok(launch_iter_batch(kPhSelFind, cl, off(kPhSelFind), ncl, ph[kPhSelFind], level, s));

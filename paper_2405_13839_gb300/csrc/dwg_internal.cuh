@@ -215,9 +215,8 @@ struct CloudIter {
 
 // phases of a batched iteration (one launch each, every cloud's blocks)
 enum BatchPhase {
-    kPhReducePoints, kPhReduceW, kPhIso, kPhMcFaces, kPhKnn, kPhKnnLists, kPhKnnFar, kPhKnnDefer, kPhUpdate, kPhSelHist,
-    kPhSelFind,
-    kPhSelSum, kPhSelFinal, kPhLeafMom, kPhMomRec, kPhListsP, kPhListsC, kPhCombineP,
+    kPhReducePoints, kPhReduceW, kPhIso, kPhMcFaces, kPhKnn, kPhKnnLists, kPhKnnFar, kPhKnnDefer, kPhUpdate,
+    kPhSelSmall, kPhSelHist, kPhSelFind, kPhSelSum, kPhSelFinal, kPhLeafMom, kPhMomRec, kPhListsP, kPhListsC, kPhCombineP,
     kPhCombineC, kPhCount
 };
 
@@ -578,6 +577,7 @@ cudaError_t launch_knn_scatter(Ctx *c);
 cudaError_t launch_normal_update(Ctx *c);
 cudaError_t launch_select(Ctx *c, cudaGraphConditionalHandle cond, int use_cond);
 int select_blocks(int64_t n);
+bool select_small(int64_t n);
 cudaError_t launch_random_normals(float4 *nrm, const int64_t *perm, int64_t n, uint64_t seed,
                                   cudaStream_t s);
 cudaError_t launch_knn_query(Ctx *c, const float4 *q, int64_t m, int k, int64_t *idx_out);

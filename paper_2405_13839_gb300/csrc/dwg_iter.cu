@@ -2240,6 +2240,40 @@ __global__ void __launch_bounds__(kSelGridThreads)
     sel_sum_body(dtheta, n, ss, part, st, blockIdx.x, gridDim.x);
 }
 
+// the statistic, the trace and the loop condition (one thread)
+__device__ __forceinline__ void sel_decide(int64_t n, float tol, int rule, unsigned prefix,
+                                           unsigned above, double sum_above, double sum_dn,
+                                           IterState *st, double *tr_iso, double *tr_stat,
+                                           double *tr_dn, long long *tr_faces,
+                                           cudaGraphConditionalHandle cond, int use_cond)
+{
+    const unsigned k = (unsigned)((n + 99) / 100);
+    const float tval = __uint_as_float(prefix);
+    double stat = (sum_above + (double)(k - above) * (double)tval) / (double)k;
+    int it = st->iter;
+    st->stat = stat;
+    if (tr_iso && it < st->max_iters) {
+        tr_iso[it] = st->iso;
+        tr_stat[it] = stat;
+        tr_dn[it] = sum_dn / (double)n;
+        tr_faces[it] = st->nfaces;
+    }
+    it += 1;
+    st->iter = it;
+    // rule 0: mean of the largest 1 % of the changes <= tol degrees (Sec. 5.1);
+    // rule 1: mean |n_new - n_old| over all points <= 2 sin(tol / 2), the
+    // chord of tol degrees (the measure plotted in Fig. 6)
+    int done;
+    if (rule == 1) {
+        const double chord = 2.0 * sin((double)tol * (kPi / 360.0));
+        done = sum_dn / (double)n <= chord;
+    } else {
+        done = stat <= (double)tol;
+    }
+    st->done = done;
+    if (use_cond) cudaGraphSetConditional(cond, (!done && it < st->max_iters) ? 1u : 0u);
+}
+
 __device__ __forceinline__ void sel_final_body(int64_t n, float tol, int rule,
                                                const SelState *__restrict__ ss,
                                                const double *__restrict__ part, int npart,
@@ -2269,28 +2303,9 @@ __device__ __forceinline__ void sel_final_body(int64_t n, float tol, int rule,
         if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        const unsigned k = (unsigned)((n + 99) / 100);
-        const float tval = __uint_as_float(ss->prefix);
-        double stat = (sum_above + (double)(k - ss->above) * (double)tval) / (double)k;
-        int it = st->iter;
-        st->stat = stat;
-        if (tr_iso && it < st->max_iters) {
-            tr_iso[it] = st->iso;
-            tr_stat[it] = stat;
-            tr_dn[it] = sh[0] / (double)n;
-            tr_faces[it] = st->nfaces;
-        }
-        it += 1;
-        st->iter = it;
-        // rule 0: mean of the largest 1 % of the changes <= tol degrees (Sec. 5.1);
-        // rule 1: mean |n_new - n_old| over all points <= 2 sin(tol / 2), the
-        // chord of tol degrees (the measure plotted in Fig. 6)
-        const double chord = 2.0 * sin((double)tol * (kPi / 360.0));
-        int done = rule == 1 ? (sh[0] / (double)n <= chord) : (stat <= (double)tol);
-        st->done = done;
-        if (use_cond) cudaGraphSetConditional(cond, (!done && it < st->max_iters) ? 1u : 0u);
-    }
+    if (threadIdx.x == 0)
+        sel_decide(n, tol, rule, ss->prefix, ss->above, sum_above, sh[0], st, tr_iso, tr_stat,
+                   tr_dn, tr_faces, cond, use_cond);
 }
 
 __global__ void __launch_bounds__(kSelThreads)
@@ -2301,6 +2316,101 @@ __global__ void __launch_bounds__(kSelThreads)
 {
     sel_final_body(n, tol, rule, ss, part, npart, st, dn_blocks, ndn, tr_iso, tr_stat, tr_dn,
                    tr_faces, cond, use_cond);
+}
+
+// The whole selection of a small cloud in one CTA: the changes in registers,
+// the bins in shared memory, no launch between the levels.  The sum's
+// partials are those of k_sel_sum's blocks, a warp each, added in the order
+// of its tree, so the statistic is the same bits either way.  It is bound by
+// the chain of barriers and by the adds of one SM: 12 us in place of 39 for the
+// eight launches at 2,000 points, 18 at 16,384, where a cloud's other phases
+// take 580; the limit is what a thread holds in registers.
+constexpr int kSelSmallPer = 16;
+constexpr int64_t kSelSmallMax = kSelSmallPer * kSelThreads;
+
+__device__ __forceinline__ void sel_small_body(const float *__restrict__ dtheta, int64_t n,
+                                               float tol, int rule, IterState *st,
+                                               const double *__restrict__ dn_blocks,
+                                               double *tr_iso, double *tr_stat, double *tr_dn,
+                                               long long *tr_faces,
+                                               cudaGraphConditionalHandle cond, int use_cond)
+{
+    if (cloud_idle(st)) return;
+    __shared__ unsigned h[2 * kSelBins + 256];  // the three levels' bins
+    __shared__ unsigned warp_sums[33];
+    __shared__ int s_bin;
+    __shared__ unsigned s_above;
+    __shared__ double part[32];
+    static_assert(kSelSmallMax <= 32 * 4 * kSelGridThreads && kSelSmallMax <= 64 * 256, "sums");
+    const unsigned *bits = reinterpret_cast<const unsigned *>(dtheta);
+    unsigned v[kSelSmallPer];
+#pragma unroll
+    for (int j = 0; j < kSelSmallPer; ++j) {
+        const int64_t i = threadIdx.x + (int64_t)j * kSelThreads;
+        v[j] = i < n ? bits[i] : 0u;
+    }
+    for (int b = threadIdx.x; b < 2 * kSelBins + 256; b += kSelThreads) h[b] = 0;
+    __syncthreads();
+    unsigned prefix = 0, above = 0, krem = (unsigned)((n + 99) / 100);
+    for (int level = 0; level < 3; ++level) {
+        unsigned *hl = h + level * kSelBins;
+        const int shift = level == 0 ? 20 : (level == 1 ? 8 : 0);
+        const unsigned mask = level == 2 ? 255u : 4095u;
+        const int sh_hi = level == 1 ? 20 : 8;
+#pragma unroll
+        for (int j = 0; j < kSelSmallPer; ++j)
+            if (threadIdx.x + (int64_t)j * kSelThreads < n &&
+                (level == 0 || (v[j] >> sh_hi) == prefix))
+                atomicAdd(&hl[(v[j] >> shift) & mask], 1u);
+        __syncthreads();
+        find_bin(hl, level == 2 ? 256 : 4096, krem, warp_sums, &s_bin, &s_above);
+        prefix = (prefix << (level == 2 ? 8 : 12)) | (unsigned)s_bin;
+        above += s_above;
+        krem -= s_above;  // (written again behind the next level's first barrier)
+    }
+    const int nblk = (int)((n + 4 * kSelGridThreads - 1) / (4 * kSelGridThreads));
+    const int lane = threadIdx.x & 31;
+    for (int b = threadIdx.x >> 5; b < nblk; b += kSelThreads / 32) {
+        double p[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            p[q] = 0.0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int64_t i =
+                    ((int64_t)k * nblk + b) * kSelGridThreads + 32 * q + lane;
+                const unsigned u = i < n ? bits[i] : 0u;
+                // one change in a hundred counts: most warps skip the add
+                if (__any_sync(0xffffffffu, u > prefix))
+                    if (u > prefix) p[q] += (double)__uint_as_float(u);
+            }
+        }
+        double t = ((p[0] + p[4]) + (p[2] + p[6])) + ((p[1] + p[5]) + (p[3] + p[7]));
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) part[b] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    // k_sel_final's trees, whose other entries are zero
+    const int ndn = (int)((n + 255) / 256);
+    double sum = lane < nblk ? part[lane] : 0.0;
+    double dn = (lane < ndn ? dn_blocks[lane] : 0.0) + (lane + 32 < ndn ? dn_blocks[lane + 32] : 0.0);
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_down_sync(0xffffffffu, sum, o);
+        dn += __shfl_down_sync(0xffffffffu, dn, o);
+    }
+    if (lane == 0)
+        sel_decide(n, tol, rule, prefix, above, sum, dn, st, tr_iso, tr_stat, tr_dn, tr_faces, cond,
+                   use_cond);
+}
+
+__global__ void __launch_bounds__(kSelThreads)
+    k_sel_small(const float *__restrict__ dtheta, int64_t n, float tol, int rule, IterState *st,
+                const double *__restrict__ dn_blocks, double *tr_iso, double *tr_stat,
+                double *tr_dn, long long *tr_faces, cudaGraphConditionalHandle cond, int use_cond)
+{
+    sel_small_body(dtheta, n, tol, rule, st, dn_blocks, tr_iso, tr_stat, tr_dn, tr_faces, cond,
+                   use_cond);
 }
 
 // ---------------------------------------------------------------------------
@@ -2786,8 +2896,16 @@ int select_blocks(int64_t n)
     return (int)std::min<int64_t>(std::max<int64_t>(ceil_div(n, 4 * kSelGridThreads), 1), 1024);
 }
 
+bool select_small(int64_t n) { return n <= kSelSmallMax; }
+
 cudaError_t launch_select(Ctx *c, cudaGraphConditionalHandle cond, int use_cond)
 {
+    if (select_small(c->n)) {
+        k_sel_small<<<1, kSelThreads, 0, c->stream>>>(
+            c->d_dtheta, c->n, c->tol, c->conv_rule, c->d_state, c->d_dn_blocks, c->d_tr_iso,
+            c->d_tr_stat, c->d_tr_dn, c->d_tr_faces, cond, use_cond);
+        return cudaGetLastError();
+    }
     const int nb = select_blocks(c->n);
     for (int level = 0; level < 3; ++level) {
         k_sel_hist<<<nb, kSelGridThreads, 0, c->stream>>>(c->d_dtheta, c->n, level, c->d_sel,
@@ -2880,9 +2998,19 @@ __global__ void __launch_bounds__(kSelGridThreads)
                   (int64_t)off[ci + 1] - off[ci]);
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_sel_find_b(const CloudIter *__restrict__ cl, int level)
+// small clouds (select_small): the whole selection in one block
+__global__ void __launch_bounds__(kSelThreads)
+    k_sel_small_b(const CloudIter *__restrict__ cl, const int *__restrict__ off, int ncl)
 {
-    const CloudIter &c = cl[blockIdx.x];
+    const CloudIter &c = cl[seg_cloud(off, ncl)];
+    sel_small_body(c.dtheta, c.n, c.tol, c.conv_rule, c.st, c.dn_blocks, c.tr_iso, c.tr_stat,
+                   c.tr_dn, c.tr_faces, 0, 0);
+}
+
+__global__ void __launch_bounds__(kSelThreads)
+    k_sel_find_b(const CloudIter *__restrict__ cl, const int *__restrict__ off, int ncl, int level)
+{
+    const CloudIter &c = cl[seg_cloud(off, ncl)];
     sel_find_body(c.n, level, c.sel, c.sel_hist, c.st);
 }
 
@@ -2895,9 +3023,10 @@ __global__ void __launch_bounds__(kSelGridThreads)
                  (int64_t)off[ci + 1] - off[ci]);
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_sel_final_b(const CloudIter *__restrict__ cl)
+__global__ void __launch_bounds__(kSelThreads)
+    k_sel_final_b(const CloudIter *__restrict__ cl, const int *__restrict__ off, int ncl)
 {
-    const CloudIter &c = cl[blockIdx.x];
+    const CloudIter &c = cl[seg_cloud(off, ncl)];
     sel_final_body(c.n, c.tol, c.conv_rule, c.sel, c.sel_part, c.sel_nb, c.st, c.dn_blocks,
                    (int)((c.n + 255) / 256), c.tr_iso, c.tr_stat, c.tr_dn, c.tr_faces, 0, 0);
 }
@@ -2917,10 +3046,11 @@ cudaError_t launch_iter_batch(int phase, const CloudIter *cl, const int *off, in
         k_knn_deferred_b<<<g, defer_threads<10>(), 0, s>>>(cl, off, ncl);
         break;
     case kPhUpdate: k_normal_update_b<<<g, 256, 0, s>>>(cl, off, ncl); break;
+    case kPhSelSmall: k_sel_small_b<<<g, kSelThreads, 0, s>>>(cl, off, ncl); break;
     case kPhSelHist: k_sel_hist_b<<<g, kSelGridThreads, 0, s>>>(cl, off, ncl, arg); break;
-    case kPhSelFind: k_sel_find_b<<<(unsigned)ncl, kSelThreads, 0, s>>>(cl, arg); break;
+    case kPhSelFind: k_sel_find_b<<<g, kSelThreads, 0, s>>>(cl, off, ncl, arg); break;
     case kPhSelSum: k_sel_sum_b<<<g, kSelGridThreads, 0, s>>>(cl, off, ncl); break;
-    case kPhSelFinal: k_sel_final_b<<<(unsigned)ncl, kSelThreads, 0, s>>>(cl); break;
+    case kPhSelFinal: k_sel_final_b<<<g, kSelThreads, 0, s>>>(cl, off, ncl); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
