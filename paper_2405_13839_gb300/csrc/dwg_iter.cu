@@ -83,52 +83,69 @@ __device__ __forceinline__ F3 lerp0(F3 xa, float fa, F3 xb, float fb)
     return {xa.x + t * (xb.x - xa.x), xa.y + t * (xb.y - xa.y), xa.z + t * (xb.z - xa.z)};
 }
 
-// polygon of one tetrahedron: returns false when the level set misses it
-__device__ __forceinline__ bool tet_face(const F3 x[4], const float f[4], const bool ab[4],
-                                         F3 &area, F3 &cen)
+// Polygon of a tetrahedron that the level set cuts; m has bit i where vertex i
+// is above.  The vertices are first put in the order lone vertex, others (one
+// on its own side) or two above, two below: by selects over all four, so that
+// nothing is indexed and everything stays in registers.
+__device__ __forceinline__ void tet_face(const F3 (&x)[4], const float (&f)[4], int m, F3 &area,
+                                         F3 &cen)
 {
-    int na = (int)ab[0] + (int)ab[1] + (int)ab[2] + (int)ab[3];
-    if (na == 0 || na == 4) return false;
+    // per mask, 2 bits a place: which vertex comes first, second, ...
+    // (mask 0 and 15 do not occur)
+    const int na = __popc(m);
+    const int mm = na == 3 ? 15 - m : m;  // the lone vertex's bit
+    // orders of the masks 1 2 3 4 5 6 8 9 10 12, 8 bits each, at 8 * mask
+    const unsigned long long t0 = 0xe4ull << 8 | 0xe1ull << 16 | 0xe4ull << 24 | 0xd2ull << 32 |
+                                  0xd8ull << 40 | 0xc9ull << 48;
+    const unsigned long long t1 = 0x93ull | 0x9cull << 8 | 0x8dull << 16 | 0x4eull << 32;
+    const unsigned perm = (unsigned)((mm < 8 ? t0 : t1) >> (8 * (mm & 7)));
+    F3 v[4];
+    float g[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int j = (perm >> (2 * i)) & 3;
+        v[i] = j == 0 ? x[0] : j == 1 ? x[1] : j == 2 ? x[2] : x[3];
+        g[i] = j == 0 ? f[0] : j == 1 ? f[1] : j == 2 ? f[2] : f[3];
+    }
     F3 P[4];
-    int np;
-    if (na == 1 || na == 3) {
-        bool want = (na == 1);
-        int lone = 0;
-        for (int i = 0; i < 4; ++i)
-            if (ab[i] == want) lone = i;
-        np = 0;
-        for (int i = 0; i < 4; ++i)
-            if (i != lone) P[np++] = lerp0(x[lone], f[lone], x[i], f[i]);
-        area = cross(P[1] - P[0], P[2] - P[0]);
-    } else {
-        int a0 = -1, a1 = -1, b0 = -1, b1 = -1;
-        for (int i = 0; i < 4; ++i) {
-            if (ab[i]) { if (a0 < 0) a0 = i; else a1 = i; }
-            else { if (b0 < 0) b0 = i; else b1 = i; }
-        }
-        P[0] = lerp0(x[a0], f[a0], x[b0], f[b0]);
-        P[1] = lerp0(x[a0], f[a0], x[b1], f[b1]);
-        P[2] = lerp0(x[a1], f[a1], x[b1], f[b1]);
-        P[3] = lerp0(x[a1], f[a1], x[b0], f[b0]);
-        np = 4;
+    F3 ca = {0, 0, 0}, cb = {0, 0, 0};
+    auto add = [](F3 &a, F3 p) { a.x += p.x; a.y += p.y; a.z += p.z; };
+    const bool quad = na == 2;
+    P[0] = lerp0(v[0], g[0], quad ? v[2] : v[1], quad ? g[2] : g[1]);
+    P[1] = lerp0(v[0], g[0], quad ? v[3] : v[2], quad ? g[3] : g[2]);
+    P[2] = lerp0(quad ? v[1] : v[0], quad ? g[1] : g[0], v[3], g[3]);
+    P[3] = lerp0(v[1], g[1], v[2], g[2]);  // of a quadrilateral
+    F3 s = {0, 0, 0};
+    if (quad) {
         area = cross(P[2] - P[0], P[3] - P[1]);
+        add(ca, v[0]);
+        add(ca, v[1]);
+        add(cb, v[2]);
+        add(cb, v[3]);
+    } else {
+        area = cross(P[1] - P[0], P[2] - P[0]);
+        add(ca, v[0]);
+        add(cb, v[1]);
+        add(cb, v[2]);
+        add(cb, v[3]);
+        if (na == 3) {
+            const F3 t = ca;
+            ca = cb;
+            cb = t;
+        }
     }
     area.x *= 0.5f; area.y *= 0.5f; area.z *= 0.5f;
-    F3 ca = {0, 0, 0}, cb = {0, 0, 0};
-    for (int i = 0; i < 4; ++i) {
-        if (ab[i]) { ca.x += x[i].x; ca.y += x[i].y; ca.z += x[i].z; }
-        else { cb.x += x[i].x; cb.y += x[i].y; cb.z += x[i].z; }
-    }
-    float ia = 1.f / na, ib = 1.f / (4 - na);
+    const float ia = 1.f / na, ib = 1.f / (4 - na);
     F3 dir = {ca.x * ia - cb.x * ib, ca.y * ia - cb.y * ib, ca.z * ia - cb.z * ib};
     if (area.x * dir.x + area.y * dir.y + area.z * dir.z < 0.f) {
         area.x = -area.x; area.y = -area.y; area.z = -area.z;
     }
-    F3 s = {0, 0, 0};
-    for (int i = 0; i < np; ++i) { s.x += P[i].x; s.y += P[i].y; s.z += P[i].z; }
-    float inv = 1.f / np;
+    add(s, P[0]);
+    add(s, P[1]);
+    add(s, P[2]);
+    if (quad) add(s, P[3]);
+    const float inv = quad ? 0.25f : 1.f / 3;
     cen = {s.x * inv, s.y * inv, s.z * inv};
-    return true;
 }
 
 // Triangles of one tetrahedron's piece of the level set (0, 1 or 2), on the
@@ -257,7 +274,13 @@ cudaError_t launch_mc_tris(Ctx *c, float *out, int64_t cap, unsigned long long *
 // Faces of the level set.  Each face record also carries its leaf's index
 // (in the area's w) and, in the centroid's w, the position in the
 // Morton-sorted points of the face's leaf cell (found once per cut leaf):
-// the k-nearest search of its faces starts there.
+// the k-nearest search of its faces starts there.  The signs at the eight
+// corners say how many faces a leaf has, so a leaf that is not cut reads
+// nothing else and the faces are written as they are computed.  Bound by the
+// latency of the gathers on a small octree, by their L2 traffic on a large
+// one: 22.5 -> 16.4 us on a 2,000-point sphere and 2.92 -> 2.37 ms on a 4M
+// union (random normals) against vertices indexed in local memory and all
+// positions read.
 __device__ __forceinline__ void mc_faces_body(const int *__restrict__ leaf_corners,
                                               const int4 *__restrict__ leaves, int64_t nl,
                                               const float4 *__restrict__ cpos,
@@ -269,31 +292,28 @@ __device__ __forceinline__ void mc_faces_body(const int *__restrict__ leaf_corne
     if (cloud_idle(st)) return;  // finished cloud of a batch
     int64_t l = bid * blockDim.x + threadIdx.x;
     const double iso = st->iso;
-    F3 area[6], cen[6];
+    // corner masks of the six tetrahedra (corners 0 and 7 and two more)
+    constexpr int tets[6][4] = {{0, 1, 3, 7}, {0, 3, 2, 7}, {0, 2, 6, 7},
+                                {0, 6, 4, 7}, {0, 4, 5, 7}, {0, 5, 1, 7}};
     int cnt = 0;
+    int ci[8];
+    float f[8];
+    bool ab[8];
     if (l < nl) {
-        F3 x[8];
-        float f[8];
-        bool ab[8];
+        const int4 c0 = reinterpret_cast<const int4 *>(leaf_corners)[2 * l];
+        const int4 c1 = reinterpret_cast<const int4 *>(leaf_corners)[2 * l + 1];
+        ci[0] = c0.x; ci[1] = c0.y; ci[2] = c0.z; ci[3] = c0.w;
+        ci[4] = c1.x; ci[5] = c1.y; ci[6] = c1.z; ci[7] = c1.w;
+#pragma unroll
         for (int v = 0; v < 8; ++v) {
-            int ci = leaf_corners[l * 8 + v];
-            x[v] = f3(cpos[ci]);
-            double df = (double)wc[ci] - iso;
+            double df = (double)wc[ci[v]] - iso;
             f[v] = (float)df;
             ab[v] = df > 0.0;
         }
 #pragma unroll
         for (int t = 0; t < 6; ++t) {
-            F3 xt[4];
-            float ft[4];
-            bool at[4];
-            for (int i = 0; i < 4; ++i) {
-                int v = c_tets[t][i];
-                xt[i] = x[v];
-                ft[i] = f[v];
-                at[i] = ab[v];
-            }
-            if (tet_face(xt, ft, at, area[cnt], cen[cnt])) ++cnt;
+            const int na = (int)ab[0] + (int)ab[tets[t][1]] + (int)ab[tets[t][2]] + (int)ab[7];
+            cnt += (na & 3) != 0;
         }
     }
     int seed = 0;
@@ -320,13 +340,26 @@ __device__ __forceinline__ void mc_faces_body(const int *__restrict__ leaf_corne
     if (lane == 31 && total > 0) base = atomicAdd(&st->nfaces, total);
     base = __shfl_sync(0xffffffffu, base, 31);
     int64_t o = (int64_t)base + incl - cnt;
-    for (int k = 0; k < cnt; ++k, ++o) {
+    if (cnt == 0) return;
+    F3 x[8];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) x[v] = f3(cpos[ci[v]]);
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+        const int m = (int)ab[0] | (int)ab[tets[t][1]] << 1 | (int)ab[tets[t][2]] << 2 |
+                      (int)ab[7] << 3;
+        if (m == 0 || m == 15) continue;
         if (o >= max_faces) {
             atomicOr(err, kErrOverflow);
             break;
         }
-        faces[2 * o] = make_float4(area[k].x, area[k].y, area[k].z, __int_as_float((int)l));
-        faces[2 * o + 1] = make_float4(cen[k].x, cen[k].y, cen[k].z, __int_as_float(seed));
+        const F3 xt[4] = {x[0], x[tets[t][1]], x[tets[t][2]], x[7]};
+        const float ft[4] = {f[0], f[tets[t][1]], f[tets[t][2]], f[7]};
+        F3 area, cen;
+        tet_face(xt, ft, m, area, cen);
+        faces[2 * o] = make_float4(area.x, area.y, area.z, __int_as_float((int)l));
+        faces[2 * o + 1] = make_float4(cen.x, cen.y, cen.z, __int_as_float(seed));
+        ++o;
     }
 }
 
