@@ -983,6 +983,7 @@ __device__ __forceinline__ void reduce_points_body(const float *__restrict__ par
     if (i < m) {
         float h[NA], l[NA];
         for (int a = 0; a < NA; ++a) { h[a] = 0.f; l[a] = 0.f; }
+#pragma unroll 4
         for (int ch = 0; ch < nchunks; ++ch)
             for (int a = 0; a < NA; ++a) {
                 float ph = part[((int64_t)(ch * NA + a) * 2 + 0) * stride + i];
@@ -1101,6 +1102,7 @@ __device__ __forceinline__ void reduce_w_body(const float *__restrict__ part, in
     int64_t i = bid * blockDim.x + threadIdx.x;
     if (i >= m) return;
     float h = 0.f, l = 0.f;
+#pragma unroll 4
     for (int ch = 0; ch < nchunks; ++ch) {
         two_sum1(h, l, part[((int64_t)ch * 2 + 0) * stride + i]);
         l = __fadd_rn(l, part[((int64_t)ch * 2 + 1) * stride + i]);
@@ -1118,6 +1120,7 @@ __device__ __forceinline__ void reduce_lattice_body(const float *__restrict__ pa
     const int to = corner[i];
     if (to < 0) return;
     float h = 0.f, l = 0.f;
+#pragma unroll 4
     for (int ch = 0; ch < nchunks; ++ch) {
         two_sum1(h, l, part[((int64_t)ch * 2 + 0) * slots + i]);
         l = __fadd_rn(l, part[((int64_t)ch * 2 + 1) * slots + i]);

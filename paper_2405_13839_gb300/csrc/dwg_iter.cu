@@ -994,7 +994,11 @@ constexpr size_t kAggSmem =
 // 64-bit keys and its own tree search (random normals / 3rd-16th iteration):
 // 2,000-point sphere 0.63 / 0.19 -> 0.10 / 0.05 ms, 100k torus 2.8 / 1.9 ->
 // 0.33 / 0.18 ms, 1M blob 13.5 / 10.2 -> 5.5 / 3.8 ms, 4M union 29 / 14.5 ->
-// 12.1 / 5.2 ms.
+// 12.1 / 5.2 ms.  On a small cloud one face's chain of dependent loads (index,
+// point, four at a time) is the time: with the next indices loading beside the
+// points, and 80 registers rather than 64, 94 / 49 -> 84 / 41 us at 2,000
+// points and 12.1 / 5.2 -> 11.5 / 4.9 ms on the 4M union; eight at a time 80 /
+// 37 us but 11.9 / 5.1 ms.
 constexpr int kScanK = 10;
 constexpr int kTabBits = 8;
 constexpr int kTabSlots = 1 << kTabBits;
@@ -1042,14 +1046,20 @@ __device__ __forceinline__ void knn_lists_body(const float4 *__restrict__ faces,
             unsigned b[kScanK + 1];
 #pragma unroll
             for (int t = 0; t <= kScanK; ++t) b[t] = 0xffffffffu;
-            for (int t = 0; t < len; t += 4) {
-                int jj[4];
-                unsigned ky[4];
+            // the indices of the next four load beside these four points
+            int jn[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) jj[u] = __ldg(&cand[min(t + u, len - 1)]);
+            for (int u = 0; u < 4; ++u) jn[u] = __ldg(&cand[min(u, len - 1)]);
+            for (int t = 0; t < len; t += 4) {
+                unsigned ky[4];
+                float4 pp[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) pp[u] = __ldg(&T.p4[jn[u]]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) jn[u] = __ldg(&cand[min(t + 4 + u, len - 1)]);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const float d = pt_d2(__ldg(&T.p4[jj[u]]), q);
+                    const float d = pt_d2(pp[u], q);
                     ky[u] = t + u < len ? (__float_as_uint(d) & 0xffffff00u) | (unsigned)(t + u)
                                         : 0xffffffffu;
                 }
@@ -1118,7 +1128,7 @@ __device__ __forceinline__ void knn_lists_body(const float4 *__restrict__ faces,
     }
 }
 
-__global__ void __launch_bounds__(32 * kScanWarps, 8)
+__global__ void __launch_bounds__(32 * kScanWarps, 6)
     k_knn_lists(const float4 *__restrict__ faces, IterState *st, int64_t max_faces, KnnTree T,
                 const int64_t *__restrict__ cell_off, const int *__restrict__ cell_idx,
                 double scale, unsigned long long *acc, int *far_q, int agg)
@@ -2975,7 +2985,7 @@ __global__ void __launch_bounds__(256)
 }
 
 // a batch has k = 10; clouds without candidate lists search the tree
-__global__ void __launch_bounds__(32 * kScanWarps, 8)
+__global__ void __launch_bounds__(32 * kScanWarps, 6)
     k_knn_lists_b(const CloudIter *__restrict__ cl, const int *__restrict__ off, int ncl)
 {
     const int ci = seg_cloud(off, ncl);
