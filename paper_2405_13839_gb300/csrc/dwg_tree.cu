@@ -613,13 +613,13 @@ __device__ __forceinline__ GrpQueries grp_queries(const float4 *__restrict__ q, 
     return G;
 }
 
-// One warp walks the tree for its group, 32 nodes per step (one per lane).
+// One warp walks the tree for its group, 32 W nodes per step (W per lane).
 // A node far from the group's box goes to on_far, a near leaf to on_near,
 // an open node pushes its children.  on_far(is_far, node, record, mask) and
 // on_near(is_near, leaf, mask) are called by every lane, on_far each step
-// and on_near where the mask is not empty (both warp-uniform).  Returns
-// false if the stack would overflow.
-template <class FarFn, class NearFn>
+// and on_near where the mask is not empty (both warp-uniform), W times a
+// step.  Returns false if the stack of W * kGrpStack entries would overflow.
+template <int W = 1, class FarFn, class NearFn>
 __device__ __forceinline__ bool grp_walk(int *stack, const float4 *__restrict__ rec,
                                          int64_t nleaf, const GrpQueries &G, int lane,
                                          FarFn &&on_far, NearFn &&on_near)
@@ -629,34 +629,41 @@ __device__ __forceinline__ bool grp_walk(int *stack, const float4 *__restrict__ 
     if (lane == 0) stack[0] = 1;
     __syncwarp();
     while (sp > 0) {
-        const int k = min(sp, 32);
+        const int k = min(sp, 32 * W);
         sp -= k;
-        const int node = lane < k ? stack[sp + lane] : 0;
+        int node[W], act[W];  // act: 1 far, 2 near leaf, 3 open
+        float4 cr[W];
+#pragma unroll
+        for (int u = 0; u < W; ++u) node[u] = 32 * u + lane < k ? stack[sp + 32 * u + lane] : 0;
         __syncwarp();  // every pop is read before pushes overwrite the slots
-        int act = 0;   // 1 far, 2 near leaf, 3 open
-        float4 cr = make_float4(0.f, 0.f, 0.f, -1.f);
-        if (lane < k) {
-            cr = rec[node];
-            if (cr.w >= 0.f) {
-                float ex = fmaxf(fmaxf(__fsub_rn(G.lox, cr.x), __fsub_rn(cr.x, G.hix)), 0.f);
-                float ey = fmaxf(fmaxf(__fsub_rn(G.loy, cr.y), __fsub_rn(cr.y, G.hiy)), 0.f);
-                float ez = fmaxf(fmaxf(__fsub_rn(G.loz, cr.z), __fsub_rn(cr.z, G.hiz)), 0.f);
+#pragma unroll
+        for (int u = 0; u < W; ++u)
+            cr[u] = 32 * u + lane < k ? rec[node[u]] : make_float4(0.f, 0.f, 0.f, -1.f);
+#pragma unroll
+        for (int u = 0; u < W; ++u) {
+            if (u > 0 && 32 * u >= k) break;
+            const float4 c = cr[u];
+            act[u] = 0;
+            if (c.w >= 0.f) {
+                float ex = fmaxf(fmaxf(__fsub_rn(G.lox, c.x), __fsub_rn(c.x, G.hix)), 0.f);
+                float ey = fmaxf(fmaxf(__fsub_rn(G.loy, c.y), __fsub_rn(c.y, G.hiy)), 0.f);
+                float ez = fmaxf(fmaxf(__fsub_rn(G.loz, c.z), __fsub_rn(c.z, G.hiz)), 0.f);
                 float d2 = fmaf(ez, ez, fmaf(ey, ey, __fmul_rn(ex, ex)));
-                act = d2 > cr.w ? 1 : ((int64_t)node >= nleaf ? 2 : 3);
+                act[u] = d2 > c.w ? 1 : ((int64_t)node[u] >= nleaf ? 2 : 3);
             }
+            on_far(act[u] == 1, node[u], c, __ballot_sync(0xffffffffu, act[u] == 1));
+            const unsigned om = __ballot_sync(0xffffffffu, act[u] == 3);
+            const int no = __popc(om);
+            if (sp + 2 * no > W * kGrpStack) return false;
+            if (act[u] == 3) {
+                const int pos = sp + 2 * __popc(om & lt);
+                stack[pos] = 2 * node[u] + 1;
+                stack[pos + 1] = 2 * node[u];
+            }
+            sp += 2 * no;
+            const unsigned nm = __ballot_sync(0xffffffffu, act[u] == 2);
+            if (nm) on_near(act[u] == 2, node[u], nm);
         }
-        on_far(act == 1, node, cr, __ballot_sync(0xffffffffu, act == 1));
-        const unsigned om = __ballot_sync(0xffffffffu, act == 3);
-        const int no = __popc(om);
-        if (sp + 2 * no > kGrpStack) return false;
-        if (act == 3) {
-            const int pos = sp + 2 * __popc(om & lt);
-            stack[pos] = 2 * node + 1;
-            stack[pos + 1] = 2 * node;
-        }
-        sp += 2 * no;
-        const unsigned nm = __ballot_sync(0xffffffffu, act == 2);
-        if (nm) on_near(act == 2, node, nm);
         __syncwarp();
     }
     return true;
@@ -787,16 +794,25 @@ __global__ void __launch_bounds__(32 * kGrpWarps)
 // iteration only evaluates them.
 // ---------------------------------------------------------------------------
 constexpr int kListWarps = 8;
+// A call's lists (eval_call_lists_t) take kWalkW nodes a lane and step: a
+// group whose box straddles a jump of the Morton order opens thousands of
+// nodes, and its warp's chain of steps holds the launch (110,592 queries of
+// 300,000 sources, the two walks of a call: 204 us at one, 165 at two, 144 at
+// four, 165 at eight, whose stacks leave too few warps).
+// The order of a list's nodes differs from the walk of one node a lane; the
+// iteration's lists, made once, keep that one.
+constexpr int kWalkW = 4;
+__host__ __device__ constexpr int list_warps(int W) { return W == 1 ? kListWarps : kListWarps / W; }
 
-template <bool FILL>
-__global__ void __launch_bounds__(32 * kListWarps)
+template <bool FILL, int W = 1>
+__global__ void __launch_bounds__(32 * list_warps(W))
     k_tree_lists(const float4 *__restrict__ q, int64_t m, const float4 *__restrict__ rec,
                  int levels, int64_t *far_n, int64_t *near_n, int *__restrict__ far_ids,
                  int *__restrict__ near_ids, int *err)
 {
-    __shared__ int stack[kListWarps][kGrpStack];
+    __shared__ int stack[list_warps(W)][W * kGrpStack];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t g = (int64_t)blockIdx.x * kListWarps + wid;
+    const int64_t g = (int64_t)blockIdx.x * list_warps(W) + wid;
     const int64_t q0 = g * kGrpQ;
     if (q0 >= m) return;
     const GrpQueries G = grp_queries(q, m, q0, lane);
@@ -804,7 +820,7 @@ __global__ void __launch_bounds__(32 * kListWarps)
     const unsigned lt = (1u << lane) - 1u;
     // FILL: far_n / near_n hold each group's first slot; else they get counts
     int64_t nf = FILL ? far_n[g] : 0, nn = FILL ? near_n[g] : 0;
-    const bool ok = grp_walk(
+    const bool ok = grp_walk<W>(
         stack[wid], rec, nleaf, G, lane,
         [&](bool is_far, int node, const float4 &, unsigned fm) {
             if (FILL && is_far) far_ids[nf + __popc(fm & lt)] = node;
@@ -1445,7 +1461,7 @@ __global__ void __launch_bounds__(1024)
 // (110,592 queries are 1,728 warps, 11 an SM, at 43 % of the FMA pipe);
 // here the lists are cut into items of at most kItemRecords records and
 // evaluated by k_tree_eval_lists.  300,000 sources, w and grad w at 110,592
-// lattice queries: 1,392 -> 690 us (walks 204, evaluation 473).  In ranges
+// lattice queries: 1,392 -> 630 us (walks 144, evaluation 473).  In ranges
 // of groups; a range whose
 // lists would take more than kCallLists bytes (queries in no order open the
 // whole tree) is walked.
@@ -1462,12 +1478,12 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
         const float4 *qr = q + g0 * kGrpQ;
         const int64_t mr = std::min<int64_t>(m - g0 * kGrpQ, (int64_t)ng * kGrpQ);
         float *pr = part + g0 * kGrpQ;
-        const unsigned blocks = (unsigned)ceil_div(ng, kListWarps);
+        const unsigned blocks = (unsigned)ceil_div(ng, list_warps(kWalkW));
         int64_t *buf = nullptr;
         DWG_CUDA_TRY(c, scratch_get(c, &buf, (5 * (int64_t)ng + 7) * sizeof(int64_t)));
         int64_t *cnt_f = buf, *cnt_n = cnt_f + ng, *far_off = cnt_n + ng, *near_off = far_off + ng + 1,
                 *item_off = near_off + ng + 1, *tot = item_off + ng + 1;
-        k_tree_lists<false><<<blocks, 32 * kListWarps, 0, c->stream>>>(
+        k_tree_lists<false, kWalkW><<<blocks, 32 * list_warps(kWalkW), 0, c->stream>>>(
             qr, mr, c->d_tree_rec, c->tree_levels, cnt_f, cnt_n, nullptr, nullptr, c->d_err);
         k_tree_list_offsets<<<1, 1024, 0, c->stream>>>(cnt_f, cnt_n, ng, c->tree_leaf, far_off,
                                                        near_off, item_off, tot);
@@ -1489,7 +1505,7 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
         DWG_CUDA_TRY(c, scratch_get(c, &near_ids, ht[1] * sizeof(int)));
         DWG_CUDA_TRY(c, scratch_get(c, &items, ht[2] * sizeof(int2)));
         DWG_CUDA_TRY(c, scratch_get(c, &ipart, ht[2] * item_bytes));
-        k_tree_lists<true><<<blocks, 32 * kListWarps, 0, c->stream>>>(
+        k_tree_lists<true, kWalkW><<<blocks, 32 * list_warps(kWalkW), 0, c->stream>>>(
             qr, mr, c->d_tree_rec, c->tree_levels, far_off, near_off, far_ids, near_ids, c->d_err);
         const int irec = (int)ht[3];
         k_tree_item_table<<<(unsigned)ceil_div(ng, 256), 256, 0, c->stream>>>(item_off, ng, irec,
