@@ -969,8 +969,8 @@ __device__ __forceinline__ int64_t warp_lower_bound(const uint64_t *__restrict__
 // The tables take 28 KB of shared memory per block, which the SM takes from
 // its L1 cache: on clouds of millions of points the searches' gathers lose
 // more to the smaller cache than the tables save (a 3M-point union: 80.8 ->
-// 40.7 ms with them; a 15M-point union: 49 -> 70 ms), so clouds above
-// kAggMaxPoints add straight to the points' sums.
+// 40.7 ms with them; a 15M-point union: 49 -> 70 ms), so in k_knn_scatter
+// clouds above kAggMaxPoints add straight to the points' sums.
 constexpr int kAggBits = 8;
 constexpr int kAggSlots = 1 << kAggBits;  // table entries per warp of 32 faces
 constexpr int kAggWarps = 4;              // warps of a 128-thread block
@@ -988,7 +988,9 @@ constexpr size_t kAggSmem =
 // key agree above them; that face is scanned again with the full (distance,
 // input index) keys.  Faces without a list are queued for k_knn_far.
 // The sums per warp are 32-bit here: a face vector is below 2^25 units (8
-// finest-cell areas) or goes straight to the points' sums.
+// finest-cell areas) or goes straight to the points' sums.  At 16 KB a block
+// the tables pay at every size (15M points: 37.4 / 15.4 ms straight to the
+// points' sums, 36.4 / 14.9 with them).
 // Bound: the gathers of the candidates (L1 wavefronts 77 % of their peak)
 // and the integer pipe.  With k_knn_far against the one thread per face with
 // 64-bit keys and its own tree search (random normals / 3rd-16th iteration):
@@ -1010,8 +1012,7 @@ __device__ __forceinline__ void knn_lists_body(const float4 *__restrict__ faces,
                                                int64_t max_faces, const KnnTree &T,
                                                const int64_t *__restrict__ cell_off,
                                                const int *__restrict__ cell_idx, double scale,
-                                               unsigned long long *acc, int *far_q, bool agg,
-                                               int64_t bid)
+                                               unsigned long long *acc, int *far_q, int64_t bid)
 {
     if (cloud_idle(st)) return;  // finished cloud of a batch
     const int64_t nf = min((int64_t)st->nfaces, max_faces);
@@ -1020,11 +1021,10 @@ __device__ __forceinline__ void knn_lists_body(const float4 *__restrict__ faces,
     extern __shared__ int s_tab[];
     int *s_key = s_tab + wid * 4 * kTabSlots;
     int *s_v = s_key + kTabSlots;
-    if (agg)
-        for (int i = lane; i < kTabSlots; i += 32) {
-            s_key[i] = -1;
-            s_v[i] = s_v[kTabSlots + i] = s_v[2 * kTabSlots + i] = 0;
-        }
+    for (int i = lane; i < kTabSlots; i += 32) {
+        s_key[i] = -1;
+        s_v[i] = s_v[kTabSlots + i] = s_v[2 * kTabSlots + i] = 0;
+    }
     const int64_t f = bid * blockDim.x + threadIdx.x;
     int bj[kScanK];
 #pragma unroll
@@ -1094,7 +1094,7 @@ __device__ __forceinline__ void knn_lists_body(const float4 *__restrict__ faces,
         atomicAdd(a + 1, (unsigned long long)vy);
         atomicAdd(a + 2, (unsigned long long)vz);
     };
-    const bool small = agg && llabs(vx) < kTabMax && llabs(vy) < kTabMax && llabs(vz) < kTabMax;
+    const bool small = llabs(vx) < kTabMax && llabs(vy) < kTabMax && llabs(vz) < kTabMax;
     __syncwarp();  // the table is cleared
 #pragma unroll
     for (int t = 0; t < kScanK; ++t) {
@@ -1116,7 +1116,6 @@ __device__ __forceinline__ void knn_lists_body(const float4 *__restrict__ faces,
         }
         if (!added) direct(j);  // a large vector, or a crowded table
     }
-    if (!agg) return;
     __syncwarp();  // every addition is in the table
     for (int i = lane; i < kTabSlots; i += 32) {
         const int j = s_key[i];
@@ -1131,10 +1130,9 @@ __device__ __forceinline__ void knn_lists_body(const float4 *__restrict__ faces,
 __global__ void __launch_bounds__(32 * kScanWarps, 6)
     k_knn_lists(const float4 *__restrict__ faces, IterState *st, int64_t max_faces, KnnTree T,
                 const int64_t *__restrict__ cell_off, const int *__restrict__ cell_idx,
-                double scale, unsigned long long *acc, int *far_q, int agg)
+                double scale, unsigned long long *acc, int *far_q)
 {
-    knn_lists_body(faces, st, max_faces, T, cell_off, cell_idx, scale, acc, far_q, agg != 0,
-                   blockIdx.x);
+    knn_lists_body(faces, st, max_faces, T, cell_off, cell_idx, scale, acc, far_q, blockIdx.x);
 }
 
 // The queued faces (in cells far from the points, over kCellCap candidates),
@@ -2649,14 +2647,13 @@ cudaError_t launch_knn_scatter(Ctx *c)
     const bool lists = cell_lists_ready(c);
     const int64_t *off = lists ? c->d_cell_off : nullptr;
     const int *idx = lists ? c->d_cell_idx : nullptr;
-    // the per-warp sum tables (dynamic shared memory) on clouds up to
-    // kAggMaxPoints; batched clouds always take them
+    // k_knn_scatter's per-warp sum tables (dynamic shared memory) on clouds up
+    // to kAggMaxPoints; batched clouds always take them
     const int agg = c->n <= kAggMaxPoints ? 1 : 0;
     const size_t smem = agg ? kAggSmem : 0;
     if (lists && c->knn == kScanK) {
-        k_knn_lists<<<blocks, 32 * kScanWarps, agg ? kTabSmem : 0, c->stream>>>(
-            c->d_faces, c->d_state, c->max_faces, T, off, idx, c->acc_scale, c->d_acc, c->d_far_q,
-            agg);
+        k_knn_lists<<<blocks, 32 * kScanWarps, kTabSmem, c->stream>>>(
+            c->d_faces, c->d_state, c->max_faces, T, off, idx, c->acc_scale, c->d_acc, c->d_far_q);
         if (c->far_cap > 0) {
             k_knn_far<<<far_blocks(c->far_cap, kFarBlocks), 32 * kFarWarps, 0, c->stream>>>(
                 c->d_faces, c->d_state, T, c->d_far_q, c->acc_scale, c->d_acc, c->d_defer,
@@ -3012,7 +3009,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, 6)
     const int ci = seg_cloud(off, ncl);
     const CloudIter &c = cl[ci];
     knn_lists_body(c.faces, c.st, c.max_faces, c.T, c.cell_off, c.cell_idx, c.acc_scale, c.acc,
-                   c.far_q, true, (int64_t)blockIdx.x - off[ci]);
+                   c.far_q, (int64_t)blockIdx.x - off[ci]);
 }
 
 __global__ void __launch_bounds__(32 * kFarWarps)
