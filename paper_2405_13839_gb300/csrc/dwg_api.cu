@@ -85,7 +85,12 @@ cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
         *p = best->p;
         return cudaSuccess;
     }
-    const cudaError_t e = cudaMalloc(p, b);
+    cudaError_t e = cudaMalloc(p, b);
+    if (e == cudaErrorMemoryAllocation && !S.blocks.empty()) {
+        cudaGetLastError();  // what the handle keeps may be what is missing
+        scratch_trim(c, 0);
+        e = cudaMalloc(p, b);
+    }
     if (e == cudaSuccess) S.blocks.push_back({*p, b, S.depth});
     return e;
 }
@@ -177,16 +182,28 @@ static bool kernel_ptr(const void *p, size_t size)
 {
     return reinterpret_cast<uintptr_t>(p) % size == 0 && is_device_ptr(p);
 }
-// Before a call's kernels touch a caller's device arrays in place, the work
-// already queued on the device is waited for, on every stream: callers fill
-// and reuse such arrays on streams of their own (a framework's default
-// stream), which the handle's stream is not ordered after.  About a
-// microsecond on an idle device.
+// Before a call's kernels touch a caller's device arrays in place, the handle's
+// stream waits for the work already queued on the default stream (and so on
+// every stream ordered with it): callers fill and reuse such arrays there, and
+// the handle's stream is not ordered after it.  Not by waiting for the whole
+// device: another thread may be capturing a graph, this library's own loop
+// among them, and a device-wide wait breaks that capture.
 static cudaError_t join_caller(Ctx *c)
 {
     if (c->scratch.joined) return cudaSuccess;
     c->scratch.joined = true;
-    return cudaDeviceSynchronize();
+    if (!c->ev_caller) {
+        const cudaError_t e = cudaEventCreateWithFlags(&c->ev_caller, cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+    }
+    const cudaError_t e = cudaEventRecord(c->ev_caller, cudaStreamLegacy);
+    if (e == cudaErrorStreamCaptureImplicit || e == cudaErrorStreamCaptureUnsupported) {
+        // a stream ordered with the default stream is being captured: nothing
+        // may be queued there, and what was queued before is the caller's care
+        cudaGetLastError();
+        return cudaSuccess;
+    }
+    return e == cudaSuccess ? cudaStreamWaitEvent(c->stream, c->ev_caller) : e;
 }
 // A caller's float array as kernels on the handle's device read it: the array
 // itself when it is there, else a scratch copy.
@@ -664,6 +681,7 @@ void dwg_destroy(dwg_handle h)
     free_lists(h->lists_c);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
+    if (h->ev_caller) cudaEventDestroy(h->ev_caller);
     if (h->own_stream) cudaStreamDestroy(h->own_stream);
     delete h;
 }

@@ -253,7 +253,7 @@ struct ScratchBlock {
 struct Scratch {
     std::vector<ScratchBlock> blocks;
     int depth = 0;
-    bool joined = false;  // this call has waited for the device (join_caller)
+    bool joined = false;  // this call waits for the default stream (join_caller)
 };
 constexpr size_t kScratchKeep = (size_t)256 << 20;
 
@@ -265,6 +265,7 @@ struct Ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     cudaStream_t own_stream = nullptr;
+    cudaEvent_t ev_caller = nullptr;  // join_caller
     std::string err;
 
     int64_t n = 0;        // points
