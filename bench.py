@@ -53,13 +53,16 @@ import synth  # noqa: E402
 #   w only, plain 12 | w and grad, plain 20 | w only, screened 16 | w and grad, screened 27
 # (screened: F / rho^3 = e inv^2 (inv + s)); each interaction also takes one
 # MUFU rsqrt and, screened, one MUFU ex2
-FP32_OPS = {("w", 0): 12, ("wg", 0): 20, ("w", 1): 16, ("wg", 1): 27}
+# The exact path's leaf corners lie on a lattice: eight corners share the terms'
+# x and y parts, 66 / 8 and 98 / 8 operations an interaction.
+FP32_OPS = {("w", 0): 12, ("wg", 0): 20, ("w", 1): 16, ("wg", 1): 27,
+            ("lattice", 0): 8.25, ("lattice", 1): 12.25}
 FP32_LANES_PER_SM = 128
 
 
 def alu_peaks(what, kind, sm_count, fmax_hz, ffma=None, rsq=None, ex2=None):
-    """Interactions per second of an evaluator.  what: "w" or "wg"; kind: 0
-    plain, 1 screened.  derived: SMs x 128 FP32 lanes x clock / FP32
+    """Interactions per second of an evaluator.  what: "w", "wg" or "lattice" (w
+    at the leaf corners on the exact path); kind: 0 plain, 1 screened.  derived: SMs x 128 FP32 lanes x clock / FP32
     operations per interaction.  With the microbenchmarks' rates (packed-FMA
     lane operations, MUFU rsqrt and ex2 per second): the FMA-pipe bound, the
     MUFU bound (one rsqrt, and for the screened kernel one ex2, per
@@ -126,21 +129,6 @@ def workload(args):
     if args.depth:
         W["depth"] = args.depth
     return W
-
-
-def profiled_traffic(kernel_file, shape):
-    """DRAM bytes per launch recorded in a committed ncu summary of the same
-    kernel shape (or None when the summary is of another shape)."""
-    got, traffic = None, None
-    try:
-        for line in open(os.path.join(ROOT, "profiles", kernel_file)):
-            if line.startswith("shape:"):
-                got = line.split(":", 1)[1].strip()
-            if line.startswith("dram_bytes_per_launch:"):
-                traffic = int(line.split(":")[1])
-    except OSError:
-        return None
-    return traffic if got == shape else None
 
 
 def profiled_bytes_per_interaction(which):
@@ -537,16 +525,13 @@ def run_ours(args, rank, world, local):
         dom = "eval_corners" if kms.get("eval_corners", 0) >= kms["eval_points"] else "eval_points"
         if dom == "eval_corners":
             work = float(nc) * n
-            what = "w"
+            what = "lattice"
         else:
             work = float(n) * n
             what = "wg"
         achieved = work / (kms[dom] / 1e3)
-        shape = f"corners_pairs={tuning['corners_pairs']},corners_threads={tuning['corners_threads']}"
-        traffic_basis = "ncu dram bytes per launch (profiles/eval_corners_torus100k.md)"
-        traffic = profiled_traffic("eval_corners_torus100k.md", shape) if (
-            dom == "eval_corners" and kind == 0 and W["name"] == "torus-100k" and
-            W["depth"] == 8) else None
+        traffic_basis = "not captured for this cloud (profiles/gwn_lattice_torus100k.md: 34 MB)"
+        traffic = None
     else:
         # Barnes-Hut: the dominant of the two tree launches (w and grad at the
         # points, w at the corners), its evaluations performed (counted on the

@@ -138,7 +138,8 @@ int dwg_set_convergence(dwg_handle h, int rule);
 /*
  * The kNN scatter of Eq. 7 (not a parameter of the paper; results do not
  * depend on it).  A face whose cell has no candidate list searches the
- * points' bucket tree in its own thread; a face that is about as far from
+ * points' bucket tree (k = 10: by a warp of its own; another k, or no lists:
+ * in its own thread); a face that is about as far from
  * many points as from its nearest (a level set far from the cloud, as near
  * the centre of a sphere) can make that search nearly exhaustive and hold
  * the whole launch.  A search that takes more than `budget` node visits and
@@ -496,8 +497,10 @@ int dwg_mlp_adam(float *params, const float *grad, float *m, float *v, int step,
  *   path:            DWG_PATH_ALLPAIRS or DWG_PATH_TREE (AUTO resolved);
  *   points_pairs, points_threads:   shape of the exact evaluator of w and
  *                    grad w at the points (query pairs per thread, CTA size);
- *   corners_pairs, corners_threads: shape of the exact evaluator of w at the
- *                    octree-leaf corners;
+ *   corners_pairs, corners_threads: shape of the exact evaluator of w alone:
+ *                    at query points, and with the modified kernel's sources
+ *                    at the octree-leaf corners (the softened kernels take
+ *                    the corners as lattice tasks, which have one shape);
  *   tree_leaf:       points per Barnes-Hut leaf (16, 32, 64 or 128);
  *   theta:           opening angle of the Barnes-Hut path (as dwg_set_tree);
  *   tree_group:      0: the opening test per query (Sec. 5.2 as printed);
