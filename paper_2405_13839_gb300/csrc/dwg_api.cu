@@ -677,6 +677,7 @@ void dwg_destroy(dwg_handle h)
                     h->d_defer, h->d_tree_dmax};
     for (void *p : bufs) cudaFree(p);
     for (ScratchBlock &k : h->scratch.blocks) cudaFree(k.p);
+    free_lattice(h);
     free_lists(h->lists_p);
     free_lists(h->lists_c);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
