@@ -136,6 +136,20 @@ int dwg_set_params(dwg_handle h, int kernel, float eps, float screening, int max
 int dwg_set_convergence(dwg_handle h, int rule);
 
 /*
+ * Device scratch of the handle's calls (not a parameter of the paper).  A
+ * call's temporary buffers stay with the handle for the next call, up to
+ * `keep` bytes of them (-1: the default, 256 MB; 0: none); what is above is
+ * given back at the end of each call and by this call at once.  `limit` >= 0
+ * bounds what a call may hold at a time: past it a call does what it does
+ * when device memory is short: it takes a way that needs less where there is
+ * one (dwg_eval_gwn on the Barnes-Hut path walks the tree instead of making
+ * lists), else it returns DWG_ERR_OOM.  -1: no limit (the default).  On a batch handle both apply to each cloud.
+ * Buffers that belong to the cloud (points, octree, lists of an orientation)
+ * are not scratch.
+ */
+int dwg_set_scratch(dwg_handle h, int64_t limit, int64_t keep);
+
+/*
  * The kNN scatter of Eq. 7 (not a parameter of the paper; results do not
  * depend on it).  A face whose cell has no candidate list searches the
  * points' bucket tree (k = 10: by a warp of its own; another k, or no lists:

@@ -85,11 +85,18 @@ cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
         *p = best->p;
         return cudaSuccess;
     }
-    cudaError_t e = cudaMalloc(p, b);
+    auto take = [&]() {
+        size_t held = 0;
+        for (const ScratchBlock &k : S.blocks) held += k.size;
+        if (b > S.limit || held > S.limit - b) return cudaErrorMemoryAllocation;
+        const cudaError_t e = cudaMalloc(p, b);
+        if (e != cudaSuccess) cudaGetLastError();  // reported here, not by the next launch
+        return e;
+    };
+    cudaError_t e = take();
     if (e == cudaErrorMemoryAllocation && !S.blocks.empty()) {
-        cudaGetLastError();  // what the handle keeps may be what is missing
-        scratch_trim(c, 0);
-        e = cudaMalloc(p, b);
+        scratch_trim(c, 0);  // what the handle keeps may be what is missing
+        e = take();
     }
     if (e == cudaSuccess) S.blocks.push_back({*p, b, S.depth});
     return e;
@@ -119,7 +126,7 @@ ScratchScope::~ScratchScope()
     for (ScratchBlock &k : S.blocks)
         if (k.scope == S.depth) k.scope = 0;
     --S.depth;
-    scratch_trim(c, kScratchKeep);
+    scratch_trim(c, S.keep);
 }
 }  // namespace dwg
 
@@ -416,7 +423,7 @@ static int ensure_iter_buffers(Ctx *c)
 {
     const uint64_t gen = c->bufgen;
     const int rc = iter_buffers(c);
-    if (c->bufgen != gen) scratch_trim(c, kScratchKeepBuilt);
+    if (c->bufgen != gen) scratch_trim(c, std::min(kScratchKeepBuilt, c->scratch.keep));
     return rc;
 }
 
@@ -879,6 +886,18 @@ int dwg_set_batch_mode(dwg_handle h, int lanes)
         h->batch_phases = lanes;
         invalidate_graph(h);
     }
+    return DWG_OK;
+}
+
+int dwg_set_scratch(dwg_handle h, int64_t limit, int64_t keep)
+{
+    if (!h) return DWG_ERR_INVALID;
+    if (limit < -1 || keep < -1) return fail(h, DWG_ERR_INVALID, "limit and keep must be >= -1");
+    cudaSetDevice(h->device);
+    h->scratch.limit = limit < 0 ? SIZE_MAX : (size_t)limit;
+    h->scratch.keep = keep < 0 ? kScratchKeep : (size_t)keep;
+    scratch_trim(h, std::min(h->scratch.keep, h->scratch.limit));
+    for (dwg_ctx *c : h->clouds) dwg_set_scratch(c, limit, keep);
     return DWG_OK;
 }
 

@@ -244,7 +244,10 @@ struct TreeLists {
 // the handle keeps when the call ends, so that a call repeated at its size
 // allocates nothing (cudaMalloc and cudaFree of a call's buffers cost tens to
 // hundreds of microseconds, and cudaFree waits for the device); together at
-// most kScratchKeep bytes between calls, all given back with the handle.
+// most `keep` bytes between calls, all given back with the handle.  A call
+// that would hold more than `limit` is told what cudaMalloc says when memory
+// is short (dwg_set_scratch).
+constexpr size_t kScratchKeep = (size_t)256 << 20;
 struct ScratchBlock {
     void *p;
     size_t size;
@@ -253,9 +256,9 @@ struct ScratchBlock {
 struct Scratch {
     std::vector<ScratchBlock> blocks;
     int depth = 0;
+    size_t keep = kScratchKeep, limit = SIZE_MAX;
     bool joined = false;  // this call waits for the default stream (join_caller)
 };
-constexpr size_t kScratchKeep = (size_t)256 << 20;
 
 // ---------------------------------------------------------------------------
 // engine context

@@ -1461,26 +1461,50 @@ __global__ void __launch_bounds__(1024)
 // (110,592 queries are 1,728 warps, 11 an SM, at 43 % of the FMA pipe);
 // here the lists are cut into items of at most kItemRecords records and
 // evaluated by k_tree_eval_lists.  300,000 sources, w and grad w at 110,592
-// lattice queries: 1,392 -> 630 us (walks 144, evaluation 473).  In ranges
-// of groups; a range whose
-// lists would take more than kCallLists bytes (queries in no order open the
-// whole tree) is walked.
-constexpr double kCallLists = 1024.0 * 1024.0 * 1024.0;
+// lattice queries: 1,392 -> 630 us (walks 144, evaluation 473).  In ranges of
+// groups.  The lists, items and partial sums of a range are one block of
+// scratch; a range for which there is no such block, or whose lists would
+// take more than kCallLists bytes (queries in no order open the whole tree),
+// is walked: in parts of 192 MB, 1M sources at 1.5M unordered queries took
+// 2,150 ms against 1,455 (a part has too few groups for the list walks).
+constexpr size_t kCallLists = (size_t)1 << 30;
+
+// the block of a range's lists and its work items of item_bytes each
+struct CallLists {
+    size_t near_at, items_at, part_at, bytes;
+    CallLists(int64_t nfar, int64_t nnear, int64_t items, size_t item_bytes)
+    {
+        auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+        near_at = up(nfar * sizeof(int));
+        items_at = near_at + up(nnear * sizeof(int));
+        part_at = items_at + up(items * sizeof(int2));
+        bytes = part_at + items * item_bytes;
+    }
+};
 
 template <bool GRAD, bool SCREENED>
 static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, int64_t stride)
 {
     const EvalParams ep = make_eval_params(c);
     const int64_t all = ceil_div(m, kGrpQ);
+    constexpr size_t item_bytes = (GRAD ? 8 : 2) * kGrpQ * sizeof(float);
+    ScratchScope scope(c);
+    int64_t *buf = nullptr;
+    const int64_t most = std::min<int64_t>(kListRange, all);
+    cudaError_t e = scratch_get(c, &buf, (5 * most + 7) * sizeof(int64_t));
+    if (e == cudaErrorMemoryAllocation) {
+        DWG_CUDA_TRY(c, launch_tree_gwn(c, q, m, GRAD, part, stride, nullptr));
+        return DWG_OK;
+    }
+    DWG_CUDA_TRY(c, e);
+    char *block = nullptr;
+    size_t held = 0;  // bytes of block
     for (int64_t g0 = 0; g0 < all; g0 += kListRange) {
-        ScratchScope scope(c);
         const int ng = (int)std::min<int64_t>(kListRange, all - g0);
         const float4 *qr = q + g0 * kGrpQ;
         const int64_t mr = std::min<int64_t>(m - g0 * kGrpQ, (int64_t)ng * kGrpQ);
         float *pr = part + g0 * kGrpQ;
         const unsigned blocks = (unsigned)ceil_div(ng, list_warps(kWalkW));
-        int64_t *buf = nullptr;
-        DWG_CUDA_TRY(c, scratch_get(c, &buf, (5 * (int64_t)ng + 7) * sizeof(int64_t)));
         int64_t *cnt_f = buf, *cnt_n = cnt_f + ng, *far_off = cnt_n + ng, *near_off = far_off + ng + 1,
                 *item_off = near_off + ng + 1, *tot = item_off + ng + 1;
         k_tree_lists<false, kWalkW><<<blocks, 32 * list_warps(kWalkW), 0, c->stream>>>(
@@ -1491,20 +1515,26 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
         int64_t ht[4];
         DWG_CUDA_TRY(c, cudaMemcpyAsync(ht, tot, sizeof ht, cudaMemcpyDeviceToHost, c->stream));
         DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-        const size_t item_bytes = (GRAD ? 8 : 2) * kGrpQ * sizeof(float);
-        const double need = 4.0 * ((double)ht[0] + (double)ht[1]) +
-                            (double)ht[2] * (sizeof(int2) + item_bytes);
-        if (need > kCallLists) {
+        const CallLists L(ht[0], ht[1], ht[2], item_bytes);
+        bool room = L.bytes <= held;
+        if (!room && L.bytes <= kCallLists) {
+            char *larger = nullptr;
+            e = scratch_get(c, &larger, L.bytes);
+            if (e != cudaErrorMemoryAllocation) {
+                DWG_CUDA_TRY(c, e);
+                block = larger;
+                held = L.bytes;
+                room = true;
+            }
+        }
+        if (!room) {
             DWG_CUDA_TRY(c, launch_tree_gwn(c, qr, mr, GRAD, pr, stride, nullptr));
             continue;
         }
-        int *far_ids = nullptr, *near_ids = nullptr;
-        int2 *items = nullptr;
-        float *ipart = nullptr;
-        DWG_CUDA_TRY(c, scratch_get(c, &far_ids, ht[0] * sizeof(int)));
-        DWG_CUDA_TRY(c, scratch_get(c, &near_ids, ht[1] * sizeof(int)));
-        DWG_CUDA_TRY(c, scratch_get(c, &items, ht[2] * sizeof(int2)));
-        DWG_CUDA_TRY(c, scratch_get(c, &ipart, ht[2] * item_bytes));
+        int *far_ids = reinterpret_cast<int *>(block);
+        int *near_ids = reinterpret_cast<int *>(block + L.near_at);
+        int2 *items = reinterpret_cast<int2 *>(block + L.items_at);
+        float *ipart = reinterpret_cast<float *>(block + L.part_at);
         k_tree_lists<true, kWalkW><<<blocks, 32 * list_warps(kWalkW), 0, c->stream>>>(
             qr, mr, c->d_tree_rec, c->tree_levels, far_off, near_off, far_ids, near_ids, c->d_err);
         const int irec = (int)ht[3];

@@ -107,6 +107,7 @@ def _load() -> ctypes.CDLL:
         "dwg_set_compensation": ([H, I], I),
         "dwg_set_batch_mode": ([H, I], I),
         "dwg_set_knn_budget": ([H, I], I),
+        "dwg_set_scratch": ([H, I64, I64], I),
         "dwg_set_weights": ([H, P], I),
         "dwg_voronoi_weights": ([H, I, P], I),
         "dwg_selfcheck_wait": ([H, I], I),
@@ -259,6 +260,12 @@ def dwg_set_knn_budget(h, budget):
     """Node visits and distances after which a face's kNN search is handed
     to a block (default 16384); -1: never.  The results do not change."""
     return _raise(h, _lib.dwg_set_knn_budget(h, int(budget)))
+
+
+def dwg_set_scratch(h, limit=-1, keep=-1):
+    """Bytes of device scratch that a call may hold (-1: no limit) and that the
+    handle keeps between calls (-1: the default, 256 MB)."""
+    return _raise(h, _lib.dwg_set_scratch(h, int(limit), int(keep)))
 
 
 def dwg_set_compensation(h, on):
