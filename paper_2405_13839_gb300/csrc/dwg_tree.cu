@@ -830,9 +830,9 @@ __global__ void __launch_bounds__(32 * list_warps(W))
             if (FILL && is_near) near_ids[nn + __popc(nm & lt)] = leaf;
             nn += __popc(nm);
         });
-    if (!ok) {
+    if (!ok) {  // no list: the callers do not use the counts of such a launch
         if (lane == 0) atomicOr(err, kErrStack);
-        return;
+        nf = nn = 0;
     }
     if (!FILL && lane == 0) {
         far_n[g] = nf;
@@ -1389,14 +1389,14 @@ cudaError_t launch_tree_moments(Ctx *c)
 
 // The offsets of up to kListRange groups' lists and work items from their
 // counts, by one block (a scan of three arrays at once); totals: far nodes,
-// near leaves, items.  The items' size follows item_records' rule.
+// near leaves, items, records of an item (item_records' rule), error flags.
 constexpr int kListRange = 16384;
 
 __global__ void __launch_bounds__(1024)
     k_tree_list_offsets(const int64_t *__restrict__ cnt_f, const int64_t *__restrict__ cnt_n,
                         int ng, int bucket, int64_t *__restrict__ far_off,
                         int64_t *__restrict__ near_off, int64_t *__restrict__ item_off,
-                        int64_t *__restrict__ totals)
+                        int64_t *__restrict__ totals, const int *__restrict__ err)
 {
     __shared__ int64_t sh[3][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1453,6 +1453,7 @@ __global__ void __launch_bounds__(1024)
         near_off[ng] = totals[1] = run[1];
         item_off[ng] = totals[2] = run[2];
         totals[3] = irec;
+        totals[4] = *err;
     }
 }
 
@@ -1491,7 +1492,7 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
     ScratchScope scope(c);
     int64_t *buf = nullptr;
     const int64_t most = std::min<int64_t>(kListRange, all);
-    cudaError_t e = scratch_get(c, &buf, (5 * most + 7) * sizeof(int64_t));
+    cudaError_t e = scratch_get(c, &buf, (5 * most + 8) * sizeof(int64_t));
     if (e == cudaErrorMemoryAllocation) {
         DWG_CUDA_TRY(c, launch_tree_gwn(c, q, m, GRAD, part, stride, nullptr));
         return DWG_OK;
@@ -1510,11 +1511,15 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
         k_tree_lists<false, kWalkW><<<blocks, 32 * list_warps(kWalkW), 0, c->stream>>>(
             qr, mr, c->d_tree_rec, c->tree_levels, cnt_f, cnt_n, nullptr, nullptr, c->d_err);
         k_tree_list_offsets<<<1, 1024, 0, c->stream>>>(cnt_f, cnt_n, ng, c->tree_leaf, far_off,
-                                                       near_off, item_off, tot);
+                                                       near_off, item_off, tot, c->d_err);
         DWG_CUDA_TRY(c, cudaGetLastError());
-        int64_t ht[4];
+        int64_t ht[5];
         DWG_CUDA_TRY(c, cudaMemcpyAsync(ht, tot, sizeof ht, cudaMemcpyDeviceToHost, c->stream));
         DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+        if (ht[4]) {  // a walk gave up: its counts are not those of the fill
+            c->err = "tree lists: traversal stack overflow";
+            return DWG_ERR_CUDA;
+        }
         const CallLists L(ht[0], ht[1], ht[2], item_bytes);
         bool room = L.bytes <= held;
         if (!room && L.bytes <= kCallLists) {
