@@ -1468,6 +1468,8 @@ __global__ void __launch_bounds__(1024)
 // take more than kCallLists bytes (queries in no order open the whole tree),
 // is walked: in parts of 192 MB, 1M sources at 1.5M unordered queries took
 // 2,150 ms against 1,455 (a part has too few groups for the list walks).
+// Ranges one after the other are walked in one launch: the two of those
+// queries by themselves 1,495 ms, each with its own last groups to wait for.
 constexpr size_t kCallLists = (size_t)1 << 30;
 
 // the block of a range's lists and its work items of item_bytes each
@@ -1499,7 +1501,15 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
     }
     DWG_CUDA_TRY(c, e);
     char *block = nullptr;
-    size_t held = 0;  // bytes of block
+    size_t held = 0;       // bytes of block
+    int64_t walk_g = all;  // groups from here to the current range are still to be walked
+    auto walk_to = [&](int64_t g1) {
+        const int64_t g = walk_g;
+        walk_g = all;
+        if (g >= g1) return cudaSuccess;
+        return launch_tree_gwn(c, q + g * kGrpQ, std::min<int64_t>(m, g1 * kGrpQ) - g * kGrpQ, GRAD,
+                               part + g * kGrpQ, stride, nullptr);
+    };
     for (int64_t g0 = 0; g0 < all; g0 += kListRange) {
         const int ng = (int)std::min<int64_t>(kListRange, all - g0);
         const float4 *qr = q + g0 * kGrpQ;
@@ -1533,9 +1543,10 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
             }
         }
         if (!room) {
-            DWG_CUDA_TRY(c, launch_tree_gwn(c, qr, mr, GRAD, pr, stride, nullptr));
+            walk_g = std::min(walk_g, g0);
             continue;
         }
+        DWG_CUDA_TRY(c, walk_to(g0));
         int *far_ids = reinterpret_cast<int *>(block);
         int *near_ids = reinterpret_cast<int *>(block + L.near_at);
         int2 *items = reinterpret_cast<int2 *>(block + L.items_at);
@@ -1552,6 +1563,7 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
             ipart, item_off, mr, pr, stride, nullptr);
         DWG_CUDA_TRY(c, cudaGetLastError());
     }
+    DWG_CUDA_TRY(c, walk_to(all));
     return DWG_OK;
 }
 

@@ -101,3 +101,18 @@ def test_more_queries_than_one_range(dwglib, torch, limit):
             _same([w[a:b], g[a:b]], _eval(dwglib, torch, h, q[a:b].contiguous()))
     finally:
         dwglib.dwg_destroy(h)
+
+
+@pytest.mark.parametrize("m", [RANGE + 130, 2 * RANGE + 130])
+def test_more_lists_than_a_call_makes(dwglib, torch, m):
+    """300,000 sources, queries in no order: every group opens most leaves, over
+    18,000 entries a group, 300M in a full range -- more than 1 GB, so one or
+    two ranges are walked; the last range's lists fit."""
+    h = _handle(dwglib, 300_000, 25.0)
+    try:
+        q = _queries(torch, m)
+        w, g = _eval(dwglib, torch, h, q)
+        for a, b in ((0, 640), (RANGE - 640, RANGE), (RANGE, RANGE + 128), (m - 130, m)):
+            _same([w[a:b], g[a:b]], _eval(dwglib, torch, h, q[a:b].contiguous()))
+    finally:
+        dwglib.dwg_destroy(h)
