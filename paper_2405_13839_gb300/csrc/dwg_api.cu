@@ -194,22 +194,26 @@ static bool kernel_ptr(const void *p, size_t size)
 // every stream ordered with it): callers fill and reuse such arrays there, and
 // the handle's stream is not ordered after it.  Not by waiting for the whole
 // device: another thread may be capturing a graph, this library's own loop
-// among them, and a device-wide wait breaks that capture.
+// among them, and a device-wide wait breaks that capture.  Nor may anything be
+// queued on the default stream while a stream ordered with it (one made
+// without cudaStreamNonBlocking) is being captured; a stream of that kind that
+// is not itself captured still runs behind what the default stream holds.
 static cudaError_t join_caller(Ctx *c)
 {
     if (c->scratch.joined) return cudaSuccess;
     c->scratch.joined = true;
-    if (!c->ev_caller) {
-        const cudaError_t e = cudaEventCreateWithFlags(&c->ev_caller, cudaEventDisableTiming);
-        if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (!c->ev_caller &&
+        (e = cudaEventCreateWithFlags(&c->ev_caller, cudaEventDisableTiming)) != cudaSuccess)
+        return e;
+    cudaStream_t on = cudaStreamLegacy;
+    cudaStreamCaptureStatus st;
+    if (cudaStreamIsCapturing(cudaStreamLegacy, &st) != cudaSuccess) {
+        cudaGetLastError();  // cudaErrorStreamCaptureImplicit: such a capture is under way
+        if (!c->join_stream && (e = cudaStreamCreate(&c->join_stream)) != cudaSuccess) return e;
+        on = c->join_stream;
     }
-    const cudaError_t e = cudaEventRecord(c->ev_caller, cudaStreamLegacy);
-    if (e == cudaErrorStreamCaptureImplicit || e == cudaErrorStreamCaptureUnsupported) {
-        // a stream ordered with the default stream is being captured: nothing
-        // may be queued there, and what was queued before is the caller's care
-        cudaGetLastError();
-        return cudaSuccess;
-    }
+    e = cudaEventRecord(c->ev_caller, on);
     return e == cudaSuccess ? cudaStreamWaitEvent(c->stream, c->ev_caller) : e;
 }
 // A caller's float array as kernels on the handle's device read it: the array
@@ -690,6 +694,7 @@ void dwg_destroy(dwg_handle h)
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->ev_caller) cudaEventDestroy(h->ev_caller);
+    if (h->join_stream) cudaStreamDestroy(h->join_stream);
     if (h->own_stream) cudaStreamDestroy(h->own_stream);
     delete h;
 }

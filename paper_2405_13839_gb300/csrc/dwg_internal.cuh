@@ -269,6 +269,7 @@ struct Ctx {
     cudaStream_t stream = nullptr;
     cudaStream_t own_stream = nullptr;
     cudaEvent_t ev_caller = nullptr;  // join_caller
+    cudaStream_t join_stream = nullptr;
     std::string err;
 
     int64_t n = 0;        // points
