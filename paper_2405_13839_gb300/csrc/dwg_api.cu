@@ -136,6 +136,13 @@ static int fail(Ctx *c, int code, const std::string &msg)
     return code;
 }
 
+// a launcher's failure: its own scratch may be what is missing
+static int fail_launch(Ctx *c, cudaError_t e, const char *what)
+{
+    return fail(c, e == cudaErrorMemoryAllocation ? DWG_ERR_OOM : DWG_ERR_CUDA,
+                std::string(what) + ": " + cudaGetErrorString(e));
+}
+
 // Memory that the library's kernels may read or write directly: device
 // memory of the current device, or managed memory.  A pointer into another
 // GPU's memory is not (without peer access a kernel could not touch it); such
@@ -600,8 +607,9 @@ static int prepare_normals(Ctx *c)
             if (launch_random_normals(c->d_nrm, c->d_perm, c->n, c->seed, c->stream) !=
                 cudaSuccess)
                 return fail(c, DWG_ERR_CUDA, "random normals launch failed");
-            if (c->init_mode == DWG_INIT_PCA && launch_init_pca(c) != cudaSuccess)
-                return fail(c, DWG_ERR_CUDA, "PCA normals launch failed");
+            cudaError_t e = cudaSuccess;
+            if (c->init_mode == DWG_INIT_PCA && (e = launch_init_pca(c)) != cudaSuccess)
+                return fail_launch(c, e, "PCA normals");
             if (c->init_mode == DWG_INIT_GAUSS && launch_init_gauss(c) != cudaSuccess)
                 return fail(c, DWG_ERR_CUDA, "Gauss-map normals launch failed");
             if (c->init_mode == DWG_INIT_LEARNED) {
@@ -611,11 +619,11 @@ static int prepare_normals(Ctx *c)
                 DWG_CUDA_TRY(c, scratch_get(c, &X, c->n * 64 * sizeof(float)));
                 DWG_CUDA_TRY(c, scratch_get(c, &Y, c->n * 3 * sizeof(float)));
                 DWG_CUDA_TRY(c, scratch_get(c, &cR, kSumDoubles * sizeof(double)));
-                if (launch_features(c, X, false, cR) != cudaSuccess ||
-                    launch_mlp_forward(c->d_mlp_params, X, c->n, Y, c->stream, c->d_err) !=
+                if ((e = launch_features(c, X, false, cR)) != cudaSuccess ||
+                    (e = launch_mlp_forward(c->d_mlp_params, X, c->n, Y, c->stream, c->d_err)) !=
                         cudaSuccess ||
-                    launch_normals_from_y(c, Y) != cudaSuccess)
-                    return fail(c, DWG_ERR_CUDA, "learned init launch failed");
+                    (e = launch_normals_from_y(c, Y)) != cudaSuccess)
+                    return fail_launch(c, e, "learned normals");
                 DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
             }
         } else {
@@ -994,8 +1002,8 @@ int dwg_set_regularization(dwg_handle h, int mode, int k, float vmin, float vmax
     float *d_out = nullptr;
     auto run = [&]() -> int {
         if (delta_out) DWG_CUDA_TRY(h, scratch_get(h, &d_out, h->n * sizeof(float)));
-        if (launch_clamp_delta(h, k, (double)vmin, (double)vmax, d_out) != cudaSuccess)
-            return fail(h, DWG_ERR_CUDA, "clamp radii launch failed");
+        const cudaError_t e = launch_clamp_delta(h, k, (double)vmin, (double)vmax, d_out);
+        if (e != cudaSuccess) return fail_launch(h, e, "clamp radii");
         int r = check_device_err(h);
         if (r) return r;
         if (delta_out) return download(h, delta_out, d_out, h->n * sizeof(float));
@@ -1126,8 +1134,8 @@ int dwg_voronoi_weights(dwg_handle h, int m, float *a_out)
     auto run = [&]() -> int {
         DWG_CUDA_TRY(h, scratch_get(h, &scratch, (h->n + kSumDoubles) * sizeof(double)));
         if (a_out) DWG_CUDA_TRY(h, scratch_get(h, &d_out, h->n * sizeof(float)));
-        if (launch_voronoi_weights(h, m, scratch, d_out) != cudaSuccess)
-            return fail(h, DWG_ERR_CUDA, "Voronoi weights launch failed");
+        const cudaError_t e = launch_voronoi_weights(h, m, scratch, d_out);
+        if (e != cudaSuccess) return fail_launch(h, e, "Voronoi weights");
         int r = check_device_err(h);
         if (r) return r;
         h->tree_built = false;  // node centres depend on the weights
@@ -1607,8 +1615,8 @@ int dwg_mlp_features(dwg_handle h, float *X_out)
     int rc = caller_out(h, X_out, count, &X);
     if (rc) return rc;
     DWG_CUDA_TRY(h, scratch_get(h, &cR, kSumDoubles * sizeof(double)));
-    if (launch_features(h, X, true, cR) != cudaSuccess)
-        return fail(h, DWG_ERR_CUDA, "features launch failed");
+    const cudaError_t e = launch_features(h, X, true, cR);
+    if (e != cudaSuccess) return fail_launch(h, e, "features");
     if ((rc = caller_done(h, X_out, X, count))) return rc;
     DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     return check_device_err(h);

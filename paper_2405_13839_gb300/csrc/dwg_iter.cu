@@ -908,18 +908,24 @@ __global__ void __launch_bounds__(32 * kShWarps)
 constexpr int kShFarBlocks = 152 * 8;
 
 // A table of the K nearest points, filled for one range of points at a time
-// (at most kKnnRange, so that the table stays small beside a large cloud):
-// `use(i0, cnt, stride, table)` launches the kernel that reads it.
+// (at most kKnnRange, so that the table stays small beside a large cloud;
+// fewer where memory is short): `use(i0, cnt, stride, table)` launches the
+// kernel that reads it.
 constexpr int64_t kKnnRange = (int64_t)3 << 20;
+constexpr int64_t kKnnRangeMin = 4096;
 
 template <int K, class UseFn>
 static cudaError_t points_nearest(Ctx *c, UseFn &&use)
 {
     const KnnTree T = knn_tree(c);
-    const int64_t stride = std::min<int64_t>(c->n, kKnnRange);
+    int64_t stride = std::min<int64_t>(c->n, kKnnRange);
     ScratchScope scope(c);
     int *buf = nullptr;  // K * stride table, queue, its length
-    cudaError_t e = scratch_get(c, &buf, ((K + 1) * stride + 1) * sizeof(int));
+    cudaError_t e;
+    while ((e = scratch_get(c, &buf, ((K + 1) * stride + 1) * sizeof(int))) ==
+               cudaErrorMemoryAllocation &&
+           stride > kKnnRangeMin)
+        stride = std::max(kKnnRangeMin, ceil_div(stride, 2));
     if (e != cudaSuccess) return e;
     int *queue = buf + K * stride, *nq = queue + stride;
     for (int64_t i0 = 0; i0 < c->n && e == cudaSuccess; i0 += stride) {
