@@ -148,7 +148,8 @@ int dwg_set_convergence(dwg_handle h, int rule);
  * bounds what a call may hold at a time: past it a call does what it does
  * when device memory is short: it takes a way that needs less where there is
  * one (dwg_eval_gwn on the Barnes-Hut path walks the tree instead of making
- * lists), else it returns DWG_ERR_OOM.  -1: no limit (the default).  On a batch handle both apply to each cloud.
+ * lists, the points' neighbours are searched in smaller ranges, the corners
+ * of the exact path are not rearranged), else it returns DWG_ERR_OOM.  -1: no limit (the default).  On a batch handle both apply to each cloud.
  * Buffers that belong to the cloud (points, octree, lists of an orientation)
  * are not scratch.
  */

@@ -24,6 +24,7 @@ struct dwg_ctx : public Ctx {
     GwnCloud *d_bcl_p = nullptr, *d_bcl_c = nullptr;
     GwnItem *d_bit_p = nullptr, *d_bit_c = nullptr;
     int64_t nit_p = 0, nit_c = 0;
+    std::vector<dwg_ctx *> general_c;  // exact clouds whose corners are not lattice tasks
     IterState **d_states = nullptr;
     bool eps_given = false;
     // fork / join of the clouds' chains in a batch iteration (each cloud runs
@@ -354,14 +355,22 @@ static unsigned nblk(int64_t n, int b = 256) { return (unsigned)ceil_div(n, b); 
 // ---------------------------------------------------------------------------
 // buffers
 // ---------------------------------------------------------------------------
+// the lattice tasks of the softened, compensated kernel; where they find no
+// memory the general evaluator takes the corners
+static int ensure_lattice(Ctx *c)
+{
+    if (c->reg_mode != DWG_REG_SOFTEN || !c->compensated) return DWG_OK;
+    const int rc = build_lattice(c);
+    return rc == DWG_ERR_OOM ? DWG_OK : rc;
+}
+
 // octree of the handle's depth, its corners and their partial sums
 static int ensure_levelset_buffers(Ctx *c, bool tree)
 {
     if (c->built_depth != c->depth) ++c->bufgen;
     int rc = build_discretization(c, c->depth);
     if (rc) return rc;
-    if (!tree && c->reg_mode == DWG_REG_SOFTEN && c->compensated && (rc = build_lattice(c)))
-        return rc;
+    if (!tree && (rc = ensure_lattice(c))) return rc;
     const int nch_c = tree ? 1 : corners_chunks(c);
     if (nch_c != c->nchunks_c) ++c->bufgen;
     c->nchunks_c = nch_c;
@@ -1863,6 +1872,7 @@ static int batch_tables(dwg_ctx *h)
 {
     std::vector<GwnCloud> cp, cc;
     std::vector<GwnItem> ip, ic;
+    h->general_c.clear();
     for (dwg_ctx *c : h->clouds) {
         if (use_tree(c)) continue;
         EvalParams ep = make_eval_params(c);
@@ -1870,6 +1880,10 @@ static int batch_tables(dwg_ctx *h)
         for (int pass = 0; pass < 2; ++pass) {
             bool grad = pass == 0;
             if (!grad && c->mode != DWG_UPDATE_LEVELSET) continue;
+            if (!grad && !corners_on_lattice(c)) {
+                h->general_c.push_back(c);
+                continue;
+            }
             int64_t m = grad ? c->n : corners_slots(c);
             int nch = grad ? c->nchunks_p : c->nchunks_c;
             GwnCloud g;
@@ -1975,15 +1989,28 @@ static cudaError_t batch_lane_phases(dwg_ctx *h, const dwg_ctx::Lane &L, bool sc
     return e;
 }
 
+// the all-pairs sums of every cloud
+static int batch_gwn(dwg_ctx *h, bool scr)
+{
+    if (launch_gwn_batch(h->d_bcl_p, h->d_bit_p, h->nit_p, true, scr, h->d_err, h->stream) !=
+            cudaSuccess ||
+        launch_gwn_batch(h->d_bcl_c, h->d_bit_c, h->nit_c, false, scr, h->d_err, h->stream) !=
+            cudaSuccess)
+        return fail(h, DWG_ERR_CUDA, "batched gwn launch failed");
+    for (dwg_ctx *c : h->general_c) {
+        c->stream = h->stream;
+        const int rc = eval_corners(c, c->nchunks_c, c->d_part_c);
+        if (rc) return fail(h, rc, "cloud: " + c->err);
+    }
+    return DWG_OK;
+}
+
 static int batch_body_phases(dwg_ctx *h)
 {
     const bool scr = h->kernel == DWG_KERNEL_SCREENED && h->lambda > 0.f;
     cudaStream_t s = h->stream;
-    if (launch_gwn_batch(h->d_bcl_p, h->d_bit_p, h->nit_p, true, scr, h->d_err, s) !=
-            cudaSuccess ||
-        launch_gwn_batch(h->d_bcl_c, h->d_bit_c, h->nit_c, false, scr, h->d_err, s) !=
-            cudaSuccess)
-        return fail(h, DWG_ERR_CUDA, "batched gwn launch failed");
+    const int rc = batch_gwn(h, scr);
+    if (rc) return rc;
     if (h->lanes.size() == 1) {
         cudaError_t e = batch_lane_phases(h, h->lanes[0], scr, s);
         if (e != cudaSuccess)
@@ -2018,11 +2045,8 @@ static int batch_body_phases(dwg_ctx *h)
 static int batch_body_branches(dwg_ctx *h, cudaGraphConditionalHandle cond)
 {
     bool scr = h->kernel == DWG_KERNEL_SCREENED && h->lambda > 0.f;
-    if (launch_gwn_batch(h->d_bcl_p, h->d_bit_p, h->nit_p, true, scr, h->d_err, h->stream) !=
-            cudaSuccess ||
-        launch_gwn_batch(h->d_bcl_c, h->d_bit_c, h->nit_c, false, scr, h->d_err, h->stream) !=
-            cudaSuccess)
-        return fail(h, DWG_ERR_CUDA, "batched gwn launch failed");
+    const int rc = batch_gwn(h, scr);
+    if (rc) return rc;
     if (!h->ev_fork)
         DWG_CUDA_TRY(h, cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     DWG_CUDA_TRY(h, cudaEventRecord(h->ev_fork, h->stream));

@@ -713,7 +713,6 @@ void free_lattice(Ctx *c)
 int build_lattice(Ctx *c)
 {
     if (c->lat_tasks > 0 || c->ncorners < 1) return DWG_OK;
-    ++c->bufgen;  // a captured graph holds other buffers
     const int64_t m = c->ncorners;
     const int bits = c->built_depth + 1;
     const int64_t nx = ((int64_t)1 << c->built_depth) + 1;
@@ -755,6 +754,7 @@ int build_lattice(Ctx *c)
                                            c->d_lat_z, c->d_lat_corner);
         DWG_CUDA_TRY(c, cudaGetLastError());
         c->lat_tasks = nt;
+        ++c->bufgen;  // a captured graph holds other buffers
         return DWG_OK;
     };
     if ((rc = fill())) free_lattice(c);
