@@ -255,6 +255,29 @@ static int caller_done(Ctx *c, float *p, const float *d, size_t count)
     return p == d ? DWG_OK : download(c, p, d, count * sizeof(float));
 }
 
+// A call that reads or writes callers' arrays in place.  Unless it comes to its
+// end (ended), what it has queued may still use them, and an error flag of its
+// inputs may still be set for the next call to find.
+struct CallEnd {
+    Ctx *c;
+    bool ended = false;
+    explicit CallEnd(Ctx *c_) : c(c_) {}
+    ~CallEnd()
+    {
+        if (ended) return;
+        cudaStreamSynchronize(c->stream);
+        cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
+    }
+    CallEnd(const CallEnd &) = delete;
+    CallEnd &operator=(const CallEnd &) = delete;
+    // the call's last result
+    int operator()(int rc)
+    {
+        ended = rc >= 0;
+        return rc;
+    }
+};
+
 // ---------------------------------------------------------------------------
 // small kernels used only by the engine
 // ---------------------------------------------------------------------------
@@ -1338,6 +1361,7 @@ int dwg_step(dwg_handle h, float *w_out, float *grad_out, float *dtheta_out, dou
     if (stat_out) *stat_out = st.stat;
     if (!w_out && !grad_out && !dtheta_out) return DWG_OK;
     ScratchScope scope(h);
+    CallEnd end(h);
     const size_t n = (size_t)h->n;
     float *w = nullptr, *g = nullptr, *d = nullptr;
     if (w_out && (rc = caller_out(h, w_out, n, &w))) return rc;
@@ -1351,7 +1375,7 @@ int dwg_step(dwg_handle h, float *w_out, float *grad_out, float *dtheta_out, dou
     if (!rc && dtheta_out) rc = caller_done(h, dtheta_out, d, n);
     const cudaError_t e = cudaStreamSynchronize(h->stream);
     if (!rc && e != cudaSuccess) rc = fail(h, DWG_ERR_CUDA, cudaGetErrorString(e));
-    return rc;
+    return end(rc);
 }
 
 int dwg_profile_step(dwg_handle h, float *ms_out, int cap, int *count)
@@ -1404,6 +1428,7 @@ int dwg_eval_gwn(dwg_handle h, const float *queries, int64_t m, float *w_out, fl
     const bool grad = grad_out != nullptr;
     const bool tree = use_tree(h);
     ScratchScope scope(h);
+    CallEnd end(h);
     const float *qx = nullptr;
     float *part = nullptr, *w = nullptr, *g = nullptr;
     float4 *q4 = nullptr;
@@ -1438,11 +1463,11 @@ int dwg_eval_gwn(dwg_handle h, const float *queries, int64_t m, float *w_out, fl
         h->stats.interactions_eval = (double)cnt;
     }
     if ((rc = check_device_err(h))) return rc;
-    if (w == w_out && g == grad_out) return DWG_OK;
+    if (w == w_out && g == grad_out) return end(DWG_OK);
     if ((rc = caller_done(h, w_out, w, m))) return rc;
     if (grad && (rc = caller_done(h, grad_out, g, 3 * m))) return rc;
     DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    return DWG_OK;
+    return end(DWG_OK);
 }
 
 int dwg_autotune(dwg_handle h, int what, double w_budget, const char *cache_path,
@@ -1618,6 +1643,7 @@ int dwg_mlp_features(dwg_handle h, float *X_out)
     if (h->is_batch) return fail(h, DWG_ERR_STATE, "not on a batch handle");
     cudaSetDevice(h->device);
     ScratchScope scope(h);
+    CallEnd end(h);
     const size_t count = (size_t)h->n * 64;
     float *X = nullptr;
     double *cR = nullptr;
@@ -1628,7 +1654,7 @@ int dwg_mlp_features(dwg_handle h, float *X_out)
     if (e != cudaSuccess) return fail_launch(h, e, "features");
     if ((rc = caller_done(h, X_out, X, count))) return rc;
     DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    return check_device_err(h);
+    return end(check_device_err(h));
 }
 
 static int mlp_check(std::initializer_list<const void *> ptrs, int64_t B)
@@ -1710,6 +1736,7 @@ int dwg_knn(dwg_handle h, const float *queries, int64_t m, int k, int64_t *idx_o
     if (m < 1 || k < 1 || k > kMaxK) return fail(h, DWG_ERR_INVALID, "need m >= 1, 1 <= k <= 32");
     cudaSetDevice(h->device);
     ScratchScope scope(h);
+    CallEnd end(h);
     const float *qx = nullptr;
     float4 *q4 = nullptr;
     int64_t *idx = idx_out;
@@ -1724,7 +1751,7 @@ int dwg_knn(dwg_handle h, const float *queries, int64_t m, int k, int64_t *idx_o
         return fail(h, DWG_ERR_CUDA, "knn launch failed");
     if (idx != idx_out && (rc = download(h, idx_out, idx, m * k * sizeof(int64_t)))) return rc;
     DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    return check_device_err(h);
+    return end(check_device_err(h));
 }
 
 // ---------------------------------------------------------------------------

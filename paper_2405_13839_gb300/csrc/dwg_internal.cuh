@@ -397,6 +397,7 @@ struct Ctx {
     do {                                                                          \
         cudaError_t e_ = (call);                                                  \
         if (e_ != cudaSuccess) {                                                  \
+            cudaGetLastError(); /* reported here, not by the next launch check */ \
             (ctx)->err = std::string(#call) + ": " + cudaGetErrorString(e_);      \
             return (e_ == cudaErrorMemoryAllocation) ? DWG_ERR_OOM : DWG_ERR_CUDA; \
         }                                                                         \
