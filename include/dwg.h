@@ -149,7 +149,9 @@ int dwg_set_convergence(dwg_handle h, int rule);
  * when device memory is short: it takes a way that needs less where there is
  * one (dwg_eval_gwn on the Barnes-Hut path walks the tree instead of making
  * lists, the points' neighbours are searched in smaller ranges, the corners
- * of the exact path are not rearranged), else it returns DWG_ERR_OOM.  -1: no limit (the default).  On a batch handle both apply to each cloud.
+ * of the exact path are not rearranged), else it returns DWG_ERR_OOM.  -1: no
+ * limit (the default).  On a batch handle `limit` applies to each cloud and
+ * `keep` to all of them together.
  * Buffers that belong to the cloud (points, octree, lists of an orientation)
  * are not scratch.
  */

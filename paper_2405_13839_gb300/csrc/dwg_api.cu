@@ -103,11 +103,12 @@ cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
     return e;
 }
 
-// frees free blocks, the largest first, until at most `keep` bytes are held
-// (cudaFree waits for the device)
+// frees free blocks, the largest first, until at most the handle's share of
+// `keep` bytes is held (cudaFree waits for the device)
 void scratch_trim(Ctx *c, size_t keep)
 {
     Scratch &S = c->scratch;
+    keep /= S.share;
     size_t total = 0;
     for (const ScratchBlock &k : S.blocks) total += k.size;
     while (total > keep) {
@@ -458,9 +459,6 @@ static int iter_buffers(Ctx *c)
     }
     return DWG_OK;
 }
-
-// what a build took and the iterations do not need
-constexpr size_t kScratchKeepBuilt = (size_t)16 << 20;
 
 static int ensure_iter_buffers(Ctx *c)
 {
@@ -816,7 +814,7 @@ static int create_impl(dwg_ctx *c, const float *points, int64_t n)
         k_iter_reset<<<1, 1, 0, c->stream>>>(c->d_state, c->max_iters, nullptr);
         DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream));
         DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-        scratch_trim(c, kScratchKeepBuilt);
+        scratch_trim(c, std::min(kScratchKeepBuilt, c->scratch.keep));
         c->stats.n_points = n;
         return DWG_OK;
     };
@@ -2228,6 +2226,7 @@ int dwg_create_batch(const float *points, const int64_t *offsets, int n_clouds, 
             dwg_ctx *s = new (std::nothrow) dwg_ctx();
             if (!s) return DWG_ERR_OOM;
             h->clouds.push_back(s);
+            s->scratch.share = n_clouds;
             int rc = create_impl(s, dpts + 3 * off[c], off[c + 1] - off[c]);
             if (rc) return fail(h, rc, "cloud " + std::to_string(c) + ": " + s->err);
             s->depth = auto_depth(s->n);

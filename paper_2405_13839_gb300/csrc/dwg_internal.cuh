@@ -248,6 +248,8 @@ struct TreeLists {
 // that would hold more than `limit` is told what cudaMalloc says when memory
 // is short (dwg_set_scratch).
 constexpr size_t kScratchKeep = (size_t)256 << 20;
+// what of it stays after a build, whose sizes the calls that follow do not need
+constexpr size_t kScratchKeepBuilt = (size_t)16 << 20;
 struct ScratchBlock {
     void *p;
     size_t size;
@@ -257,6 +259,7 @@ struct Scratch {
     std::vector<ScratchBlock> blocks;
     int depth = 0;
     size_t keep = kScratchKeep, limit = SIZE_MAX;
+    int share = 1;        // handles that keep as much together (the clouds of a batch)
     bool joined = false;  // this call waits for the default stream (join_caller)
 };
 
@@ -517,7 +520,7 @@ inline cudaError_t scratch_get(Ctx *c, T **p, size_t bytes)
 {
     return scratch_get(c, reinterpret_cast<void **>(p), bytes);
 }
-void scratch_trim(Ctx *c, size_t keep);
+void scratch_trim(Ctx *c, size_t keep);  // to this handle's share of keep
 struct ScratchScope {
     Ctx *c;
     explicit ScratchScope(Ctx *c_) : c(c_)
