@@ -379,15 +379,6 @@ static unsigned nblk(int64_t n, int b = 256) { return (unsigned)ceil_div(n, b); 
 // ---------------------------------------------------------------------------
 // buffers
 // ---------------------------------------------------------------------------
-// the lattice tasks of the softened, compensated kernel; where they find no
-// memory the general evaluator takes the corners
-static int ensure_lattice(Ctx *c)
-{
-    if (c->reg_mode != DWG_REG_SOFTEN || !c->compensated) return DWG_OK;
-    const int rc = build_lattice(c);
-    return rc == DWG_ERR_OOM ? DWG_OK : rc;
-}
-
 // octree of the handle's depth, its corners and their partial sums
 static int ensure_levelset_buffers(Ctx *c, bool tree)
 {

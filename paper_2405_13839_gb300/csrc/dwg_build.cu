@@ -710,7 +710,7 @@ void free_lattice(Ctx *c)
     c->lat_tasks = 0;
 }
 
-int build_lattice(Ctx *c)
+static int build_lattice(Ctx *c)
 {
     if (c->lat_tasks > 0 || c->ncorners < 1) return DWG_OK;
     const int64_t m = c->ncorners;
@@ -759,6 +759,15 @@ int build_lattice(Ctx *c)
     };
     if ((rc = fill())) free_lattice(c);
     return rc;
+}
+
+// the tasks of the softened, compensated kernel; where they find no memory the
+// general evaluator takes the corners
+int ensure_lattice(Ctx *c)
+{
+    if (c->reg_mode != DWG_REG_SOFTEN || !c->compensated) return DWG_OK;
+    const int rc = build_lattice(c);
+    return rc == DWG_ERR_OOM ? DWG_OK : rc;
 }
 
 }  // namespace dwg

@@ -464,7 +464,7 @@ cudaError_t launch_gather_points(const float *xyz, const float *a, const int64_t
                                  int64_t n, float4 *p4, cudaStream_t s);
 int build_knn_tree(Ctx *c);
 int build_discretization(Ctx *c, int depth);
-int build_lattice(Ctx *c);
+int ensure_lattice(Ctx *c);
 void free_lattice(Ctx *c);
 
 // dwg_eval.cu

@@ -385,7 +385,10 @@ int autotune(Ctx *c, int what, double budget, const char *cache_path, dwg_tuning
         if ((rc = tune_shape(c, c->d_p4, c->n, true, &vg, &ap_ms_p))) return rc;
         if (lset && (rc = tune_shape(c, c->d_corner_pos, c->ncorners, false, &vw, &ap_ms_c)))
             return rc;
-        if (lset && corners_on_lattice(c)) {  // what an iteration runs at the corners
+        // what an iteration of the exact path runs at the corners (on a handle
+        // whose path resolves to the tree so far the tasks are not made yet)
+        if (lset && (rc = ensure_lattice(c))) return rc;
+        if (lset && corners_on_lattice(c)) {
             const int nch = corners_chunks(c);
             Buf part;
             TUNE_TRY(cudaMalloc(&part.p, (size_t)nch * 2 * corners_slots(c) * sizeof(float)));
