@@ -910,13 +910,21 @@ constexpr int kShFarBlocks = 152 * 8;
 // A table of the K nearest points, filled for one range of points at a time
 // (at most kKnnRange, so that the table stays small beside a large cloud;
 // fewer where memory is short): `use(i0, cnt, stride, table)` launches the
-// kernel that reads it.
+// kernel that reads it.  A cloud of at most kKnnDirect points gets none: there
+// the launches that fill a table are the time, and the kernel that would read
+// it searches by itself (features of 10 points: 67 us by a table, 47 by itself;
+// of 100 points 74 by a table, 99).
 constexpr int64_t kKnnRange = (int64_t)3 << 20;
 constexpr int64_t kKnnRangeMin = 4096;
+constexpr int64_t kKnnDirect = 48;
 
 template <int K, class UseFn>
 static cudaError_t points_nearest(Ctx *c, UseFn &&use)
 {
+    if (c->n <= kKnnDirect) {
+        use(0, (int)c->n, 0, (const int *)nullptr);
+        return cudaGetLastError();
+    }
     const KnnTree T = knn_tree(c);
     int64_t stride = std::min<int64_t>(c->n, kKnnRange);
     ScratchScope scope(c);
@@ -941,6 +949,20 @@ static cudaError_t points_nearest(Ctx *c, UseFn &&use)
         e = cudaGetLastError();
     }
     return e;
+}
+
+// the neighbours of a point, from its column of the table or by a search
+template <int K, bool TABLE>
+__device__ __forceinline__ void point_neighbours(const KnnTree &T, float4 p, int64_t stride,
+                                                 const int *__restrict__ nbr, int r, int (&bj)[K],
+                                                 int *err)
+{
+    if constexpr (TABLE) {
+#pragma unroll
+        for (int t = 0; t < K; ++t) bj[t] = __ldg(&nbr[t * stride + r]);
+    } else {
+        knn_search<K, true>(T, F3{p.x, p.y, p.z}, K, bj, err);
+    }
 }
 
 __device__ __forceinline__ uint64_t point_code(const KnnTree &T, F3 q)
@@ -1485,7 +1507,8 @@ cudaError_t launch_spacing(Ctx *c, int64_t m, float *d_out)
 // centre b (so that mean |p - c|^2 = mean |p - b|^2 - |c - b|^2 loses nothing):
 // per-block sums in a fixed order, then one block over the blocks' sums.  As
 // one block over all points it was a chain of loads: 913 us for 200,000
-// points, 13 us as two launches.
+// points, 13 us as two launches.  Up to kSumOne points one block is enough.
+constexpr int64_t kSumOne = 512;
 constexpr int kSumBlocks = 304;
 
 __device__ __forceinline__ double block_sum(double v, double *sh)
@@ -1501,9 +1524,20 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
     return r;
 }
 
+// mean offset m[0..2] from b and mean squared distance m[3] -> cx, cy, cz, R
+__device__ __forceinline__ void centroid_out(const double (&m)[4], double bx, double by, double bz,
+                                             double *out)
+{
+    out[0] = bx + m[0];
+    out[1] = by + m[1];
+    out[2] = bz + m[2];
+    out[3] = sqrt(fmax(0.0, m[3] - (m[0] * m[0] + m[1] * m[1] + m[2] * m[2])));
+}
+
+// (one block: the result at once)
 __global__ void __launch_bounds__(256)
     k_centroid_part(const float4 *__restrict__ p4, int64_t n, double bx, double by, double bz,
-                    double *__restrict__ part)
+                    double *__restrict__ part, double *__restrict__ out)
 {
     __shared__ double sh[256];
     double s[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1517,14 +1551,16 @@ __global__ void __launch_bounds__(256)
         s[3] += dx * dx + dy * dy + dz * dz;
     }
     for (int k = 0; k < 4; ++k) {
-        const double v = block_sum(s[k], sh);
-        if (threadIdx.x == 0) part[4 * blockIdx.x + k] = v;
+        s[k] = block_sum(s[k], sh);
+        if (threadIdx.x == 0) part[4 * blockIdx.x + k] = s[k];
+        s[k] /= n;
     }
+    if (gridDim.x == 1 && threadIdx.x == 0) centroid_out(s, bx, by, bz, out);
 }
 
 __global__ void __launch_bounds__(256)
     k_centroid(const double *__restrict__ part, int nb, int64_t n, double bx, double by, double bz,
-               double *out /* cx,cy,cz,R */)
+               double *out)
 {
     __shared__ double sh[256];
     double m[4];
@@ -1533,12 +1569,7 @@ __global__ void __launch_bounds__(256)
         for (int b = threadIdx.x; b < nb; b += blockDim.x) v += part[4 * b + k];
         m[k] = block_sum(v, sh) / n;
     }
-    if (threadIdx.x == 0) {
-        out[0] = bx + m[0];
-        out[1] = by + m[1];
-        out[2] = bz + m[2];
-        out[3] = sqrt(fmax(0.0, m[3] - (m[0] * m[0] + m[1] * m[1] + m[2] * m[2])));
-    }
+    if (threadIdx.x == 0) centroid_out(m, bx, by, bz, out);
 }
 
 // Feature row of sorted point i: offsets to its 16 nearest other points (in
@@ -1550,9 +1581,10 @@ __global__ void __launch_bounds__(256)
 constexpr int kFeatWarps = 4;
 constexpr int kFeatRow = 51;
 
+template <bool TABLE>
 __global__ void __launch_bounds__(32 * kFeatWarps)
     k_features(KnnTree T, int64_t i0, int cnt_i, int64_t stride, const int *__restrict__ nbr,
-               const double *__restrict__ cR, float *__restrict__ X, int by_input)
+               const double *__restrict__ cR, float *__restrict__ X, int by_input, int *err)
 {
     __shared__ float rows[kFeatWarps][32][kFeatRow];
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1566,10 +1598,12 @@ __global__ void __launch_bounds__(32 * kFeatWarps)
     if (r < cnt_i) {
         const int64_t i = i0 + r;
         const float4 pi = T.p4[i];
+        int bj[17];
+        point_neighbours<17, TABLE>(T, pi, stride, nbr, r, bj, err);
         float ss = 0.f;
 #pragma unroll
         for (int t = 0; t < 17; ++t) {
-            int j = __ldg(&nbr[t * stride + r]);
+            const int j = bj[t];
             if (j < 0 || j == (int)i || cnt == 16) continue;
             float4 pj = T.p4[j];
             float dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
@@ -1612,14 +1646,16 @@ __global__ void k_normals_from_y(const float *__restrict__ Y, int64_t n, float4 
 
 cudaError_t launch_features(Ctx *c, float *X, bool by_input, double *cR)
 {
-    const int nb = (int)std::min<int64_t>(ceil_div(c->n, 256), kSumBlocks);
+    const int nb = c->n <= kSumOne ? 1 : (int)std::min<int64_t>(ceil_div(c->n, 256), kSumBlocks);
     k_centroid_part<<<nb, 256, 0, c->stream>>>(c->d_p4, c->n, c->bbox_c[0], c->bbox_c[1],
-                                               c->bbox_c[2], cR + 4);
-    k_centroid<<<1, 256, 0, c->stream>>>(cR + 4, nb, c->n, c->bbox_c[0], c->bbox_c[1],
-                                         c->bbox_c[2], cR);
+                                               c->bbox_c[2], cR + 4, cR);
+    if (nb > 1)
+        k_centroid<<<1, 256, 0, c->stream>>>(cR + 4, nb, c->n, c->bbox_c[0], c->bbox_c[1],
+                                             c->bbox_c[2], cR);
     return points_nearest<17>(c, [&](int64_t i0, int cnt, int64_t stride, const int *nbr) {
-        k_features<<<(unsigned)ceil_div(cnt, 32 * kFeatWarps), 32 * kFeatWarps, 0, c->stream>>>(
-            knn_tree(c), i0, cnt, stride, nbr, cR, X, by_input ? 1 : 0);
+        auto k = nbr ? k_features<true> : k_features<false>;
+        k<<<(unsigned)ceil_div(cnt, 32 * kFeatWarps), 32 * kFeatWarps, 0, c->stream>>>(
+            knn_tree(c), i0, cnt, stride, nbr, cR, X, by_input ? 1 : 0, c->d_err);
     });
 }
 
@@ -1687,19 +1723,22 @@ __device__ bool sym3_min_eigvec(double a[3][3], double out[3])
 // from the bounding-box centre c (the Gauss-map side, n . (p_i - c) > 0),
 // and +z, then +y, then +x where that dot product is zero.  Where the
 // covariance is zero the random normal already in nrm stays.
+template <bool TABLE>
 __global__ void __launch_bounds__(128)
     k_init_pca(KnnTree T, int64_t i0, int cnt_i, int64_t stride, const int *__restrict__ nbr,
-               double cx, double cy, double cz, float4 *__restrict__ nrm)
+               double cx, double cy, double cz, float4 *__restrict__ nrm, int *err)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= cnt_i) return;
     const int64_t i = i0 + r;
     const float4 pi = T.p4[i];
+    int bj[kPcaK];
+    point_neighbours<kPcaK, TABLE>(T, pi, stride, nbr, r, bj, err);
     double d[kPcaK][3], mean[3] = {0.0, 0.0, 0.0};
     int cnt = 0;
 #pragma unroll
     for (int t = 0; t < kPcaK; ++t) {
-        const int j = __ldg(&nbr[t * stride + r]);
+        const int j = bj[t];
         if (j < 0) continue;
         const float4 pj = T.p4[j];
         d[cnt][0] = (double)pj.x - (double)pi.x;
@@ -1746,8 +1785,10 @@ __global__ void k_init_gauss(const float4 *__restrict__ p4, int64_t n, double cx
 cudaError_t launch_init_pca(Ctx *c)
 {
     return points_nearest<kPcaK>(c, [&](int64_t i0, int cnt, int64_t stride, const int *nbr) {
-        k_init_pca<<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(
-            knn_tree(c), i0, cnt, stride, nbr, c->bbox_c[0], c->bbox_c[1], c->bbox_c[2], c->d_nrm);
+        auto k = nbr ? k_init_pca<true> : k_init_pca<false>;
+        k<<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(knn_tree(c), i0, cnt, stride, nbr,
+                                                               c->bbox_c[0], c->bbox_c[1],
+                                                               c->bbox_c[2], c->d_nrm, c->d_err);
     });
 }
 
@@ -1847,7 +1888,7 @@ __device__ double vor_disk_area(const double *px, const double *py, int k, doubl
 // plane through it, the projected neighbours as Voronoi seeds, the cell of
 // the origin cut to the disk of half the largest projected distance.  A
 // neighbourhood with no extent gives 0 (the caller substitutes the mean).
-template <int KMAX, bool FIXED>
+template <int KMAX, bool FIXED, bool TABLE>
 __global__ void __launch_bounds__(128)
     k_voronoi_area(KnnTree T, int64_t i0, int cnt_i, int64_t stride, const int *__restrict__ nbr,
                    int m, double *__restrict__ area, int *err)
@@ -1858,12 +1899,10 @@ __global__ void __launch_bounds__(128)
     const int64_t i = i0 + r;
     const float4 pi = T.p4[i];
     int bj[KMAX];
-    if constexpr (FIXED) {
-#pragma unroll
-        for (int t = 0; t < KMAX; ++t) bj[t] = __ldg(&nbr[t * stride + r]);
-    } else {
-        knn_search<KMAX, FIXED>(T, F3{pi.x, pi.y, pi.z}, m + 1, bj, err);
-    }
+    if constexpr (FIXED)
+        point_neighbours<KMAX, TABLE>(T, pi, stride, nbr, r, bj, err);
+    else
+        knn_search<KMAX, false>(T, F3{pi.x, pi.y, pi.z}, m + 1, bj, err);
     double d[KMAX][3];
     double mean[3] = {0.0, 0.0, 0.0};
     int cnt = 0;
@@ -1925,9 +1964,14 @@ __global__ void __launch_bounds__(128)
 }
 
 // mean of the positive areas: per-block sums in a fixed order, then one
-// block over them (1,050 us for 1M points as one block)
+// block over them (1,050 us for 1M points as one block); up to kAreaOne points
+// one block is enough.  No positive area at all (a cloud of one point, or all
+// copies of one): the paper's default weight 1.
+constexpr int64_t kAreaOne = 2048;
+
 __global__ void __launch_bounds__(256)
-    k_area_part(const double *__restrict__ area, int64_t n, double *__restrict__ part)
+    k_area_part(const double *__restrict__ area, int64_t n, double *__restrict__ part,
+                double *__restrict__ out)
 {
     __shared__ double sh[256];
     double s = 0.0, c = 0.0;
@@ -1940,6 +1984,7 @@ __global__ void __launch_bounds__(256)
     if (threadIdx.x == 0) {
         part[2 * blockIdx.x] = ss;
         part[2 * blockIdx.x + 1] = sc;
+        if (gridDim.x == 1) out[0] = sc > 0.0 ? ss / sc : 1.0;
     }
 }
 
@@ -1953,8 +1998,6 @@ __global__ void __launch_bounds__(256)
         c += part[2 * b + 1];
     }
     const double ss = block_sum(s, sh), sc = block_sum(c, sh);
-    // no positive area at all (a cloud of one point, or all copies of one):
-    // the paper's default weight 1
     if (threadIdx.x == 0) out[0] = sc > 0.0 ? ss / sc : 1.0;
 }
 
@@ -1978,16 +2021,18 @@ cudaError_t launch_voronoi_weights(Ctx *c, int m, double *scratch, float *a_out)
     cudaError_t e = cudaSuccess;
     if (m == 15)
         e = points_nearest<16>(c, [&](int64_t i0, int cnt, int64_t stride, const int *nbr) {
-            k_voronoi_area<16, true><<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(
-                knn_tree(c), i0, cnt, stride, nbr, m, scratch, c->d_err);
+            auto k = nbr ? k_voronoi_area<16, true, true> : k_voronoi_area<16, true, false>;
+            k<<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(knn_tree(c), i0, cnt, stride,
+                                                                   nbr, m, scratch, c->d_err);
         });
     else
-        k_voronoi_area<32, false><<<(unsigned)ceil_div(c->n, 128), 128, 0, c->stream>>>(
+        k_voronoi_area<32, false, false><<<(unsigned)ceil_div(c->n, 128), 128, 0, c->stream>>>(
             knn_tree(c), 0, (int)c->n, 0, nullptr, m, scratch, c->d_err);
     if (e != cudaSuccess) return e;
-    const int nb = (int)std::min<int64_t>(ceil_div(c->n, 256), kSumBlocks);
-    k_area_part<<<nb, 256, 0, c->stream>>>(scratch, c->n, scratch + c->n + 1);
-    k_area_mean<<<1, 256, 0, c->stream>>>(scratch + c->n + 1, nb, scratch + c->n);
+    const int nb = c->n <= kAreaOne ? 1 : (int)std::min<int64_t>(ceil_div(c->n, 256), kSumBlocks);
+    double *mean = scratch + c->n;
+    k_area_part<<<nb, 256, 0, c->stream>>>(scratch, c->n, mean + 1, mean);
+    if (nb > 1) k_area_mean<<<1, 256, 0, c->stream>>>(mean + 1, nb, mean);
     k_area_install<<<(unsigned)ceil_div(c->n, 256), 256, 0, c->stream>>>(
         scratch, scratch + c->n, c->d_perm, c->n, c->d_p4, a_out, c->d_err);
     return cudaGetLastError();
@@ -2000,7 +2045,7 @@ cudaError_t launch_voronoi_weights(Ctx *c, int m, double *scratch, float *a_out)
 // points whose distance lies in [vmin, vmax]; if none does, the mean of all
 // k distances clamped to [vmin, vmax].  Stored as delta^2 in float32 (sorted
 // order) and, when asked, delta in input order.
-template <int KMAX, bool FIXED>
+template <int KMAX, bool FIXED, bool TABLE>
 __global__ void __launch_bounds__(128)
     k_clamp_delta(KnnTree T, int64_t i0, int cnt_i, int64_t stride, const int *__restrict__ nbr,
                   int k, double vmin, double vmax, float *__restrict__ delta2,
@@ -2011,12 +2056,10 @@ __global__ void __launch_bounds__(128)
     const int64_t i = i0 + r;
     const float4 pi = T.p4[i];
     int bj[KMAX];
-    if constexpr (FIXED) {
-#pragma unroll
-        for (int t = 0; t < KMAX; ++t) bj[t] = __ldg(&nbr[t * stride + r]);
-    } else {
-        knn_search<KMAX, FIXED>(T, F3{pi.x, pi.y, pi.z}, k + 1, bj, err);
-    }
+    if constexpr (FIXED)
+        point_neighbours<KMAX, TABLE>(T, pi, stride, nbr, r, bj, err);
+    else
+        knn_search<KMAX, false>(T, F3{pi.x, pi.y, pi.z}, k + 1, bj, err);
     double sum_in = 0.0, sum_all = 0.0;
     int n_in = 0, cnt = 0;
 #pragma unroll
@@ -2045,10 +2088,11 @@ cudaError_t launch_clamp_delta(Ctx *c, int k, double vmin, double vmax, float *d
 {
     if (k == 10)
         return points_nearest<11>(c, [&](int64_t i0, int cnt, int64_t stride, const int *nbr) {
-            k_clamp_delta<11, true><<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(
+            auto kern = nbr ? k_clamp_delta<11, true, true> : k_clamp_delta<11, true, false>;
+            kern<<<(unsigned)ceil_div(cnt, 128), 128, 0, c->stream>>>(
                 knn_tree(c), i0, cnt, stride, nbr, k, vmin, vmax, c->d_delta2, delta_out, c->d_err);
         });
-    k_clamp_delta<32, false><<<(unsigned)ceil_div(c->n, 128), 128, 0, c->stream>>>(
+    k_clamp_delta<32, false, false><<<(unsigned)ceil_div(c->n, 128), 128, 0, c->stream>>>(
         knn_tree(c), 0, (int)c->n, 0, nullptr, k, vmin, vmax, c->d_delta2, delta_out, c->d_err);
     return cudaGetLastError();
 }
