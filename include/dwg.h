@@ -458,7 +458,9 @@ int dwg_get_corners(dwg_handle h, int64_t *keys_out, int64_t cap, int64_t *count
  *   cloud on that path are one kernel launch.  normals_out (total x 3, host
  *   or device, may be NULL) in the input layout; iters_out (host, n_clouds,
  *   may be NULL).  Returns DWG_NOT_CONVERGED if any cloud reached the cap.
- * dwg_orient and dwg_step return DWG_ERR_STATE on a batch handle.
+ * Calls on one cloud (dwg_orient, dwg_step, dwg_set_weights, dwg_set_normals,
+ * dwg_get_normals, dwg_eval_gwn, dwg_knn, dwg_get_leaves and the like) return
+ * DWG_ERR_STATE on a batch handle.
  */
 int dwg_create_batch(const float *points, const int64_t *offsets, int n_clouds,
                      dwg_handle *out);

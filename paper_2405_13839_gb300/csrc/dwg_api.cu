@@ -138,6 +138,14 @@ static int fail(Ctx *c, int code, const std::string &msg)
     return code;
 }
 
+// A batch handle has no points, normals or octree of its own: calls on one
+// cloud would launch on null arrays.
+static bool batch_refused(dwg_ctx *h)
+{
+    if (h->is_batch) fail(h, DWG_ERR_STATE, "a call on one cloud, not on a batch handle");
+    return h->is_batch;
+}
+
 // a launcher's failure: its own scratch may be what is missing
 static int fail_launch(Ctx *c, cudaError_t e, const char *what)
 {
@@ -978,6 +986,7 @@ int dwg_set_tree(dwg_handle h, int path, float theta)
 int dwg_set_weights(dwg_handle h, const float *a)
 {
     if (!h || !a) return DWG_ERR_INVALID;
+    if (batch_refused(h)) return DWG_ERR_STATE;
     cudaSetDevice(h->device);
     ScratchScope scope(h);
     const float *d = nullptr;
@@ -1226,6 +1235,7 @@ int dwg_set_init(dwg_handle h, int mode, uint64_t seed, const float *normals)
 int dwg_set_normals(dwg_handle h, const float *normals)
 {
     if (!h || !normals) return DWG_ERR_INVALID;
+    if (batch_refused(h)) return DWG_ERR_STATE;
     cudaSetDevice(h->device);
     int rc = normals_from_caller(h, normals, h->d_nrm);
     if (rc) return rc;
@@ -1236,6 +1246,7 @@ int dwg_set_normals(dwg_handle h, const float *normals)
 int dwg_get_normals(dwg_handle h, float *normals_out)
 {
     if (!h || !normals_out) return DWG_ERR_INVALID;
+    if (batch_refused(h)) return DWG_ERR_STATE;
     cudaSetDevice(h->device);
     if (h->normals_pending) {
         int rc = prepare_normals(h);
@@ -1370,6 +1381,7 @@ int dwg_step(dwg_handle h, float *w_out, float *grad_out, float *dtheta_out, dou
 int dwg_profile_step(dwg_handle h, float *ms_out, int cap, int *count)
 {
     if (!h) return DWG_ERR_INVALID;
+    if (batch_refused(h)) return DWG_ERR_STATE;
     cudaSetDevice(h->device);
     int rc = ensure_iter_buffers(h);
     if (rc) return rc;
@@ -1410,6 +1422,7 @@ int dwg_profile_step(dwg_handle h, float *ms_out, int cap, int *count)
 int dwg_eval_gwn(dwg_handle h, const float *queries, int64_t m, float *w_out, float *grad_out)
 {
     if (!h || !queries || !w_out) return DWG_ERR_INVALID;
+    if (batch_refused(h)) return DWG_ERR_STATE;
     if (m < 1) return fail(h, DWG_ERR_INVALID, "m must be >= 1");
     cudaSetDevice(h->device);
     int rc;
@@ -1543,6 +1556,7 @@ int dwg_get_trace(dwg_handle h, double *iso, double *stat, double *mean_dn, int6
 int dwg_get_leaves(dwg_handle h, int64_t *leaves_out, int64_t cap, int64_t *count)
 {
     if (!h || !count) return DWG_ERR_INVALID;
+    if (batch_refused(h)) return DWG_ERR_STATE;
     cudaSetDevice(h->device);
     int rc = build_discretization(h, h->depth);
     if (rc) return rc;
@@ -1580,6 +1594,7 @@ int dwg_get_leaves(dwg_handle h, int64_t *leaves_out, int64_t cap, int64_t *coun
 int dwg_get_corners(dwg_handle h, int64_t *keys_out, int64_t cap, int64_t *count)
 {
     if (!h || !count) return DWG_ERR_INVALID;
+    if (batch_refused(h)) return DWG_ERR_STATE;
     cudaSetDevice(h->device);
     int rc = build_discretization(h, h->depth);
     if (rc) return rc;
@@ -1722,6 +1737,7 @@ int dwg_mlp_adam(float *params, const float *grad, float *m, float *v, int step,
 int dwg_knn(dwg_handle h, const float *queries, int64_t m, int k, int64_t *idx_out)
 {
     if (!h || !queries || !idx_out) return DWG_ERR_INVALID;
+    if (batch_refused(h)) return DWG_ERR_STATE;
     if (m < 1 || k < 1 || k > kMaxK) return fail(h, DWG_ERR_INVALID, "need m >= 1, 1 <= k <= 32");
     cudaSetDevice(h->device);
     ScratchScope scope(h);
