@@ -75,12 +75,12 @@ cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
     Scratch &S = c->scratch;
     const size_t b = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
     *p = nullptr;
-    // the smallest free block that holds it, none far too large
+    // the smallest free block that holds it, none far too large (under a limit
+    // none larger at all: what a call can do would depend on the calls before)
+    const size_t most = S.limit == SIZE_MAX ? 4 * b + ((size_t)1 << 20) : b;
     ScratchBlock *best = nullptr;
     for (ScratchBlock &k : S.blocks)
-        if (!k.scope && k.size >= b && k.size <= 4 * b + ((size_t)1 << 20) &&
-            (!best || k.size < best->size))
-            best = &k;
+        if (!k.scope && k.size >= b && k.size <= most && (!best || k.size < best->size)) best = &k;
     if (best) {
         best->scope = S.depth;
         *p = best->p;
