@@ -150,8 +150,7 @@ int dwg_set_convergence(dwg_handle h, int rule);
  * one (dwg_eval_gwn on the Barnes-Hut path walks the tree instead of making
  * lists, the points' neighbours are searched in smaller ranges, the corners
  * of the exact path are not rearranged), else it returns DWG_ERR_OOM.  -1: no
- * limit (the default).  On a batch handle `limit` applies to each cloud and
- * `keep` to all of them together.
+ * limit (the default).  The clouds of a batch handle share its scratch.
  * Buffers that belong to the cloud (points, octree, lists of an orientation)
  * are not scratch.
  */

@@ -72,7 +72,7 @@ bool use_tree(const Ctx *c)
 namespace dwg {
 cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
 {
-    Scratch &S = c->scratch;
+    Scratch &S = *c->scratch;
     const size_t b = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
     *p = nullptr;
     // the smallest free block that holds it, none far too large (under a limit
@@ -103,12 +103,11 @@ cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
     return e;
 }
 
-// frees free blocks, the largest first, until at most the handle's share of
-// `keep` bytes is held (cudaFree waits for the device)
+// frees free blocks, the largest first, until at most `keep` bytes are held
+// (cudaFree waits for the device)
 void scratch_trim(Ctx *c, size_t keep)
 {
-    Scratch &S = c->scratch;
-    keep /= S.share;
+    Scratch &S = *c->scratch;
     size_t total = 0;
     for (const ScratchBlock &k : S.blocks) total += k.size;
     while (total > keep) {
@@ -124,7 +123,7 @@ void scratch_trim(Ctx *c, size_t keep)
 
 ScratchScope::~ScratchScope()
 {
-    Scratch &S = c->scratch;
+    Scratch &S = *c->scratch;
     for (ScratchBlock &k : S.blocks)
         if (k.scope == S.depth) k.scope = 0;
     --S.depth;
@@ -217,8 +216,8 @@ static bool kernel_ptr(const void *p, size_t size)
 // is not itself captured still runs behind what the default stream holds.
 static cudaError_t join_caller(Ctx *c)
 {
-    if (c->scratch.joined) return cudaSuccess;
-    c->scratch.joined = true;
+    if (c->joined) return cudaSuccess;
+    c->joined = true;
     cudaError_t e = cudaSuccess;
     if (!c->ev_caller &&
         (e = cudaEventCreateWithFlags(&c->ev_caller, cudaEventDisableTiming)) != cudaSuccess)
@@ -463,7 +462,7 @@ static int ensure_iter_buffers(Ctx *c)
 {
     const uint64_t gen = c->bufgen;
     const int rc = iter_buffers(c);
-    if (c->bufgen != gen) scratch_trim(c, std::min(kScratchKeepBuilt, c->scratch.keep));
+    if (c->bufgen != gen) scratch_trim(c, std::min(kScratchKeepBuilt, c->scratch->keep));
     return rc;
 }
 
@@ -724,7 +723,7 @@ void dwg_destroy(dwg_handle h)
                     h->d_delta2, h->d_src16, h->d_cell_off, h->d_cell_idx, h->d_far_q,
                     h->d_defer, h->d_tree_dmax};
     for (void *p : bufs) cudaFree(p);
-    for (ScratchBlock &k : h->scratch.blocks) cudaFree(k.p);
+    for (ScratchBlock &k : h->own_scratch.blocks) cudaFree(k.p);
     free_lattice(h);
     free_lists(h->lists_p);
     free_lists(h->lists_c);
@@ -813,7 +812,7 @@ static int create_impl(dwg_ctx *c, const float *points, int64_t n)
         k_iter_reset<<<1, 1, 0, c->stream>>>(c->d_state, c->max_iters, nullptr);
         DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream));
         DWG_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-        scratch_trim(c, std::min(kScratchKeepBuilt, c->scratch.keep));
+        scratch_trim(c, std::min(kScratchKeepBuilt, c->scratch->keep));
         c->stats.n_points = n;
         return DWG_OK;
     };
@@ -936,10 +935,9 @@ int dwg_set_scratch(dwg_handle h, int64_t limit, int64_t keep)
     if (!h) return DWG_ERR_INVALID;
     if (limit < -1 || keep < -1) return fail(h, DWG_ERR_INVALID, "limit and keep must be >= -1");
     cudaSetDevice(h->device);
-    h->scratch.limit = limit < 0 ? SIZE_MAX : (size_t)limit;
-    h->scratch.keep = keep < 0 ? kScratchKeep : (size_t)keep;
-    scratch_trim(h, std::min(h->scratch.keep, h->scratch.limit));
-    for (dwg_ctx *c : h->clouds) dwg_set_scratch(c, limit, keep);
+    h->scratch->limit = limit < 0 ? SIZE_MAX : (size_t)limit;
+    h->scratch->keep = keep < 0 ? kScratchKeep : (size_t)keep;
+    scratch_trim(h, std::min(h->scratch->keep, h->scratch->limit));
     return DWG_OK;
 }
 
@@ -1159,6 +1157,7 @@ int dwg_voronoi_weights(dwg_handle h, int m, float *a_out)
     }
     int rc;
     ScratchScope scope(h);
+    CallEnd end(h);
     double *scratch = nullptr;
     float *d_out = nullptr;
     auto run = [&]() -> int {
@@ -1177,7 +1176,7 @@ int dwg_voronoi_weights(dwg_handle h, int m, float *a_out)
         cudaError_t e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) rc = fail(h, DWG_ERR_CUDA, cudaGetErrorString(e));
     }
-    return rc;
+    return end(rc);
 }
 
 static int normals_from_caller(dwg_handle h, const float *normals, float4 *dst)
@@ -2233,7 +2232,7 @@ int dwg_create_batch(const float *points, const int64_t *offsets, int n_clouds, 
             dwg_ctx *s = new (std::nothrow) dwg_ctx();
             if (!s) return DWG_ERR_OOM;
             h->clouds.push_back(s);
-            s->scratch.share = n_clouds;
+            s->scratch = &h->own_scratch;
             int rc = create_impl(s, dpts + 3 * off[c], off[c + 1] - off[c]);
             if (rc) return fail(h, rc, "cloud " + std::to_string(c) + ": " + s->err);
             s->depth = auto_depth(s->n);

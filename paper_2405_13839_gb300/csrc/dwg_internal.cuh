@@ -259,15 +259,17 @@ struct Scratch {
     std::vector<ScratchBlock> blocks;
     int depth = 0;
     size_t keep = kScratchKeep, limit = SIZE_MAX;
-    int share = 1;        // handles that keep as much together (the clouds of a batch)
-    bool joined = false;  // this call waits for the default stream (join_caller)
 };
 
 // ---------------------------------------------------------------------------
 // engine context
 // ---------------------------------------------------------------------------
 struct Ctx {
-    Scratch scratch;
+    // the clouds of a batch take their scratch from the batch's: their calls
+    // follow one another, each at its end when the next begins
+    Scratch own_scratch;
+    Scratch *scratch = &own_scratch;
+    bool joined = false;  // this call waits for the default stream (join_caller)
     int device = 0;
     cudaStream_t stream = nullptr;
     cudaStream_t own_stream = nullptr;
@@ -520,12 +522,12 @@ inline cudaError_t scratch_get(Ctx *c, T **p, size_t bytes)
 {
     return scratch_get(c, reinterpret_cast<void **>(p), bytes);
 }
-void scratch_trim(Ctx *c, size_t keep);  // to this handle's share of keep
+void scratch_trim(Ctx *c, size_t keep);
 struct ScratchScope {
     Ctx *c;
     explicit ScratchScope(Ctx *c_) : c(c_)
     {
-        if (++c->scratch.depth == 1) c->scratch.joined = false;
+        if (++c->scratch->depth == 1) c->joined = false;
     }
     ~ScratchScope();
     ScratchScope(const ScratchScope &) = delete;
