@@ -268,9 +268,9 @@ int radix_sort_pairs(Ctx *c, uint64_t *keys, int64_t *vals, int64_t n, int key_b
     // frees were 40-60 us of dwg_create from 200,000 points on)
     ScratchScope scope(c);
     uint64_t *k2 = nullptr;
-    const int64_t nhist = (int64_t)256 * nblocks;
-    DWG_CUDA_TRY(c, scratch_get(c, &k2, (2 * n + 2 * nhist + 1) * sizeof(int64_t)));
-    int64_t *v2 = reinterpret_cast<int64_t *>(k2 + n), *hist = v2 + n, *offs = hist + nhist,
+    const int64_t ns = ceil_div(n, 32) * 32, nhist = (int64_t)256 * nblocks;
+    DWG_CUDA_TRY(c, scratch_get(c, &k2, (2 * ns + 2 * nhist + 1) * sizeof(int64_t)));
+    int64_t *v2 = reinterpret_cast<int64_t *>(k2 + ns), *hist = v2 + ns, *offs = hist + nhist,
             *tot = offs + nhist;
     uint64_t *ka = keys, *kb = k2;
     int64_t *va = vals, *vb = v2;
@@ -529,13 +529,14 @@ int build_discretization(Ctx *c, int d)
 
     ScratchScope scope(c);
     auto body = [&]() -> int {
-        DWG_CUDA_TRY(c, scratch_get(c, &flags, n * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &pos, n * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &cnt, n * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &tot, sizeof(int64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &nodes_a, n * sizeof(uint64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &nodes_b, n * sizeof(uint64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &mask, n * sizeof(unsigned)));
+        const int64_t ns = ceil_div(n, 32) * 32;  // 256-byte steps
+        DWG_CUDA_TRY(c, scratch_get(c, &flags, (5 * ns + ns / 2 + 1) * sizeof(int64_t)));
+        pos = flags + ns;
+        cnt = pos + ns;
+        nodes_a = reinterpret_cast<uint64_t *>(cnt + ns);
+        nodes_b = nodes_a + ns;
+        mask = reinterpret_cast<unsigned *>(nodes_b + ns);
+        tot = reinterpret_cast<int64_t *>(mask + ns);
 
         // unique level-l prefixes of the sorted codes, in Morton order
         auto level_nodes = [&](int lvl, uint64_t *out, int64_t &cntn) -> int {
@@ -584,10 +585,11 @@ int build_discretization(Ctx *c, int d)
 
         // distinct corners: sort the 8 corner keys of every leaf, keep the first of each run
         int64_t m = nleaves * 8;
-        DWG_CUDA_TRY(c, scratch_get(c, &keys, m * sizeof(uint64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &slots, m * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &kf, m * sizeof(int64_t)));
-        DWG_CUDA_TRY(c, scratch_get(c, &kp, m * sizeof(int64_t)));
+        const int64_t ms = ceil_div(m, 32) * 32;
+        DWG_CUDA_TRY(c, scratch_get(c, &keys, 4 * ms * sizeof(int64_t)));
+        slots = reinterpret_cast<int64_t *>(keys + ms);
+        kf = slots + ms;
+        kp = kf + ms;
         k_corner_keys<<<(unsigned)ceil_div(m, B), B, 0, c->stream>>>(leaves, nleaves, d, keys,
                                                                       slots);
         int rc = radix_sort_pairs(c, keys, slots, m, 3 * (d + 1));
@@ -700,10 +702,7 @@ __global__ void k_lat_fill(const uint64_t *__restrict__ keys, const int64_t *__r
 
 void free_lattice(Ctx *c)
 {
-    cudaFree(c->d_lat_x);
-    cudaFree(c->d_lat_y);
-    cudaFree(c->d_lat_z);
-    cudaFree(c->d_lat_corner);
+    cudaFree(c->d_lat_x);  // one allocation
     c->d_lat_x = c->d_lat_y = c->d_lat_z = nullptr;
     c->d_lat_corner = nullptr;
     c->lat_tasks = 0;
@@ -719,16 +718,10 @@ static int build_lattice(Ctx *c)
     const unsigned g = (unsigned)ceil_div(m, B), gx = (unsigned)ceil_div(nx, B);
     ScratchScope scope(c);
     uint64_t *keys = nullptr;
-    int64_t *idx = nullptr, *flags = nullptr, *piece = nullptr, *first = nullptr, *tasks = nullptr,
-            *base = nullptr, *tot = nullptr;
-    DWG_CUDA_TRY(c, scratch_get(c, &keys, m * sizeof(uint64_t)));
-    DWG_CUDA_TRY(c, scratch_get(c, &idx, m * sizeof(int64_t)));
-    DWG_CUDA_TRY(c, scratch_get(c, &flags, m * sizeof(int64_t)));
-    DWG_CUDA_TRY(c, scratch_get(c, &piece, m * sizeof(int64_t)));
-    DWG_CUDA_TRY(c, scratch_get(c, &first, nx * sizeof(int64_t)));
-    DWG_CUDA_TRY(c, scratch_get(c, &tasks, nx * sizeof(int64_t)));
-    DWG_CUDA_TRY(c, scratch_get(c, &base, nx * sizeof(int64_t)));
-    DWG_CUDA_TRY(c, scratch_get(c, &tot, 2 * sizeof(int64_t)));
+    const int64_t ms = ceil_div(m, 32) * 32;
+    DWG_CUDA_TRY(c, scratch_get(c, &keys, (4 * ms + 3 * nx + 2) * sizeof(int64_t)));
+    int64_t *idx = reinterpret_cast<int64_t *>(keys + ms), *flags = idx + ms, *piece = flags + ms,
+            *first = piece + ms, *tasks = first + nx, *base = tasks + nx, *tot = base + nx;
     k_lat_keys<<<g, B, 0, c->stream>>>(c->d_corner_keys, m, bits, keys, idx);
     int rc = radix_sort_pairs(c, keys, idx, m, 3 * bits);
     if (rc) return rc;
@@ -740,13 +733,12 @@ static int build_lattice(Ctx *c)
     if ((rc = read_count(c, tot + 1, &nt))) return rc;
     nt = ceil_div(nt, kLatThreads) * kLatThreads;
     auto fill = [&]() -> int {
-        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_x, nt * sizeof(float)));
-        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_y, nt * kLatCols * sizeof(float)));
-        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_z, nt * kLatQ * sizeof(float)));
-        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_corner, nt * kLatQ * sizeof(int)));
-        DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_x, 0, nt * sizeof(float), c->stream));
-        DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_y, 0, nt * kLatCols * sizeof(float), c->stream));
-        DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_z, 0, nt * kLatQ * sizeof(float), c->stream));
+        const size_t words = (1 + kLatCols + kLatQ) * (size_t)nt;
+        DWG_CUDA_TRY(c, cudaMalloc(&c->d_lat_x, (words + kLatQ * nt) * sizeof(float)));
+        c->d_lat_y = c->d_lat_x + nt;
+        c->d_lat_z = c->d_lat_y + kLatCols * nt;
+        c->d_lat_corner = reinterpret_cast<int *>(c->d_lat_z + kLatQ * nt);
+        DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_x, 0, words * sizeof(float), c->stream));
         DWG_CUDA_TRY(c, cudaMemsetAsync(c->d_lat_corner, 0xff, nt * kLatQ * sizeof(int), c->stream));
         k_lat_fill<<<g, B, 0, c->stream>>>(keys, idx, flags, piece, m, bits, first, base,
                                            c->d_corner_pos, nt, c->d_lat_x, c->d_lat_y,
