@@ -889,9 +889,10 @@ int eval_launch(Ctx *c, const float4 *q, int64_t m, bool grad, int nchunks, floa
 }
 
 constexpr int kPGrad = 2;   // query pairs per thread, gradient kernel (batched launches)
-// query pairs per thread, w-only kernel (raw launches): 20,000 sources at
-// 60,001 queries, screened, 675 us a call with 4 pairs, 696 with 2; 60,000
-// sources at 200,000 queries 6.27 ms with 4, 6.10 ms with 2
+// query pairs per thread, w-only kernel (raw launches).  Screened, 4 pairs
+// against 2: 65,536 sources at 1,000 queries 134 us against 97, 2,000 at 2,000
+// 59 against 50, 60,000 at 200,000 6.27 ms against 6.10; 20,000 at 60,001 680 us
+// against 703, 2,000 at 262,144 360 against 371
 constexpr int kPW = 2;
 
 bool corners_on_lattice(const Ctx *c)

@@ -87,6 +87,10 @@ struct EvalParams {
     int screened;
 };
 
+// Streaming multiprocessors of a GB300: the launch sizes that need not follow a
+// problem's size are multiples of it.
+constexpr int kSMs = 152;
+
 // The octree's leaf corners arranged for the exact evaluator of w: a task is
 // a thread's eight corners of one lattice plane x, in four (x, y) columns of
 // two z each (kLatQ; places with no corner repeat the origin).  Tasks are
@@ -598,7 +602,7 @@ cudaError_t launch_init_pca(Ctx *c);
 cudaError_t launch_init_gauss(Ctx *c);
 // scratch doubles of launch_voronoi_weights beside its n areas, and of
 // launch_features
-constexpr int kSumDoubles = 4 + 4 * 304;
+constexpr int kSumDoubles = 4 + 4 * 2 * kSMs;
 // local-Voronoi area weights of the m nearest points into p4.w (scratch: n +
 // kSumDoubles doubles; a_out: n floats in input order, device, or null)
 cudaError_t launch_voronoi_weights(Ctx *c, int m, double *scratch, float *a_out);

@@ -555,7 +555,8 @@ __device__ __forceinline__ void warp_sort(uint64_t &key, int &j, int lane)
 
 // The batch (nk, nj), one pair per lane (~0: none), merged into the sorted
 // list: one pair at a time while few are below the k-th key, else by sorting
-// the batch and a bitonic merge of the two lists' 32 smallest.
+// the batch and a bitonic merge of the two lists' 32 smallest (the line between
+// them at 6, 12, 20 or all 32: within 1 % of each other).
 __device__ __forceinline__ void warp_merge(uint64_t &key, int &j, uint64_t &kth, uint64_t nk, int nj,
                                            int k, int lane)
 {
@@ -698,7 +699,9 @@ constexpr int kShWarps = 4;       // warps per CTA of the kernels that use it
 constexpr int kShStack = 96;      // at most 3 siblings per two levels stay behind
 // A warp stops after this many buckets: the lanes that still need a node (an
 // outlier, a cell far from the points) are searched by a warp each instead,
-// so that one such query does not hold its 31 neighbours.
+// so that one such query does not hold its 31 neighbours.  With 32 buckets the
+// features of a 1M blob take 2.28 ms, with 64 1.77, with 128 1.91 (1 % outliers;
+// 200,000 points 541, 538 and 700 us).
 constexpr int kShBuckets = 64;
 
 struct ShSmem {
@@ -905,7 +908,7 @@ __global__ void __launch_bounds__(32 * kShWarps)
     }
 }
 
-constexpr int kShFarBlocks = 152 * 8;
+constexpr int kShFarBlocks = kSMs * 8;
 
 // A table of the K nearest points, filled for one range of points at a time
 // (at most kKnnRange, so that the table stays small beside a large cloud;
@@ -1019,14 +1022,14 @@ constexpr size_t kAggSmem =
 // finest-cell areas) or goes straight to the points' sums.  At 16 KB a block
 // the tables pay at every size (15M points: 37.4 / 15.4 ms straight to the
 // points' sums, 36.4 / 14.9 with them).
-// Bound: the gathers of the candidates (L1 wavefronts 77 % of their peak)
+// Bound: the gathers of the candidates (L1 wavefronts 81-85 % of their peak)
 // and the integer pipe.  With k_knn_far against the one thread per face with
 // 64-bit keys and its own tree search (random normals / 3rd-16th iteration):
 // 2,000-point sphere 0.63 / 0.19 -> 0.10 / 0.05 ms, 100k torus 2.8 / 1.9 ->
 // 0.33 / 0.18 ms, 1M blob 13.5 / 10.2 -> 5.5 / 3.8 ms, 4M union 29 / 14.5 ->
 // 12.1 / 5.2 ms.  On a small cloud one face's chain of dependent loads (index,
 // point, four at a time) is the time: with the next indices loading beside the
-// points, and 80 registers rather than 64, 94 / 49 -> 84 / 41 us at 2,000
+// points, and six CTAs an SM asked for rather than eight, 94 / 49 -> 84 / 41 us at 2,000
 // points and 12.1 / 5.2 -> 11.5 / 4.9 ms on the 4M union; eight at a time 80 /
 // 37 us but 11.9 / 5.1 ms.
 constexpr int kScanK = 10;
@@ -1218,7 +1221,7 @@ static int far_blocks(int64_t cap, int most)
 {
     return (int)std::min<int64_t>(ceil_div(cap, kFarWarps), most);
 }
-constexpr int kFarBlocks = 152 * 8;      // one cloud
+constexpr int kFarBlocks = kSMs * 8;      // one cloud
 constexpr int kFarBlocksBatch = 64;      // a cloud's part of a batch
 
 // A face whose own search (no candidate list for its cell) runs past
@@ -1507,9 +1510,9 @@ cudaError_t launch_spacing(Ctx *c, int64_t m, float *d_out)
 // centre b (so that mean |p - c|^2 = mean |p - b|^2 - |c - b|^2 loses nothing):
 // per-block sums in a fixed order, then one block over the blocks' sums.  As
 // one block over all points it was a chain of loads: 913 us for 200,000
-// points, 13 us as two launches.  Up to kSumOne points one block is enough.
+// points, 24 us as two launches.  Up to kSumOne points one block is enough.
 constexpr int64_t kSumOne = 512;
-constexpr int kSumBlocks = 304;
+constexpr int kSumBlocks = 2 * kSMs;
 
 __device__ __forceinline__ double block_sum(double v, double *sh)
 {

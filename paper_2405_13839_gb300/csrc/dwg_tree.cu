@@ -877,7 +877,7 @@ constexpr int kItemRecords = 2048;
 
 __host__ __device__ static int item_records(int64_t records, int64_t ng)
 {
-    const int64_t places = (int64_t)152 * 16;
+    const int64_t places = (int64_t)kSMs * 16;
     const int64_t items = records / kItemRecords + ng / 2;
     return items < 4 * places ? kItemRecords / 4 : items < 8 * places ? kItemRecords / 2
                                                                      : kItemRecords;
