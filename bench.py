@@ -144,6 +144,20 @@ def profiled_bytes_per_interaction(which):
     return None
 
 
+def profiled_lattice_bytes(corners):
+    """DRAM bytes of one corner launch of the exact path from the committed ncu
+    summary (None when absent or of another cloud)."""
+    got = {}
+    try:
+        for line in open(os.path.join(ROOT, "profiles", "gwn_lattice_torus100k.md")):
+            for key in ("corners:", "dram_bytes_per_launch:"):
+                if line.startswith(key):
+                    got[key] = int(line.split(":")[1])
+    except OSError:
+        return None
+    return got.get("dram_bytes_per_launch:") if got.get("corners:") == corners else None
+
+
 def measured_peaks():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -530,8 +544,10 @@ def run_ours(args, rank, world, local):
             work = float(n) * n
             what = "wg"
         achieved = work / (kms[dom] / 1e3)
-        traffic_basis = "not captured for this cloud (profiles/gwn_lattice_torus100k.md: 34 MB)"
-        traffic = None
+        # DRAM bytes of the launch as captured by ncu (the torus cloud's corners)
+        traffic = profiled_lattice_bytes(nc) if dom == "eval_corners" else None
+        traffic_basis = ("ncu dram bytes of k_gwn_lattice (profiles/gwn_lattice_torus100k.md)"
+                         if traffic is not None else "not captured for this launch")
     else:
         # Barnes-Hut: the dominant of the two tree launches (w and grad at the
         # points, w at the corners), its evaluations performed (counted on the
