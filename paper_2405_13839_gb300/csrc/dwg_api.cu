@@ -74,60 +74,96 @@ cudaError_t scratch_get(Ctx *c, void **p, size_t bytes)
 {
     Scratch &S = *c->scratch;
     const size_t b = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
+    const bool limited = S.limit != SIZE_MAX;
     *p = nullptr;
-    // the smallest free block that holds it, none far too large (under a limit
-    // none larger at all: what a call can do would depend on the calls before)
-    const size_t most = S.limit == SIZE_MAX ? 4 * b + ((size_t)1 << 20) : b;
-    ScratchBlock *best = nullptr;
-    for (ScratchBlock &k : S.blocks)
-        if (!k.scope && k.size >= b && k.size <= most && (!best || k.size < best->size)) best = &k;
-    if (best) {
-        best->scope = S.depth;
-        *p = best->p;
-        return cudaSuccess;
+    // The smallest free piece that holds it; what it does not need stays free.
+    // Under a limit a piece of its size only: what a call can do would depend on
+    // the calls before it.
+    size_t best = S.pieces.size();
+    for (size_t i = 0; i < S.pieces.size(); ++i) {
+        const ScratchPiece &k = S.pieces[i];
+        if (!k.scope && (limited ? k.size == b : k.size >= b) &&
+            (best == S.pieces.size() || k.size < S.pieces[best].size))
+            best = i;
     }
-    auto take = [&]() {
-        size_t held = 0;
-        for (const ScratchBlock &k : S.blocks) held += k.size;
-        if (b > S.limit || held > S.limit - b) return cudaErrorMemoryAllocation;
-        const cudaError_t e = cudaMalloc(p, b);
-        if (e != cudaSuccess) cudaGetLastError();  // reported here, not by the next launch
-        return e;
-    };
-    cudaError_t e = take();
-    if (e == cudaErrorMemoryAllocation && !S.blocks.empty()) {
-        scratch_trim(c, 0);  // what the handle keeps may be what is missing
-        e = take();
+    if (best == S.pieces.size()) {
+        const size_t seg = limited ? b : std::max(b, kScratchSegment);
+        char *q = nullptr;
+        auto take = [&]() {
+            size_t held = 0;
+            for (const ScratchPiece &k : S.pieces) held += k.size;
+            if (seg > S.limit || held > S.limit - seg) return cudaErrorMemoryAllocation;
+            const cudaError_t e = cudaMalloc(&q, seg);
+            if (e != cudaSuccess) cudaGetLastError();  // reported here, not by the next launch
+            return e;
+        };
+        cudaError_t e = take();
+        if (e == cudaErrorMemoryAllocation && !S.pieces.empty()) {
+            scratch_trim(c, 0);  // what the handle keeps may be what is missing
+            e = take();
+        }
+        if (e != cudaSuccess) return e;
+        best = S.pieces.size();
+        S.pieces.push_back({q, seg, 0, true});
     }
-    if (e == cudaSuccess) S.blocks.push_back({*p, b, S.depth});
-    return e;
+    if (S.pieces[best].size > b) {
+        const ScratchPiece rest{S.pieces[best].p + b, S.pieces[best].size - b, 0, false};
+        S.pieces[best].size = b;
+        S.pieces.insert(S.pieces.begin() + best + 1, rest);
+    }
+    S.pieces[best].scope = S.depth;
+    *p = S.pieces[best].p;
+    return cudaSuccess;
 }
 
-// frees free blocks, the largest first, until at most `keep` bytes are held
+cudaError_t scratch_parts(Ctx *c, std::initializer_list<ScratchPart> parts)
+{
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    size_t total = 0;
+    for (const ScratchPart &q : parts) total += up(q.bytes);
+    char *piece = nullptr;
+    const cudaError_t e = scratch_get(c, &piece, total);
+    if (e != cudaSuccess) return e;
+    for (const ScratchPart &q : parts) {
+        *q.p = piece;
+        piece += up(q.bytes);
+    }
+    return cudaSuccess;
+}
+
+// frees free segments, the largest first, until at most `keep` bytes are held
 // (cudaFree waits for the device)
 void scratch_trim(Ctx *c, size_t keep)
 {
-    Scratch &S = *c->scratch;
+    std::vector<ScratchPiece> &P = c->scratch->pieces;
     size_t total = 0;
-    for (const ScratchBlock &k : S.blocks) total += k.size;
+    for (const ScratchPiece &k : P) total += k.size;
     while (total > keep) {
-        auto big = S.blocks.end();
-        for (auto k = S.blocks.begin(); k != S.blocks.end(); ++k)
-            if (!k->scope && (big == S.blocks.end() || k->size > big->size)) big = k;
-        if (big == S.blocks.end()) break;
-        total -= big->size;
-        cudaFree(big->p);
-        S.blocks.erase(big);
+        size_t big = P.size();
+        for (size_t i = 0; i < P.size(); ++i)
+            if (P[i].head && !P[i].scope && (i + 1 == P.size() || P[i + 1].head) &&
+                (big == P.size() || P[i].size > P[big].size))
+                big = i;
+        if (big == P.size()) break;
+        total -= P[big].size;
+        cudaFree(P[big].p);
+        P.erase(P.begin() + big);
     }
 }
 
 ScratchScope::~ScratchScope()
 {
     Scratch &S = *c->scratch;
-    for (ScratchBlock &k : S.blocks)
+    size_t n = 0;  // pieces kept, free neighbours of a segment as one
+    for (ScratchPiece k : S.pieces) {
         if (k.scope == S.depth) k.scope = 0;
-    --S.depth;
-    scratch_trim(c, S.keep);
+        if (n > 0 && !k.head && !k.scope && !S.pieces[n - 1].scope)
+            S.pieces[n - 1].size += k.size;
+        else
+            S.pieces[n++] = k;
+    }
+    S.pieces.resize(n);
+    if (--S.depth == 0) scratch_trim(c, S.keep);
 }
 }  // namespace dwg
 
@@ -723,7 +759,8 @@ void dwg_destroy(dwg_handle h)
                     h->d_delta2, h->d_src16, h->d_cell_off, h->d_cell_idx, h->d_far_q,
                     h->d_defer, h->d_tree_dmax};
     for (void *p : bufs) cudaFree(p);
-    for (ScratchBlock &k : h->own_scratch.blocks) cudaFree(k.p);
+    for (ScratchPiece &k : h->own_scratch.pieces)
+        if (k.head) cudaFree(k.p);
     free_lattice(h);
     free_lists(h->lists_p);
     free_lists(h->lists_c);

@@ -182,9 +182,8 @@ int scan_i64(Ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *d_tota
         k_scan_block<<<1, kScanBlock, 0, c->stream>>>(in, out, n, nullptr);
     } else {
         ScratchScope scope(c);
-        int64_t *sums = nullptr;
-        DWG_CUDA_TRY(c, scratch_get(c, &sums, (2 * nb + 1) * sizeof(int64_t)));
-        int64_t *soffs = sums + nb, *stot = soffs + nb;
+        int64_t *sums = nullptr, *soffs = nullptr, *stot = nullptr;
+        DWG_CUDA_TRY(c, scratch_parts(c, {{&sums, nb}, {&soffs, nb}, {&stot, 1}}));
         k_scan_block<<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, out, n, sums);
         int rc = scan_i64(c, sums, soffs, nb, stot);
         if (rc) return rc;
@@ -264,14 +263,11 @@ int radix_sort_pairs(Ctx *c, uint64_t *keys, int64_t *vals, int64_t n, int key_b
 {
     if (n <= 1) return DWG_OK;
     int nblocks = (int)ceil_div(n, kSortItems);
-    // one block: a new handle's sort allocates once (five allocations and their
-    // frees were 40-60 us of dwg_create from 200,000 points on)
     ScratchScope scope(c);
     uint64_t *k2 = nullptr;
-    const int64_t ns = ceil_div(n, 32) * 32, nhist = (int64_t)256 * nblocks;
-    DWG_CUDA_TRY(c, scratch_get(c, &k2, (2 * ns + 2 * nhist + 1) * sizeof(int64_t)));
-    int64_t *v2 = reinterpret_cast<int64_t *>(k2 + ns), *hist = v2 + ns, *offs = hist + nhist,
-            *tot = offs + nhist;
+    int64_t *v2 = nullptr, *hist = nullptr, *offs = nullptr, *tot = nullptr;
+    const int64_t nhist = (int64_t)256 * nblocks;
+    DWG_CUDA_TRY(c, scratch_parts(c, {{&k2, n}, {&v2, n}, {&hist, nhist}, {&offs, nhist}, {&tot, 1}}));
     uint64_t *ka = keys, *kb = k2;
     int64_t *va = vals, *vb = v2;
     int passes = (key_bits + 7) / 8;
@@ -529,14 +525,8 @@ int build_discretization(Ctx *c, int d)
 
     ScratchScope scope(c);
     auto body = [&]() -> int {
-        const int64_t ns = ceil_div(n, 32) * 32;  // 256-byte steps
-        DWG_CUDA_TRY(c, scratch_get(c, &flags, (5 * ns + ns / 2 + 1) * sizeof(int64_t)));
-        pos = flags + ns;
-        cnt = pos + ns;
-        nodes_a = reinterpret_cast<uint64_t *>(cnt + ns);
-        nodes_b = nodes_a + ns;
-        mask = reinterpret_cast<unsigned *>(nodes_b + ns);
-        tot = reinterpret_cast<int64_t *>(mask + ns);
+        DWG_CUDA_TRY(c, scratch_parts(c, {{&flags, n}, {&pos, n}, {&cnt, n}, {&tot, 1},
+                                          {&nodes_a, n}, {&nodes_b, n}, {&mask, n}}));
 
         // unique level-l prefixes of the sorted codes, in Morton order
         auto level_nodes = [&](int lvl, uint64_t *out, int64_t &cntn) -> int {
@@ -585,11 +575,7 @@ int build_discretization(Ctx *c, int d)
 
         // distinct corners: sort the 8 corner keys of every leaf, keep the first of each run
         int64_t m = nleaves * 8;
-        const int64_t ms = ceil_div(m, 32) * 32;
-        DWG_CUDA_TRY(c, scratch_get(c, &keys, 4 * ms * sizeof(int64_t)));
-        slots = reinterpret_cast<int64_t *>(keys + ms);
-        kf = slots + ms;
-        kp = kf + ms;
+        DWG_CUDA_TRY(c, scratch_parts(c, {{&keys, m}, {&slots, m}, {&kf, m}, {&kp, m}}));
         k_corner_keys<<<(unsigned)ceil_div(m, B), B, 0, c->stream>>>(leaves, nleaves, d, keys,
                                                                       slots);
         int rc = radix_sort_pairs(c, keys, slots, m, 3 * (d + 1));
@@ -718,10 +704,10 @@ static int build_lattice(Ctx *c)
     const unsigned g = (unsigned)ceil_div(m, B), gx = (unsigned)ceil_div(nx, B);
     ScratchScope scope(c);
     uint64_t *keys = nullptr;
-    const int64_t ms = ceil_div(m, 32) * 32;
-    DWG_CUDA_TRY(c, scratch_get(c, &keys, (4 * ms + 3 * nx + 2) * sizeof(int64_t)));
-    int64_t *idx = reinterpret_cast<int64_t *>(keys + ms), *flags = idx + ms, *piece = flags + ms,
-            *first = piece + ms, *tasks = first + nx, *base = tasks + nx, *tot = base + nx;
+    int64_t *idx = nullptr, *flags = nullptr, *piece = nullptr, *first = nullptr, *tasks = nullptr,
+            *base = nullptr, *tot = nullptr;
+    DWG_CUDA_TRY(c, scratch_parts(c, {{&keys, m}, {&idx, m}, {&flags, m}, {&piece, m}, {&first, nx},
+                                      {&tasks, nx}, {&base, nx}, {&tot, 2}}));
     k_lat_keys<<<g, B, 0, c->stream>>>(c->d_corner_keys, m, bits, keys, idx);
     int rc = radix_sort_pairs(c, keys, idx, m, 3 * bits);
     if (rc) return rc;

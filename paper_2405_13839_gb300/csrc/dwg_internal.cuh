@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -244,23 +245,26 @@ struct TreeLists {
     bool valid = false;
 };
 
-// Scratch of the calls on a handle.  A call's device buffers are blocks that
-// the handle keeps when the call ends, so that a call repeated at its size
-// allocates nothing (cudaMalloc and cudaFree of a call's buffers cost tens to
-// hundreds of microseconds, and cudaFree waits for the device); together at
-// most `keep` bytes between calls, all given back with the handle.  A call
-// that would hold more than `limit` is told what cudaMalloc says when memory
-// is short (dwg_set_scratch).
+// Scratch of the calls on a handle.  A call's device buffers are pieces of
+// segments (one cudaMalloc each) that the handle keeps when the call ends, so
+// that a call repeated at its size allocates nothing (cudaMalloc and cudaFree of
+// a call's buffers cost tens to hundreds of microseconds, and cudaFree waits for
+// the device), and a new handle's calls share what its build took; together at
+// most `keep` bytes between calls, all given back with the handle.  A call that
+// would hold more than `limit` is told what cudaMalloc says when memory is short
+// (dwg_set_scratch).
 constexpr size_t kScratchKeep = (size_t)256 << 20;
 // what of it stays after a build, whose sizes the calls that follow do not need
 constexpr size_t kScratchKeepBuilt = (size_t)16 << 20;
-struct ScratchBlock {
-    void *p;
+constexpr size_t kScratchSegment = (size_t)256 << 10;  // at least so much a segment
+struct ScratchPiece {
+    char *p;
     size_t size;
     int scope;  // nesting depth of the scope that holds it, 0: free
+    bool head;  // the first piece of its segment
 };
 struct Scratch {
-    std::vector<ScratchBlock> blocks;
+    std::vector<ScratchPiece> pieces;  // segment by segment, in address order
     int depth = 0;
     size_t keep = kScratchKeep, limit = SIZE_MAX;
 };
@@ -517,8 +521,8 @@ cudaError_t launch_reduce_w_raw(const float *part, int nchunks, int64_t m, float
                                 cudaStream_t s);
 
 // dwg_api.cu
-// a block of the handle's scratch, held until the innermost ScratchScope ends
-// (the work of a handle is ordered on its stream, so a block handed out again
+// a piece of the handle's scratch, held until the innermost ScratchScope ends
+// (the work of a handle is ordered on its stream, so a piece handed out again
 // is only written after what read it before)
 cudaError_t scratch_get(Ctx *c, void **p, size_t bytes);
 template <class T>
@@ -526,6 +530,16 @@ inline cudaError_t scratch_get(Ctx *c, T **p, size_t bytes)
 {
     return scratch_get(c, reinterpret_cast<void **>(p), bytes);
 }
+// several buffers held together, as one piece
+struct ScratchPart {
+    void **p;
+    size_t bytes;
+    template <class T>
+    ScratchPart(T **p_, int64_t count) : p(reinterpret_cast<void **>(p_)), bytes(count * sizeof(T))
+    {
+    }
+};
+cudaError_t scratch_parts(Ctx *c, std::initializer_list<ScratchPart> parts);
 void scratch_trim(Ctx *c, size_t keep);
 struct ScratchScope {
     Ctx *c;

@@ -1463,27 +1463,13 @@ __global__ void __launch_bounds__(1024)
 // here the lists are cut into items of at most kItemRecords records and
 // evaluated by k_tree_eval_lists.  300,000 sources, w and grad w at 110,592
 // lattice queries: 1,392 -> 630 us (walks 144, evaluation 473).  In ranges of
-// groups.  The lists, items and partial sums of a range are one block of
-// scratch; a range for which there is no such block, or whose lists would
-// take more than kCallLists bytes (queries in no order open the whole tree),
+// groups.  A range whose lists, items and partial sums find no scratch, or
+// would take more than kCallLists bytes (queries in no order open the whole tree),
 // is walked: in parts of 192 MB, 1M sources at 1.5M unordered queries took
 // 2,150 ms against 1,455 (a part has too few groups for the list walks).
 // Ranges one after the other are walked in one launch: the two of those
 // queries by themselves 1,495 ms, each with its own last groups to wait for.
-constexpr size_t kCallLists = (size_t)1 << 30;
-
-// the block of a range's lists and its work items of item_bytes each
-struct CallLists {
-    size_t near_at, items_at, part_at, bytes;
-    CallLists(int64_t nfar, int64_t nnear, int64_t items, size_t item_bytes)
-    {
-        auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-        near_at = up(nfar * sizeof(int));
-        items_at = near_at + up(nnear * sizeof(int));
-        part_at = items_at + up(items * sizeof(int2));
-        bytes = part_at + items * item_bytes;
-    }
-};
+constexpr double kCallLists = 1024.0 * 1024.0 * 1024.0;
 
 template <bool GRAD, bool SCREENED>
 static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, int64_t stride)
@@ -1500,8 +1486,6 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
         return DWG_OK;
     }
     DWG_CUDA_TRY(c, e);
-    char *block = nullptr;
-    size_t held = 0;       // bytes of block
     int64_t walk_g = all;  // groups from here to the current range are still to be walked
     auto walk_to = [&](int64_t g1) {
         const int64_t g = walk_g;
@@ -1530,27 +1514,23 @@ static int eval_call_lists_t(Ctx *c, const float4 *q, int64_t m, float *part, in
             c->err = "tree lists: traversal stack overflow";
             return DWG_ERR_CUDA;
         }
-        const CallLists L(ht[0], ht[1], ht[2], item_bytes);
-        bool room = L.bytes <= held;
-        if (!room && L.bytes <= kCallLists) {
-            char *larger = nullptr;
-            e = scratch_get(c, &larger, L.bytes);
-            if (e != cudaErrorMemoryAllocation) {
-                DWG_CUDA_TRY(c, e);
-                block = larger;
-                held = L.bytes;
-                room = true;
-            }
-        }
-        if (!room) {
+        const double need = sizeof(int) * ((double)ht[0] + (double)ht[1]) +
+                            (double)ht[2] * (sizeof(int2) + item_bytes);
+        ScratchScope range(c);
+        int *far_ids = nullptr, *near_ids = nullptr;
+        int2 *items = nullptr;
+        float *ipart = nullptr;
+        e = need <= kCallLists ? cudaSuccess : cudaErrorMemoryAllocation;
+        if (e == cudaSuccess) e = scratch_get(c, &far_ids, ht[0] * sizeof(int));
+        if (e == cudaSuccess) e = scratch_get(c, &near_ids, ht[1] * sizeof(int));
+        if (e == cudaSuccess) e = scratch_get(c, &items, ht[2] * sizeof(int2));
+        if (e == cudaSuccess) e = scratch_get(c, &ipart, ht[2] * item_bytes);
+        if (e == cudaErrorMemoryAllocation) {
             walk_g = std::min(walk_g, g0);
             continue;
         }
+        DWG_CUDA_TRY(c, e);
         DWG_CUDA_TRY(c, walk_to(g0));
-        int *far_ids = reinterpret_cast<int *>(block);
-        int *near_ids = reinterpret_cast<int *>(block + L.near_at);
-        int2 *items = reinterpret_cast<int2 *>(block + L.items_at);
-        float *ipart = reinterpret_cast<float *>(block + L.part_at);
         k_tree_lists<true, kWalkW><<<blocks, 32 * list_warps(kWalkW), 0, c->stream>>>(
             qr, mr, c->d_tree_rec, c->tree_levels, far_off, near_off, far_ids, near_ids, c->d_err);
         const int irec = (int)ht[3];
