@@ -36,11 +36,13 @@
  *   - All GPU work is issued on the handle's stream (dwg_set_stream), and
  *     every function returns only after its results are in the caller's
  *     buffers.
- *   - Device arrays are read and written in place, behind the work that the
- *     caller has queued on the default stream (and on streams ordered with
- *     it) or on the handle's stream.  Work on any other stream is not waited
- *     for: synchronise it first, or pass it to dwg_set_stream.  Calls may run
- *     while another thread captures a graph; they neither join nor break it.
+ *   - Device arrays are read and written behind the work that the caller has
+ *     queued on the default stream (and on streams ordered with it) or on the
+ *     handle's stream, most of them in place.  Work on any other stream is not
+ *     waited for: synchronise it first, or pass it to dwg_set_stream.  (The
+ *     calls without a handle run on the stream they are given.)  Calls may run
+ *     while another thread captures a graph in the relaxed or thread-local
+ *     mode; they neither join nor break that capture.
  *   - A handle is not thread-safe; distinct handles are independent.
  */
 #ifndef DWG_H

@@ -221,16 +221,20 @@ static bool is_host_ptr(const void *p)
     return a.type == cudaMemoryTypeUnregistered || a.type == cudaMemoryTypeHost;
 }
 
+static cudaError_t join_caller(Ctx *c);
+
 // Copy bytes between a caller buffer (host memory, or device memory of any
 // GPU) and the handle's device memory; the unified address space tells the
 // copy which kind it is.
 static int upload(Ctx *c, void *dst, const void *src, size_t bytes)
 {
+    if (is_device_ptr(src)) DWG_CUDA_TRY(c, join_caller(c));
     DWG_CUDA_TRY(c, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, c->stream));
     return DWG_OK;
 }
 static int download(Ctx *c, void *dst, const void *src, size_t bytes)
 {
+    if (is_device_ptr(dst)) DWG_CUDA_TRY(c, join_caller(c));
     DWG_CUDA_TRY(c, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, c->stream));
     return DWG_OK;
 }
@@ -241,7 +245,7 @@ static bool kernel_ptr(const void *p, size_t size)
 {
     return reinterpret_cast<uintptr_t>(p) % size == 0 && is_device_ptr(p);
 }
-// Before a call's kernels touch a caller's device arrays in place, the handle's
+// Before a call's kernels or copies touch a caller's device arrays, the handle's
 // stream waits for the work already queued on the default stream (and so on
 // every stream ordered with it): callers fill and reuse such arrays there, and
 // the handle's stream is not ordered after it.  Not by waiting for the whole
@@ -1140,7 +1144,9 @@ int dwg_extract_level_set(dwg_handle h, float *tri_out, int64_t cap, int64_t *co
         }
         if (!tri_out || (int64_t)nt > cap || nt == 0) return check_device_err(h);
         float *dst = tri_out;
-        if (!is_device_ptr(tri_out)) {
+        if (is_device_ptr(tri_out)) {
+            DWG_CUDA_TRY(h, join_caller(h));
+        } else {
             DWG_CUDA_TRY(h, scratch_get(h, &d_tri, nt * 9 * sizeof(float)));
             dst = d_tri;
         }
@@ -1251,6 +1257,7 @@ int dwg_set_init(dwg_handle h, int mode, uint64_t seed, const float *normals)
         if (!normals) return fail(h, DWG_ERR_INVALID, "DWG_INIT_LEARNED needs the parameters");
         if (!h->d_mlp_params)
             DWG_CUDA_TRY(h, cudaMalloc(&h->d_mlp_params, kMlpParamCount * sizeof(float)));
+        ScratchScope scope(h);
         int rc = upload(h, h->d_mlp_params, normals, kMlpParamCount * sizeof(float));
         if (rc) return rc;
         DWG_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
@@ -1594,6 +1601,7 @@ int dwg_get_leaves(dwg_handle h, int64_t *leaves_out, int64_t cap, int64_t *coun
     if (!h || !count) return DWG_ERR_INVALID;
     if (batch_refused(h)) return DWG_ERR_STATE;
     cudaSetDevice(h->device);
+    ScratchScope scope(h);
     int rc = build_discretization(h, h->depth);
     if (rc) return rc;
     *count = h->nleaves;
@@ -1632,6 +1640,7 @@ int dwg_get_corners(dwg_handle h, int64_t *keys_out, int64_t cap, int64_t *count
     if (!h || !count) return DWG_ERR_INVALID;
     if (batch_refused(h)) return DWG_ERR_STATE;
     cudaSetDevice(h->device);
+    ScratchScope scope(h);
     int rc = build_discretization(h, h->depth);
     if (rc) return rc;
     *count = h->ncorners;
@@ -1660,6 +1669,7 @@ int dwg_get_tree(dwg_handle h, int64_t cap, int64_t *nodes_out, int *leaf_out, i
     if (!h || !nodes_out || !leaf_out) return DWG_ERR_INVALID;
     if (h->is_batch) return fail(h, DWG_ERR_STATE, "read the tree of a cloud handle");
     cudaSetDevice(h->device);
+    ScratchScope scope(h);
     int rc;
     if ((rc = build_tree(h)) || (rc = tree_records(h))) return rc;
     const int64_t nn = (int64_t)2 << h->tree_levels;
