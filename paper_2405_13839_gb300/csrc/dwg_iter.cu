@@ -1510,7 +1510,7 @@ cudaError_t launch_spacing(Ctx *c, int64_t m, float *d_out)
 // centre b (so that mean |p - c|^2 = mean |p - b|^2 - |c - b|^2 loses nothing):
 // per-block sums in a fixed order, then one block over the blocks' sums.  As
 // one block over all points it was a chain of loads: 913 us for 200,000
-// points, 24 us as two launches.  Up to kSumOne points one block is enough.
+// points, 23 us as two launches.  Up to kSumOne points one block is enough.
 constexpr int64_t kSumOne = 512;
 constexpr int kSumBlocks = 2 * kSMs;
 
